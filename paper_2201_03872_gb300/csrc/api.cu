@@ -82,8 +82,7 @@ int upload_mu(tmamg_ctx* ctx, const double* mu, int nsys) {
                     "upload mu");
 }
 
-static int ensure_scratch(tmamg_ctx* ctx, size_t bytes) {
-  if (bytes <= ctx->scratch_bytes) return TMAMG_OK;
+static int grow_scratch(tmamg_ctx* ctx, size_t bytes) {
   for (int i = 0; i < 2; ++i) {
     if (ctx->scratch[i]) cudaFree(ctx->scratch[i]);
     ctx->scratch[i] = nullptr;
@@ -95,6 +94,11 @@ static int ensure_scratch(tmamg_ctx* ctx, size_t bytes) {
   }
   ctx->scratch_bytes = bytes;
   return TMAMG_OK;
+}
+
+static int ensure_scratch(tmamg_ctx* ctx, size_t bytes) {
+  if (bytes <= ctx->scratch_bytes) return TMAMG_OK;
+  return with_optional_memory(ctx, [&] { return grow_scratch(ctx, bytes); });
 }
 
 }  // namespace tmamg
@@ -166,6 +170,7 @@ int tmamg_create(const int L[4], int bc_t, void* cuda_stream, tmamg_ctx** out) {
     tmamg_destroy(ctx);
     return rc;
   }
+  alloc_fixed(ctx->g);  // optional copies of the operator
   *out = ctx;
   return TMAMG_OK;
 }
@@ -181,6 +186,7 @@ int tmamg_destroy(tmamg_ctx* ctx) {
   cudaFree(ctx->U32);
   cudaFree(ctx->C64);
   cudaFree(ctx->C32);
+  free_fixed(ctx->g);
   cudaFree(ctx->mu_dev);
   cudaFree(ctx->eps_dev);
   for (int i = 0; i < 2; ++i) cudaFree(ctx->scratch[i]);
@@ -214,6 +220,7 @@ int tmamg_load_gauge(tmamg_ctx* ctx, const double* U, int on_device) {
     src = tmp;
   }
   launch_convert_gauge(ctx->g, src, ctx->U64, ctx->U32, ctx->stream);
+  launch_fixed_links(ctx->g, ctx->U64, ctx->stream);
   int rc = check_cuda(ctx, cudaGetLastError(), "convert_gauge launch");
   if (tmp) {
     cudaStreamSynchronize(ctx->stream);
@@ -233,6 +240,7 @@ int tmamg_set_operator(tmamg_ctx* ctx, double kappa, double c_sw) {
   ctx->kappa = kappa;
   ctx->c_sw = c_sw;
   launch_build_clover(ctx->g, ctx->U64, kappa, c_sw, ctx->C64, ctx->C32, ctx->stream);
+  launch_fixed_clover(ctx->g, ctx->C64, ctx->stream);
   int rc = check_cuda(ctx, cudaGetLastError(), "build_clover launch");
   if (rc) return rc;
   ctx->have_op = true;

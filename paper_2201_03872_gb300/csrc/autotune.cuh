@@ -23,14 +23,24 @@ int tune_lookup(const char* family, int64_t key);
 // each), records the fastest for (family, key) and returns it
 int tune_run(const char* family, int64_t key, int nvar, const std::function<void(int)>& launch, cudaStream_t st);
 
-// the variant to use: tuned on first use when tuning is on, else variant 0
-inline int tune_pick(const char* family, int64_t key, int nvar, const std::function<void(int)>& launch,
-                     cudaStream_t st) {
+// the variant to use: the forced one, else the one tuned on first use when tuning is on; tuning (which
+// runs every variant on this call's data) only when `may_tune`, i.e. when the launch is repeatable
+inline int tune_variant(const char* family, int64_t key, int nvar, bool may_tune,
+                        const std::function<void(int)>& launch, cudaStream_t st) {
   const int f = tune_forced();
   if (f >= 0) return f < nvar ? f : 0;
   if (!autotune_on() || nvar < 2) return 0;
   const int v = tune_lookup(family, key);
-  return v >= 0 ? v : tune_run(family, key, nvar, launch, st);
+  if (v >= 0) return v;
+  return may_tune ? tune_run(family, key, nvar, launch, st) : 0;
+}
+
+// largest divisor of nt that keeps a CTA of bx x ty threads at <= maxthreads threads
+inline int pick_ty(int nt, int bx, int maxthreads) {
+  int best = 1;
+  for (int d = 1; d * bx <= maxthreads && d <= nt; ++d)
+    if (nt % d == 0) best = d;
+  return best;
 }
 
 }  // namespace tmamg

@@ -13,6 +13,7 @@
 #include <vector>
 
 #include "../../include/tmamg.h"
+#include "fixed64.cuh"
 
 namespace tmamg {
 
@@ -28,6 +29,7 @@ struct Geom {
   int L[4];     // x, y, z, t
   int64_t V;
   int bc_t;
+  FixedOp fx;  // fixed-point copies of the FP64 links and clover for the FP64 stencil (null if they do not fit)
 };
 
 __host__ __device__ inline void site_coords(int64_t s, const int* L, int* c) {
@@ -118,9 +120,30 @@ int set_err(tmamg_ctx* ctx, int code, const std::string& msg);
 int check_cuda(tmamg_ctx* ctx, cudaError_t e, const char* what);
 int upload_mu(tmamg_ctx* ctx, const double* mu, int nsys);
 
+// runs f; if it found no device memory while the context holds optional copies of the operator, gives
+// those back (the FP64 stencil then runs in FP64 arithmetic) and runs it again. f leaves nothing half
+// allocated behind when it returns TMAMG_ERR_OOM.
+void free_fixed(Geom& g);
+template <class F>
+int with_optional_memory(tmamg_ctx* ctx, F f) {
+  int rc = f();
+  if (rc == TMAMG_ERR_OOM && ctx->g.fx.U) {
+    cudaStreamSynchronize(ctx->stream);
+    free_fixed(ctx->g);
+    cudaGetLastError();
+    rc = f();
+  }
+  return rc;
+}
+
 // kernels launched from other translation units
 void launch_build_clover(const Geom& g, const double2* U64, double kappa, double c_sw, double* C64, float* C32,
                          cudaStream_t st);
+// the fixed-point copies (dirac64.cu): allocation (optional: without them the FP64 stencil runs in FP64
+// arithmetic), release, and conversion from the FP64 links and clover
+int alloc_fixed(Geom& g);
+void launch_fixed_links(const Geom& g, const double2* U64, cudaStream_t st);
+void launch_fixed_clover(const Geom& g, const double* C64, cudaStream_t st);
 void launch_convert_gauge(const Geom& g, const double* Uin, double2* U64, float2* U32, cudaStream_t st);
 // eps (optional): the non-degenerate doublet form, per doublet splittings (device): FP32 tiles hold the
 // flavours u, d of one doublet (eps per tile), FP64 tiles 2p and 2p + 1 those of doublet p

@@ -233,17 +233,17 @@ void launch_build_clover(const Geom& g, const double2* U64, double kappa, double
                                                                        c_sw, C64, C32); TM_COUNT();
 }
 
-// FP32: 192-thread CTAs, two per SM, up to 170 registers (no spills); FP64: 256 threads, one per SM
-// RES: residual form y = b - D x (b = bsub, tile tile / nshift), else y = D x (bsub unused).
+// The FP32 form (dirac64.cu holds the FP64 one): 192-thread CTAs, two per SM, up to 170 registers.
+// RES: residual form y = b - D x (b = bsub, tile for tile), else y = D x (bsub unused).
 // MAXT, MINB: the launch variant's largest CTA and the CTAs per SM it is compiled for (which sets the
 // register budget); every variant does the same per-thread arithmetic.
-template <typename real, int T, int BX, bool RES, int MAXT, int MINB>
-__global__ void __launch_bounds__(MAXT, MINB) dirac_kernel(const typename LinkT<real>::t* __restrict__ U,
-                                                    const real* __restrict__ C, const real* __restrict__ x,
-                                                    real* y, const double* __restrict__ mu, int nsys,
-                                                    int ntile, int Lx, int Ly, int Lz, int Lt, real bc_t,
-                                                    const real* bsub, int nshift,
-                                                    const double* __restrict__ eps) {
+template <int BX, bool RES, int MAXT, int MINB>
+__global__ void __launch_bounds__(MAXT, MINB) dirac_kernel(const float2* __restrict__ U, const float* __restrict__ C,
+                                                           const float* __restrict__ x, float* y,
+                                                           const double* __restrict__ mu, int nsys, int ntile, int Lx,
+                                                           int Ly, int Lz, int Lt, float bc_t, const float* bsub,
+                                                           const double* __restrict__ eps) {
+  constexpr int T = 2;
   // y is not restrict-qualified: the residual form may run in place (bsub == y), every thread
   // reading b at its own site before it writes y there; x never overlaps y
   const int64_t V = (int64_t)Lx * Ly * Lz * Lt;
@@ -254,210 +254,100 @@ __global__ void __launch_bounds__(MAXT, MINB) dirac_kernel(const typename LinkT<
   int c[4];
   site_coords(s, L, c);
   const int64_t tstride = (int64_t)12 * V * 2 * T;
-  const real* xt = x + tile * tstride;
+  const float* xt = x + tile * tstride;
   const int64_t strides[4] = {1, (int64_t)Lx, (int64_t)Lx * Ly, (int64_t)Lx * Ly * Lz};
-  if constexpr (sizeof(real) == 4) {
-    // packed FP32x2 arithmetic over the tile's two systems
-    Spinor2 acc;
+  // packed FP32x2 arithmetic over the tile's two systems
+  Spinor2 acc;
+#pragma unroll
+  for (int k = 0; k < 12; ++k) {
+    acc.c[k].re = make_float2(0.f, 0.f);
+    acc.c[k].im = make_float2(0.f, 0.f);
+  }
+  // software pipeline over the eight hops: the neighbour spinor of hop k + 1 is loaded before
+  // the colour multiply of hop k, so its latency overlaps that arithmetic (loading the site's own
+  // spinor for the local term the same way measured slower)
+  int64_t nb[8];
+#pragma unroll
+  for (int nu = 0; nu < 4; ++nu) {
+    nb[2 * nu] = c[nu] + 1 < L[nu] ? s + strides[nu] : s - (int64_t)(L[nu] - 1) * strides[nu];
+    nb[2 * nu + 1] = c[nu] > 0 ? s - strides[nu] : s + (int64_t)(L[nu] - 1) * strides[nu];
+  }
+  const float pf = c[3] == Lt - 1 ? bc_t : 1.f, pb = c[3] == 0 ? bc_t : 1.f;
+  Raw2 raw;
+  CV2 h[2][3];
+  ld_raw2(raw, xt + nb[0] * 4, V);
+#define TM_PHOP(NU, FWD, K)                                                                          \
+  proj_raw2<NU, FWD>(h, raw);                                                                      \
+  if (K < 7) ld_raw2(raw, xt + nb[K < 7 ? K + 1 : 0] * 4, V);                                        \
+  mul_acc2<NU, FWD>(acc, h, U + (int64_t)NU * 9 * V, V, FWD ? s : nb[K], NU == 3 ? (FWD ? pf : pb) : 1.f);
+  TM_PHOP(0, true, 0)
+  TM_PHOP(0, false, 1)
+  TM_PHOP(1, true, 2)
+  TM_PHOP(1, false, 3)
+  TM_PHOP(2, true, 4)
+  TM_PHOP(2, false, 5)
+  TM_PHOP(3, true, 6)
+  TM_PHOP(3, false, 7)
+#undef TM_PHOP
+  const int n0 = tile * 2;
+  const float2 m2 = make_float2(n0 < nsys ? (float)mu[n0] : 0.f, n0 + 1 < nsys ? (float)mu[n0 + 1] : 0.f);
+  // eps (doublet form): the tile's two systems are the flavours u, d of one doublet
+  local2(acc, xt + s * 4, V, C, V, s, m2, eps ? (float)eps[tile] : 0.f);
+  float* yo = y + tile * tstride + s * 4;
+  if constexpr (RES) {
+    const float* bo = bsub + tile * tstride + s * 4;
 #pragma unroll
     for (int k = 0; k < 12; ++k) {
-      acc.c[k].re = make_float2(0.f, 0.f);
-      acc.c[k].im = make_float2(0.f, 0.f);
+      const CV2 bv = ld2(bo + (int64_t)k * V * 4);
+      acc.c[k].re = sub2(bv.re, acc.c[k].re);
+      acc.c[k].im = sub2(bv.im, acc.c[k].im);
     }
-    // software pipeline over the eight hops: the neighbour spinor of hop k + 1 is loaded before
-    // the colour multiply of hop k, so its latency overlaps that arithmetic (loading the site's own
-    // spinor for the local term the same way measured slower)
-    int64_t nb[8];
-#pragma unroll
-    for (int nu = 0; nu < 4; ++nu) {
-      nb[2 * nu] = c[nu] + 1 < L[nu] ? s + strides[nu] : s - (int64_t)(L[nu] - 1) * strides[nu];
-      nb[2 * nu + 1] = c[nu] > 0 ? s - strides[nu] : s + (int64_t)(L[nu] - 1) * strides[nu];
-    }
-    const float pf = c[3] == Lt - 1 ? (float)bc_t : 1.f, pb = c[3] == 0 ? (float)bc_t : 1.f;
-    Raw2 raw;
-    CV2 h[2][3];
-    ld_raw2(raw, xt + nb[0] * 4, V);
-#define TM_PHOP(NU, FWD, K)                                                                          \
-    proj_raw2<NU, FWD>(h, raw);                                                                      \
-    if (K < 7) ld_raw2(raw, xt + nb[K < 7 ? K + 1 : 0] * 4, V);                                        \
-    mul_acc2<NU, FWD>(acc, h, U + (int64_t)NU * 9 * V, V, FWD ? s : nb[K], NU == 3 ? (FWD ? pf : pb) : 1.f);
-    TM_PHOP(0, true, 0)
-    TM_PHOP(0, false, 1)
-    TM_PHOP(1, true, 2)
-    TM_PHOP(1, false, 3)
-    TM_PHOP(2, true, 4)
-    TM_PHOP(2, false, 5)
-    TM_PHOP(3, true, 6)
-    TM_PHOP(3, false, 7)
-#undef TM_PHOP
-    const int n0 = tile * 2;
-    const float2 m2 = make_float2(n0 < nsys ? (float)mu[n0] : 0.f, n0 + 1 < nsys ? (float)mu[n0 + 1] : 0.f);
-    // eps (doublet form): the tile's two systems are the flavours u, d of one doublet
-    local2(acc, xt + s * 4, V, C, V, s, m2, eps ? (float)eps[tile] : 0.f);
-    real* yo = y + tile * tstride + s * 4;
-    if constexpr (RES) {
-      // residual form y = b - D x (b tile tile / nshift)
-      const real* bo = bsub + (int64_t)(tile / nshift) * tstride + s * 4;
-#pragma unroll
-      for (int k = 0; k < 12; ++k) {
-        const CV2 bv = ld2(bo + (int64_t)k * V * 4);
-        acc.c[k].re = sub2(bv.re, acc.c[k].re);
-        acc.c[k].im = sub2(bv.im, acc.c[k].im);
-      }
-    }
-#pragma unroll
-    for (int k = 0; k < 12; ++k) st2(yo + (int64_t)k * V * 4, acc.c[k]);
-  } else {
-    Spinor<real, T> acc;
-#pragma unroll
-    for (int k = 0; k < 12; ++k)
-#pragma unroll
-      for (int l = 0; l < T; ++l) { acc.c[k].re[l] = 0; acc.c[k].im[l] = 0; }
-
-#define TM_HOP(NU)                                                                                   \
-    {                                                                                                  \
-      int64_t sf = c[NU] + 1 < L[NU] ? s + strides[NU] : s - (int64_t)(L[NU] - 1) * strides[NU];      \
-      int64_t sb = c[NU] > 0 ? s - strides[NU] : s + (int64_t)(L[NU] - 1) * strides[NU];               \
-      real pf = (NU == 3 && c[3] == Lt - 1) ? bc_t : real(1);                                         \
-      real pb = (NU == 3 && c[3] == 0) ? bc_t : real(1);                                              \
-      hop<NU, true, real, T>(acc, xt + sf * 2 * T, V, U + (int64_t)NU * 9 * V, V, s, pf);               \
-      hop<NU, false, real, T>(acc, xt + sb * 2 * T, V, U + (int64_t)NU * 9 * V, V, sb, pb);             \
-    }
-    TM_HOP(0)
-    TM_HOP(1)
-    TM_HOP(2)
-    TM_HOP(3)
-#undef TM_HOP
-    real m[T];
-#pragma unroll
-    for (int l = 0; l < T; ++l) {
-      int n = tile * T + l;
-      m[l] = n < nsys ? (real)mu[n] : real(0);
-    }
-    // eps (doublet form, one system per tile): tiles 2p and 2p + 1 are the flavours u, d of doublet p
-    const real* xp = eps ? x + (int64_t)(tile ^ 1) * tstride + s * 2 * T : nullptr;
-    local_term<real, T>(acc, xt + s * 2 * T, V, C, V, s, m, xp, eps ? (real)eps[tile >> 1] : real(0));
-    real* yo = y + tile * tstride + s * 2 * T;
-    if constexpr (RES) {
-      // residual form y = b - D x, with b stored once per right-hand side (tile / nshift; for a
-      // doublet, once per right-hand side and flavour: tile (p / nshift) 2 + f of doublet p = tile / 2)
-      const int bt = eps ? ((tile >> 1) / nshift) * 2 + (tile & 1) : tile / nshift;
-      const real* bo = bsub + (int64_t)bt * tstride + s * 2 * T;
-#pragma unroll
-      for (int k = 0; k < 12; ++k) {
-        CV<real, T> bv;
-        ldcv(bv, bo + (int64_t)k * V * 2 * T);
-#pragma unroll
-        for (int l = 0; l < T; ++l) {
-          acc.c[k].re[l] = bv.re[l] - acc.c[k].re[l];
-          acc.c[k].im[l] = bv.im[l] - acc.c[k].im[l];
-        }
-      }
-    }
-#pragma unroll
-    for (int k = 0; k < 12; ++k) stcv(yo + (int64_t)k * V * 2 * T, acc.c[k]);
   }
+#pragma unroll
+  for (int k = 0; k < 12; ++k) st2(yo + (int64_t)k * V * 4, acc.c[k]);
 }
 
-// largest divisor of nt that keeps the CTA at <= maxthreads threads
-static inline int pick_ty(int nt, int bx, int maxthreads) {
-  int best = 1;
-  for (int d = 1; d * bx <= maxthreads && d <= nt; ++d)
-    if (nt % d == 0) best = d;
-  return best;
-}
-
-// launch variants: (sites per CTA row, largest CTA, CTAs per SM). FP32: 168 registers at 12 warps
-// per SM, or 128 registers (a few bytes of spills) at 16 warps per SM; FP64: 254 registers at 8
-// warps, or 168 registers (about 100 bytes of spills) at 12 warps.
-template <typename real, bool RES, int BX, int MAXT, int MINB>
-static void launch_variant(const Geom& g, const void* U, const real* C, const real* x, real* y, const double* mu,
-                           int nsys, const real* b, int nshift, const double* eps, cudaStream_t st) {
-  constexpr int T = Tile<real>::T;
-  const int nt = ntiles(nsys, T);
+// launch variants: (sites per CTA row, largest CTA, CTAs per SM): 168 registers at 12 warps per SM, or
+// 128 registers (a few bytes of spills) at 16 warps per SM
+template <bool RES, int BX, int MAXT, int MINB>
+static void launch_variant(const Geom& g, const float2* U, const float* C, const float* x, float* y, const double* mu,
+                           int nsys, const float* b, const double* eps, cudaStream_t st) {
+  const int nt = ntiles(nsys, 2);
   const int ty = pick_ty(nt, BX, MAXT);
   dim3 block(BX, ty);
   dim3 grid((unsigned)((g.V + BX - 1) / BX), (unsigned)(nt / ty));
-  dirac_kernel<real, T, BX, RES, MAXT, MINB><<<grid, block, 0, st>>>(
-      reinterpret_cast<const typename LinkT<real>::t*>(U), C, x, y, mu, nsys, nt, g.L[0], g.L[1], g.L[2], g.L[3],
-      (real)g.bc_t, b, nshift, eps); TM_COUNT();
+  dirac_kernel<BX, RES, MAXT, MINB><<<grid, block, 0, st>>>(U, C, x, y, mu, nsys, nt, g.L[0], g.L[1], g.L[2], g.L[3],
+                                                            (float)g.bc_t, b, eps); TM_COUNT();
 }
 
-template <typename real, bool RES>
-static void launch_variant_k(int v, const Geom& g, const void* U, const real* C, const real* x, real* y,
-                             const double* mu, int nsys, const real* b, int nshift, const double* eps,
-                             cudaStream_t st) {
-  if constexpr (sizeof(real) == 4) {
-    switch (v) {
-      case 1: launch_variant<real, RES, 32, 256, 2>(g, U, C, x, y, mu, nsys, b, nshift, eps, st); return;
-      case 2: launch_variant<real, RES, 64, 256, 2>(g, U, C, x, y, mu, nsys, b, nshift, eps, st); return;
-      case 3: launch_variant<real, RES, 32, 128, 4>(g, U, C, x, y, mu, nsys, b, nshift, eps, st); return;
-      default: launch_variant<real, RES, 32, 192, 2>(g, U, C, x, y, mu, nsys, b, nshift, eps, st); return;
-    }
-  } else {
-    switch (v) {
-      case 1: launch_variant<real, RES, 64, 192, 2>(g, U, C, x, y, mu, nsys, b, nshift, eps, st); return;
-      case 2: launch_variant<real, RES, 32, 192, 2>(g, U, C, x, y, mu, nsys, b, nshift, eps, st); return;
-      default: launch_variant<real, RES, 64, 256, 1>(g, U, C, x, y, mu, nsys, b, nshift, eps, st); return;
-    }
-  }
-}
-
-template <typename real>
-static constexpr int n_variants() {
-  return sizeof(real) == 4 ? 4 : 3;
-}
-
-// the tuned variant of a family for this lattice and system count; tuning (which runs every variant
-// on this call's data) only when `may_tune`, i.e. when the launch is repeatable
-template <typename real, bool RES>
-static void launch_tuned(const char* family, bool may_tune, const Geom& g, const void* U, const real* C, const real* x,
-                         real* y, const double* mu, int nsys, const real* b, int nshift, const double* eps,
+template <bool RES>
+static void launch_tuned(const char* family, bool may_tune, const Geom& g, const float2* U, const float* C,
+                         const float* x, float* y, const double* mu, int nsys, const float* b, const double* eps,
                          cudaStream_t st) {
-  const int64_t key = g.V * 4096 + nsys;
-  int v = 0;
-  if (tune_forced() >= 0) {
-    v = tune_forced() < n_variants<real>() ? tune_forced() : 0;
-  } else if (autotune_on()) {
-    v = tune_lookup(family, key);
-    if (v < 0)
-      v = may_tune ? tune_run(family, key, n_variants<real>(),
-                              [&](int k) {
-                                launch_variant_k<real, RES>(k, g, U, C, x, y, mu, nsys, b, nshift, eps, st);
-                              },
-                              st)
-                   : 0;
-  }
-  launch_variant_k<real, RES>(v, g, U, C, x, y, mu, nsys, b, nshift, eps, st);
+  auto launch = [&](int v) {
+    switch (v) {
+      case 1: launch_variant<RES, 32, 256, 2>(g, U, C, x, y, mu, nsys, b, eps, st); return;
+      case 2: launch_variant<RES, 64, 256, 2>(g, U, C, x, y, mu, nsys, b, eps, st); return;
+      case 3: launch_variant<RES, 32, 128, 4>(g, U, C, x, y, mu, nsys, b, eps, st); return;
+      default: launch_variant<RES, 32, 192, 2>(g, U, C, x, y, mu, nsys, b, eps, st); return;
+    }
+  };
+  launch(tune_variant(family, g.V * 4096 + nsys, 4, may_tune, launch, st));
 }
 
-template <typename real>
-void launch_dirac(const Geom& g, const void* U, const real* C, const real* x, real* y, const double* mu, int nsys,
-                  cudaStream_t st, const double* eps) {
-  TM_PROF(st, sizeof(real) == 4 ? "dirac_f32" : "dirac_f64");
-  launch_tuned<real, false>(sizeof(real) == 4 ? "dirac_f32" : "dirac_f64", true, g, U, C, x, y, mu, nsys, nullptr, 1,
-                            eps, st);
+template <>
+void launch_dirac<float>(const Geom& g, const void* U, const float* C, const float* x, float* y, const double* mu,
+                         int nsys, cudaStream_t st, const double* eps) {
+  TM_PROF(st, "dirac_f32");
+  launch_tuned<false>("dirac_f32", true, g, reinterpret_cast<const float2*>(U), C, x, y, mu, nsys, nullptr, eps, st);
 }
 
 void launch_residual32(const Geom& g, const float2* U, const float* C, const float* x, const float* b, float* r,
                        const double* mu, int nsys, cudaStream_t st, const double* eps) {
   TM_PROF(st, "residual_f32");
   // tuned only out of place (in place, b == r, the launch is not repeatable)
-  launch_tuned<float, true>("residual_f32", b != r, g, reinterpret_cast<const void*>(U), C, x, r, mu, nsys, b, 1, eps,
-                            st);
+  launch_tuned<true>("residual_f32", b != r, g, U, C, x, r, mu, nsys, b, eps, st);
 }
-
-void launch_residual64(const Geom& g, const double2* U, const double* C, const double* x, const double* b, int nshift,
-                       double* r, const double* mu, int nsys, cudaStream_t st, const double* eps) {
-  TM_PROF(st, "residual_f64");
-  launch_tuned<double, true>("residual_f64", b != r, g, reinterpret_cast<const void*>(U), C, x, r, mu, nsys, b, nshift,
-                             eps, st);
-}
-
-template void launch_dirac<float>(const Geom&, const void*, const float*, const float*, float*, const double*, int,
-                                  cudaStream_t, const double*);
-template void launch_dirac<double>(const Geom&, const void*, const double*, const double*, double*, const double*,
-                                   int, cudaStream_t, const double*);
 
 // ---------------------------------------------------------------- pack / unpack
 // field: complex [nsys][V][12]; bundle: [ntile][12][V][2][T]

@@ -199,14 +199,15 @@ static int ensure_ws(tmamg_ctx* ctx, int nsys, const tmamg_solve_params& p) {
     ws_free(w);
     return check_cuda(ctx, e, "workspace allocation");
   }
-  if (w->top.alloc(mm, ns, partial_elems(12 * V, ns, mm + 1, 2))) return set_err(ctx, TMAMG_ERR_OOM, "gmres state");
-  if (w->coarse.alloc(mcc, ns, partial_elems((int64_t)nc * Vc, ns, mcc + 1, 2)))
-    return set_err(ctx, TMAMG_ERR_OOM, "gmres state");
-  if (three && w->mid.alloc(mmm, ns, partial_elems((int64_t)ncm * Vm, ns, mmm + 1, 2)))
-    return set_err(ctx, TMAMG_ERR_OOM, "gmres state");
+  auto oom = [&](const char* what) {
+    ws_free(w);
+    return set_err(ctx, TMAMG_ERR_OOM, what);
+  };
+  if (w->top.alloc(mm, ns, partial_elems(12 * V, ns, mm + 1, 2))) return oom("gmres state");
+  if (w->coarse.alloc(mcc, ns, partial_elems((int64_t)nc * Vc, ns, mcc + 1, 2))) return oom("gmres state");
+  if (three && w->mid.alloc(mmm, ns, partial_elems((int64_t)ncm * Vm, ns, mmm + 1, 2))) return oom("gmres state");
   // the grid for one tile is the largest any system count uses
-  if (w->cg.alloc(mcc, ns, coarse_gmres_grid(1), w->cb32, cm_x16_bytes(Vc, nc, ns)))
-    return set_err(ctx, TMAMG_ERR_OOM, "coarse gmres state");
+  if (w->cg.alloc(mcc, ns, coarse_gmres_grid(1), w->cb32, cm_x16_bytes(Vc, nc, ns))) return oom("coarse gmres state");
   fill_c_kernel<<<(ns + 127) / 128, 128, 0, ctx->stream>>>(w->ones, ns, 1.0); TM_COUNT();
   fill_c_kernel<<<(ns + 127) / 128, 128, 0, ctx->stream>>>(w->mones, ns, -1.0); TM_COUNT();
   return check_cuda(ctx, cudaGetLastError(), "workspace init");
@@ -963,8 +964,10 @@ static int ensure_ws64(tmamg_ctx* ctx, int nsys, int m, int mc) {
     return check_cuda(ctx, e, "FP64 workspace allocation");
   }
   if (w->top.alloc(mm, ns, partial_elems(12 * V, ns, mm + 1, 1)) ||
-      w->coarse.alloc(mcc, ns, partial_elems((int64_t)w->nc * w->Vc, ns, mcc + 1, 1)))
+      w->coarse.alloc(mcc, ns, partial_elems((int64_t)w->nc * w->Vc, ns, mcc + 1, 1))) {
+    ws64_free(w);
     return set_err(ctx, TMAMG_ERR_OOM, "FP64 gmres state");
+  }
   fill_c_kernel<<<(ns + 127) / 128, 128, 0, ctx->stream>>>(w->ones, ns, 1.0); TM_COUNT();
   fill_c_kernel<<<(ns + 127) / 128, 128, 0, ctx->stream>>>(w->mones, ns, -1.0); TM_COUNT();
   return check_cuda(ctx, cudaGetLastError(), "FP64 workspace init");
@@ -1318,13 +1321,13 @@ int tmamg_debug_bounded_wait(long long limit_cycles, int unreachable_next) {
 int tmamg_setup(tmamg_ctx* ctx, const tmamg_setup_params* p, const float* start_vectors) {
   if (!ctx || !p) return set_err(ctx, TMAMG_ERR_ARG, "setup: null argument");
   if (!ctx->have_op) return set_err(ctx, TMAMG_ERR_STATE, "setup: operator not set");
-  return do_setup(ctx, p, start_vectors, true);
+  return with_optional_memory(ctx, [&] { return do_setup(ctx, p, start_vectors, true); });
 }
 
 int tmamg_setup_from_vectors(tmamg_ctx* ctx, const tmamg_setup_params* p, const float* test_vectors) {
   if (!ctx || !p || !test_vectors) return set_err(ctx, TMAMG_ERR_ARG, "setup_from_vectors: null argument");
   if (!ctx->have_op) return set_err(ctx, TMAMG_ERR_STATE, "setup_from_vectors: operator not set");
-  return do_setup(ctx, p, test_vectors, false);
+  return with_optional_memory(ctx, [&] { return do_setup(ctx, p, test_vectors, false); });
 }
 
 int tmamg_solve(tmamg_ctx* ctx, const double* b, int nrhs, const double* mu, int nshift, double* x, int on_device,
@@ -1334,7 +1337,7 @@ int tmamg_solve(tmamg_ctx* ctx, const double* b, int nrhs, const double* mu, int
   if (!ctx->have_setup) return set_err(ctx, TMAMG_ERR_STATE, "solve: no multigrid setup");
   tmamg_solve_params def;
   tmamg_default_solve_params(&def);
-  return do_solve(ctx, b, nrhs, mu, nshift, x, on_device, p ? p : &def, stats, nullptr);
+  return with_optional_memory(ctx, [&] { return do_solve(ctx, b, nrhs, mu, nshift, x, on_device, p ? p : &def, stats, nullptr); });
 }
 
 int tmamg_solve_doublet(tmamg_ctx* ctx, const double* b, int nrhs, const double* mu, const double* eps, int nshift,
@@ -1345,7 +1348,7 @@ int tmamg_solve_doublet(tmamg_ctx* ctx, const double* b, int nrhs, const double*
   if (!ctx->have_setup) return set_err(ctx, TMAMG_ERR_STATE, "solve_doublet: no multigrid setup");
   tmamg_solve_params def;
   tmamg_default_solve_params(&def);
-  return do_solve(ctx, b, nrhs, mu, nshift, x, on_device, p ? p : &def, stats, eps);
+  return with_optional_memory(ctx, [&] { return do_solve(ctx, b, nrhs, mu, nshift, x, on_device, p ? p : &def, stats, eps); });
 }
 
 size_t tmamg_coarse_bundle_bytes(const tmamg_ctx* ctx, int level, int nsys) {
@@ -1366,7 +1369,7 @@ int tmamg_sap(tmamg_ctx* ctx, void* r_bundle, void* e_bundle, int nsys, const do
   if (rc) return rc;
   float* delta = nullptr;
   size_t bytes = (size_t)ntiles(nsys, 2) * 12 * ctx->g.V * 4 * sizeof(float);
-  rc = check_cuda(ctx, cudaMalloc(&delta, bytes), "cudaMalloc(sap scratch)");
+  rc = with_optional_memory(ctx, [&] { return check_cuda(ctx, cudaMalloc(&delta, bytes), "cudaMalloc(sap scratch)"); });
   if (rc) return rc;
   sap_apply(ctx->g, block, ctx->U32, ctx->C32, (float*)r_bundle, (float*)e_bundle, delta, ctx->mu_dev, nsys, cycles,
             mr_steps, ctx->stream);
@@ -1428,7 +1431,7 @@ int tmamg_coarse_solve(tmamg_ctx* ctx, int level, const void* rc_bundle, void* x
       p->coarse_restart < 1 || p->coarse_restart > 64 || p->coarse_maxiter < 1 ||
       (p->coarse_precision != 0 && p->coarse_precision != 16 && p->coarse_precision != 32))
     return set_err(ctx, TMAMG_ERR_ARG, "coarse_solve: bad parameters");
-  int rc = ensure_ws(ctx, nsys, *p);
+  int rc = with_optional_memory(ctx, [&] { return ensure_ws(ctx, nsys, *p); });
   if (rc) return rc;
   std::vector<double> musys(nsys);
   for (int n = 0; n < nsys; ++n) musys[n] = mu[n % nshift];
