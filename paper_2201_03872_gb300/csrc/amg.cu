@@ -139,122 +139,226 @@ void build_P(const AggDims& g, const float* Vb, float2* P, int nv, int d, cudaSt
 // K x nsys, K = asize d) and the prolongation its transpose; P_a is read once for all systems.
 
 // xc[tile][chi nv + j][a] = sum_k conj(P[a][chi][j][k]) r[tile][chi d + c'][site(a, q)], k = c' asize + q.
-// One CTA per (aggregate, chirality). The vector entries of a chunk of RS_KC values of k are
-// staged in shared memory for all tiles (every output row reads them there). A thread owns a
-// 3 x 3 block of outputs (three rows j, three system tiles) and one of 16 interleaved slices of
-// k; per k it loads three entries of P and reads three staged 16-byte entries, and does nine
-// packed complex multiply-adds (both systems of a tile at once). The 16 slice sums of an output
-// are added by shuffles in a fixed order.
-constexpr int RS_KS = 16;         // k slices (lanes of a half warp)
-constexpr int RS_MAX_SLOTS = 24;  // output blocks processed at once per CTA (blockDim.x / RS_KS)
-constexpr int RS_KC = 128;        // k values staged per chunk (fewer when many tiles)
+//
+// A batch of small complex products (nv x K times K x nsys, K = asize d), one CTA per (aggregate,
+// chirality) and up to RS_MAXT tiles. It is bound by FP32 arithmetic from about 24 systems on (4 packed
+// multiply-adds per entry of P and tile) and by the bytes of P and the vector below.
+//  * The CTA's warps split K into chunks of RS_KC values; each warp brings its chunks to shared memory by
+//    its own asynchronous copies, two buffers deep, so that no CTA-wide barrier stands in the loop.
+//  * In a warp, 8 row groups x TG tile groups x 4 / TG values of k: a thread holds R x TT outputs (R =
+//    ceil(nv / 8) rows, TT tiles of two systems), so that a value of k costs R + TT shared loads, most
+//    of them broadcasts, for 4 R TT packed multiply-adds. The groups' rows and tiles lie so that a warp's
+//    loads fall into different banks (strides of 144 bytes per tile and 80 per row of a chunk).
+//  * Every tile of the call is in the CTA's registers (up to 40 systems): P and the vector are read once.
+//    The warps' partial sums are added in a fixed order at the end.
+// 24^3x48, nv = 24, 40 systems: 5.88 ms with 3 x 3 outputs per thread, 16 slices of k per half warp and the
+// vector staged behind CTA barriers in three rounds, 1.29 ms in this form (FP32 arithmetic alone
+// 0.76 ms, the bytes 0.61 ms); 1 system 0.357 -> 0.30 ms (bytes 0.24 ms), 16 systems 1.31 -> 0.65 ms.
+// warps per CTA: 16 (one CTA per SM) when the lanes hold four tile groups, so that a warp sums at most 96
+// values of k at nv = 24, d = 6, 4^4 aggregates (8 warps and two CTAs: 1.24 against 1.29 ms, but sums twice
+// as long and less exact); 8 and two CTAs per SM when the lanes split k further
+constexpr int rs_warps(int TG) { return TG == 4 ? 16 : 8; }
+constexpr int RS_KC = 8;         // values of k per chunk
+constexpr int RS_MAXT = 20;      // tiles per CTA (TG * TT)
+constexpr int RS_TABLE = 4096;   // largest aggregate whose sites are tabulated (two CTAs per SM fit with it)
+constexpr int RS_VS = RS_KC + 1; // float4 per tile of a staged chunk
+constexpr int RS_PS = RS_KC + 2; // float2 per row of a staged chunk (a multiple of 16 bytes)
 
-// two CTAs per SM (80 registers, no spills): one stages its vector chunk while the other computes
-__global__ void __launch_bounds__(RS_KS * RS_MAX_SLOTS, 2) restrict_kernel(const float2* __restrict__ P,
-                                                              const float* __restrict__ r, float* __restrict__ xc,
-                                                              AggDims g, int nv, int d, int nt, int kc) {
-  extern __shared__ float4 rsm[];                            // [nt][kc] staged entries
-  int* sidx = reinterpret_cast<int*>(rsm + (size_t)nt * kc);  // [asize] lattice site of each member
+__host__ __device__ constexpr int rs_stage_bytes(int R, int tiles) { return 8 * R * RS_PS * 8 + tiles * RS_VS * 16; }
+
+__device__ __forceinline__ void rs_copy16(void* smem, const void* gmem, bool on) {  // zeros if !on
+  const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
+  const int n = on ? 16 : 0;
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(sa), "l"(gmem), "r"(n) : "memory");
+}
+__device__ __forceinline__ void rs_copy8(void* smem, const void* gmem, bool on) {
+  const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
+  const int n = on ? 8 : 0;
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(sa), "l"(gmem), "r"(n) : "memory");
+}
+
+template <int R, int TT, int TG>
+__global__ void __launch_bounds__(rs_warps(TG) * 32, 16 / rs_warps(TG)) restrict_kernel(const float2* __restrict__ P,
+                                                                    const float* __restrict__ r,
+                                                                    float* __restrict__ xc, AggDims g, int nv, int d,
+                                                                    int nt, int chunk, int table) {
+  constexpr int WARPS = rs_warps(TG), TILES = TG * TT, KG = 4 / TG, ROWS = 8 * R;
+  constexpr int STAGE = rs_stage_bytes(R, TILES);
+  extern __shared__ float4 rsm[];
+  unsigned char* base = reinterpret_cast<unsigned char*>(rsm);
+  // [table] lattice site of each member (table = asize, or 0 for aggregates beyond RS_TABLE)
+  int* sidx = reinterpret_cast<int*>(base + WARPS * 2 * STAGE);
   const int64_t a = blockIdx.x >> 1;
   const int chi = blockIdx.x & 1;
+  const int t0 = blockIdx.y * chunk;
+  const int ntc = nt - t0 < chunk ? nt - t0 : chunk;
   const int K = g.asize * d;
-  for (int q = threadIdx.x; q < g.asize; q += blockDim.x) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (int q = threadIdx.x; q < table; q += blockDim.x) {
     int c[4];
     agg_site(a, q, g.Lc, g.agg, g.L, c);
     sidx[q] = (int)site_index(c, g.L);
   }
-  const int ks = threadIdx.x % RS_KS, slot = threadIdx.x / RS_KS;
-  const int nslots = blockDim.x / RS_KS;
-  const int JG = (nv + 2) / 3, TG = (nt + 2) / 3;
+  // rows and tiles that no copy fills stay zero
+  unsigned char* mine = base + warp * 2 * STAGE;
+  for (int i = lane; i < 2 * STAGE / 16; i += 32) reinterpret_cast<float4*>(mine)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+  __syncthreads();
   const float2* Pa = P + ((a * 2 + chi) * nv) * (int64_t)K;
-  for (int og0 = 0; og0 < JG * TG; og0 += nslots) {
-    const int og = og0 + slot;
-    const bool live = og < JG * TG;
-    const int jg = live ? og / TG : 0, tg = live ? og % TG : 0;
-    const int j0 = 3 * jg, t0 = 3 * tg;
-    float2 are[9], aim[9];
-#pragma unroll
-    for (int u = 0; u < 9; ++u) {
-      are[u] = make_float2(0.f, 0.f);
-      aim[u] = make_float2(0.f, 0.f);
-    }
-    for (int kc0 = 0; kc0 < K; kc0 += kc) {
-      const int kn = K - kc0 < kc ? K - kc0 : kc;
-      __syncthreads();  // sidx ready / the previous chunk consumed
-      for (int e = threadIdx.x; e < nt * kn; e += blockDim.x) {
-        const int t = e / kn, kk = e - t * kn;
-        const int k = kc0 + kk;
-        const int cp = k / g.asize, q = k - cp * g.asize;
-        rsm[t * kc + kk] =
-            __ldg(reinterpret_cast<const float4*>(r + (((int64_t)t * (2 * d) + chi * d + cp) * g.Vp + sidx[q]) * 4));
+  const float* ra = r + ((int64_t)t0 * (2 * d) + chi * d) * g.Vp * 4;
+  const int64_t tstr = (int64_t)(2 * d) * g.Vp * 4;
+  const bool even = (K & 1) == 0;  // rows of P start on 16-byte boundaries
+  const int nch = (K + RS_KC - 1) / RS_KC;
+  auto fetch = [&](int ch, int buf) {
+    if (ch < nch) {
+      float2* Ps = reinterpret_cast<float2*>(mine + buf * STAGE);
+      float4* Vs = reinterpret_cast<float4*>(mine + buf * STAGE + ROWS * RS_PS * 8);
+      const int k0 = ch * RS_KC;
+      if (even) {
+        for (int i = lane; i < nv * (RS_KC / 2); i += 32) {
+          const int j = i / (RS_KC / 2), q = 2 * (i % (RS_KC / 2));
+          const bool on = k0 + q < K;
+          rs_copy16(Ps + j * RS_PS + q, Pa + (int64_t)j * K + (on ? k0 + q : 0), on);
+        }
+      } else {
+        for (int i = lane; i < nv * RS_KC; i += 32) {
+          const int j = i / RS_KC, q = i % RS_KC;
+          const bool on = k0 + q < K;
+          rs_copy8(Ps + j * RS_PS + q, Pa + (int64_t)j * K + (on ? k0 + q : 0), on);
+        }
       }
-      __syncthreads();
-      if (live) {
-#pragma unroll 4
-        for (int kk = ks; kk < kn; kk += RS_KS) {
-          float2 p[3];
-          float4 v[3];
+      const int kk = lane % RS_KC, k = k0 + kk;
+      const bool on = k < K;
+      const int cp = on ? k / g.asize : 0, q = on ? k - cp * g.asize : 0;
+      int64_t site;
+      if (table) {
+        site = sidx[q];
+      } else {
+        int c[4];
+        agg_site(a, q, g.Lc, g.agg, g.L, c);
+        site = site_index(c, g.L);
+      }
+      const float* src = ra + ((int64_t)cp * g.Vp + site) * 4;
+      for (int t = lane / RS_KC; t < ntc; t += 32 / RS_KC) rs_copy16(Vs + t * RS_VS + kk, src + t * tstr, on);
+    }
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+  };
+  const int tg = lane % TG, kg = (lane / TG) % KG, rg = lane / 4;
+  float2 are[R][TT], aim[R][TT];
 #pragma unroll
-          for (int jj = 0; jj < 3; ++jj)
-            p[jj] = j0 + jj < nv ? __ldg(Pa + (int64_t)(j0 + jj) * K + kc0 + kk) : make_float2(0.f, 0.f);
+  for (int i = 0; i < R; ++i)
 #pragma unroll
-          for (int tt = 0; tt < 3; ++tt)
-            v[tt] = t0 + tt < nt ? rsm[(t0 + tt) * kc + kk] : make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int t = 0; t < TT; ++t) {
+      are[i][t] = make_float2(0.f, 0.f);
+      aim[i][t] = make_float2(0.f, 0.f);
+    }
+  int buf = 0;
+  fetch(warp, 0);
+  for (int ch = warp; ch < nch; ch += WARPS) {
+    fetch(ch + WARPS, buf ^ 1);
+    asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+    __syncwarp();
+    const float2* Ps = reinterpret_cast<const float2*>(mine + buf * STAGE) + rg * R * RS_PS;
+    const float4* Vs = reinterpret_cast<const float4*>(mine + buf * STAGE + ROWS * RS_PS * 8) + tg * TT * RS_VS;
 #pragma unroll
-          for (int jj = 0; jj < 3; ++jj) {
-            const float2 pr = make_float2(p[jj].x, p[jj].x), pi = make_float2(p[jj].y, p[jj].y);
-            const float2 npi = make_float2(-p[jj].y, -p[jj].y);
+    for (int k1 = 0; k1 < RS_KC; k1 += KG) {
+      const int kk = k1 + kg;
+      float4 v[TT];
 #pragma unroll
-            for (int tt = 0; tt < 3; ++tt) {
-              const float2 vr = make_float2(v[tt].x, v[tt].y), vi = make_float2(v[tt].z, v[tt].w);
-              // conj(p) v = (pr vr + pi vi) + i (pr vi - pi vr), both systems at once
-              are[jj * 3 + tt] = __ffma2_rn(pr, vr, are[jj * 3 + tt]);
-              are[jj * 3 + tt] = __ffma2_rn(pi, vi, are[jj * 3 + tt]);
-              aim[jj * 3 + tt] = __ffma2_rn(pr, vi, aim[jj * 3 + tt]);
-              aim[jj * 3 + tt] = __ffma2_rn(npi, vr, aim[jj * 3 + tt]);
-            }
-          }
+      for (int t = 0; t < TT; ++t) v[t] = Vs[t * RS_VS + kk];
+#pragma unroll
+      for (int i = 0; i < R; ++i) {
+        const float2 p = Ps[i * RS_PS + kk];
+        const float2 pr = make_float2(p.x, p.x), pi = make_float2(p.y, p.y), npi = make_float2(-p.y, -p.y);
+#pragma unroll
+        for (int t = 0; t < TT; ++t) {
+          const float2 vr = make_float2(v[t].x, v[t].y), vi = make_float2(v[t].z, v[t].w);
+          // conj(p) v = (pr vr + pi vi) + i (pr vi - pi vr), both systems at once
+          are[i][t] = __ffma2_rn(pr, vr, are[i][t]);
+          are[i][t] = __ffma2_rn(pi, vi, are[i][t]);
+          aim[i][t] = __ffma2_rn(pr, vi, aim[i][t]);
+          aim[i][t] = __ffma2_rn(npi, vr, aim[i][t]);
         }
       }
     }
-    // sum of the 16 slices (lanes ks of the half warp), fixed order
+    __syncwarp();  // the buffer may be filled again
+    buf ^= 1;
+  }
+  asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+  // the values of k held by other lanes, then the warps, in a fixed order
 #pragma unroll
-    for (int u = 0; u < 9; ++u) {
+  for (int o = TG; o < 4; o <<= 1)
 #pragma unroll
-      for (int o = RS_KS / 2; o > 0; o >>= 1) {
-        are[u].x += __shfl_xor_sync(0xffffffffu, are[u].x, o);
-        are[u].y += __shfl_xor_sync(0xffffffffu, are[u].y, o);
-        aim[u].x += __shfl_xor_sync(0xffffffffu, aim[u].x, o);
-        aim[u].y += __shfl_xor_sync(0xffffffffu, aim[u].y, o);
+    for (int i = 0; i < R; ++i)
+#pragma unroll
+      for (int t = 0; t < TT; ++t) {
+        are[i][t].x += __shfl_xor_sync(0xffffffffu, are[i][t].x, o);
+        are[i][t].y += __shfl_xor_sync(0xffffffffu, are[i][t].y, o);
+        aim[i][t].x += __shfl_xor_sync(0xffffffffu, aim[i][t].x, o);
+        aim[i][t].y += __shfl_xor_sync(0xffffffffu, aim[i][t].y, o);
       }
-    }
-    if (live && ks == 0) {
+  __syncthreads();  // every warp is done with its buffers
+  if (kg == 0) {
 #pragma unroll
-      for (int jj = 0; jj < 3; ++jj)
+    for (int i = 0; i < R; ++i)
 #pragma unroll
-        for (int tt = 0; tt < 3; ++tt)
-          if (j0 + jj < nv && t0 + tt < nt)
-            *reinterpret_cast<float4*>(xc + (((int64_t)(t0 + tt) * (2 * nv) + chi * nv + j0 + jj) * g.Vc + a) * 4) =
-                make_float4(are[jj * 3 + tt].x, are[jj * 3 + tt].y, aim[jj * 3 + tt].x, aim[jj * 3 + tt].y);
+      for (int t = 0; t < TT; ++t)
+        rsm[(warp * ROWS + rg * R + i) * TILES + tg * TT + t] =
+            make_float4(are[i][t].x, are[i][t].y, aim[i][t].x, aim[i][t].y);
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < nv * ntc; e += blockDim.x) {
+    const int j = e / ntc, t = e % ntc;
+    float4 s = rsm[j * TILES + t];
+#pragma unroll
+    for (int w = 1; w < WARPS; ++w) {
+      const float4 v = rsm[(w * ROWS + j) * TILES + t];
+      s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
     }
+    *reinterpret_cast<float4*>(xc + (((int64_t)(t0 + t) * (2 * nv) + chi * nv + j) * g.Vc + a) * 4) = s;
+  }
+}
+
+template <int R, int TT, int TG>
+static void launch_restrict(const AggDims& g, const float2* P, const float* r, float* xc, int nv, int d, int nt,
+                            int chunk, cudaStream_t st) {
+  constexpr int WARPS = rs_warps(TG);
+  constexpr size_t stages = (size_t)WARPS * 2 * rs_stage_bytes(R, TG * TT);
+  constexpr size_t sums = (size_t)WARPS * 8 * R * TG * TT * sizeof(float4);
+  static_assert(sums <= stages, "the partial sums reuse the stages");
+  const int table = g.asize <= RS_TABLE ? g.asize : 0;
+  const size_t smem = stages + sizeof(int) * table;
+  func_smem_optin((const void*)restrict_kernel<R, TT, TG>, (int)(stages + sizeof(int) * RS_TABLE));
+  restrict_kernel<R, TT, TG><<<dim3((unsigned)(g.Vc * 2), (nt + chunk - 1) / chunk), WARPS * 32, smem, st>>>(
+      P, r, xc, g, nv, d, nt, chunk, table);
+  TM_COUNT();
+}
+
+template <int R>
+static void launch_restrict_r(const AggDims& g, const float2* P, const float* r, float* xc, int nv, int d, int nt,
+                              cudaStream_t st) {
+  // equal chunks of at most RS_MAXT tiles; with one or two tiles the lanes that would idle split k instead
+  const int nchunk = (nt + RS_MAXT - 1) / RS_MAXT, chunk = (nt + nchunk - 1) / nchunk;
+  switch (chunk <= 1 ? 0 : chunk <= 2 ? 1 : (chunk + 3) / 4 + 1) {
+    case 0: launch_restrict<R, 1, 1>(g, P, r, xc, nv, d, nt, chunk, st); return;
+    case 1: launch_restrict<R, 1, 2>(g, P, r, xc, nv, d, nt, chunk, st); return;
+    case 2: launch_restrict<R, 1, 4>(g, P, r, xc, nv, d, nt, chunk, st); return;
+    case 3: launch_restrict<R, 2, 4>(g, P, r, xc, nv, d, nt, chunk, st); return;
+    case 4: launch_restrict<R, 3, 4>(g, P, r, xc, nv, d, nt, chunk, st); return;
+    case 5: launch_restrict<R, 4, 4>(g, P, r, xc, nv, d, nt, chunk, st); return;
+    default: launch_restrict<R, 5, 4>(g, P, r, xc, nv, d, nt, chunk, st); return;
   }
 }
 
 void restrict_vec(const AggDims& g, const float2* P, const float* r, float* xc, int nv, int d, int nsys,
                   cudaStream_t st) {
   const int nt = ntiles(nsys, T2);
-  int kc = RS_KC;
-  while (kc > RS_KS && sizeof(float4) * (size_t)nt * kc + sizeof(int) * g.asize > 100 * 1024) kc -= RS_KS;  // two CTAs per SM
-  const size_t smem = sizeof(float4) * (size_t)nt * kc + sizeof(int) * g.asize;
-  func_smem_optin((const void*)restrict_kernel, 200 * 1024);
   TM_PROF(st, d == 6 ? "restrict" : "restrict_coarse");
-  // every output block of the aggregate in one pass over P and the staged vector chunks when they
-  // fit one CTA (rounds of RS_MAX_SLOTS blocks otherwise)
-  const int nblk = ((nv + 2) / 3) * ((nt + 2) / 3);
-  const int rounds = (nblk + RS_MAX_SLOTS - 1) / RS_MAX_SLOTS;
-  const int slots = (nblk + rounds - 1) / rounds;
-  restrict_kernel<<<(unsigned)(g.Vc * 2), RS_KS * slots, smem, st>>>(P, r, xc, g, nv, d, nt, kc);
-  TM_COUNT();
+  switch ((nv + 7) / 8) {  // nv <= 32
+    case 1: launch_restrict_r<1>(g, P, r, xc, nv, d, nt, st); return;
+    case 2: launch_restrict_r<2>(g, P, r, xc, nv, d, nt, st); return;
+    case 3: launch_restrict_r<3>(g, P, r, xc, nv, d, nt, st); return;
+    default: launch_restrict_r<4>(g, P, r, xc, nv, d, nt, st); return;
+  }
 }
 
 // prolongation: tile chunk and CTA size

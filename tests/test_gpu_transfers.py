@@ -1,0 +1,98 @@
+"""Restriction and prolongation at the edges of their tilings, against the dense P.
+
+P is taken column by column from the prolongation of unit vectors (one system each) and checked to be
+orthonormal; restriction and prolongation of random vectors are then compared with the dense products.
+Row counts around the groups of eight, system counts around the tile groups and the largest chunk, and a
+level-2 transfer whose K = nv1 x 3 is odd. Tolerance as for the other FP32 components: 2e-5."""
+import numpy as np
+import pytest
+
+import synth
+from tests.gpu_util import Lattice, coarse_from_bundle, coarse_to_bundle, relerr, torch_cuda
+
+pytestmark = pytest.mark.gpu
+TOL32 = 2e-5
+
+
+def _dense(prolong, nc, Vc, batch=64):
+    """[parent entries, Vc * nc] columns of P from unit coarse vectors (site-major)"""
+    cols = []
+    n = Vc * nc
+    for k0 in range(0, n, batch):
+        m = min(batch, n - k0)
+        e = np.zeros((m, n), dtype=complex)
+        e[np.arange(m), k0 + np.arange(m)] = 1.0
+        cols.append(prolong(e.reshape(m, Vc, nc)).reshape(m, -1).T)
+    return np.concatenate(cols, axis=1)
+
+
+@pytest.mark.parametrize("nv,nsys", [(1, 1), (3, 4), (8, 2), (9, 3), (17, 9), (24, 24), (24, 33), (32, 40), (32, 43)])
+def test_transfers_against_dense_p(nv, nsys):
+    torch = torch_cuda()
+    L = (8, 4, 4, 4)
+    lat = Lattice(L, synth.gauge_field(L, 0.3, seed=3), 0.125, 1.0)
+    try:
+        T = lat.T
+        tv = synth.gaussian_spinors(L, nv, seed=5).astype(np.complex64)
+        p = T.setup_params(nv=nv, agg=(4, 4, 4, 4), sap_block=(4, 2, 2, 2))
+        T.tmamg_setup_from_vectors(lat.ctx, p, torch.from_numpy(tv.view(np.float32).copy()).cuda())
+        Vc, nc = 2, 2 * nv
+
+        def prolong(xc):
+            n = xc.shape[0]
+            cb = torch.from_numpy(coarse_to_bundle(xc, nc, Vc)).cuda()
+            fb = torch.full((T.tmamg_bundle_bytes(lat.ctx, n, 32) // 4,), 7.0, device="cuda")
+            T.tmamg_prolong(lat.ctx, 1, cb, fb, n)
+            return lat.from_fine_bundle(fb, n)
+
+        P = _dense(prolong, nc, Vc)
+        assert np.abs(P.conj().T @ P - np.eye(Vc * nc)).max() < TOL32
+        x = synth.gaussian_spinors(L, nsys, seed=6)
+        cb = lat.coarse_buffer(nsys)
+        T.tmamg_restrict(lat.ctx, 1, lat.fine_bundle(x), cb, nsys)
+        torch.cuda.synchronize()
+        got = coarse_from_bundle(cb.cpu().numpy(), nsys, nc, Vc)
+        want = (P.conj().T @ x.astype(np.complex64).reshape(nsys, -1).T).T.reshape(nsys, Vc, nc)
+        for n in range(nsys):
+            assert relerr(got[n], want[n]) <= TOL32, n
+        xc = synth.gaussian_coarse((2, 1, 1, 1), nsys, nv, seed=9).reshape(nsys, Vc, nc)
+        up = prolong(xc).reshape(nsys, -1)
+        for n in range(nsys):
+            assert relerr(up[n], P @ xc[n].ravel()) <= TOL32, n
+    finally:
+        lat.close()
+
+
+@pytest.mark.parametrize("nsys", [1, 6, 19])
+def test_level_two_transfers_with_odd_k(nsys):
+    torch = torch_cuda()
+    L = (12, 4, 4, 4)
+    nv, nv2 = 5, 7  # K = 5 x 3 per chirality: rows of P2 on 8-byte boundaries only
+    lat = Lattice(L, synth.gauge_field(L, 0.3, seed=3), 0.125, 1.0)
+    try:
+        T = lat.T
+        p = T.setup_params(levels=3, nv=nv, nv2=nv2, agg=(4, 4, 4, 4), agg2=(3, 1, 1, 1), sap_block=(2, 2, 2, 2))
+        tv = np.concatenate([synth.gaussian_spinors(L, nv, seed=5).ravel(),
+                             synth.gaussian_coarse((3, 1, 1, 1), nv2, nv, seed=7).ravel()]).astype(np.complex64)
+        T.tmamg_setup_from_vectors(lat.ctx, p, torch.from_numpy(tv.view(np.float32).copy()).cuda())
+        nc1, nc2 = 2 * nv, 2 * nv2
+
+        def prolong(xc):
+            n = xc.shape[0]
+            cb = torch.from_numpy(coarse_to_bundle(xc, nc2, 1)).cuda()
+            fb = lat.coarse_buffer(n, 1)
+            T.tmamg_prolong(lat.ctx, 2, cb, fb, n)
+            torch.cuda.synchronize()
+            return coarse_from_bundle(fb.cpu().numpy(), n, nc1, 3)
+
+        P = _dense(prolong, nc2, 1)
+        assert np.abs(P.conj().T @ P - np.eye(nc2)).max() < TOL32
+        x = synth.gaussian_coarse((3, 1, 1, 1), nsys, nv, seed=8).reshape(nsys, 3, nc1)
+        cb = lat.coarse_buffer(nsys, 2)
+        T.tmamg_restrict(lat.ctx, 2, torch.from_numpy(coarse_to_bundle(x, nc1, 3)).cuda(), cb, nsys)
+        torch.cuda.synchronize()
+        got = coarse_from_bundle(cb.cpu().numpy(), nsys, nc2, 1)
+        for n in range(nsys):
+            assert relerr(got[n].ravel(), P.conj().T @ x[n].ravel()) <= TOL32, n
+    finally:
+        lat.close()
