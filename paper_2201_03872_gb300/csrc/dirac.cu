@@ -233,11 +233,42 @@ void launch_build_clover(const Geom& g, const double2* U64, double kappa, double
                                                                        c_sw, C64, C32); TM_COUNT();
 }
 
-// The FP32 form (dirac64.cu holds the FP64 one): 192-thread CTAs, two per SM, up to 170 registers.
+__device__ __forceinline__ void dr_copy16(void* smem, const void* gmem) {
+  const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem) : "memory");
+}
+__device__ __forceinline__ void dr_copy8(void* smem, const void* gmem) {
+  const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(sa), "l"(gmem) : "memory");
+}
+__device__ __forceinline__ void dr_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void dr_wait_sync() {  // all but the last N groups of every thread have landed
+  asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
+  __syncthreads();
+}
+
+// bytes of the staged operator data of a CTA row of bx sites: links of the sites, links of their backward
+// neighbours, clover blocks
+__host__ __device__ constexpr int dr_stage_bytes(int bx) { return bx * (36 * 8 + 36 * 8 + 72 * 4); }
+
+// The FP32 form (dirac64.cu holds the FP64 one).
 // RES: residual form y = b - D x (b = bsub, tile for tile), else y = D x (bsub unused).
+// STAGED: the links and clover blocks of the CTA's sites come to shared memory by asynchronous copies, once
+// for all tiles of the CTA and ahead of their use; otherwise every thread loads them where it needs them.
+//  What bounds the direct form is latency: 12 warps per SM, and each hop starts with nine loads of links
+//  that the previous hop's arithmetic does not cover (33% of the issue slots used, 5.3 of 8.7 cycles per
+//  instruction waiting for global loads, 24^3x48 x 16 systems). Staged in three groups, waited for as
+//  they are needed, those loads are off the critical path and a quarter of the L1 lookups is gone; the
+//  site's own spinor for the local term then joins the software pipeline (it gained nothing before).
+//  Direct against staged: 40^3x80 x 16 systems 8.2 and 6.6 ms (2.7 ms at the HBM rate), 16^3x32 x 12 152
+//  and 124 us; issue slots used 33% and 44%, L1 data path 43% and 60%. With one tile (one or two systems)
+//  nothing is shared and the direct form is the faster one (24^3x48, one system: 137 against 177 us), so
+//  both are launch variants. Prefetching the neighbours' lines into L1 (9.2 ms) and wider CTA rows (8.9 to 9.1
+//  ms) measured slower.
 // MAXT, MINB: the launch variant's largest CTA and the CTAs per SM it is compiled for (which sets the
 // register budget); every variant does the same per-thread arithmetic.
-template <int BX, bool RES, int MAXT, int MINB>
+template <int BX, bool RES, bool STAGED, int MAXT, int MINB>
 __global__ void __launch_bounds__(MAXT, MINB) dirac_kernel(const float2* __restrict__ U, const float* __restrict__ C,
                                                            const float* __restrict__ x, float* y,
                                                            const double* __restrict__ mu, int nsys, int ntile, int Lx,
@@ -247,9 +278,11 @@ __global__ void __launch_bounds__(MAXT, MINB) dirac_kernel(const float2* __restr
   // y is not restrict-qualified: the residual form may run in place (bsub == y), every thread
   // reading b at its own site before it writes y there; x never overlaps y
   const int64_t V = (int64_t)Lx * Ly * Lz * Lt;
-  const int64_t s = blockIdx.x * (int64_t)BX + threadIdx.x;
+  const int64_t s0 = blockIdx.x * (int64_t)BX;
   const int tile = blockIdx.y * blockDim.y + threadIdx.y;
-  if (s >= V || tile >= ntile) return;
+  const bool live = s0 + threadIdx.x < V;
+  if (!STAGED && !live) return;
+  const int64_t s = live ? s0 + threadIdx.x : V - 1;
   const int L[4] = {Lx, Ly, Lz, Lt};
   int c[4];
   site_coords(s, L, c);
@@ -264,26 +297,59 @@ __global__ void __launch_bounds__(MAXT, MINB) dirac_kernel(const float2* __restr
     acc.c[k].im = make_float2(0.f, 0.f);
   }
   // software pipeline over the eight hops: the neighbour spinor of hop k + 1 is loaded before
-  // the colour multiply of hop k, so its latency overlaps that arithmetic (loading the site's own
-  // spinor for the local term the same way measured slower)
+  // the colour multiply of hop k, so its latency overlaps that arithmetic
   int64_t nb[8];
 #pragma unroll
   for (int nu = 0; nu < 4; ++nu) {
     nb[2 * nu] = c[nu] + 1 < L[nu] ? s + strides[nu] : s - (int64_t)(L[nu] - 1) * strides[nu];
     nb[2 * nu + 1] = c[nu] > 0 ? s - strides[nu] : s + (int64_t)(L[nu] - 1) * strides[nu];
   }
+  extern __shared__ float4 dr_smem[];
+  float2* Lf = reinterpret_cast<float2*>(dr_smem);  // [4 nu][9][BX] U_nu(s)
+  float2* Lb = Lf + 36 * BX;                        // [4 nu][9][BX] U_nu(s - nu)
+  float* Cs = reinterpret_cast<float*>(Lb + 36 * BX);  // [72][BX]
+  if constexpr (STAGED) {
+    // V is a multiple of 16 (even extents): the rows of a site range start on 16-byte boundaries
+    const int nt = BX * blockDim.y, tid = threadIdx.y * BX + threadIdx.x;
+    const int n = V - s0 < BX ? (int)(V - s0) : BX;
+#pragma unroll
+    for (int half = 0; half < 2; ++half) {  // directions x, y, then z, t
+      for (int i = tid; i < 18 * (BX / 2); i += nt) {
+        const int q = 18 * half + i / (BX / 2), e = 2 * (i % (BX / 2));
+        if (e < n) dr_copy16(Lf + q * BX + e, U + (int64_t)q * V + s0 + e);
+      }
+      if (live) {
+#pragma unroll
+        for (int nu = 2 * half; nu < 2 * half + 2; ++nu)
+          for (int k = threadIdx.y; k < 9; k += blockDim.y)
+            dr_copy8(Lb + (nu * 9 + k) * BX + threadIdx.x, U + (int64_t)(nu * 9 + k) * V + nb[2 * nu + 1]);
+      }
+      dr_commit();
+    }
+    for (int i = tid; i < 72 * (BX / 4); i += nt) {
+      const int q = i / (BX / 4), e = 4 * (i % (BX / 4));
+      if (e < n) dr_copy16(Cs + q * BX + e, C + (int64_t)q * V + s0 + e);
+    }
+    dr_commit();
+  }
   const float pf = c[3] == Lt - 1 ? bc_t : 1.f, pb = c[3] == 0 ? bc_t : 1.f;
   Raw2 raw;
   CV2 h[2][3];
   ld_raw2(raw, xt + nb[0] * 4, V);
+  if constexpr (STAGED) dr_wait_sync<2>();
 #define TM_PHOP(NU, FWD, K)                                                                          \
-  proj_raw2<NU, FWD>(h, raw);                                                                      \
-  if (K < 7) ld_raw2(raw, xt + nb[K < 7 ? K + 1 : 0] * 4, V);                                        \
-  mul_acc2<NU, FWD>(acc, h, U + (int64_t)NU * 9 * V, V, FWD ? s : nb[K], NU == 3 ? (FWD ? pf : pb) : 1.f);
+  proj_raw2<NU, FWD>(h, raw);                                                                        \
+  if (STAGED || K < 7) ld_raw2(raw, xt + (K < 7 ? nb[K < 7 ? K + 1 : 0] : s) * 4, V);                \
+  if constexpr (STAGED)                                                                              \
+    mul_acc2<NU, FWD>(acc, h, (FWD ? Lf : Lb) + NU * 9 * BX, BX, threadIdx.x,                        \
+                      NU == 3 ? (FWD ? pf : pb) : 1.f);                                              \
+  else                                                                                               \
+    mul_acc2<NU, FWD>(acc, h, U + (int64_t)NU * 9 * V, V, FWD ? s : nb[K], NU == 3 ? (FWD ? pf : pb) : 1.f);
   TM_PHOP(0, true, 0)
   TM_PHOP(0, false, 1)
   TM_PHOP(1, true, 2)
   TM_PHOP(1, false, 3)
+  if constexpr (STAGED) dr_wait_sync<1>();
   TM_PHOP(2, true, 4)
   TM_PHOP(2, false, 5)
   TM_PHOP(3, true, 6)
@@ -292,7 +358,14 @@ __global__ void __launch_bounds__(MAXT, MINB) dirac_kernel(const float2* __restr
   const int n0 = tile * 2;
   const float2 m2 = make_float2(n0 < nsys ? (float)mu[n0] : 0.f, n0 + 1 < nsys ? (float)mu[n0 + 1] : 0.f);
   // eps (doublet form): the tile's two systems are the flavours u, d of one doublet
-  local2(acc, xt + s * 4, V, C, V, s, m2, eps ? (float)eps[tile] : 0.f);
+  const float ep = eps ? (float)eps[tile] : 0.f;
+  if constexpr (STAGED) {
+    dr_wait_sync<0>();
+    local2(acc, raw, Cs, BX, threadIdx.x, m2, ep);
+    if (!live) return;
+  } else {
+    local2(acc, xt + s * 4, V, C, V, s, m2, ep);
+  }
   float* yo = y + tile * tstride + s * 4;
   if constexpr (RES) {
     const float* bo = bsub + tile * tstride + s * 4;
@@ -307,17 +380,18 @@ __global__ void __launch_bounds__(MAXT, MINB) dirac_kernel(const float2* __restr
   for (int k = 0; k < 12; ++k) st2(yo + (int64_t)k * V * 4, acc.c[k]);
 }
 
-// launch variants: (sites per CTA row, largest CTA, CTAs per SM): 168 registers at 12 warps per SM, or
-// 128 registers (a few bytes of spills) at 16 warps per SM
-template <bool RES, int BX, int MAXT, int MINB>
+// launch variants: (sites per CTA row, staged, largest CTA, CTAs per SM): 168 registers at 12 warps per SM,
+// or 128 registers (a few bytes of spills) at 16 warps per SM
+template <bool RES, int BX, bool STAGED, int MAXT, int MINB>
 static void launch_variant(const Geom& g, const float2* U, const float* C, const float* x, float* y, const double* mu,
                            int nsys, const float* b, const double* eps, cudaStream_t st) {
   const int nt = ntiles(nsys, 2);
   const int ty = pick_ty(nt, BX, MAXT);
   dim3 block(BX, ty);
   dim3 grid((unsigned)((g.V + BX - 1) / BX), (unsigned)(nt / ty));
-  dirac_kernel<BX, RES, MAXT, MINB><<<grid, block, 0, st>>>(U, C, x, y, mu, nsys, nt, g.L[0], g.L[1], g.L[2], g.L[3],
-                                                            (float)g.bc_t, b, eps); TM_COUNT();
+  if (STAGED) func_smem_optin((const void*)dirac_kernel<BX, RES, STAGED, MAXT, MINB>, dr_stage_bytes(BX));
+  dirac_kernel<BX, RES, STAGED, MAXT, MINB><<<grid, block, STAGED ? dr_stage_bytes(BX) : 0, st>>>(
+      U, C, x, y, mu, nsys, nt, g.L[0], g.L[1], g.L[2], g.L[3], (float)g.bc_t, b, eps); TM_COUNT();
 }
 
 template <bool RES>
@@ -326,10 +400,10 @@ static void launch_tuned(const char* family, bool may_tune, const Geom& g, const
                          cudaStream_t st) {
   auto launch = [&](int v) {
     switch (v) {
-      case 1: launch_variant<RES, 32, 256, 2>(g, U, C, x, y, mu, nsys, b, eps, st); return;
-      case 2: launch_variant<RES, 64, 256, 2>(g, U, C, x, y, mu, nsys, b, eps, st); return;
-      case 3: launch_variant<RES, 32, 128, 4>(g, U, C, x, y, mu, nsys, b, eps, st); return;
-      default: launch_variant<RES, 32, 192, 2>(g, U, C, x, y, mu, nsys, b, eps, st); return;
+      case 1: launch_variant<RES, 32, false, 192, 2>(g, U, C, x, y, mu, nsys, b, eps, st); return;
+      case 2: launch_variant<RES, 32, true, 256, 2>(g, U, C, x, y, mu, nsys, b, eps, st); return;
+      case 3: launch_variant<RES, 64, true, 128, 3>(g, U, C, x, y, mu, nsys, b, eps, st); return;
+      default: launch_variant<RES, 32, true, 192, 2>(g, U, C, x, y, mu, nsys, b, eps, st); return;
     }
   };
   launch(tune_variant(family, g.V * 4096 + nsys, 4, may_tune, launch, st));

@@ -395,16 +395,16 @@ __device__ __forceinline__ void mul_acc2(Spinor2& acc, const CV2 (&h)[2][3], con
 // local_term<> for FP32 tiles of two systems in packed arithmetic: acc <- A_chi x_chi +
 // i s mu x_chi - 1/2 acc per chirality; mu: the two systems' twisted masses. ep != 0: the tile's two
 // systems are the flavours of a non-degenerate doublet, coupled by -ep (each lane gets -ep times
-// the other lane's entry)
-__device__ __forceinline__ void local2(Spinor2& acc, const float* __restrict__ x0, int64_t cstride,
-                                       const float* __restrict__ C, int64_t V, int64_t s, float2 mu,
-                                       float ep = 0.f) {
+// the other lane's entry). entry(k): component k of the site's own spinor
+template <class Entry>
+__device__ __forceinline__ void local2_of(Spinor2& acc, Entry entry, const float* __restrict__ C, int64_t V, int64_t s,
+                                          float2 mu, float ep) {
 #pragma unroll
   for (int chi = 0; chi < 2; ++chi) {
     const float* Cc = C + (int64_t)chi * 36 * V + s;
     CV2 xc[6];
 #pragma unroll
-    for (int i = 0; i < 6; ++i) xc[i] = ld2(x0 + (int64_t)(chi * 6 + i) * cstride * 4);
+    for (int i = 0; i < 6; ++i) xc[i] = entry(chi * 6 + i);
     const float2 smu = chi == 0 ? mu : make_float2(-mu.x, -mu.y);
     const float2 nsmu = make_float2(-smu.x, -smu.y);
 #pragma unroll
@@ -440,6 +440,18 @@ __device__ __forceinline__ void local2(Spinor2& acc, const float* __restrict__ x
       hv.im = fma2(f2(-0.5f), hv.im, o.im);
     }
   }
+}
+
+// the site's own spinor at x0, components strided by cstride entries
+__device__ __forceinline__ void local2(Spinor2& acc, const float* __restrict__ x0, int64_t cstride,
+                                       const float* __restrict__ C, int64_t V, int64_t s, float2 mu,
+                                       float ep = 0.f) {
+  local2_of(acc, [&](int k) { return ld2(x0 + (int64_t)k * cstride * 4); }, C, V, s, mu, ep);
+}
+// the site's own spinor in registers
+__device__ __forceinline__ void local2(Spinor2& acc, const Raw2& r, const float* __restrict__ C, int64_t V, int64_t s,
+                                       float2 mu, float ep) {
+  local2_of(acc, [&](int k) { return r.v[k]; }, C, V, s, mu, ep);
 }
 
 }  // namespace tmamg
