@@ -114,12 +114,12 @@ def dirac_bytes_per_site(nsys, prec):
 # the same kernel on another volume is reported as the captured bytes times the volume ratio.
 # Valid only for the kernel sources the capture was taken on (SHA-1 of the files), else null.
 KERNEL_TRAFFIC = {
-    "dirac_f32": {"bytes": 1975047424 + 996297216, "L": (24, 24, 24, 48), "nsys": 16,
+    "dirac_f32": {"bytes": 1972962304 + 996601856, "L": (24, 24, 24, 48), "nsys": 16,
                   "sha1": {"dirac.cu": "9f157006078c6ab5accc5809e79ffb8d99d40f1c",
-                           "stencil.cuh": "18a3bd554cd420934e3562a1ed82099499fa41ab"}},
-    "sap_mr": {"bytes": 3087883264 + 1500493824, "L": (24, 24, 24, 48), "nsys": 16,
-               "sha1": {"sap.cu": "f57da3cd9bff38252df3a6da1a335eaf2ab9f83a",
-                        "stencil.cuh": "bbe52b7b1bde87326034de584ba1950fba6a7d1b"}},
+                           "stencil.cuh": "76df2d28f1ae9c55ef0539b804f08d293db5940f"}},
+    "sap_mr": {"bytes": 2211575552 + 1500810240, "L": (24, 24, 24, 48), "nsys": 16,
+               "sha1": {"sap.cu": "0d16cf72354ebde8b86ec57456174d79eaed40f0",
+                        "stencil.cuh": "76df2d28f1ae9c55ef0539b804f08d293db5940f"}},
 }
 
 

@@ -82,6 +82,12 @@ int upload_mu(tmamg_ctx* ctx, const double* mu, int nsys) {
                     "upload mu");
 }
 
+void free_sap_delta(tmamg_ctx* ctx) {
+  cudaFree(ctx->sap_delta);
+  ctx->sap_delta = nullptr;
+  ctx->sap_delta_bytes = 0;
+}
+
 static int grow_scratch(tmamg_ctx* ctx, size_t bytes) {
   for (int i = 0; i < 2; ++i) {
     if (ctx->scratch[i]) cudaFree(ctx->scratch[i]);
@@ -187,6 +193,7 @@ int tmamg_destroy(tmamg_ctx* ctx) {
   cudaFree(ctx->C64);
   cudaFree(ctx->C32);
   free_fixed(ctx->g);
+  free_sap_delta(ctx);
   cudaFree(ctx->mu_dev);
   cudaFree(ctx->eps_dev);
   for (int i = 0; i < 2; ++i) cudaFree(ctx->scratch[i]);

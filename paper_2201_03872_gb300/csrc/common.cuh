@@ -94,6 +94,9 @@ struct tmamg_ctx {
   // scratch for tmamg_apply
   void* scratch[2] = {nullptr, nullptr};
   size_t scratch_bytes = 0;
+  // correction buffer of tmamg_sap (grown on demand)
+  float* sap_delta = nullptr;
+  size_t sap_delta_bytes = 0;
   // multigrid hierarchy
   tmamg_setup_params sp;
   std::vector<tmamg::CoarseLevel> levels;
@@ -120,15 +123,17 @@ int set_err(tmamg_ctx* ctx, int code, const std::string& msg);
 int check_cuda(tmamg_ctx* ctx, cudaError_t e, const char* what);
 int upload_mu(tmamg_ctx* ctx, const double* mu, int nsys);
 
-// runs f; if it found no device memory while the context holds optional copies of the operator, gives
-// those back (the FP64 stencil then runs in FP64 arithmetic) and runs it again. f leaves nothing half
-// allocated behind when it returns TMAMG_ERR_OOM.
+// runs f; if it found no device memory while the context holds some that it can do without (the correction
+// buffer of tmamg_sap, the optional copies of the operator: the FP64 stencil then runs in FP64 arithmetic),
+// gives that back and runs it again. f leaves nothing half allocated behind when it returns TMAMG_ERR_OOM.
 void free_fixed(Geom& g);
+void free_sap_delta(tmamg_ctx* ctx);
 template <class F>
 int with_optional_memory(tmamg_ctx* ctx, F f) {
   int rc = f();
-  if (rc == TMAMG_ERR_OOM && ctx->g.fx.U) {
+  if (rc == TMAMG_ERR_OOM && (ctx->g.fx.U || ctx->sap_delta)) {
     cudaStreamSynchronize(ctx->stream);
+    free_sap_delta(ctx);
     free_fixed(ctx->g);
     cudaGetLastError();
     rc = f();

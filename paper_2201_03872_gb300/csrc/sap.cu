@@ -5,13 +5,12 @@
 // then black. Here each block solve is `steps` minimal-residual steps on the block
 // operator D_B (hops that leave the block dropped) from a zero start.
 //
-// GPU design: one CTA per (block, system tile), one thread per block site. The block
-// residual rho and the block correction live in shared memory; the block operator reads
-// neighbours from shared memory and links/clover from global memory (L1/L2 resident
-// across the MR steps). Because neighbouring blocks always have the other colour, the
-// residual on a block right after its solve is exactly the final MR residual, and the
-// residual on the other colour changes only through hops that cross a block face: a
-// second kernel subtracts those hops, so SAP needs no full-lattice operator application.
+// GPU design: one CTA per SM works through (block, system tile) items, one thread per block site. The
+// block residual rho, the links and the clover blocks live in shared memory, the block correction in
+// registers. Because neighbouring blocks always have the other colour, the residual on a block right
+// after its solve is exactly the final MR residual, and the residual on the other colour changes only
+// through hops that cross a block face: a second kernel subtracts those hops, so SAP needs no
+// full-lattice operator application.
 #include "sap.cuh"
 #include "profile.cuh"
 #include "stencil.cuh"
@@ -48,37 +47,57 @@ __device__ __forceinline__ int local_index(const int* lc, const SapDims& d) {
   return ((lc[3] * d.bs[2] + lc[2]) * d.bs[1] + lc[1]) * d.bs[0] + lc[0];
 }
 
-template <int N>
-__device__ __forceinline__ void block_reduce(float (&v)[N], float* red) {
-  // sums v[0..N) over the CTA; every thread gets the totals (N <= 8); blockDim.x is a
-  // multiple of 32, so every warp is full. Fixed-size and fully unrolled, so v stays in registers.
-  // One barrier: the caller alternates between two scratch buffers `red`, so a buffer is written
-  // again only after a later barrier that every reader of its previous contents has passed.
+// Sums v[0..2] (system 0 of the tile) and v[3..5] (system 1) over the CTA; every thread gets the totals;
+// blockDim.x is a multiple of 32, so every warp is full. The first exchange leaves each half warp with one
+// system's three sums, which halves the shuffles. One barrier: the caller alternates between two scratch
+// buffers `red` (two float4 per warp), so a buffer is written again only after a later barrier that every
+// reader of its previous contents has passed.
+__device__ __forceinline__ void block_reduce(float (&v)[6], float4* red) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nw = (blockDim.x + 31) >> 5;
+  const bool up = lane >= 16;
+  float t[3];
 #pragma unroll
-  for (int i = 0; i < N; ++i) {
-    float x = v[i];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-    v[i] = x;
+  for (int i = 0; i < 3; ++i) {
+    const float keep = up ? v[3 + i] : v[i], give = up ? v[i] : v[3 + i];
+    t[i] = keep + __shfl_xor_sync(0xffffffffu, give, 16);
   }
-  if (lane == 0) {
 #pragma unroll
-    for (int i = 0; i < N; ++i) red[warp * 8 + i] = v[i];
-  }
+  for (int o = 8; o > 0; o >>= 1)
+#pragma unroll
+    for (int i = 0; i < 3; ++i) t[i] += __shfl_xor_sync(0xffffffffu, t[i], o);
+  if ((lane & 15) == 0) red[2 * warp + (lane >> 4)] = make_float4(t[0], t[1], t[2], 0.f);
   __syncthreads();
 #pragma unroll
-  for (int i = 0; i < N; ++i) {
-    float s = 0;
-    for (int w = 0; w < nw; ++w) s += red[w * 8 + i];
-    v[i] = s;
+  for (int i = 0; i < 6; ++i) v[i] = 0.f;
+  for (int w = 0; w < nw; ++w) {
+    const float4 a = red[2 * w], b = red[2 * w + 1];
+    v[0] += a.x; v[1] += a.y; v[2] += a.z;
+    v[3] += b.x; v[4] += b.y; v[5] += b.z;
   }
 }
 
+// Entries of one block row are 64 contiguous bytes (4 sites) between rows of the other colour: every load asks
+// L2 for 64 bytes, not for the whole 128-byte line whose other half this colour never touches
+__device__ __forceinline__ CV2 sap_ld(const float* p) {
+  float4 a;
+  asm volatile("ld.global.L2::64B.v4.f32 {%0, %1, %2, %3}, [%4];\n" : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(a.w) : "l"(p));
+  CV2 v;
+  v.re = make_float2(a.x, a.y);
+  v.im = make_float2(a.z, a.w);
+  return v;
+}
 __device__ __forceinline__ void sap_cp_async16(void* smem, const void* gmem) {
   const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem) : "memory");
+  asm volatile("cp.async.cg.shared.global.L2::64B [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem) : "memory");
+}
+__device__ __forceinline__ void sap_cp_async8(void* smem, const void* gmem) {
+  const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
+  asm volatile("cp.async.ca.shared.global.L2::64B [%0], [%1], 8;\n" ::"r"(sa), "l"(gmem) : "memory");
+}
+__device__ __forceinline__ void sap_cp_async4(void* smem, const void* gmem) {
+  const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
+  asm volatile("cp.async.ca.shared.global.L2::64B [%0], [%1], 4;\n" ::"r"(sa), "l"(gmem) : "memory");
 }
 __device__ __forceinline__ void sap_cp_async_wait() {
   asm volatile("cp.async.commit_group;\n" ::: "memory");
@@ -93,8 +112,16 @@ __device__ __forceinline__ void sap_cp_async_wait() {
 // packed FP32x2 arithmetic; CTA of ceil(bv / 32) * 32 threads (the threads past bv only take
 // part in the reductions and barriers).
 //
+// What bounds it: a 4^4 block fills the shared memory and, at 246 registers, the register file of an SM, so 8
+// warps have to cover their own waits (34% of the issue slots used; spills would go to L2, the L1 being all
+// shared memory). Hence asynchronous staging, few loads of rho (the dot products are taken while the local
+// term holds it), a reduction of 15 shuffles, no load of e in the first cycle, and e on its way to L2 while
+// the item runs. 32^3x64, 8 systems, 4 MR steps, per launch: 3.59 ms before these, 3.11 ms with them (1.4 ms at
+// the FP32 rate); 16^3x32, 12 systems: 342 and 303 us. Two threads per site (16 warps at 128 registers) measured
+// 3.9 ms: links and clover then pass through the shared-memory pipe twice.
+//
 // shared memory: links [4 nu][9][bv] float2, clover [72][bv] float, rho [12][bv] float4,
-// reduction scratch [2][nwarps][8] float
+// reduction scratch [2][2 nwarps] float4
 constexpr int SAP_THREADS = 256;
 constexpr int SAP_MAX_TILES = 128;  // system tiles per call (256 systems)
 
@@ -126,19 +153,21 @@ __device__ __forceinline__ int colour_block(const SapDims& d, int colour, int k)
   return ((c[3] * d.nb[2] + c[2]) * d.nb[1] + c[1]) * d.nb[0] + c[0];
 }
 
+// fresh: e holds nothing yet (e = correction; delta, which would equal it, is not written); else e += and
+// delta = correction
 __global__ void __launch_bounds__(SAP_THREADS, 1) sap_mr_kernel(const float2* __restrict__ U,
                                                                 const float* __restrict__ C, float* __restrict__ r,
                                                                 float* __restrict__ delta, float* __restrict__ e,
                                                                 const double* __restrict__ mu, int nsys, SapDims d,
                                                                 int colour, int steps, int nitems, int ntile,
-                                                                const double* __restrict__ eps) {
+                                                                const double* __restrict__ eps, int fresh) {
   constexpr int T = 2;  // systems per tile
   extern __shared__ float4 sm[];
   const int bv = d.bv;
   float2* Ls = reinterpret_cast<float2*>(sm);              // [4][9][bv]
   float* Cs = reinterpret_cast<float*>(Ls + 36 * bv);      // [72][bv]
   float4* rho = reinterpret_cast<float4*>(Cs + 72 * bv);   // [12][bv]
-  float* red = reinterpret_cast<float*>(rho + 12 * bv);    // [nwarps][8]
+  float4* red = rho + 12 * bv;                             // [2][2 nwarps]
   const int tid = threadIdx.x;
   const bool act = tid < bv;
   const int64_t V = (int64_t)d.L[0] * d.L[1] * d.L[2] * d.L[3];
@@ -186,9 +215,9 @@ __global__ void __launch_bounds__(SAP_THREADS, 1) sap_mr_kernel(const float2* __
         // links of the block: U_nu(x) for x in the block (forward hops, and backward hops
         // through the in-block neighbour x - nu, whose own forward link it is)
 #pragma unroll 12
-        for (int q = 0; q < 36; ++q) Ls[q * bv + tid] = U[(int64_t)q * V + s];
+        for (int q = 0; q < 36; ++q) sap_cp_async8(&Ls[q * bv + tid], U + (int64_t)q * V + s);
 #pragma unroll 12
-        for (int q = 0; q < 72; ++q) Cs[q * bv + tid] = C[(int64_t)q * V + s];
+        for (int q = 0; q < 72; ++q) sap_cp_async4(&Cs[q * bv + tid], C + (int64_t)q * V + s);
       }
 #pragma unroll
       for (int nu = 0; nu < 4; ++nu) {
@@ -226,6 +255,11 @@ __global__ void __launch_bounds__(SAP_THREADS, 1) sap_mr_kernel(const float2* __
       eb[k2].im = make_float2(0.f, 0.f);
     }
     sap_cp_async_wait();  // this thread's residual entries are in rho (the barrier below publishes them)
+    if (act && !fresh) {  // e is wanted at the end of the item: from HBM to L2 meanwhile
+#pragma unroll
+      for (int k2 = 0; k2 < 12; ++k2)
+        asm volatile("prefetch.global.L2 [%0];\n" ::"l"(e + tile * tstride + ((int64_t)k2 * V + s) * 2 * T));
+    }
     const float2 m2 = mu_s[tile];
     // doublet form (eps): the tile's two systems are the flavours of one doublet, one MR system
     const float ep = ep_s[tile];
@@ -252,25 +286,22 @@ __global__ void __launch_bounds__(SAP_THREADS, 1) sap_mr_kernel(const float2* __
         TM_BHOP(2)
         TM_BHOP(3)
 #undef TM_BHOP
-        local2(q, rb + tid * 4, bv, Cs, bv, tid, m2, ep);
-        // partial <q, q> and <q, rho> per system (packed over the two systems)
+        // the local term, and the partial <q, q> and <q, rho> per system (packed over the two systems)
         float2 qq = make_float2(0.f, 0.f), qr = qq, qi = qq;
-#pragma unroll
-        for (int k2 = 0; k2 < 12; ++k2) {
-          const float4 rr = rho[k2 * bv + tid];
-          const float2 rre = make_float2(rr.x, rr.y), rim = make_float2(rr.z, rr.w);
-          const CV2& qv = q.c[k2];
-          qq = fma2(qv.re, qv.re, qq);
-          qq = fma2(qv.im, qv.im, qq);
-          qr = fma2(qv.re, rre, qr);
-          qr = fma2(qv.im, rim, qr);
-          qi = fma2(qv.re, rim, qi);
-          qi = fma2(f2(-1.f), mul2(qv.im, rre), qi);
-        }
+        local2_of(
+            q, [&](int k2) { return ld2(rb + (k2 * bv + tid) * 4); }, Cs, bv, tid, m2, ep,
+            [&](const CV2& qv, const CV2& x) {
+              qq = fma2(qv.re, qv.re, qq);
+              qq = fma2(qv.im, qv.im, qq);
+              qr = fma2(qv.re, x.re, qr);
+              qr = fma2(qv.im, x.im, qr);
+              qi = fma2(qv.re, x.im, qi);
+              qi = fma2(f2(-1.f), mul2(qv.im, x.re), qi);
+            });
         v[0] = qq.x; v[1] = qr.x; v[2] = qi.x;
         v[3] = qq.y; v[4] = qr.y; v[5] = qi.y;
       }
-      block_reduce(v, red + (it & 1) * 8 * nwarps);  // its barrier: every q is computed, rho may change
+      block_reduce(v, red + (it & 1) * 2 * nwarps);  // its barrier: every q is computed, rho may change
       if (eps) {  // one minimal-residual step for the doublet: the dots summed over both flavours
 #pragma unroll
         for (int u = 0; u < 3; ++u) {
@@ -304,18 +335,27 @@ __global__ void __launch_bounds__(SAP_THREADS, 1) sap_mr_kernel(const float2* __
     if (act) {
       float* dt = delta + tile * tstride;
       float* et = e + tile * tstride;
-      // every load of e first (twelve in flight), then the stores
-      CV2 e0[12];
+      if (fresh) {
 #pragma unroll
-      for (int k2 = 0; k2 < 12; ++k2) e0[k2] = ld2(et + ((int64_t)k2 * V + s) * 2 * T);
+        for (int k2 = 0; k2 < 12; ++k2) {
+          const int64_t o = ((int64_t)k2 * V + s) * 2 * T;
+          st2(et + o, eb[k2]);
+          *reinterpret_cast<float4*>(rt + o) = rho[k2 * bv + tid];
+        }
+      } else {
+        // every load of e first (twelve in flight), then the stores
+        CV2 e0[12];
 #pragma unroll
-      for (int k2 = 0; k2 < 12; ++k2) {
-        const int64_t o = ((int64_t)k2 * V + s) * 2 * T;
-        st2(dt + o, eb[k2]);
-        e0[k2].re = add2(e0[k2].re, eb[k2].re);
-        e0[k2].im = add2(e0[k2].im, eb[k2].im);
-        st2(et + o, e0[k2]);
-        *reinterpret_cast<float4*>(rt + o) = rho[k2 * bv + tid];
+        for (int k2 = 0; k2 < 12; ++k2) e0[k2] = sap_ld(et + ((int64_t)k2 * V + s) * 2 * T);
+#pragma unroll
+        for (int k2 = 0; k2 < 12; ++k2) {
+          const int64_t o = ((int64_t)k2 * V + s) * 2 * T;
+          st2(dt + o, eb[k2]);
+          e0[k2].re = add2(e0[k2].re, eb[k2].re);
+          e0[k2].im = add2(e0[k2].im, eb[k2].im);
+          st2(et + o, e0[k2]);
+          *reinterpret_cast<float4*>(rt + o) = rho[k2 * bv + tid];
+        }
       }
     }
     // rho is private per thread from the last barrier on (neighbour reads ended before it): the
@@ -324,14 +364,83 @@ __global__ void __launch_bounds__(SAP_THREADS, 1) sap_mr_kernel(const float2* __
   }
 }
 
+// One block-crossing hop of the face update, its direction sign a value of the thread (sgn = +1 forward, -1
+// backward): the backward projection and scatter are the forward ones with the sign of K flipped, so one code
+// serves both faces of a block. r: the neighbour's spinor; W: the link, stride V, used as it is (forward) or
+// as its adjoint.
+__device__ __forceinline__ void ld_raw64(Raw2& r, const float* __restrict__ xs, int64_t cstride) {
+#pragma unroll
+  for (int k = 0; k < 12; ++k) r.v[k] = sap_ld(xs + (int64_t)k * cstride * 4);
+}
+template <int NU>
+__device__ __forceinline__ void face_hop(Spinor2& acc, const Raw2& r, const float2* __restrict__ W, int64_t V, bool fwd,
+                                         float phase) {
+  using P = Proj<NU, true>;
+  const float sg = fwd ? 1.f : -1.f;
+  // u + sgn K(d)
+  auto proj = [&](int K, const CV2& u, const CV2& d) {
+    CV2 h;
+    const float c = (K & 1) ? -sg : sg;  // K: +1, -1, +i, -i
+    if (K < 2) {
+      h.re = fma2(f2(c), d.re, u.re);
+      h.im = fma2(f2(c), d.im, u.im);
+    } else {
+      h.re = fma2(f2(-c), d.im, u.re);
+      h.im = fma2(f2(c), d.re, u.im);
+    }
+    return h;
+  };
+  CV2 h[2][3];
+#pragma unroll
+  for (int col = 0; col < 3; ++col) {
+    h[0][col] = proj(P::c0, r.v[col], r.v[(2 + P::p0) * 3 + col]);
+    h[1][col] = proj(P::c1, r.v[3 + col], r.v[(2 + P::p1) * 3 + col]);
+  }
+  const int64_t sa = fwd ? 3 * V : V, sb = fwd ? V : 3 * V;  // row and column strides of W (its adjoint backward)
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    float2 w[3];
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      w[b] = W[a * sa + b * sb];
+      w[b] = make_float2(w[b].x * phase, w[b].y * (sg * phase));
+    }
+    CV2 g[2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      g[k].re = mul2(f2(w[0].x), h[k][0].re);
+      g[k].im = mul2(f2(w[0].x), h[k][0].im);
+      g[k].re = fma2(f2(-w[0].y), h[k][0].im, g[k].re);
+      g[k].im = fma2(f2(w[0].y), h[k][0].re, g[k].im);
+#pragma unroll
+      for (int b = 1; b < 3; ++b) {
+        g[k].re = fma2(f2(w[b].x), h[k][b].re, g[k].re);
+        g[k].re = fma2(f2(-w[b].y), h[k][b].im, g[k].re);
+        g[k].im = fma2(f2(w[b].x), h[k][b].im, g[k].im);
+        g[k].im = fma2(f2(w[b].y), h[k][b].re, g[k].im);
+      }
+    }
+    acc2<0>(acc.c[a], g[0]);
+    acc2<0>(acc.c[3 + a], g[1]);
+    acc.c[6 + a] = proj(P::b0, acc.c[6 + a], g[P::p0]);
+    acc.c[9 + a] = proj(P::b1, acc.c[9 + a], g[P::p1]);
+  }
+}
+
 // r(s) -= (D delta)(s) on the sites of the blocks of colour `other`, where delta is nonzero
 // only on the blocks of the other colour: only hops across a block face contribute,
 // D's hop term is -1/2 sum hops, so r += 1/2 sum_{crossing hops} hop(delta).
-template <typename real, int T>
-__global__ void __launch_bounds__(256) sap_face_kernel(const float2* __restrict__ U, const real* __restrict__ delta,
-                                                       real* __restrict__ r, SapDims d, int other, int ntile) {
+//
+// A site crosses at most once per direction (blocks of extent one cross both ways: the second pass), so a
+// direction is one body for both faces of a block. The kernel is bound by memory: its rows of 64 bytes
+// alternate with rows of the other colour, and with whole lines fetched for every load it moved 423 MB where
+// 281 MB suffice (16^3x32, 12 systems: 114 us; with 64-byte requests 82 us; 32^3x64, 8 systems: 1.10 and
+// 0.80 ms; 0.4 ms at the HBM rate). Loading the next direction ahead (168 registers) measured slower.
+__global__ void __launch_bounds__(128, 4) sap_face_kernel(const float2* __restrict__ U, const float* __restrict__ delta,
+                                                          float* __restrict__ r, SapDims d, int other, int ntile) {
   // threads over the sites of the blocks of colour `other` only (block k of that colour, site q
   // in the block), so that no lane of a warp idles on a site of the wrong colour
+  constexpr int T = 2;
   const int64_t V = (int64_t)d.L[0] * d.L[1] * d.L[2] * d.L[3];
   const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int tile = blockIdx.y;
@@ -341,51 +450,56 @@ __global__ void __launch_bounds__(256) sap_face_kernel(const float2* __restrict_
   int bc[4], lc[4], c[4];
   block_site(d, colour_block(d, other, k), q, bc, lc, c);
   const int64_t s = site_index(c, d.L);
-  bool fwd[4], bwd[4];
-#pragma unroll
-  for (int nu = 0; nu < 4; ++nu) {
-    fwd[nu] = d.nb[nu] > 1 && lc[nu] == d.bs[nu] - 1;
-    bwd[nu] = d.nb[nu] > 1 && lc[nu] == 0;
-  }
-  if (!(fwd[0] || fwd[1] || fwd[2] || fwd[3] || bwd[0] || bwd[1] || bwd[2] || bwd[3])) return;
+  const int64_t strides[4] = {1, (int64_t)d.L[0], (int64_t)d.L[0] * d.L[1], (int64_t)d.L[0] * d.L[1] * d.L[2]};
   const int64_t tstride = (int64_t)12 * V * 2 * T;
-  const real* dt = delta + tile * tstride;
-  static_assert(sizeof(real) == 4 && T == 2, "packed FP32 tiles");
+  const float* dt = delta + tile * tstride;
   Spinor2 acc;
 #pragma unroll
-  for (int k = 0; k < 12; ++k) {
-    acc.c[k].re = make_float2(0.f, 0.f);
-    acc.c[k].im = make_float2(0.f, 0.f);
+  for (int j = 0; j < 12; ++j) {
+    acc.c[j].re = make_float2(0.f, 0.f);
+    acc.c[j].im = make_float2(0.f, 0.f);
   }
-  const int64_t strides[4] = {1, (int64_t)d.L[0], (int64_t)d.L[0] * d.L[1], (int64_t)d.L[0] * d.L[1] * d.L[2]};
-#define TM_FHOP(NU)                                                                                   \
-  {                                                                                                   \
-    if (fwd[NU]) {                                                                                    \
-      int64_t sf = c[NU] + 1 < d.L[NU] ? s + strides[NU] : s - (int64_t)(d.L[NU] - 1) * strides[NU];  \
-      real ph = (NU == 3 && c[3] == d.L[3] - 1) ? (real)d.bc_t : real(1);                           \
-      hop2<NU, true>(acc, dt + sf * 2 * T, V, U + (int64_t)NU * 9 * V, V, s, ph);                      \
-    }                                                                                                 \
-    if (bwd[NU]) {                                                                                    \
-      int64_t sb = c[NU] > 0 ? s - strides[NU] : s + (int64_t)(d.L[NU] - 1) * strides[NU];             \
-      real ph = (NU == 3 && c[3] == 0) ? (real)d.bc_t : real(1);                                     \
-      hop2<NU, false>(acc, dt + sb * 2 * T, V, U + (int64_t)NU * 9 * V, V, sb, ph);                    \
-    }                                                                                                 \
-  }
-  TM_FHOP(0)
-  TM_FHOP(1)
-  TM_FHOP(2)
-  TM_FHOP(3)
-#undef TM_FHOP
-  real* rt = r + tile * tstride;
+  bool any = false;
+#pragma unroll 1
+  for (int pass = 0; pass < 2; ++pass) {
+    bool on[4], fwd[4];
+    int64_t nb[4];
 #pragma unroll
-  for (int k = 0; k < 12; ++k) {
-    int64_t o = ((int64_t)k * V + s) * 2 * T;
-    float4 v = *reinterpret_cast<const float4*>(rt + o);
-    v.x += 0.5f * acc.c[k].re.x;
-    v.y += 0.5f * acc.c[k].re.y;
-    v.z += 0.5f * acc.c[k].im.x;
-    v.w += 0.5f * acc.c[k].im.y;
-    *reinterpret_cast<float4*>(rt + o) = v;
+    for (int nu = 0; nu < 4; ++nu) {
+      const bool up = d.nb[nu] > 1 && lc[nu] == d.bs[nu] - 1, dn = d.nb[nu] > 1 && lc[nu] == 0;
+      fwd[nu] = up && pass == 0;
+      on[nu] = pass == 0 ? up || dn : up && dn;
+      nb[nu] = fwd[nu] ? (c[nu] + 1 < d.L[nu] ? s + strides[nu] : s - (int64_t)(d.L[nu] - 1) * strides[nu])
+                       : (c[nu] > 0 ? s - strides[nu] : s + (int64_t)(d.L[nu] - 1) * strides[nu]);
+      any |= on[nu];
+    }
+    if (pass == 1 && !(d.bs[0] == 1 || d.bs[1] == 1 || d.bs[2] == 1 || d.bs[3] == 1)) break;
+    const float pt = c[3] == (fwd[3] ? d.L[3] - 1 : 0) ? (float)d.bc_t : 1.f;
+#define TM_FHOP(NU)                                                                                     \
+    {                                                                                                   \
+      if (on[NU]) {                                                                                     \
+        Raw2 raw;                                                                                       \
+        ld_raw64(raw, dt + nb[NU] * 2 * T, V);                                                          \
+        face_hop<NU>(acc, raw, U + (int64_t)NU * 9 * V + (fwd[NU] ? s : nb[NU]), V, fwd[NU], NU == 3 ? pt : 1.f); \
+      }                                                                                                 \
+    }
+    TM_FHOP(0)
+    TM_FHOP(1)
+    TM_FHOP(2)
+    TM_FHOP(3)
+#undef TM_FHOP
+  }
+  if (!any) return;
+  float* rt = r + tile * tstride;
+  CV2 rv[12];
+#pragma unroll
+  for (int j = 0; j < 12; ++j) rv[j] = sap_ld(rt + ((int64_t)j * V + s) * 2 * T);
+#pragma unroll
+  for (int j = 0; j < 12; ++j) {
+    const int64_t o = ((int64_t)j * V + s) * 2 * T;
+    *reinterpret_cast<float4*>(rt + o) = make_float4(
+        rv[j].re.x + 0.5f * acc.c[j].re.x, rv[j].re.y + 0.5f * acc.c[j].re.y, rv[j].im.x + 0.5f * acc.c[j].im.x,
+        rv[j].im.y + 0.5f * acc.c[j].im.y);
   }
 }
 
@@ -428,14 +542,12 @@ void sap_apply(const Geom& g, const int bs[4], const float2* U32, const float* C
     if (d.nb[k] >= 2) d.pdim = k;
   constexpr int T = Tile<float>::T;
   int nt = ntiles(nsys, T);
-  size_t M = (size_t)12 * g.V * 2 * T * nt;
-  if (!accumulate) cudaMemsetAsync(e, 0, M * sizeof(float), st);
   const int nthreads = (d.bv + 31) / 32 * 32;  // one thread per block site
   const int nwarps = nthreads / 32;
   if (nt > SAP_MAX_TILES) return;  // callers check (at most 256 systems)
   // links [4][9][bv] float2 + clover [72][bv] + rho [12][bv] float4 + reduction scratch (two buffers)
   size_t smem = sizeof(float2) * 36 * d.bv + sizeof(float) * 72 * d.bv + sizeof(float4) * 12 * d.bv +
-                sizeof(float) * 2 * 8 * nwarps;
+                sizeof(float4) * 4 * nwarps;
   const int sms = device_sms();
   func_smem_optin((const void*)sap_mr_kernel, 200 * 1024);
   // persistent grid: as many CTAs as fit on the device at once (smaller blocks fit two per SM)
@@ -448,19 +560,22 @@ void sap_apply(const Geom& g, const int bs[4], const float2* U32, const float* C
     for (int colour = 0; colour < 2; ++colour) {
       const int nb_c = d.pdim < 0 ? (colour == 0 ? 1 : 0) : per_colour;
       const int nitems = nb_c * nt;
+      // from a zero start the first cycle's corrections are e itself: both colours cover every site
+      const int fresh = !accumulate && cy == 0;
       if (nitems > 0) {
         const int grid = nitems < sms * per_sm ? nitems : sms * per_sm;
         TM_PROF(st, "sap_mr");
         sap_mr_kernel<<<grid, nthreads, smem, st>>>(U32, C32, r, delta, e, mu, nsys, d, colour, steps, nitems, nt,
-                                                    eps);
+                                                    eps, fresh);
         TM_COUNT();
       }
       bool last = (cy == cycles - 1) && colour == 1;
       if (!last && d.pdim >= 0) {
         TM_PROF(st, "sap_face");
         const int64_t nsite = (int64_t)(nblocks / 2) * d.bv;  // sites of the blocks of the other colour
-        sap_face_kernel<float, T><<<dim3((unsigned)((nsite + 255) / 256), nt), 256, 0, st>>>(U32, delta, r, d,
-                                                                                            1 - colour, nt); TM_COUNT();
+sap_face_kernel<<<dim3((unsigned)((nsite + 127) / 128), nt), 128, 0, st>>>(U32, fresh ? e : delta, r, d,
+                                                                                   1 - colour, nt);
+        TM_COUNT();
       }
     }
   }

@@ -1367,15 +1367,20 @@ int tmamg_sap(tmamg_ctx* ctx, void* r_bundle, void* e_bundle, int nsys, const do
   if (sap_check_blocks(ctx->g, block, why)) return set_err(ctx, TMAMG_ERR_ARG, "sap: " + why);
   int rc = upload_mu(ctx, mu, nsys);
   if (rc) return rc;
-  float* delta = nullptr;
-  size_t bytes = (size_t)ntiles(nsys, 2) * 12 * ctx->g.V * 4 * sizeof(float);
-  rc = with_optional_memory(ctx, [&] { return check_cuda(ctx, cudaMalloc(&delta, bytes), "cudaMalloc(sap scratch)"); });
-  if (rc) return rc;
-  sap_apply(ctx->g, block, ctx->U32, ctx->C32, (float*)r_bundle, (float*)e_bundle, delta, ctx->mu_dev, nsys, cycles,
-            mr_steps, ctx->stream);
+  // the correction buffer stays with the context: allocating and freeing it cost more than a small smoother
+  const size_t bytes = (size_t)ntiles(nsys, 2) * 12 * ctx->g.V * 4 * sizeof(float);
+  if (bytes > ctx->sap_delta_bytes) {
+    free_sap_delta(ctx);
+    rc = with_optional_memory(ctx, [&] {
+      return check_cuda(ctx, cudaMalloc(&ctx->sap_delta, bytes), "cudaMalloc(sap scratch)");
+    });
+    if (rc) return rc;
+    ctx->sap_delta_bytes = bytes;
+  }
+  sap_apply(ctx->g, block, ctx->U32, ctx->C32, (float*)r_bundle, (float*)e_bundle, ctx->sap_delta, ctx->mu_dev, nsys,
+            cycles, mr_steps, ctx->stream);
   rc = check_cuda(ctx, cudaGetLastError(), "sap launch");
   cudaStreamSynchronize(ctx->stream);
-  cudaFree(delta);
   return rc;
 }
 

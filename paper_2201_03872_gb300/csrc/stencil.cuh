@@ -395,10 +395,11 @@ __device__ __forceinline__ void mul_acc2(Spinor2& acc, const CV2 (&h)[2][3], con
 // local_term<> for FP32 tiles of two systems in packed arithmetic: acc <- A_chi x_chi +
 // i s mu x_chi - 1/2 acc per chirality; mu: the two systems' twisted masses. ep != 0: the tile's two
 // systems are the flavours of a non-degenerate doublet, coupled by -ep (each lane gets -ep times
-// the other lane's entry). entry(k): component k of the site's own spinor
-template <class Entry>
+// the other lane's entry). entry(k): component k of the site's own spinor; done(acc_k, x_k) is called with
+// every finished component and the site's own entry
+template <class Entry, class Done>
 __device__ __forceinline__ void local2_of(Spinor2& acc, Entry entry, const float* __restrict__ C, int64_t V, int64_t s,
-                                          float2 mu, float ep) {
+                                          float2 mu, float ep, Done done) {
 #pragma unroll
   for (int chi = 0; chi < 2; ++chi) {
     const float* Cc = C + (int64_t)chi * 36 * V + s;
@@ -438,6 +439,7 @@ __device__ __forceinline__ void local2_of(Spinor2& acc, Entry entry, const float
       CV2& hv = acc.c[chi * 6 + i];
       hv.re = fma2(f2(-0.5f), hv.re, o.re);
       hv.im = fma2(f2(-0.5f), hv.im, o.im);
+      done(hv, xc[i]);
     }
   }
 }
@@ -446,12 +448,13 @@ __device__ __forceinline__ void local2_of(Spinor2& acc, Entry entry, const float
 __device__ __forceinline__ void local2(Spinor2& acc, const float* __restrict__ x0, int64_t cstride,
                                        const float* __restrict__ C, int64_t V, int64_t s, float2 mu,
                                        float ep = 0.f) {
-  local2_of(acc, [&](int k) { return ld2(x0 + (int64_t)k * cstride * 4); }, C, V, s, mu, ep);
+  local2_of(acc, [&](int k) { return ld2(x0 + (int64_t)k * cstride * 4); }, C, V, s, mu, ep,
+            [](const CV2&, const CV2&) {});
 }
 // the site's own spinor in registers
 __device__ __forceinline__ void local2(Spinor2& acc, const Raw2& r, const float* __restrict__ C, int64_t V, int64_t s,
                                        float2 mu, float ep) {
-  local2_of(acc, [&](int k) { return r.v[k]; }, C, V, s, mu, ep);
+  local2_of(acc, [&](int k) { return r.v[k]; }, C, V, s, mu, ep, [](const CV2&, const CV2&) {});
 }
 
 }  // namespace tmamg
