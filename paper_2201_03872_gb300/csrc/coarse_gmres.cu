@@ -897,7 +897,7 @@ int coarse_gmres_solve(CoarseGmres& s, const CoarseDims& cd, const float2* A, co
   if (G > s.G || m > s.m || nsys > s.NS || m > CG_MAXM || cd.nc > 64 || (cd.nc % 2) || need > s.hbytes) return -2;
   const size_t cap = dyn_smem_cap();
   const int nstage = A16 ? cm_nstage(cd.nc, nsys, cap) : 0;
-  if (A16 && (nstage < 2 || cm_x16_bytes(cd.Vc, cd.nc, nsys) > s.x16_bytes)) return -2;
+  if (A16 && (nstage == 0 || cm_x16_bytes(cd.Vc, cd.nc, nsys) > s.x16_bytes)) return -2;
   const size_t dyn = dyn_smem_bytes(m, cd.nc, nsys, A16 != nullptr, nstage);
   if (dyn > cap) return -2;
   CGArgs p;

@@ -105,7 +105,7 @@ int coarse_apply_f16(const CoarseDims& cd, const __half* A16, const float* x, fl
   if (nsys <= 0) return 0;
   if (cd.nc > CM_MAXNC || cd.nc < 1 || nsys > CM_MAXSYS) return -2;
   const int nstage = cm_nstage(cd.nc, nsys, cap);
-  if (nstage < 2) return -2;
+  if (nstage == 0) return -2;
   const int nt = ntiles(nsys, 2);
   const int64_t M = (int64_t)cd.nc * cd.Vc;
   cudaMemsetAsync(mx, 0, sizeof(float) * nsys, st);

@@ -18,9 +18,9 @@
 // Both operands are kept in HBM in the no-swizzle K-major core-matrix layout (8 rows x 16 B per
 // core matrix, contiguous) in which the tensor cores read them from shared memory: the
 // operator once (setup), the B images of a vector by a conversion pass before each product.
-// The product is then a pipeline of bulk copies (one producer thread), MMAs (one issuing
-// thread) and a tensor-memory epilogue (two warps), over a ring of shared-memory stages of
-// one hop each and two accumulators. The accumulator uses M = 128 rows of which the first nc
+// The product is then a pipeline of bulk copies (one producer lane per stage), MMAs (one issuing
+// thread per accumulator) and a tensor-memory epilogue (two warps), over a ring of shared-memory stages of
+// three hops each and two accumulators. The accumulator uses M = 128 rows of which the first nc
 // are read; the descriptor's remaining row groups alias other staged data and are never read.
 #pragma once
 #include <cuda_fp16.h>
@@ -37,6 +37,10 @@ constexpr int CM_TMEM_COLS = 64;  // tensor-memory columns held per CTA (two acc
 constexpr int CM_SLACK = 2048;    // bytes past the last stage the M = 128 descriptor may touch
 constexpr int CM_MAXNC = 64;      // rows of D read back by the two epilogue warps
 constexpr int CM_MAXSTG = 16;     // stages in the shared-memory ring
+// hops per stage: a stage costs its issuing thread a wait and a commit of about 440 cycles together, as much as
+// eight MMAs, and its operator blocks are one copy
+constexpr int CM_HOPS = 3;
+constexpr int CM_USTG = 9 / CM_HOPS;  // stages of a unit (one site, one chunk)
 constexpr int CM_EPI0 = 4;        // first epilogue warp (warps 4 and 5 read TMEM lanes 0..63)
 constexpr int CM_TAB = 256;       // systems whose epilogue factors are tabulated in shared memory per call
 
@@ -54,13 +58,13 @@ __host__ __device__ inline int64_t cm_img_bytes(int nc, int S) { return 8LL * cm
 inline size_t cm_x16_bytes(int64_t Vc, int nc, int nsys) {
   return (size_t)Vc * cm_nchunk(nsys) * cm_img_bytes(nc, cm_chunk(nsys));
 }
-inline size_t cm_stage_bytes(int nc, int S) { return (size_t)(cm_hop_bytes(nc) + cm_img_bytes(nc, S)); }
-// stages that fit in cap bytes of dynamic shared memory (0 if fewer than two)
+inline size_t cm_stage_bytes(int nc, int S) { return (size_t)CM_HOPS * (cm_hop_bytes(nc) + cm_img_bytes(nc, S)); }
+// stages that fit in cap bytes of dynamic shared memory (0 if not a unit's; n_c = 64 with 16 systems takes
+// 223 KB for its three)
 inline int cm_nstage(int nc, int nsys, size_t cap) {
-  const size_t st = cm_stage_bytes(nc, cm_chunk(nsys));
-  if (cap < CM_SLACK + 2 * st) return 0;
-  const size_t n = (cap - CM_SLACK) / st;
-  return n < (size_t)CM_MAXSTG ? (int)n : CM_MAXSTG;
+  if (cap < CM_SLACK) return 0;
+  const size_t n = (cap - CM_SLACK) / cm_stage_bytes(nc, cm_chunk(nsys));
+  return n < (size_t)CM_USTG ? 0 : n < (size_t)CM_MAXSTG ? (int)n : CM_MAXSTG;
 }
 inline size_t cm_smem_bytes(int nc, int nsys, int nstage) {
   return (size_t)nstage * cm_stage_bytes(nc, cm_chunk(nsys)) + CM_SLACK;
@@ -71,6 +75,7 @@ struct CmShared {
   unsigned long long tfull[CM_ACCS], tempty[CM_ACCS];    // accumulator ready / drained
   unsigned tmem;
   int fail;
+  int seen[CM_ACCS];  // per MMA issuer: stages (counted over the whole pipeline) it has seen loaded
   // per-system epilogue factors of the current call (systems n < CM_TAB): output scale so[n] and
   // twist dmu mu_n si[n], in FP32, so that the epilogue does no FP64 arithmetic (FP64 runs at a
   // small fraction of the FP32 rate on this GPU)
@@ -86,6 +91,7 @@ struct CmPipe {
   unsigned phase = 0;
   int acc = 0;
   unsigned aphase = 0;
+  int count = 0;  // stages of the units passed so far
 };
 
 // per-system scaling of the FP16 vector entries (the FP16 range is kept for any input):
@@ -127,6 +133,7 @@ __device__ __forceinline__ bool cm_try_wait(uint32_t mb, uint32_t parity) {
 
 // bounded wait (about one second at 2 GHz); gives up early when another thread failed
 __device__ __forceinline__ bool cm_wait(uint32_t mb, uint32_t parity, volatile int* fail) {
+  if (cm_try_wait(mb, parity)) return true;
   const long long t0 = clock64();
   while (!cm_try_wait(mb, parity)) {
     if (*fail) return false;
@@ -164,6 +171,7 @@ __device__ __forceinline__ void cm_begin(CmShared& cs) {
     }
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     cs.fail = 0;
+    for (int k = 0; k < CM_ACCS; ++k) cs.seen[k] = 0;
   }
   if (threadIdx.x < 32) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(cm_smem(&cs.tmem)),
@@ -246,9 +254,10 @@ __device__ __forceinline__ int cm_neighbour(const CmCoord& k, int h, int L0, int
   return ((c3 * L2 + c2) * L1 + c1) * L0 + c0;
 }
 
-// The B images of x for all sites: item = ((a chunks + c) TP + tp) MG + g covers the eight
-// components 8g .. 8g+7 of tile c TP + tp at site a. sin: input factor per system (shared
-// memory, [nsys]). Items first .. total step stride; the caller fences the generic writes
+// The B images of x for all sites: item = ((c TP + tp) MG + g) Vc + a covers the eight components 8g .. 8g+7
+// of tile c TP + tp at site a (consecutive items are consecutive sites, so that a warp reads whole lines of
+// the bundle; with the site slowest a product's conversion took twice as long). sin: input factor per system
+// (shared memory, [nsys]). Items first .. total step stride; the caller fences the generic writes
 // against the bulk copies that read them (fence.proxy.async.global) before its barrier.
 __device__ __forceinline__ void cm_convert(const float* __restrict__ x, __half* X16, int64_t Vc, int nc, int nsys,
                                            const float* sin, int64_t first, int64_t stride) {
@@ -259,12 +268,12 @@ __device__ __forceinline__ void cm_convert(const float* __restrict__ x, __half* 
   const int64_t total = Vc * nchunk * TP * MG;
   for (int64_t item = first; item < total; item += stride) {
     const int it32 = (int)item;  // Vc * chunks * TP * MG < 2^31 for every supported size
-    const int g = it32 % MG;
-    int r = it32 / MG;
+    const int64_t a = it32 % (int)Vc;
+    int r = it32 / (int)Vc;
+    const int g = r % MG;
+    r /= MG;
     const int tp = r % TP;
-    r /= TP;
-    const int c = r % nchunk;
-    const int64_t a = r / nchunk;
+    const int c = r / TP;
     const int t = c * TP + tp;
     float4 v[8];
 #pragma unroll
@@ -297,21 +306,127 @@ __device__ __forceinline__ void cm_convert(const float* __restrict__ x, __half* 
 
 __device__ __forceinline__ void cm_fence_global_async() { asm volatile("fence.proxy.async.global;\n" ::: "memory"); }
 
-// The stencil over the units (site a, chunk c), a = cta, cta + ncta, ..., from the B images in
-// q.X16 (every thread of the CTA calls it). Thread 0 loads stages (operator block of one hop
-// plus the B image of that hop's neighbour), thread 32 issues the MMAs of a unit into one of
-// two accumulators, warps 4 and 5 drain an accumulator while the next unit accumulates.
+// bounded wait until *seen has reached `want` (stages of one launch: far below 2^31; <= 0: before stage 0)
+__device__ __forceinline__ bool cm_wait_seen(volatile int* seen, int want, volatile int* fail) {
+  if (want <= 0 || *seen >= want) return true;
+  const long long t0 = clock64();
+  while (*seen < want) {
+    if (*fail) return false;
+    if (clock64() - t0 > 2000000000LL) {
+      *fail = 1;
+      return false;
+    }
+  }
+  return true;
+}
+
+// the stages of a unit passed (the ring holds at least a unit)
+__device__ __forceinline__ void cm_advance_unit(CmPipe& pipe, int NS) {
+  pipe.count += CM_USTG;
+  pipe.stage += CM_USTG;
+  if (pipe.stage >= NS) {
+    pipe.stage -= NS;
+    pipe.phase ^= 1u;
+  }
+}
+
+// The MMAs of one hop's stage into the accumulator at TMEM address dt: KS steps over [Re | Im]. Fully
+// unrolled: the k-step descriptors are the stage's plus constants (the start-address field, address / 16 in
+// 14 bits, advances by the k offset; every address stays below 2^18 bytes, so there is no carry), and the
+// issuing thread spends most of its time on moving descriptors to uniform registers.
+template <int KS>
+__device__ __forceinline__ void cm_issue_hop(uint32_t dt, uint64_t ad, uint64_t bd, uint32_t astep, uint32_t bstep,
+                                             uint32_t idesc, uint32_t accum0) {
+#pragma unroll
+  for (int k = 0; k < KS; ++k) {
+    const uint32_t accum = k == 0 ? accum0 : 1u;
+    asm volatile(
+        "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(dt),
+        "l"(ad + (uint64_t)(k * astep)), "l"(bd + (uint64_t)(k * bstep)), "r"(idesc), "r"(accum));
+  }
+}
+
+// The MMA role (one thread per accumulator): nine hops x KS steps for every unit that goes to accumulator
+// `mine`; the units alternate between the accumulators, so the two threads' issuing overlaps. A stage holds
+// CM_HOPS operator blocks and behind them their images.
+// A wait on a barrier's parity is only meaningful within one phase of it: before a thread waits for the
+// load of stage number g it makes sure that the other thread has seen the slot's previous load (number
+// g - NS, where that belongs to the other's unit).
+template <int KS>
+__device__ __forceinline__ void cm_mma_role(const CmArgs& q, CmShared& cs, CmPipe& pipe, int mine, uint32_t s0,
+                                            uint32_t HA, uint32_t IB, int N, int NG, int nchunk, int64_t cta,
+                                            int64_t ncta) {
+  constexpr int MG = KS;  // row groups of A, one K step of 16 per group of 8 components
+  volatile int* fail = &cs.fail;
+  const int NS = q.nstage;
+  const uint32_t idesc = (1u << 4)                        // FP32 accumulator
+                         | ((uint32_t)(N >> 3) << 17)     // N
+                         | ((uint32_t)(128 >> 4) << 24);  // M = 128; FP16 A and B, both K-major
+  const uint32_t astep = (2 * MG * 128) >> 4, bstep = (uint32_t)(2 * NG * 128) >> 4;
+  for (int64_t a = q.Vc * cta / ncta, a1 = q.Vc * (cta + 1) / ncta; a < a1 && !*fail; ++a)
+    for (int c = 0; c < nchunk && !*fail; ++c) {
+      const int d = pipe.acc;
+      if (d == mine) {
+        if (!cm_wait(cm_smem(&cs.tempty[d]), pipe.aphase ^ 1u, fail)) return;
+        cm_fence_after();
+        const uint32_t dt = cs.tmem + (uint32_t)(d * 32);
+        int st = pipe.stage;
+        unsigned ph = pipe.phase;
+#pragma unroll 1
+        for (int h = 0; h < CM_USTG; ++h) {
+          const int g = pipe.count + h;
+          if (h >= NS - CM_USTG && !cm_wait_seen(&cs.seen[mine ^ 1], g - NS + 1, fail)) return;
+          if (!cm_wait(cm_smem(&cs.full[st]), ph, fail)) return;
+          *(volatile int*)&cs.seen[mine] = g + 1;
+          cm_fence_after();
+          const uint32_t ab = s0 + st * CM_HOPS * (HA + IB);
+#pragma unroll 1
+          for (int j = 0; j < CM_HOPS; ++j)
+            cm_issue_hop<KS>(dt, cm_desc(ab + j * HA, MG * 128, 128), cm_desc(ab + CM_HOPS * HA + j * IB, NG * 128, 128),
+                             astep, bstep, idesc, h + j != 0);
+          // the stage is free once these MMAs have read it
+          asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
+                           cm_smem(&cs.empty[st]))
+                       : "memory");
+          if (++st == NS) {
+            st = 0;
+            ph ^= 1u;
+          }
+        }
+        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
+                         cm_smem(&cs.tfull[d]))
+                     : "memory");
+      }
+      cm_advance_unit(pipe, NS);
+      if (++pipe.acc == CM_ACCS) {
+        pipe.acc = 0;
+        pipe.aphase ^= 1u;
+      }
+    }
+}
+
+// The stencil over the units (site a, chunk c) of the CTA's contiguous share of the sites, from the B images in
+// q.X16 (every thread of the CTA calls it). Lanes of warp 0 load the stages of a unit (the operator blocks of
+// CM_HOPS hops plus the B images of those hops' neighbours), threads 32 and 64 issue the MMAs of the units of
+// their accumulator, warps 4 and 5 drain an accumulator while the other one accumulates.
 // pipe: this thread's role state. Returns false when a bounded wait gave up (q.err = 2).
+//
+// Bound by HBM: the operator passes once (680 of 790 MB at 32^3x64, n_c = 48, 16 systems), 162 us, 5.2 TB/s
+// of DRAM traffic. What it took, each alone (same size): one producer thread and one issuer, one hop per stage
+// 275 us (a unit was as long as its issuing thread, which spends about 440 cycles on a stage's wait and commit
+// and 55 per MMA, whatever M and N); one producer lane per stage and unrolled K steps 208 us; an issuer per
+// accumulator 180 us; contiguous sites per CTA, so that neighbours share lines of x, y and images 172 us (the
+// twist's entries loaded a unit ahead and three hops per stage take another 1 us); the operator evicted first from
+// L2, where it had pushed out images that eight more sites read (955 to 815 MB read) 162 us.
 static __device__ __forceinline__ bool cm_apply(const CmArgs& q, CmShared& cs, unsigned char* dsm, CmPipe& pipe,
                                                 int64_t cta, int64_t ncta) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int nc = q.nc, ncp = cm_ncp(nc);
-  const int MG = ncp / 8;   // row groups of A (and k-groups per half of K)
-  const int KS = ncp / 8;   // K steps of 16 over [Re | Im]
   const int S = cm_chunk(q.nsys), N = 2 * S, NG = S / 4, TP = S / 2;
   const int nchunk = cm_nchunk(q.nsys);
   const int nt = (q.nsys + 1) / 2;
-  const uint32_t HA = (uint32_t)cm_hop_bytes(nc), IB = (uint32_t)cm_img_bytes(nc, S), ST = HA + IB;
+  const uint32_t HA = (uint32_t)cm_hop_bytes(nc), IB = (uint32_t)cm_img_bytes(nc, S), ST = CM_HOPS * (HA + IB);
   const int NS = q.nstage;
   volatile int* fail = &cs.fail;
   // shared memory last written through the generic proxy (other phases) is next written by
@@ -327,110 +442,91 @@ static __device__ __forceinline__ bool cm_apply(const CmArgs& q, CmShared& cs, u
   __syncthreads();
   const uint32_t s0 = cm_smem(dsm);
 
-  if (tid == 0) {
-    // ---- producer: one stage per (unit, hop)
-    cm_fence_global_async();
-    const unsigned char* Ag = reinterpret_cast<const unsigned char*>(q.A16);
-    const unsigned char* Xg = reinterpret_cast<const unsigned char*>(q.X16);
-    const int L0 = q.L[0], L1 = q.L[1], L2 = q.L[2], L3 = q.L[3];
-    for (int64_t a = cta; a < q.Vc && !*fail; a += ncta) {
-      const CmCoord kc = cm_coords((int)a, L0, L1, L2);
-      int nbs[9];
-#pragma unroll
-      for (int h = 0; h < 9; ++h) nbs[h] = cm_neighbour(kc, h, L0, L1, L2, L3);
-      for (int c = 0; c < nchunk && !*fail; ++c)
-#pragma unroll 1
-        for (int h = 0; h < 9; ++h) {
-          const int st = pipe.stage;
-          if (!cm_wait(cm_smem(&cs.empty[st]), pipe.phase ^ 1u, fail)) break;
-          const uint32_t fb = cm_smem(&cs.full[st]);
-          asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(fb), "r"(ST) : "memory");
-          int nb = nbs[0];
-#pragma unroll
-          for (int q2 = 1; q2 < 9; ++q2)
-            if (h == q2) nb = nbs[q2];
-          asm volatile(
-              "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(
-                  s0 + st * ST),
-              "l"(Ag + (a * 9 + h) * (int64_t)HA), "r"(HA), "r"(fb)
-              : "memory");
-          asm volatile(
-              "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(
-                  s0 + st * ST + HA),
-              "l"(Xg + ((int64_t)nb * nchunk + c) * (int64_t)IB), "r"(IB), "r"(fb)
-              : "memory");
-          if (++pipe.stage == NS) {
-            pipe.stage = 0;
-            pipe.phase ^= 1u;
+  if (warp == 0) {
+    // ---- producer: lane h for stage h of a unit. The lanes keep step (the warp barrier), so that every
+    // slot's previous load has been issued when a lane waits for the slot.
+    if (lane < CM_USTG) {
+      cm_fence_global_async();
+      const unsigned mask = (1u << CM_USTG) - 1u;
+      // the last chunk's operator makes way in L2 for the images, which nine sites read
+      uint64_t last, again;
+      asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;\n" : "=l"(last));
+      asm("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;\n" : "=l"(again));
+      const unsigned char* Ag = reinterpret_cast<const unsigned char*>(q.A16);
+      const unsigned char* Xg = reinterpret_cast<const unsigned char*>(q.X16);
+      const int L0 = q.L[0], L1 = q.L[1], L2 = q.L[2], L3 = q.L[3];
+      for (int64_t a = q.Vc * cta / ncta, a1 = q.Vc * (cta + 1) / ncta; a < a1; ++a) {
+        const CmCoord kc = cm_coords((int)a, L0, L1, L2);
+        for (int c = 0; c < nchunk; ++c) {
+          int st = pipe.stage + lane;
+          unsigned ph = pipe.phase;
+          if (st >= NS) {
+            st -= NS;
+            ph ^= 1u;
           }
-        }
-    }
-  } else if (tid == 32) {
-    // ---- MMA issuer: nine hops x KS steps per unit into accumulator pipe.acc
-    const uint32_t idesc = (1u << 4)                        // FP32 accumulator
-                           | ((uint32_t)(N >> 3) << 17)     // N
-                           | ((uint32_t)(128 >> 4) << 24);  // M = 128; FP16 A and B, both K-major
-    for (int64_t a = cta; a < q.Vc && !*fail; a += ncta)
-      for (int c = 0; c < nchunk && !*fail; ++c) {
-        const int d = pipe.acc;
-        if (!cm_wait(cm_smem(&cs.tempty[d]), pipe.aphase ^ 1u, fail)) break;
-        cm_fence_after();
-        const uint32_t dt = cs.tmem + (uint32_t)(d * 32);
-        bool ok = true;
-        for (int h = 0; h < 9; ++h) {
-          const int st = pipe.stage;
-          if (!cm_wait(cm_smem(&cs.full[st]), pipe.phase, fail)) {
-            ok = false;
+          if (cm_wait(cm_smem(&cs.empty[st]), ph ^ 1u, fail)) {
+            const uint32_t fb = cm_smem(&cs.full[st]);
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(fb), "r"(ST) : "memory");
+            asm volatile(
+                "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], "
+                "%4;\n" ::"r"(s0 + st * ST),
+                "l"(Ag + (a * 9 + lane * CM_HOPS) * (int64_t)HA), "r"(CM_HOPS * HA), "r"(fb), "l"(c + 1 < nchunk ? again : last)
+                : "memory");
+            for (int j = 0; j < CM_HOPS; ++j) {
+              const int nb = cm_neighbour(kc, lane * CM_HOPS + j, L0, L1, L2, L3);
+              asm volatile(
+                  "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(
+                      s0 + st * ST + CM_HOPS * HA + j * IB),
+                  "l"(Xg + ((int64_t)nb * nchunk + c) * (int64_t)IB), "r"(IB), "r"(fb)
+                  : "memory");
+            }
+          }
+          cm_advance_unit(pipe, NS);
+          __syncwarp(mask);
+          if (__any_sync(mask, *fail != 0)) {  // the lanes leave together
+            a = a1;
             break;
           }
-          cm_fence_after();
-          const uint32_t ab = s0 + st * ST, bb = ab + HA;
-          // k-step descriptors: the start-address field (address / 16, 14 bits) of the stage's
-          // descriptor advanced by the k offset (every address stays below 2^18 bytes: no carry)
-          const uint64_t ad0 = cm_desc(ab, MG * 128, 128), bd0 = cm_desc(bb, NG * 128, 128);
-          for (int k = 0; k < KS; ++k) {
-            const uint64_t ad = ad0 + (uint64_t)((2 * k * MG * 128) >> 4);
-            const uint64_t bd = bd0 + (uint64_t)((2 * k * NG * 128) >> 4);
-            const uint32_t accum = (h | k) != 0;
-            asm volatile(
-                "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-                "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(dt),
-                "l"(ad), "l"(bd), "r"(idesc), "r"(accum));
-          }
-          // the stage is free once these MMAs have read it
-          asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
-                           cm_smem(&cs.empty[st]))
-                       : "memory");
-          if (++pipe.stage == NS) {
-            pipe.stage = 0;
-            pipe.phase ^= 1u;
-          }
-        }
-        if (!ok) break;
-        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
-                         cm_smem(&cs.tfull[d]))
-                     : "memory");
-        if (++pipe.acc == CM_ACCS) {
-          pipe.acc = 0;
-          pipe.aphase ^= 1u;
         }
       }
+    }
+  } else if (tid == 32 || tid == 64) {
+    // ---- MMA issuers, one per accumulator
+    const int mine = warp - 1;
+    switch (ncp / 8) {
+      case 1: cm_mma_role<1>(q, cs, pipe, mine, s0, HA, IB, N, NG, nchunk, cta, ncta); break;
+      case 2: cm_mma_role<2>(q, cs, pipe, mine, s0, HA, IB, N, NG, nchunk, cta, ncta); break;
+      case 3: cm_mma_role<3>(q, cs, pipe, mine, s0, HA, IB, N, NG, nchunk, cta, ncta); break;
+      case 4: cm_mma_role<4>(q, cs, pipe, mine, s0, HA, IB, N, NG, nchunk, cta, ncta); break;
+      case 5: cm_mma_role<5>(q, cs, pipe, mine, s0, HA, IB, N, NG, nchunk, cta, ncta); break;
+      case 6: cm_mma_role<6>(q, cs, pipe, mine, s0, HA, IB, N, NG, nchunk, cta, ncta); break;
+      case 7: cm_mma_role<7>(q, cs, pipe, mine, s0, HA, IB, N, NG, nchunk, cta, ncta); break;
+      default: cm_mma_role<8>(q, cs, pipe, mine, s0, HA, IB, N, NG, nchunk, cta, ncta); break;  // nc <= CM_MAXNC
+    }
   } else if (warp == CM_EPI0 || warp == CM_EPI0 + 1) {
     // ---- epilogue: rows i = 32 (warp - 4) + lane of the accumulator, twist term, scaling
     const int i = (warp - CM_EPI0) * 32 + lane;
     const float g5 = i < nc / 2 ? 1.f : -1.f;
-    for (int64_t a = cta; a < q.Vc && !*fail; a += ncta)
+    // the site's own entries for the twist term, fetched a unit ahead
+    float4 xn[CM_MAXS / 2];
+    auto load_x = [&](int64_t a, int c) {
+#pragma unroll
+      for (int tp = 0; tp < CM_MAXS / 2; ++tp) {
+        const int t = c * TP + tp;
+        xn[tp] = (i < nc && tp < TP && t < nt)
+                     ? __ldcg(reinterpret_cast<const float4*>(q.x + ((((int64_t)t * nc + i) * q.Vc) + a) * 4))
+                     : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+    };
+    if (q.Vc * cta / ncta < q.Vc * (cta + 1) / ncta) load_x(q.Vc * cta / ncta, 0);
+    for (int64_t a = q.Vc * cta / ncta, a1 = q.Vc * (cta + 1) / ncta; a < a1 && !*fail; ++a)
       for (int c = 0; c < nchunk && !*fail; ++c) {
         const int d = pipe.acc;
-        // the site's own entries for the twist term, fetched while the MMAs run
         float4 xv[CM_MAXS / 2];
 #pragma unroll
-        for (int tp = 0; tp < CM_MAXS / 2; ++tp) {
-          const int t = c * TP + tp;
-          xv[tp] = (i < nc && tp < TP && t < nt)
-                       ? __ldcg(reinterpret_cast<const float4*>(q.x + ((((int64_t)t * nc + i) * q.Vc) + a) * 4))
-                       : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
+        for (int tp = 0; tp < CM_MAXS / 2; ++tp) xv[tp] = xn[tp];
+        const bool more = c + 1 < nchunk;
+        if (more || a + 1 < a1) load_x(more ? a : a + 1, more ? c + 1 : 0);
         if (!cm_wait(cm_smem(&cs.tfull[d]), pipe.aphase, fail)) break;
         cm_fence_after();
         uint32_t r[32] = {};
