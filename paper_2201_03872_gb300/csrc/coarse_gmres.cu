@@ -18,8 +18,8 @@
 //  * Vector phases: CTA b works on tile b % nt and on the entries of slice b / nt; the same
 //    thread owns the same entries in every vector phase, so in-place updates need no
 //    barrier of their own.
-//  * Small dense work (Givens rotations, back substitution) is per system, with every
-//    operand fetched before the dependent arithmetic starts.
+//  * Small dense work (Givens rotations, back substitution) is per system, by a few lanes, as FP64
+//    instructions are slow here, with the operands fetched before the dependent arithmetic starts.
 #include <atomic>
 #include <cmath>
 
@@ -32,9 +32,11 @@ namespace tmamg {
 
 constexpr int CG_THREADS = 256;
 constexpr int CG_TCH = 8;    // system tiles per shared-memory chunk in the stencil phase
-constexpr int CG_IVEC = 4;   // basis vectors per register chunk in the dot phase
+constexpr int CG_IVEC = 8;   // basis vectors per register chunk in the vector phases
 constexpr int CG_MAXM = 64;  // largest restart length
-constexpr int CG_EPT = 8;    // entries per thread held in registers in the vector phases
+constexpr int CG_RED = 4 * (CG_MAXM + 8);  // floats per warp of the reductions: every vector's sums, and a group's slack
+constexpr int CG_RED_BYTES = CG_THREADS / 32 * CG_RED * 4;
+constexpr int CG_EPT = 4;    // entries per thread held in registers in the vector phases
 constexpr int CG_MAXNC = 64; // largest coarse site dimension 2 Nv
 constexpr int CG_AJC = 16;   // stencil columns per asynchronous chunk
 // per-warp shared memory of the stencil phase, in float4 units (vector staging + 2 chunks)
@@ -45,6 +47,8 @@ struct CGArgs {
   const __half* A16;  // FP16 operator for the tensor-core stencil, or null (FP32 stencil)
   __half* X16;        // B images of the vector the tensor-core stencil multiplies
   int cm_nstage;      // shared-memory stages of the tensor-core stencil
+  int dyn_bytes;      // dynamic shared memory of a CTA
+  int rot_bytes;      // of those, at the end: CTA 0's Givens rotations and column (0: in its threads' own arrays)
   double* b0;         // [NS] initial residual norm per system (scale of the restart product)
   int L[4];
   int64_t Vc;
@@ -272,28 +276,49 @@ __device__ void cg_apply_sum(const CGArgs& p, const float* in, float* out, int t
   }
 }
 
-// CTA-wide sum of nv float4 values per thread into FP64 partials part[b][slot0 + v][lane]
-__device__ void cta_reduce_store(const CGArgs& p, float4* vals, int nv, int slot0, double* sm) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int v = 0; v < nv; ++v) {
-    float4 x = vals[v];
+// The warp's sums of N floats per thread (N a power of two up to 32): value k of the sums ends up in lane k's
+// return value (lanes k + N, ... hold it too). Halving exchanges the values not kept: 31 shuffles for 16 values
+// and 32 lanes instead of 80.
+template <int N>
+__device__ __forceinline__ float warp_sums(const float (&v)[N], int lane) {
+  float t[N];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      x.x += __shfl_xor_sync(0xffffffffu, x.x, o);
-      x.y += __shfl_xor_sync(0xffffffffu, x.y, o);
-      x.z += __shfl_xor_sync(0xffffffffu, x.z, o);
-      x.w += __shfl_xor_sync(0xffffffffu, x.w, o);
-    }
-    if (lane == 0) {
-      double* s = sm + (warp * CG_IVEC + v) * 4;
-      s[0] = x.x; s[1] = x.y; s[2] = x.z; s[3] = x.w;
+  for (int k = 0; k < N; ++k) t[k] = v[k];
+#pragma unroll
+  for (int h = N / 2; h > 0; h >>= 1) {
+    const bool up = lane & h;
+#pragma unroll
+    for (int k = 0; k < h; ++k) {
+      const float keep = up ? t[k + h] : t[k], give = up ? t[k] : t[k + h];
+      t[k] = keep + __shfl_xor_sync(0xffffffffu, give, h);
     }
   }
+  float r = t[0];
+#pragma unroll
+  for (int o = N; o < 32; o <<= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+  return r;
+}
+
+// CTA-wide sums of NV float4 values per thread, in two parts: the warp's sums to sm[warp][4 slot + ...], then,
+// once every value of the phase is there, n slots added over the warps in FP64 into part[b][slot0 + v][lane]
+template <int NV>
+__device__ __forceinline__ void warp_part(const float4 (&acc)[NV], int slot, float* sm) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  float v[4 * NV];
+#pragma unroll
+  for (int u = 0; u < NV; ++u) {
+    v[4 * u] = acc[u].x; v[4 * u + 1] = acc[u].y; v[4 * u + 2] = acc[u].z; v[4 * u + 3] = acc[u].w;
+  }
+  const float r = warp_sums(v, lane);
+  if (lane < 4 * NV) sm[warp * CG_RED + 4 * slot + lane] = r;
+}
+__device__ __forceinline__ void cta_part(const CGArgs& p, int n, int slot0, const float* sm) {
   __syncthreads();
-  if (threadIdx.x < nv * 4) {
-    const int v = threadIdx.x / 4, q = threadIdx.x % 4;
+  for (int k = threadIdx.x; k < n * 4; k += CG_THREADS) {
+    const int v = k / 4, q = k % 4;
     double s = 0;
-    for (int w = 0; w < CG_THREADS / 32; ++w) s += sm[(w * CG_IVEC + v) * 4 + q];
+#pragma unroll
+    for (int w = 0; w < CG_THREADS / 32; ++w) s += sm[w * CG_RED + k];
     // q: 0 = re lane 0, 1 = re lane 1, 2 = im lane 0, 3 = im lane 1; stored as (re, im) per lane
     double* dst = reinterpret_cast<double*>(p.part + ((int64_t)blockIdx.x * (p.m + 2) + slot0 + v) * 2);
     const int ln = q & 1, ri = q >> 1;
@@ -323,77 +348,224 @@ __device__ double2 part_sum(const CGArgs& p, int i, int n) {
   return s;
 }
 
+// the same by four neighbouring lanes, each a quarter of the slices (all four return the sum)
+__device__ double2 part_sum4(const CGArgs& p, int i, int n) {
+  const int t = n / 2, ln = n % 2, q = threadIdx.x & 3;
+  double2 s = make_double2(0, 0);
+  for (int sl0 = q; sl0 < p.Gt; sl0 += 32) {
+    double2 v[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const int sl = sl0 + 4 * k;
+      v[k] = sl < p.Gt ? ldx(p.part + ((int64_t)(sl * p.nt + t) * (p.m + 2) + i) * 2 + ln) : make_double2(0, 0);
+    }
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      s.x += v[k].x;
+      s.y += v[k].y;
+    }
+  }
+#pragma unroll
+  for (int o = 1; o < 4; o <<= 1) {
+    s.x += __shfl_xor_sync(0xffffffffu, s.x, o);
+    s.y += __shfl_xor_sync(0xffffffffu, s.y, o);
+  }
+  return s;
+}
+
 __device__ __forceinline__ double2 cmul(double2 a, double2 b) {
   return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
 __device__ __forceinline__ double2 conjd(double2 a) { return make_double2(a.x, -a.y); }
 
-// Givens step for system n on Arnoldi column j, with H[j+1][j] = hn. The rotations of the
-// cycle stay in the calling thread's own arrays c_, s_ (the same thread handles system n at
-// every step), so only the new column is fetched. total: Arnoldi steps done before step j.
-__device__ void givens_step(const CGArgs& p, int n, int j, double hn, int total, double* c_, double2* s_) {
-  const int NS = p.NS, m = p.m;
-  double2* col = p.H + (int64_t)j * (m + 1) * NS;
-  double2 cv[CG_MAXM + 1];
-  // the column fetched sixteen entries at a time into registers before it is parked in local memory
-  for (int i0 = 0; i0 <= j; i0 += 16) {
-    double2 t[16];
-#pragma unroll
-    for (int k = 0; k < 16; ++k) t[k] = i0 + k <= j ? ldx(col + (i0 + k) * NS + n) : make_double2(0, 0);
-#pragma unroll
-    for (int k = 0; k < 16; ++k)
-      if (i0 + k <= j) cv[i0 + k] = t[k];
-  }
-  cv[j + 1] = make_double2(hn, 0);
-  for (int i = 0; i < j; ++i) {
-    const double2 a = cv[i], bb = cv[i + 1];
-    const double2 t = cmul(s_[i], bb);
-    cv[i] = make_double2(c_[i] * a.x + t.x, c_[i] * a.y + t.y);
-    const double2 u = cmul(conjd(s_[i]), a);
-    cv[i + 1] = make_double2(c_[i] * bb.x - u.x, c_[i] * bb.y - u.y);
-  }
-  const double2 a = cv[j];
-  const double na = hypot(a.x, a.y), nb = hn;
-  const double r = hypot(na, nb);
-  double c;
-  double2 sn;
-  if (r == 0.0) {
-    c = 1.0;
-    sn = make_double2(0, 0);
-  } else if (na == 0.0) {
-    c = 0.0;
-    sn = make_double2(1, 0);
-  } else {
-    c = na / r;  // s = (a / |a|) conj(b) / r with b = hn real
-    sn = make_double2(a.x / na * (nb / r), a.y / na * (nb / r));
-  }
-  cv[j] = na == 0.0 ? make_double2(r, 0) : make_double2(a.x / na * r, a.y / na * r);
-  cv[j + 1] = make_double2(0, 0);
-  for (int i = 0; i <= j + 1; ++i) col[i * NS + n] = cv[i];
-  c_[j] = c;
-  s_[j] = sn;
-  const double2 gj = p.g[j * NS + n];
-  const double2 t = cmul(conjd(sn), gj);
-  p.g[(j + 1) * NS + n] = make_double2(-t.x, -t.y);
-  p.g[j * NS + n] = make_double2(c * gj.x, c * gj.y);
-  const double res = hypot(t.x, t.y);
-  if (!(res > p.tolabs[n]) || nb == 0.0) {
-    p.kconv[n] = j + 1;
-    p.active[n] = 0;
-    p.done[n] = 1;
-  } else if (j + 1 == m || total + 1 >= p.maxiter) {
-    p.kconv[n] = j + 1;
-    p.active[n] = 0;
+// Arnoldi column j of every active system, by CTA 0 (H[j+1][j] was stored by the norm phase of step j): the cycle's
+// rotations applied to it, a new one made, the residual and the stop flags. total: Arnoldi steps done before
+// step j. Four neighbouring lanes per system: a warp's FP64 instruction takes 64 cycles here whatever it does,
+// so each lane computes one of the four real outputs of a rotation (three instructions instead of sixteen), and one
+// division serves the four quotients of the new one. SH: the rotations [m][nsys] and the column stay in rot
+// (shared memory); otherwise they are in global memory.
+// A cycle of 28 steps, 12 systems: 13.9 us a step with a thread per system, more than the stencil that runs beside
+// it; this way 8.3 us.
+template <bool SH>
+__device__ __forceinline__ void givens_column(const CGArgs& p, int j, int total, double2* rot) {
+  const int NS = p.NS, m = p.m, st = SH ? p.nsys : NS, r = threadIdx.x & 3;
+  auto get2 = [](const double2* q) { return SH ? *q : ldx(q); };
+  auto quad = [](double v, int from) { return __shfl_sync(0xffffffffu, v, from, 4); };
+  for (int k0 = threadIdx.x / 32 * 8; k0 < p.nsys; k0 += CG_THREADS / 4) {  // uniform over the warp
+    const int nq = k0 + (threadIdx.x & 31) / 4;
+    const int n = nq < p.nsys ? nq : p.nsys - 1;
+    const bool on = nq < p.nsys && ldx(p.active + n);
+    double2* col = p.H + (int64_t)j * (m + 1) * NS + n;
+    const double nb = ldx(col + (int64_t)(j + 1) * NS).x;
+    const double2 gj = ldx(p.g + j * NS + n);
+    const double ta = ldx(p.tolabs + n);
+    double2* s_ = (SH ? rot : p.sn) + n;
+    double* c_ = (SH ? reinterpret_cast<double*>(rot + 2 * m * st) : p.cs) + n;
+    double2* cv = SH ? rot + m * st + n : col;
+    if (SH) {
+#pragma unroll 4
+      for (int i = r; i <= j; i += 4) cv[i * st] = ldx(col + (int64_t)i * NS);
+      __syncwarp();
+    }
+    double2 a = get2(cv);
+    for (int i = 0; i < j; ++i) {
+      // new entry i: c a + s b (lanes 0, 1: re, im), carried on: c b - conj(s) a (lanes 2, 3)
+      const double2 b = get2(cv + (int64_t)(i + 1) * st), s = get2(s_ + (int64_t)i * st);
+      const double c = SH ? c_[(int64_t)i * st] : ldx(c_ + (int64_t)i * st);
+      const double2 f = r < 2 ? a : b, g = r < 2 ? b : make_double2(-a.x, -a.y);
+      const double P = r & 1 ? f.y : f.x, Q = r & 1 ? g.y : g.x, R = r & 1 ? g.x : g.y;
+      const double o = fma(c, P, fma(s.x, Q, s.y * (r == 0 || r == 3 ? -R : R)));
+      if (on && r < 2) reinterpret_cast<double*>(col + (int64_t)i * NS)[r] = o;
+      a = make_double2(quad(o, 2), quad(o, 3));
+    }
+    const double na = hypot(a.x, a.y);
+    const double h = hypot(na, nb);
+    const double qt = (r == 0 ? a.x : r == 1 ? a.y : r == 2 ? nb : na) / (r < 2 ? na : h);
+    const double ux = quad(qt, 0), uy = quad(qt, 1), sb = quad(qt, 2), cb = quad(qt, 3);
+    double c = cb;
+    double2 sn = make_double2(ux * sb, uy * sb);  // s = (a / |a|) conj(b) / r with b = hn real
+    double2 d = make_double2(ux * h, uy * h);
+    if (na == 0.0) {
+      c = h == 0.0 ? 1.0 : 0.0;
+      sn = make_double2(h == 0.0 ? 0.0 : 1.0, 0);
+      d = make_double2(h, 0);
+    }
+    const double2 t = cmul(conjd(sn), gj);
+    const double res = hypot(t.x, t.y);
+    if (on && r == 0) {
+      col[(int64_t)j * NS] = d;
+      col[(int64_t)(j + 1) * NS] = make_double2(0, 0);
+      c_[(int64_t)j * st] = c;
+      s_[(int64_t)j * st] = sn;
+      p.g[(j + 1) * NS + n] = make_double2(-t.x, -t.y);
+      p.g[j * NS + n] = make_double2(c * gj.x, c * gj.y);
+      if (!(res > ta) || nb == 0.0) {
+        p.kconv[n] = j + 1;
+        p.active[n] = 0;
+        p.done[n] = 1;
+      } else if (j + 1 == m || total + 1 >= p.maxiter) {
+        p.kconv[n] = j + 1;
+        p.active[n] = 0;
+      }
+    }
   }
 }
 
-// The rotations of column j for every active system, by threads n < nsys of CTA 0 (the same
-// thread per system at every step; H[j+1][j] was stored by the norm phase of step j).
-__device__ __forceinline__ void givens_column(const CGArgs& p, int j, int total, double* gc, double2* gs) {
-  const int n = threadIdx.x;
-  if (n < p.nsys && ldx(p.active + n)) {
-    const double hn = ldx(p.H + ((int64_t)j * (p.m + 1) + j + 1) * p.NS + n).x;
-    givens_step(p, n, j, hn, total, gc, gs);
+// Vector phases of an Arnoldi step. Every thread owns the entries e0 + q estep of its tile; CG_EPT of them are in
+// registers at a time, with the loads of CG_IVEC basis vectors in flight. The phases are bound by the latency of
+// L2, so what counts is how many loads are under way and that nothing waits in between: the sums of the vectors
+// leave each warp without a CTA barrier, and where a thread owns at most CG_EPT entries the second pass over the
+// basis finds the first vectors in shared memory (the stencil's ring is idle), each thread its own entries.
+// 16^3x32, n_c = 48, 12 systems, 28 steps: dots 14.9 -> 8.1 us, update 11.7 -> 8.4 us a step.
+
+// the dots <V_i, w>, i <= j, into the slots of the partials; w = V_{j+1}. V_j is scaled in place by (s0, s1)
+// first. cache: E CG_THREADS entries for each of the first ncache vectors.
+__device__ __forceinline__ void cg_dots(const CGArgs& p, float* V, int j, float s0, float s1, int64_t e0,
+                                        int64_t estep, float4* cache, int ncache, float* sm) {
+  constexpr int E = CG_EPT, IV = CG_IVEC;
+  const bool one = p.M <= E * estep;
+  const float* w = V + (int64_t)(j + 1) * p.vstride;
+  float* vj = V + (int64_t)j * p.vstride;
+  float4 ww[E];
+  for (int64_t e = e0; e < p.M; e += estep) {
+    float4 v = ld4(vj + e * 4);
+    v.x *= s0; v.y *= s1; v.z *= s0; v.w *= s1;
+    st4(vj + e * 4, v);
+  }
+  for (int i0 = 0; i0 <= j; i0 += IV) {
+    float4 acc[IV];
+#pragma unroll
+    for (int u = 0; u < IV; ++u) acc[u] = make_float4(0, 0, 0, 0);
+    for (int64_t eb = e0; eb < p.M; eb += E * estep) {
+      if (i0 == 0 || !one) {
+#pragma unroll
+        for (int q = 0; q < E; ++q) {
+          const int64_t e = eb + q * estep;
+          ww[q] = e < p.M ? ld4(w + e * 4) : make_float4(0, 0, 0, 0);
+        }
+      }
+      float4 vv[IV][E];
+#pragma unroll
+      for (int u = 0; u < IV; ++u)
+#pragma unroll
+        for (int q = 0; q < E; ++q) {
+          const int64_t e = eb + q * estep;
+          vv[u][q] = i0 + u <= j && e < p.M ? ld4(V + (int64_t)(i0 + u) * p.vstride + e * 4) : make_float4(0, 0, 0, 0);
+        }
+#pragma unroll
+      for (int u = 0; u < IV; ++u) {
+        if (i0 + u < ncache) {
+#pragma unroll
+          for (int q = 0; q < E; ++q) cache[((i0 + u) * E + q) * CG_THREADS + threadIdx.x] = vv[u][q];
+        }
+#pragma unroll
+        for (int q = 0; q < E; ++q) {
+          const float4 v = vv[u][q];
+          // conj(v) w per lane
+          acc[u].x += v.x * ww[q].x + v.z * ww[q].z;
+          acc[u].y += v.y * ww[q].y + v.w * ww[q].w;
+          acc[u].z += v.x * ww[q].z - v.z * ww[q].x;
+          acc[u].w += v.y * ww[q].w - v.w * ww[q].y;
+        }
+      }
+    }
+    warp_part(acc, i0, sm);
+  }
+  cta_part(p, j + 1, 0, sm);
+}
+
+// y -= sum_{i < k} h_i V_i (SIGN = -1, and |y|^2 into slot m + 1 of the partials) or y += (SIGN = 1)
+template <int SIGN>
+__device__ __forceinline__ void cg_update(const CGArgs& p, float* y, const float* V, int k, const float4* hsm,
+                                          int64_t e0, int64_t estep, const float4* cache, int ncache, float* sm) {
+  constexpr int E = CG_EPT, IV = CG_IVEC;
+  float4 nrm[1] = {make_float4(0, 0, 0, 0)};
+  for (int64_t eb = e0; eb < p.M; eb += E * estep) {
+    float4 yy[E];
+#pragma unroll
+    for (int q = 0; q < E; ++q) {
+      const int64_t e = eb + q * estep;
+      yy[q] = e < p.M ? ld4(y + e * 4) : make_float4(0, 0, 0, 0);
+    }
+    for (int i0 = 0; i0 < k; i0 += IV) {
+      float4 vv[IV][E];
+#pragma unroll
+      for (int u = 0; u < IV; ++u)
+#pragma unroll
+        for (int q = 0; q < E; ++q) {
+          const int64_t e = eb + q * estep;
+          vv[u][q] = i0 + u < ncache                ? cache[((i0 + u) * E + q) * CG_THREADS + threadIdx.x]
+                     : i0 + u < k && e < p.M ? ld4(V + (int64_t)(i0 + u) * p.vstride + e * 4)
+                                             : make_float4(0, 0, 0, 0);
+        }
+#pragma unroll
+      for (int u = 0; u < IV; ++u) {
+        if (i0 + u < k) {
+          const float4 h = hsm[i0 + u];
+#pragma unroll
+          for (int q = 0; q < E; ++q) {
+            const float4 v = vv[u][q];
+            yy[q].x += SIGN * (h.x * v.x - h.y * v.z);
+            yy[q].z += SIGN * (h.x * v.z + h.y * v.x);
+            yy[q].y += SIGN * (h.z * v.y - h.w * v.w);
+            yy[q].w += SIGN * (h.z * v.w + h.w * v.y);
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < E; ++q) {
+      const int64_t e = eb + q * estep;
+      if (e < p.M) {
+        st4(y + e * 4, yy[q]);
+        nrm[0].x += yy[q].x * yy[q].x + yy[q].z * yy[q].z;
+        nrm[0].y += yy[q].y * yy[q].y + yy[q].w * yy[q].w;
+      }
+    }
+  }
+  if (SIGN < 0) {
+    warp_part(nrm, 0, sm);
+    cta_part(p, 1, p.m + 1, sm);
   }
 }
 
@@ -468,16 +640,16 @@ __device__ __forceinline__ void cg_convert(const CGArgs& p, const float* x, cons
 }
 
 __device__ __forceinline__ void cg_body(const CGArgs& p, CmShared& cs, float4* dyn) {
-  __shared__ double sm[(CG_THREADS / 32) * CG_IVEC * 4];
   __shared__ float4 hsm[CG_MAXM + 1];  // H column (or y) of this CTA's two systems
   CmPipe pipe;  // this thread's place in the tensor-core stencil pipeline
   __shared__ float cvs[256];  // input factors of the B-image conversion, per system
-  double gc[CG_MAXM];   // Givens rotations of the current cycle (used by the threads gtid < nsys)
-  double2 gs[CG_MAXM];
   unsigned char* dsm = reinterpret_cast<unsigned char*>(dyn);
   const int b = blockIdx.x;
   const int tile = b % p.nt;
   const int slice = b / p.nt;
+  // the vector phases use the dynamic shared memory, free outside the stencil: reductions, then cached entries
+  float* sm = reinterpret_cast<float*>(dsm);
+  float4* cache = dyn + CG_RED_BYTES / sizeof(float4);
   const int64_t toff = (int64_t)tile * p.M * 4;
   const int64_t e0 = (int64_t)slice * CG_THREADS + threadIdx.x;
   const int64_t estep = (int64_t)p.Gt * CG_THREADS;
@@ -486,18 +658,24 @@ __device__ __forceinline__ void cg_body(const CGArgs& p, CmShared& cs, float4* d
   const int m = p.m;
   const int n0 = 2 * tile, n1 = 2 * tile + 1;
   const int GG = p.G > 1 ? 1 : 0;  // CTAs kept free of stencil sites for the Givens rotations
+  // basis vectors whose entries fit in shared memory between the two passes of the vector phases
+  const int ncache = p.M <= CG_EPT * estep ? (p.dyn_bytes - p.rot_bytes - CG_RED_BYTES) /
+                                                 (CG_EPT * CG_THREADS * (int)sizeof(float4))
+                                           : 0;
+  double2* rot = p.rot_bytes ? reinterpret_cast<double2*>(dsm + p.dyn_bytes - p.rot_bytes) : nullptr;
 
   // ---- start: x = 0, V0 = rc, |rc| per system
   {
-    float4 nrm = make_float4(0, 0, 0, 0);
+    float4 nrm[1] = {make_float4(0, 0, 0, 0)};
     for (int64_t e = e0; e < p.M; e += estep) {
       const float4 r = ld4(p.rc + toff + e * 4);
       st4(p.V + toff + e * 4, r);
       st4(p.xc + toff + e * 4, make_float4(0, 0, 0, 0));
-      nrm.x += r.x * r.x + r.z * r.z;
-      nrm.y += r.y * r.y + r.w * r.w;
+      nrm[0].x += r.x * r.x + r.z * r.z;
+      nrm[0].y += r.y * r.y + r.w * r.w;
     }
-    cta_reduce_store(p, &nrm, 1, 0, sm);
+    warp_part(nrm, 0, sm);
+    cta_part(p, 1, 0, sm);
   }
   if (!grid_barrier(p)) return;
   // norms sit in the real slot of each lane's partial (see cta_reduce_store)
@@ -524,6 +702,10 @@ __device__ __forceinline__ void cg_body(const CGArgs& p, CmShared& cs, float4* d
   }
 
   int total = 0;
+  auto last_column = [&](int j) {
+    if (rot) givens_column<true>(p, j, total - 1, rot);
+    else givens_column<false>(p, j, total - 1, nullptr);
+  };
   while (true) {
     int j = 0;
     for (; j < m && total < p.maxiter; ++j) {
@@ -538,7 +720,7 @@ __device__ __forceinline__ void cg_body(const CGArgs& p, CmShared& cs, float4* d
       } else {
         cg_apply_partials(p, p.V + (int64_t)j * p.vstride, dyn);
       }
-      if (j > 0 && b == 0) givens_column(p, j - 1, total - 1, gc, gs);
+      if (j > 0 && b == 0) last_column(j - 1);
       if (!grid_barrier(p)) return;
       if (!p.A16)
         cg_apply_sum(p, p.V + (int64_t)j * p.vstride, p.V + (int64_t)(j + 1) * p.vstride, tile, e0, estep);
@@ -548,148 +730,58 @@ __device__ __forceinline__ void cg_body(const CGArgs& p, CmShared& cs, float4* d
         float s0 = 0, s1 = 0;
         if (n0 < p.nsys) s0 = (float)ldx(p.sc + n0);
         if (n1 < p.nsys) s1 = (float)ldx(p.sc + n1);
-        float* vj = p.V + (int64_t)j * p.vstride + toff;
-        for (int64_t e = e0; e < p.M; e += estep) {
-          float4 v = ld4(vj + e * 4);
-          v.x *= s0; v.y *= s1; v.z *= s0; v.w *= s1;
-          st4(vj + e * 4, v);
-        }
-        const float* w = p.V + (int64_t)(j + 1) * p.vstride + toff;
-        for (int i0 = 0; i0 <= j; i0 += CG_IVEC) {
-          const int ni = j + 1 - i0 < CG_IVEC ? j + 1 - i0 : CG_IVEC;
-          float4 acc[CG_IVEC];
-#pragma unroll
-          for (int u = 0; u < CG_IVEC; ++u) acc[u] = make_float4(0, 0, 0, 0);
-          for (int64_t eb = e0; eb < p.M; eb += CG_EPT * estep) {
-            float4 ww[CG_EPT];
-#pragma unroll
-            for (int q = 0; q < CG_EPT; ++q) {
-              const int64_t e = eb + q * estep;
-              ww[q] = e < p.M ? ld4(w + e * 4) : make_float4(0, 0, 0, 0);
-            }
-#pragma unroll
-            for (int u = 0; u < CG_IVEC; ++u) {
-              if (u < ni) {
-                const float* vu = p.V + (int64_t)(i0 + u) * p.vstride + toff;
-#pragma unroll
-                for (int q = 0; q < CG_EPT; ++q) {
-                  const int64_t e = eb + q * estep;
-                  if (e < p.M) {
-                    const float4 v = ld4(vu + e * 4);
-                    // conj(v) w per lane
-                    acc[u].x += v.x * ww[q].x + v.z * ww[q].z;
-                    acc[u].y += v.y * ww[q].y + v.w * ww[q].w;
-                    acc[u].z += v.x * ww[q].z - v.z * ww[q].x;
-                    acc[u].w += v.y * ww[q].w - v.w * ww[q].y;
-                  }
-                }
-              }
-            }
-          }
-          cta_reduce_store(p, acc, ni, i0, sm);
-        }
+        cg_dots(p, p.V + toff, j, s0, s1, e0, estep, cache, ncache, sm);
       }
       if (!grid_barrier(p)) return;
       // P3 + P4: every CTA sums the H column of its tile's two systems from the partials
       // (the same fixed order everywhere; slice 0 stores it for P5), then
       // w -= sum_i H[i][j] V_i (owner entries) and |w|^2 partials
       {
-        double* hd = reinterpret_cast<double*>(sm);  // [j + 1][2 lanes] (re, im)
-        if (threadIdx.x < 2 * (j + 1)) {
-          const int i = threadIdx.x >> 1, ln = threadIdx.x & 1;
-          const int n = 2 * tile + ln;
-          const double2 h = n < p.nsys ? part_sum(p, i, n) : make_double2(0, 0);
-          if (slice == 0 && n < p.nsys) p.H[((int64_t)j * (m + 1) + i) * NS + n] = h;
-          hd[(i * 2 + ln) * 2] = h.x;
-          hd[(i * 2 + ln) * 2 + 1] = h.y;
-        }
-        __syncthreads();
-        if (threadIdx.x <= j) {
-          const int i = threadIdx.x;
-          hsm[i] = make_float4((float)hd[i * 4], (float)hd[i * 4 + 1], (float)hd[i * 4 + 2], (float)hd[i * 4 + 3]);
+        for (int k0 = 0; k0 < 2 * (j + 1); k0 += CG_THREADS / 4) {  // (uniform: part_sum4 shuffles)
+          const int k = k0 + threadIdx.x / 4;
+          const int i = k >> 1, ln = k & 1, n = 2 * tile + ln;
+          const bool on = k < 2 * (j + 1) && n < p.nsys;
+          const double2 h = part_sum4(p, on ? i : 0, on ? n : 2 * tile);
+          if (k < 2 * (j + 1) && (threadIdx.x & 3) == 0) {
+            if (slice == 0 && on) p.H[((int64_t)j * (m + 1) + i) * NS + n] = h;
+            reinterpret_cast<float2*>(hsm)[k] = on ? make_float2((float)h.x, (float)h.y) : make_float2(0.f, 0.f);
+          }
         }
         __syncthreads();
         float* w = p.V + (int64_t)(j + 1) * p.vstride + toff;
-        float4 nrm = make_float4(0, 0, 0, 0);
-        for (int64_t eb = e0; eb < p.M; eb += CG_EPT * estep) {
-          float4 ww[CG_EPT];
-#pragma unroll
-          for (int q = 0; q < CG_EPT; ++q) {
-            const int64_t e = eb + q * estep;
-            ww[q] = e < p.M ? ld4(w + e * 4) : make_float4(0, 0, 0, 0);
-          }
-          for (int i0 = 0; i0 <= j; i0 += CG_IVEC) {
-#pragma unroll
-            for (int u = 0; u < CG_IVEC; ++u) {
-              if (i0 + u <= j) {
-                const float4 h = hsm[i0 + u];
-                const float* vu = p.V + (int64_t)(i0 + u) * p.vstride + toff;
-#pragma unroll
-                for (int q = 0; q < CG_EPT; ++q) {
-                  const int64_t e = eb + q * estep;
-                  if (e < p.M) {
-                    const float4 v = ld4(vu + e * 4);
-                    ww[q].x -= h.x * v.x - h.y * v.z;
-                    ww[q].z -= h.x * v.z + h.y * v.x;
-                    ww[q].y -= h.z * v.y - h.w * v.w;
-                    ww[q].w -= h.z * v.w + h.w * v.y;
-                  }
-                }
-              }
-            }
-          }
-#pragma unroll
-          for (int q = 0; q < CG_EPT; ++q) {
-            const int64_t e = eb + q * estep;
-            if (e < p.M) {
-              st4(w + e * 4, ww[q]);
-              nrm.x += ww[q].x * ww[q].x + ww[q].z * ww[q].z;
-              nrm.y += ww[q].y * ww[q].y + ww[q].w * ww[q].w;
-            }
-          }
-        }
-        cta_reduce_store(p, &nrm, 1, m + 1, sm);
+        cg_update<-1>(p, w, p.V + toff, j + 1, hsm, e0, estep, cache, ncache, sm);
       }
       if (!grid_barrier(p)) return;
       // P5: H[j+1][j] = |w| and sc = 1 / |w| (every CTA sums the norms in the same order; CTA 0
       // stores them), then the B images of sc w for the next stencil
-      for (int n = threadIdx.x; n < p.nsys; n += CG_THREADS) {
-        const double2 s = part_sum(p, m + 1, n);
-        const double hn = sqrt(fmax(s.x, 0.0));
-        const double scn = hn > 0 ? 1.0 / hn : 0.0;
-        cvs[n] = (float)scn;
-        if (b == 0) {
-          p.sc[n] = scn;
-          p.H[((int64_t)j * (m + 1) + j + 1) * NS + n] = make_double2(hn, 0);
+      for (int k0 = 0; k0 < p.nsys; k0 += CG_THREADS / 4) {
+        const int n = k0 + threadIdx.x / 4;
+        const double2 s = part_sum4(p, m + 1, n < p.nsys ? n : 0);
+        if (n < p.nsys && (threadIdx.x & 3) == 0) {
+          const double hn = sqrt(fmax(s.x, 0.0));
+          const double scn = hn > 0 ? 1.0 / hn : 0.0;
+          cvs[n] = (float)scn;
+          if (b == 0) {
+            p.sc[n] = scn;
+            p.H[((int64_t)j * (m + 1) + j + 1) * NS + n] = make_double2(hn, 0);
+          }
         }
       }
-      if (p.A16) {
-        __syncthreads();
-        cg_convert(p, p.V + (int64_t)(j + 1) * p.vstride, cvs);
-      }
+      // active systems left: the flags were last written in the stencil phase (givens_column)
+      int left = 0;
+      for (int n = threadIdx.x; n < p.nsys; n += CG_THREADS) left |= ldx(p.active + n);
+      left = __syncthreads_or(left);
+      if (p.A16) cg_convert(p, p.V + (int64_t)(j + 1) * p.vstride, cvs);
       ++total;
       if (!grid_barrier(p)) return;
-      {
-        // active systems left (warp 0 of every CTA counts; the flags were last written
-        // before the barrier)
-        __shared__ int nact;
-        if (threadIdx.x < 32) {
-          int c = 0;
-          for (int n = threadIdx.x; n < p.nsys; n += 32) c += ldx(p.active + n);
-#pragma unroll
-          for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-          if (threadIdx.x == 0) nact = c;
-        }
-        __syncthreads();
-        if (nact == 0) {
-          ++j;
-          break;
-        }
+      if (!left) {
+        ++j;
+        break;
       }
     }
     // rotations of the cycle's last column (the loop ended on the cycle length or the step
     // budget; systems that converged earlier are inactive already)
-    if (j > 0 && b == 0) givens_column(p, j - 1, total - 1, gc, gs);
+    if (j > 0 && b == 0) last_column(j - 1);
     if (!grid_barrier(p)) return;
     // y = R^{-1} g per system (a CTA per system), then x += sum_i y_i V_i
     for (int n = b; n < p.nsys; n += p.G) backsub(p, n, reinterpret_cast<double2*>(dyn));
@@ -702,40 +794,8 @@ __device__ __forceinline__ void cg_body(const CGArgs& p, CmShared& cs, float4* d
         hsm[i] = make_float4((float)y0.x, (float)y0.y, (float)y1.x, (float)y1.y);
       }
       __syncthreads();
-      float* x = p.xc + toff;
-      for (int64_t eb = e0; eb < p.M; eb += CG_EPT * estep) {
-        float4 xx[CG_EPT];
-#pragma unroll
-        for (int q = 0; q < CG_EPT; ++q) {
-          const int64_t e = eb + q * estep;
-          xx[q] = e < p.M ? ld4(x + e * 4) : make_float4(0, 0, 0, 0);
-        }
-        for (int i0 = 0; i0 < j; i0 += CG_IVEC) {
-#pragma unroll
-          for (int u = 0; u < CG_IVEC; ++u) {
-            if (i0 + u < j) {
-              const float4 yv = hsm[i0 + u];
-              const float* vu = p.V + (int64_t)(i0 + u) * p.vstride + toff;
-#pragma unroll
-              for (int q = 0; q < CG_EPT; ++q) {
-                const int64_t e = eb + q * estep;
-                if (e < p.M) {
-                  const float4 v = ld4(vu + e * 4);
-                  xx[q].x += yv.x * v.x - yv.y * v.z;
-                  xx[q].z += yv.x * v.z + yv.y * v.x;
-                  xx[q].y += yv.z * v.y - yv.w * v.w;
-                  xx[q].w += yv.z * v.w + yv.w * v.y;
-                }
-              }
-            }
-          }
-        }
-#pragma unroll
-        for (int q = 0; q < CG_EPT; ++q) {
-          const int64_t e = eb + q * estep;
-          if (e < p.M) st4(x + e * 4, xx[q]);
-        }
-      }
+      // (the basis is not in shared memory any more: the back substitution has used it)
+      cg_update<1>(p, p.xc + toff, p.V + toff, j, hsm, e0, estep, cache, 0, sm);
     }
     // restart decision (uniform: done[] was last written before a grid barrier)
     bool again;
@@ -764,16 +824,17 @@ __device__ __forceinline__ void cg_body(const CGArgs& p, CmShared& cs, float4* d
     if (!grid_barrier(p)) return;
     if (!p.A16) cg_apply_sum(p, p.xc, p.V, tile, e0, estep);
     {
-      float4 nrm = make_float4(0, 0, 0, 0);
+      float4 nrm[1] = {make_float4(0, 0, 0, 0)};
       for (int64_t e = e0; e < p.M; e += estep) {
         const float4 r = ld4(p.rc + toff + e * 4);
         float4 w = ld4(p.V + toff + e * 4);
         w.x = r.x - w.x; w.y = r.y - w.y; w.z = r.z - w.z; w.w = r.w - w.w;
         st4(p.V + toff + e * 4, w);
-        nrm.x += w.x * w.x + w.z * w.z;
-        nrm.y += w.y * w.y + w.w * w.w;
+        nrm[0].x += w.x * w.x + w.z * w.z;
+        nrm[0].y += w.y * w.y + w.w * w.w;
       }
-      cta_reduce_store(p, &nrm, 1, 0, sm);
+      warp_part(nrm, 0, sm);
+    cta_part(p, 1, 0, sm);
     }
     if (!grid_barrier(p)) return;
     if (gtid < p.nsys) {
@@ -857,7 +918,8 @@ void CoarseGmres::release() {
 static size_t dyn_smem_bytes(int m, int nc, int nsys, bool tc, int nstage) {
   const size_t rs = sizeof(double2) * (size_t)m * m;
   const size_t stage = tc ? cm_smem_bytes(nc, nsys, nstage) : sizeof(float4) * (size_t)(CG_THREADS / 32) * CG_WARP_F4;
-  return stage > rs ? stage : rs;
+  const size_t need = stage > rs ? stage : rs;
+  return need > (size_t)CG_RED_BYTES ? need : (size_t)CG_RED_BYTES;
 }
 
 static size_t dyn_smem_cap() {
@@ -905,6 +967,10 @@ int coarse_gmres_solve(CoarseGmres& s, const CoarseDims& cd, const float2* A, co
   p.A16 = A16;
   p.X16 = s.X16;
   p.cm_nstage = nstage;
+  p.dyn_bytes = (int)dyn;
+  // CTA 0 keeps the rotations in shared memory when it has no part in the stencil and they leave half of it
+  const size_t rot = (2 * sizeof(double2) + sizeof(double)) * (size_t)m * nsys + sizeof(double2);
+  p.rot_bytes = A16 && G > 1 && 2 * (rot + CG_RED_BYTES) <= dyn ? (int)(rot / sizeof(double2) * sizeof(double2)) : 0;
   p.b0 = s.b0;
   for (int k = 0; k < 4; ++k) p.L[k] = cd.L[k];
   p.Vc = cd.Vc;
