@@ -110,21 +110,74 @@ __global__ void __launch_bounds__(RED_THREADS, 4) mdot_partial_kernel(const real
   }
 }
 
-// out[i * ostride + n] = sum_blk partial  (system n = tile * T + lane), n < nsys
+// The same for a vector with itself (k = 1): partial = (sum |w|^2, 0). NU entries per thread are in flight, which
+// the general kernel's loop does not get to (24^3x48, 16 FP32 systems: 278 -> 144 us), and the FP64 form, bound by FP64
+// arithmetic, does half of it (16 systems: 1400 -> 705 us).
+template <typename real, int T>
+__global__ void __launch_bounds__(RED_THREADS, 4) norm_partial_kernel(const real* __restrict__ w, int64_t M,
+                                                                   double2* __restrict__ partial) {
+  constexpr int NU = 4;
+  __shared__ double red[RED_THREADS / 32][T];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const real* ww = w + (int64_t)blockIdx.y * M * 2 * T;
+  const int64_t step = (int64_t)gridDim.x * RED_THREADS;
+  real acc[NU][T];
+#pragma unroll
+  for (int u = 0; u < NU; ++u)
+#pragma unroll
+    for (int l = 0; l < T; ++l) acc[u][l] = 0;
+  for (int64_t m = blockIdx.x * (int64_t)RED_THREADS + threadIdx.x; m < M; m += NU * step) {
+    Ent<real, T> e[NU];
+#pragma unroll
+    for (int u = 0; u < NU; ++u) {
+      if (m + u * step < M) {
+        e[u] = lde<real, T>(ww + (m + u * step) * 2 * T);
+      } else {
+#pragma unroll
+        for (int l = 0; l < T; ++l) e[u].re[l] = e[u].im[l] = 0;
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < NU; ++u)
+#pragma unroll
+      for (int l = 0; l < T; ++l) acc[u][l] += e[u].re[l] * e[u].re[l] + e[u].im[l] * e[u].im[l];
+  }
+#pragma unroll
+  for (int l = 0; l < T; ++l) {
+    double d = (double)(acc[0][l] + acc[1][l]) + (double)(acc[2][l] + acc[3][l]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+    if (lane == 0) red[warp][l] = d;
+  }
+  __syncthreads();
+  if (threadIdx.x < T) {
+    double s = 0;
+    for (int q = 0; q < RED_THREADS / 32; ++q) s += red[q][threadIdx.x];
+    partial[((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * T + threadIdx.x] = make_double2(s, 0);
+  }
+}
+
+// out[i * ostride + n] = sum_blk partial  (system n = tile * T + lane), n < nsys. A warp per output: a thread per
+// output waited for one load and one FP64 addition after the other (14 to 36 us; this 4 us).
 template <int T>
 __global__ void mdot_final_kernel(const double2* __restrict__ partial, int nblk, int k, int nsys, double2* out,
                                   int64_t ostride, double scale) {
-  int t = blockIdx.x * blockDim.x + threadIdx.x;
+  const int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, ln = threadIdx.x & 31;
   if (t >= nsys * k) return;
   int n = t % nsys, i = t / nsys;
   int tile = n / T, lane = n % T;
   double2 s = make_double2(0, 0);
-  for (int b = 0; b < nblk; ++b) {
+  for (int b = ln; b < nblk; b += 32) {
     double2 p = partial[(((int64_t)tile * nblk + b) * k + i) * T + lane];
     s.x += p.x;
     s.y += p.y;
   }
-  out[i * ostride + n] = make_double2(s.x * scale, s.y * scale);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    s.x += __shfl_xor_sync(0xffffffffu, s.x, o);
+    s.y += __shfl_xor_sync(0xffffffffu, s.y, o);
+  }
+  if (ln == 0) out[i * ostride + n] = make_double2(s.x * scale, s.y * scale);
 }
 
 static thread_local bool t_pair_fold = false;
@@ -156,13 +209,15 @@ void mdot(const real* V, int64_t vstride, int k, const real* w, int64_t M, int n
   constexpr int T = Tile<real>::T;
   int nt = ntiles(nsys, T);
   int nblk = red_blocks(M, nt);
-  if (k == 1)
+  if (k == 1 && V == w)
+    norm_partial_kernel<real, T><<<dim3(nblk, nt), RED_THREADS, 0, st>>>(w, M, partial);
+  else if (k == 1)
     mdot_partial_kernel<real, T, 1><<<dim3(nblk, nt), RED_THREADS, 0, st>>>(V, vstride, k, w, M, partial);
   else
     mdot_partial_kernel<real, T, 4><<<dim3(nblk, nt), RED_THREADS, 0, st>>>(V, vstride, k, w, M, partial);
   TM_COUNT();
   int tot = nsys * k;
-  mdot_final_kernel<T><<<(tot + 127) / 128, 128, 0, st>>>(partial, nblk, k, nsys, out, ostride, 1.0); TM_COUNT();
+  mdot_final_kernel<T><<<(tot + 3) / 4, 128, 0, st>>>(partial, nblk, k, nsys, out, ostride, 1.0); TM_COUNT();
   if (t_pair_fold) {
     const int np = nsys / 2;
     pair_fold_kernel<<<(k * np + 127) / 128, 128, 0, st>>>(out, ostride, k, np); TM_COUNT();
