@@ -380,8 +380,131 @@ __global__ void __launch_bounds__(MAXT, MINB) dirac_kernel(const float2* __restr
   for (int k = 0; k < 12; ++k) st2(yo + (int64_t)k * V * 4, acc.c[k]);
 }
 
+// The split form for lattices too small to fill the chip with a thread per site: twelve warps per 32 sites and tile.
+// Warps 0 to 7 multiply one hop each and leave its two colour vectors in shared memory, every warp then computes one
+// component of the local term and adds that component's hop parts in the order of the other forms (same bits).
+// It is then one or two load latencies long instead of eight: 8^3x16, one system, 9.0 -> 8.0 us with cold caches and
+// 10.3 -> 8.2 us per call of many; with four times the sites 20.5 us against 12.0, so it is a launch variant.
+constexpr int DS_WARPS = 12;
+
+template <int NU, bool FWD>
+__device__ __forceinline__ void split_hop(float4* g, const float2* __restrict__ U, const float* __restrict__ xt, int V,
+                                          int s, int c, int ext, int stride, float phase) {
+  const int nb = FWD ? (c + 1 < ext ? s + stride : s - (ext - 1) * stride) : (c > 0 ? s - stride : s + (ext - 1) * stride);
+  Raw2 raw;
+  ld_raw2(raw, xt + (int64_t)nb * 4, V);
+  CV2 h[2][3];
+  proj_raw2<NU, FWD>(h, raw);
+  Spinor2 a;
+#pragma unroll
+  for (int k = 0; k < 12; ++k) a.c[k].re = a.c[k].im = make_float2(0.f, 0.f);
+  mul_acc2<NU, FWD>(a, h, U + (int64_t)NU * 9 * V, V, FWD ? s : nb, phase);
+#pragma unroll
+  for (int k = 0; k < 6; ++k) g[k * 32] = make_float4(a.c[k].re.x, a.c[k].re.y, a.c[k].im.x, a.c[k].im.y);  // spins 0, 1
+}
+
+template <int NU, bool FWD, int SPIN>
+__device__ __forceinline__ void split_add(CV2& acc, const float4* g, int col) {
+  using P = Proj<NU, FWD>;
+  constexpr int K = SPIN < 2 ? 0 : SPIN == 2 ? P::b0 : P::b1;
+  constexpr int half = SPIN < 2 ? SPIN : (SPIN == 2 ? P::p0 : P::p1);
+  acc2<K>(acc, ld2(reinterpret_cast<const float*>(g + (half * 3 + col) * 32)));
+}
+
+// the sum over the hops of component (SPIN, col)
+template <int SPIN>
+__device__ __forceinline__ CV2 split_sum(const float4* g, int col) {
+  CV2 a;
+  a.re = a.im = make_float2(0.f, 0.f);
+  split_add<0, true, SPIN>(a, g, col);
+  split_add<0, false, SPIN>(a, g + 192, col);
+  split_add<1, true, SPIN>(a, g + 2 * 192, col);
+  split_add<1, false, SPIN>(a, g + 3 * 192, col);
+  split_add<2, true, SPIN>(a, g + 4 * 192, col);
+  split_add<2, false, SPIN>(a, g + 5 * 192, col);
+  split_add<3, true, SPIN>(a, g + 6 * 192, col);
+  split_add<3, false, SPIN>(a, g + 7 * 192, col);
+  return a;
+}
+
+template <bool RES>
+__global__ void __launch_bounds__(DS_WARPS * 32, 2) dirac_split_kernel(
+    const float2* __restrict__ U, const float* __restrict__ C, const float* __restrict__ x, float* y,
+    const double* __restrict__ mu, int nsys, int Lx, int Ly, int Lz, int Lt, float bc_t, const float* bsub,
+    const double* __restrict__ eps) {
+  __shared__ float4 gs[8 * 192];  // [hop][half spinor component][site]
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int V = Lx * Ly * Lz * Lt, tile = blockIdx.y;
+  const int s0 = blockIdx.x * 32 + lane;
+  const bool live = s0 < V;
+  const int s = live ? s0 : V - 1;
+  const float* xt = x + (int64_t)tile * 12 * V * 4;
+  float4* g = gs + warp * 192 + lane;
+  const int sy = Lx, sz = Lx * Ly, st = sz * Lz;
+  switch (warp) {
+    case 0: split_hop<0, true>(g, U, xt, V, s, s % Lx, Lx, 1, 1.f); break;
+    case 1: split_hop<0, false>(g, U, xt, V, s, s % Lx, Lx, 1, 1.f); break;
+    case 2: split_hop<1, true>(g, U, xt, V, s, s / sy % Ly, Ly, sy, 1.f); break;
+    case 3: split_hop<1, false>(g, U, xt, V, s, s / sy % Ly, Ly, sy, 1.f); break;
+    case 4: split_hop<2, true>(g, U, xt, V, s, s / sz % Lz, Lz, sz, 1.f); break;
+    case 5: split_hop<2, false>(g, U, xt, V, s, s / sz % Lz, Lz, sz, 1.f); break;
+    case 6: split_hop<3, true>(g, U, xt, V, s, s / st, Lt, st, s / st == Lt - 1 ? bc_t : 1.f); break;
+    case 7: split_hop<3, false>(g, U, xt, V, s, s / st, Lt, st, s / st == 0 ? bc_t : 1.f); break;
+    default: break;
+  }
+  // component `warp` of the local term (local2_of: the same operations in the same order)
+  const int chi = warp / 6, i = warp % 6;
+  const int n0 = tile * 2;
+  const float2 m2 = make_float2(n0 < nsys ? (float)mu[n0] : 0.f, n0 + 1 < nsys ? (float)mu[n0 + 1] : 0.f);
+  const float ep = eps ? (float)eps[tile] : 0.f;
+  const float* Cc = C + (int64_t)chi * 36 * V + s;
+  const float* xc = xt + ((int64_t)chi * 6 * V + s) * 4;
+  const CV2 xi = ld2(xc + (int64_t)i * V * 4);
+  const float2 smu = chi == 0 ? m2 : make_float2(-m2.x, -m2.y);
+  const float2 nsmu = make_float2(-smu.x, -smu.y);
+  const float d = Cc[(int64_t)i * V];
+  CV2 o;
+  o.re = fma2(f2(d), xi.re, mul2(nsmu, xi.im));
+  o.im = fma2(f2(d), xi.im, mul2(smu, xi.re));
+#pragma unroll
+  for (int j = 0; j < 6; ++j) {
+    if (j == i) continue;
+    const CV2 xj = ld2(xc + (int64_t)j * V * 4);
+    const int k = i > j ? 6 + 2 * (i * (i - 1) / 2 + j) : 6 + 2 * (j * (j - 1) / 2 + i);
+    const float ar = Cc[(int64_t)k * V], ci = Cc[(int64_t)(k + 1) * V];
+    const float ai = i > j ? ci : -ci;
+    o.re = fma2(f2(ar), xj.re, o.re);
+    o.re = fma2(f2(-ai), xj.im, o.re);
+    o.im = fma2(f2(ar), xj.im, o.im);
+    o.im = fma2(f2(ai), xj.re, o.im);
+  }
+  if (ep != 0.f) {
+    o.re = fma2(f2(-ep), make_float2(xi.re.y, xi.re.x), o.re);
+    o.im = fma2(f2(-ep), make_float2(xi.im.y, xi.im.x), o.im);
+  }
+  __syncthreads();
+  const int col = warp % 3;
+  CV2 a;
+  switch (warp / 3) {
+    case 0: a = split_sum<0>(gs + lane, col); break;
+    case 1: a = split_sum<1>(gs + lane, col); break;
+    case 2: a = split_sum<2>(gs + lane, col); break;
+    default: a = split_sum<3>(gs + lane, col); break;
+  }
+  a.re = fma2(f2(-0.5f), a.re, o.re);
+  a.im = fma2(f2(-0.5f), a.im, o.im);
+  if (!live) return;
+  const int64_t at = (((int64_t)tile * 12 + warp) * V + s) * 4;
+  if constexpr (RES) {
+    const CV2 bv = ld2(bsub + at);
+    a.re = sub2(bv.re, a.re);
+    a.im = sub2(bv.im, a.im);
+  }
+  st2(y + at, a);
+}
+
 // launch variants: (sites per CTA row, staged, largest CTA, CTAs per SM): 168 registers at 12 warps per SM,
-// or 128 registers (a few bytes of spills) at 16 warps per SM
+// or 128 registers (a few bytes of spills) at 16 warps per SM; and the split form
 template <bool RES, int BX, bool STAGED, int MAXT, int MINB>
 static void launch_variant(const Geom& g, const float2* U, const float* C, const float* x, float* y, const double* mu,
                            int nsys, const float* b, const double* eps, cudaStream_t st) {
@@ -402,7 +525,11 @@ static void launch_tuned(const char* family, bool may_tune, const Geom& g, const
     switch (v) {
       case 1: launch_variant<RES, 32, false, 192, 2>(g, U, C, x, y, mu, nsys, b, eps, st); return;
       case 2: launch_variant<RES, 32, true, 256, 2>(g, U, C, x, y, mu, nsys, b, eps, st); return;
-      case 3: launch_variant<RES, 64, true, 128, 3>(g, U, C, x, y, mu, nsys, b, eps, st); return;
+      case 3:
+        dirac_split_kernel<RES><<<dim3((unsigned)((g.V + 31) / 32), ntiles(nsys, 2)), DS_WARPS * 32, 0, st>>>(
+            U, C, x, y, mu, nsys, g.L[0], g.L[1], g.L[2], g.L[3], (float)g.bc_t, b, eps);
+        TM_COUNT();
+        return;
       default: launch_variant<RES, 32, true, 192, 2>(g, U, C, x, y, mu, nsys, b, eps, st); return;
     }
   };
