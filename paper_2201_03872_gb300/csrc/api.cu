@@ -280,11 +280,25 @@ int tmamg_unpack(tmamg_ctx* ctx, const void* x_bundle, void* x_field, int nsys, 
   return check_cuda(ctx, cudaGetLastError(), "unpack launch");
 }
 
+// whether the FP32 stencil takes this call's masses as values (not while the stream is being captured: a replay
+// reads them where the caller keeps them)
+static bool takes_values(tmamg_ctx* ctx, int nsys, int prec) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  return prec == 32 && dirac32_takes_values(ctx->g, nsys) &&
+         cudaStreamIsCapturing(ctx->stream, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
+}
+
 int tmamg_dirac(tmamg_ctx* ctx, const void* x_bundle, void* y_bundle, int nsys, const double* mu, int prec) {
   if (!ctx) return TMAMG_ERR_ARG;
   if (!x_bundle || !y_bundle || !mu || nsys <= 0) return set_err(ctx, TMAMG_ERR_ARG, "dirac: bad argument");
   if (x_bundle == y_bundle) return set_err(ctx, TMAMG_ERR_ARG, "dirac: x and y must not overlap");
   if (!ctx->have_op) return set_err(ctx, TMAMG_ERR_STATE, "dirac: operator not set");
+  if (takes_values(ctx, nsys, prec)) {
+    MassArgs ma;
+    for (int n = 0; n < nsys; ++n) ma.v[n] = mu[n];
+    launch_dirac32_values(ctx->g, ctx->U32, ctx->C32, (const float*)x_bundle, (float*)y_bundle, ma, nsys, ctx->stream);
+    return check_cuda(ctx, cudaGetLastError(), "dirac launch");
+  }
   int rc = upload_mu(ctx, mu, nsys);
   if (rc) return rc;
   if (prec == 32)
@@ -306,6 +320,17 @@ int tmamg_dirac_doublet(tmamg_ctx* ctx, const void* x_bundle, void* y_bundle, in
   if (x_bundle == y_bundle) return set_err(ctx, TMAMG_ERR_ARG, "dirac_doublet: x and y must not overlap");
   if (!ctx->have_op) return set_err(ctx, TMAMG_ERR_STATE, "dirac_doublet: operator not set");
   const int nsys = 2 * npair;
+  if (takes_values(ctx, nsys, prec)) {
+    MassArgs ma;
+    ma.doublet = 1;
+    for (int q = 0; q < npair; ++q) {
+      ma.v[2 * q] = mu[q];
+      ma.v[2 * q + 1] = -mu[q];
+      ma.e[q] = eps[q];
+    }
+    launch_dirac32_values(ctx->g, ctx->U32, ctx->C32, (const float*)x_bundle, (float*)y_bundle, ma, nsys, ctx->stream);
+    return check_cuda(ctx, cudaGetLastError(), "dirac_doublet launch");
+  }
   std::vector<double> ms(nsys);
   for (int q = 0; q < npair; ++q) {
     ms[2 * q] = mu[q];

@@ -35,6 +35,13 @@ inline int tune_variant(const char* family, int64_t key, int nvar, bool may_tune
   return may_tune ? tune_run(family, key, nvar, launch, st) : 0;
 }
 
+// the variant that a launch would use now without tuning first, or -1 if it would tune
+inline int tune_peek(const char* family, int64_t key, int nvar) {
+  const int f = tune_forced();
+  if (f >= 0) return f < nvar ? f : 0;
+  return autotune_on() ? tune_lookup(family, key) : 0;
+}
+
 // largest divisor of nt that keeps a CTA of bx x ty threads at <= maxthreads threads
 inline int pick_ty(int nt, int bx, int maxthreads) {
   int best = 1;

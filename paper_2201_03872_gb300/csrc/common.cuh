@@ -155,6 +155,22 @@ void launch_convert_gauge(const Geom& g, const double* Uin, double2* U64, float2
 template <typename real>
 void launch_dirac(const Geom& g, const void* U, const real* C, const real* x, real* y, const double* mu, int nsys,
                   cudaStream_t st, const double* eps = nullptr);
+// Twisted masses and, for the doublet form, splittings of a stencil launch: device arrays, or, for up to
+// MASS_VALUES systems, the values themselves in the kernel's arguments.
+constexpr int MASS_VALUES = 32;
+struct MassArgs {
+  const double* mu = nullptr;   // device, or null: v
+  const double* eps = nullptr;  // device, or null: e
+  int doublet = 0;
+  double v[MASS_VALUES];
+  double e[MASS_VALUES / 2];
+};
+// y = D(mu) x in FP32 with the masses as values, which spares a small lattice's call the copy that it otherwise
+// starts with (8^3x16, one system: 8.2 us a call with it, 6.2 without): for the split form only, where the call has
+// that choice already. The forms for larger lattices are fast enough to hide the copy, and lose 6% to other registers.
+bool dirac32_takes_values(const Geom& g, int nsys);
+void launch_dirac32_values(const Geom& g, const float2* U, const float* C, const float* x, float* y, const MassArgs& ma,
+                           int nsys, cudaStream_t st);
 // r = b - D(mu) x on FP32 bundles in one pass (b with the same tiles as x)
 void launch_residual32(const Geom& g, const float2* U, const float* C, const float* x, const float* b, float* r,
                        const double* mu, int nsys, cudaStream_t st, const double* eps = nullptr);

@@ -430,8 +430,7 @@ __device__ __forceinline__ CV2 split_sum(const float4* g, int col) {
 template <bool RES>
 __global__ void __launch_bounds__(DS_WARPS * 32, 2) dirac_split_kernel(
     const float2* __restrict__ U, const float* __restrict__ C, const float* __restrict__ x, float* y,
-    const double* __restrict__ mu, int nsys, int Lx, int Ly, int Lz, int Lt, float bc_t, const float* bsub,
-    const double* __restrict__ eps) {
+    const __grid_constant__ MassArgs ma, int nsys, int Lx, int Ly, int Lz, int Lt, float bc_t, const float* bsub) {
   __shared__ float4 gs[8 * 192];  // [hop][half spinor component][site]
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int V = Lx * Ly * Lz * Lt, tile = blockIdx.y;
@@ -455,8 +454,9 @@ __global__ void __launch_bounds__(DS_WARPS * 32, 2) dirac_split_kernel(
   // component `warp` of the local term (local2_of: the same operations in the same order)
   const int chi = warp / 6, i = warp % 6;
   const int n0 = tile * 2;
+  const double* mu = ma.mu ? ma.mu : ma.v;
   const float2 m2 = make_float2(n0 < nsys ? (float)mu[n0] : 0.f, n0 + 1 < nsys ? (float)mu[n0 + 1] : 0.f);
-  const float ep = eps ? (float)eps[tile] : 0.f;
+  const float ep = ma.doublet ? (float)(ma.eps ? ma.eps : ma.e)[tile] : 0.f;
   const float* Cc = C + (int64_t)chi * 36 * V + s;
   const float* xc = xt + ((int64_t)chi * 6 * V + s) * 4;
   const CV2 xi = ld2(xc + (int64_t)i * V * 4);
@@ -503,6 +503,14 @@ __global__ void __launch_bounds__(DS_WARPS * 32, 2) dirac_split_kernel(
   st2(y + at, a);
 }
 
+template <bool RES>
+static void launch_split(const Geom& g, const float2* U, const float* C, const float* x, float* y, const MassArgs& ma,
+                         int nsys, const float* b, cudaStream_t st) {
+  dirac_split_kernel<RES><<<dim3((unsigned)((g.V + 31) / 32), ntiles(nsys, 2)), DS_WARPS * 32, 0, st>>>(
+      U, C, x, y, ma, nsys, g.L[0], g.L[1], g.L[2], g.L[3], (float)g.bc_t, b);
+  TM_COUNT();
+}
+
 // launch variants: (sites per CTA row, staged, largest CTA, CTAs per SM): 168 registers at 12 warps per SM,
 // or 128 registers (a few bytes of spills) at 16 warps per SM; and the split form
 template <bool RES, int BX, bool STAGED, int MAXT, int MINB>
@@ -517,6 +525,9 @@ static void launch_variant(const Geom& g, const float2* U, const float* C, const
       U, C, x, y, mu, nsys, nt, g.L[0], g.L[1], g.L[2], g.L[3], (float)g.bc_t, b, eps); TM_COUNT();
 }
 
+constexpr int NVARIANTS = 4, SPLIT_VARIANT = 3;
+static int64_t tune_key(const Geom& g, int nsys) { return g.V * 4096 + nsys; }
+
 template <bool RES>
 static void launch_tuned(const char* family, bool may_tune, const Geom& g, const float2* U, const float* C,
                          const float* x, float* y, const double* mu, int nsys, const float* b, const double* eps,
@@ -525,15 +536,28 @@ static void launch_tuned(const char* family, bool may_tune, const Geom& g, const
     switch (v) {
       case 1: launch_variant<RES, 32, false, 192, 2>(g, U, C, x, y, mu, nsys, b, eps, st); return;
       case 2: launch_variant<RES, 32, true, 256, 2>(g, U, C, x, y, mu, nsys, b, eps, st); return;
-      case 3:
-        dirac_split_kernel<RES><<<dim3((unsigned)((g.V + 31) / 32), ntiles(nsys, 2)), DS_WARPS * 32, 0, st>>>(
-            U, C, x, y, mu, nsys, g.L[0], g.L[1], g.L[2], g.L[3], (float)g.bc_t, b, eps);
-        TM_COUNT();
+      case SPLIT_VARIANT: {
+        MassArgs ma;
+        ma.mu = mu;
+        ma.eps = eps;
+        ma.doublet = eps != nullptr;
+        launch_split<RES>(g, U, C, x, y, ma, nsys, b, st);
         return;
+      }
       default: launch_variant<RES, 32, true, 192, 2>(g, U, C, x, y, mu, nsys, b, eps, st); return;
     }
   };
-  launch(tune_variant(family, g.V * 4096 + nsys, 4, may_tune, launch, st));
+  launch(tune_variant(family, tune_key(g, nsys), NVARIANTS, may_tune, launch, st));
+}
+
+bool dirac32_takes_values(const Geom& g, int nsys) {
+  return nsys <= MASS_VALUES && tune_peek("dirac_f32", tune_key(g, nsys), NVARIANTS) == SPLIT_VARIANT;
+}
+
+void launch_dirac32_values(const Geom& g, const float2* U, const float* C, const float* x, float* y, const MassArgs& ma,
+                           int nsys, cudaStream_t st) {
+  TM_PROF(st, "dirac_f32");
+  launch_split<false>(g, U, C, x, y, ma, nsys, nullptr, st);
 }
 
 template <>

@@ -1,5 +1,5 @@
 """The FP32 stencil's split form against the direct form, bit for bit: lattices whose sites do not fill the last 32,
-one site per direction pair (extent 2: both neighbours are the same site), one to three tiles, the antiperiodic
+one site per direction pair (extent 2: both neighbours are the same site), one to three tiles, more systems than the kernel takes masses as values, the antiperiodic
 boundary and the doublet's coupling. (The direct form is compared with the oracle elsewhere.)"""
 import numpy as np
 import pytest
@@ -10,7 +10,7 @@ from tests.gpu_util import Lattice, torch_cuda
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("L,nsys", [((2, 2, 2, 2), 1), ((2, 2, 2, 6), 2), ((6, 2, 4, 2), 3), ((4, 4, 4, 4), 5), ((10, 2, 6, 4), 6)])
+@pytest.mark.parametrize("L,nsys", [((2, 2, 2, 2), 1), ((2, 2, 2, 6), 2), ((6, 2, 4, 2), 3), ((4, 4, 4, 4), 5), ((10, 2, 6, 4), 6), ((4, 4, 4, 4), 34)])
 def test_split_form_same_bits(L, nsys):
     torch = torch_cuda()
     lat = Lattice(L, synth.gauge_field(L, 0.4, seed=6), 0.124, 1.1)
