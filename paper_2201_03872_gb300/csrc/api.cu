@@ -385,6 +385,13 @@ int tmamg_apply(tmamg_ctx* ctx, const void* x_field, void* y_field, int nsys, co
   int rc = ensure_scratch(ctx, bytes);
   if (rc) return rc;
   rc = tmamg_pack(ctx, x_field, ctx->scratch[0], nsys, prec);
+  if (!rc && prec == 32 && ctx->have_op && dirac32_to_field(ctx->g, nsys)) {
+    rc = upload_mu(ctx, mu, nsys);
+    if (rc) return rc;
+    launch_dirac32_field(ctx->g, ctx->U32, ctx->C32, (const float*)ctx->scratch[0], (float*)y_field, ctx->mu_dev, nsys,
+                         ctx->stream);
+    return check_cuda(ctx, cudaGetLastError(), "apply launch");
+  }
   if (!rc) rc = tmamg_dirac(ctx, ctx->scratch[0], ctx->scratch[1], nsys, mu, prec);
   if (!rc) rc = tmamg_unpack(ctx, ctx->scratch[1], y_field, nsys, prec);
   return rc;

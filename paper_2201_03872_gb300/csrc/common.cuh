@@ -171,6 +171,10 @@ struct MassArgs {
 bool dirac32_takes_values(const Geom& g, int nsys);
 void launch_dirac32_values(const Geom& g, const float2* U, const float* C, const float* x, float* y, const MassArgs& ma,
                            int nsys, cudaStream_t st);
+// D(mu) x in FP32 from a bundle to a user field in one kernel, where the stencil's form for this call allows it
+bool dirac32_to_field(const Geom& g, int nsys);
+void launch_dirac32_field(const Geom& g, const float2* U, const float* C, const float* x, float* y, const double* mu,
+                          int nsys, cudaStream_t st);
 // r = b - D(mu) x on FP32 bundles in one pass (b with the same tiles as x)
 void launch_residual32(const Geom& g, const float2* U, const float* C, const float* x, const float* b, float* r,
                        const double* mu, int nsys, cudaStream_t st, const double* eps = nullptr);

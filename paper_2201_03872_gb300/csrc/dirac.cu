@@ -266,9 +266,12 @@ __host__ __device__ constexpr int dr_stage_bytes(int bx) { return bx * (36 * 8 +
 //  nothing is shared and the direct form is the faster one (24^3x48, one system: 137 against 177 us), so
 //  both are launch variants. Prefetching the neighbours' lines into L1 (9.2 ms) and wider CTA rows (8.9 to 9.1
 //  ms) measured slower.
+// FIELD (staged, BX = 32, not RES): y is a user field [nsys][V][12], a warp's rows transposed through the staging
+//  space, which spares the call the bundle's way to HBM and back: 20x12x28x44, 5 systems, 138 + 58 us as two
+//  kernels, 166 us as one.
 // MAXT, MINB: the launch variant's largest CTA and the CTAs per SM it is compiled for (which sets the
 // register budget); every variant does the same per-thread arithmetic.
-template <int BX, bool RES, bool STAGED, int MAXT, int MINB>
+template <int BX, bool RES, bool STAGED, int MAXT, int MINB, bool FIELD = false>
 __global__ void __launch_bounds__(MAXT, MINB) dirac_kernel(const float2* __restrict__ U, const float* __restrict__ C,
                                                            const float* __restrict__ x, float* y,
                                                            const double* __restrict__ mu, int nsys, int ntile, int Lx,
@@ -362,6 +365,28 @@ __global__ void __launch_bounds__(MAXT, MINB) dirac_kernel(const float2* __restr
   if constexpr (STAGED) {
     dr_wait_sync<0>();
     local2(acc, raw, Cs, BX, threadIdx.x, m2, ep);
+    if constexpr (FIELD) {
+      static_assert(STAGED && !RES && BX == 32, "a warp holds 32 sites of one tile");
+      constexpr int PITCH = 26;  // 24 reals per site, and 2 that keep the transposed access off the same banks
+      __syncthreads();           // the staged operator data is no longer needed
+      float* sm = reinterpret_cast<float*>(dr_smem) + threadIdx.y * 32 * PITCH;
+      const int ns = V - s0 < 32 ? (int)(V - s0) : 32;
+#pragma unroll
+      for (int l = 0; l < 2; ++l) {
+        if (n0 + l >= nsys) break;
+#pragma unroll
+        for (int k = 0; k < 12; ++k)
+          *reinterpret_cast<float2*>(sm + threadIdx.x * PITCH + 2 * k) =
+              l ? make_float2(acc.c[k].re.y, acc.c[k].im.y) : make_float2(acc.c[k].re.x, acc.c[k].im.x);
+        __syncwarp();
+        float* dst = y + ((int64_t)(n0 + l) * V + s0) * 24;
+#pragma unroll
+        for (int k = threadIdx.x; k < 32 * 24; k += 32)
+          if (k < ns * 24) dst[k] = sm[k + (PITCH - 24) * (k / 24)];
+        __syncwarp();
+      }
+      return;
+    }
     if (!live) return;
   } else {
     local2(acc, xt + s * 4, V, C, V, s, m2, ep);
@@ -548,6 +573,26 @@ static void launch_tuned(const char* family, bool may_tune, const Geom& g, const
     }
   };
   launch(tune_variant(family, tune_key(g, nsys), NVARIANTS, may_tune, launch, st));
+}
+
+bool dirac32_to_field(const Geom& g, int nsys) {
+  const int v = tune_peek("dirac_f32", tune_key(g, nsys), NVARIANTS);
+  return v == 0 || v == 2;
+}
+
+void launch_dirac32_field(const Geom& g, const float2* U, const float* C, const float* x, float* y, const double* mu,
+                          int nsys, cudaStream_t st) {
+  TM_PROF(st, "dirac_f32");
+  const int nt = ntiles(nsys, 2);
+  const bool wide = tune_peek("dirac_f32", tune_key(g, nsys), NVARIANTS) == 2;
+  const int ty = pick_ty(nt, 32, wide ? 256 : 192);
+  const dim3 block(32, ty), grid((unsigned)((g.V + 31) / 32), (unsigned)(nt / ty));
+  static_assert(8 * 32 * 26 * 4 <= dr_stage_bytes(32), "eight warps transpose in the staging space");
+  const auto kernel = wide ? dirac_kernel<32, false, true, 256, 2, true> : dirac_kernel<32, false, true, 192, 2, true>;
+  func_smem_optin((const void*)kernel, dr_stage_bytes(32));
+  kernel<<<grid, block, dr_stage_bytes(32), st>>>(U, C, x, y, mu, nsys, nt, g.L[0], g.L[1], g.L[2], g.L[3],
+                                                  (float)g.bc_t, nullptr, nullptr);
+  TM_COUNT();
 }
 
 bool dirac32_takes_values(const Geom& g, int nsys) {

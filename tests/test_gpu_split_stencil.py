@@ -1,6 +1,7 @@
 """The FP32 stencil's split form against the direct form, bit for bit: lattices whose sites do not fill the last 32,
-one site per direction pair (extent 2: both neighbours are the same site), one to three tiles, more systems than the kernel takes masses as values, the antiperiodic
-boundary and the doublet's coupling. (The direct form is compared with the oracle elsewhere.)"""
+one site per direction pair (extent 2: both neighbours are the same site), one to three tiles, more systems than
+the kernel takes masses for as values, the antiperiodic boundary and the doublet's coupling. (The direct form is
+compared with the oracle elsewhere.)"""
 import numpy as np
 import pytest
 
