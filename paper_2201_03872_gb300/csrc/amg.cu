@@ -434,11 +434,142 @@ __global__ void __launch_bounds__(RP_THREADS) prolong_kernel(const float2* __res
   }
 }
 
+// few systems: entries k per thread, and the ring of P ahead of its use: RP_NST stages of RP_JS rows j
+constexpr int RP_R = 2;
+constexpr int RP_JS = 4;
+constexpr int RP_NST = 6;
+constexpr size_t RP_RING = sizeof(float2) * RP_NST * RP_JS * RP_R * RP_THREADS;
+
+// The same for up to TCH tiles, few enough that the kernel is bound by HBM and not by arithmetic. There the general
+// kernel waits for P, of which it has eight rows at a time on their way to registers (32 KB per SM). Here every
+// thread keeps 160 KB per SM of its own P entries on their way to shared memory, and two entries k share each
+// broadcast of the coarse vector. 24^3x48, nv = 24: 1 system 494 -> 335 us, 4 systems 513 -> 357, 8 systems 540 -> 452;
+// at 16 systems the general kernel is the faster one (615 against 698 us, its arithmetic has fewer other instructions).
+template <int TCH>
+__global__ void __launch_bounds__(RP_THREADS, 2) prolong_few_kernel(const float2* __restrict__ P,
+                                                                    const float* __restrict__ xc,
+                                                                    float* __restrict__ e, AggDims g, int nv, int d,
+                                                                    int nt, int accumulate) {
+  __shared__ float4 Xs[32][TCH];    // [j][tile] for this chirality (nv <= 32)
+  extern __shared__ float2 ring[];  // [RP_NST][RP_JS][RP_R][RP_THREADS], each thread its own entries
+  int* sidx = reinterpret_cast<int*>(ring + RP_NST * RP_JS * RP_R * RP_THREADS);  // [asize]
+  const int64_t a = blockIdx.x >> 1;
+  const int chi = blockIdx.x & 1;
+  const int nc = 2 * nv;
+  const int K = g.asize * d;
+  for (int q = threadIdx.x; q < g.asize; q += RP_THREADS) {
+    int c[4];
+    agg_site(a, q, g.Lc, g.agg, g.L, c);
+    sidx[q] = (int)site_index(c, g.L);
+  }
+  const float2* Pa = P + ((a * 2 + chi) * nv) * (int64_t)K;
+  const int nblk = (nv + RP_JS - 1) / RP_JS;
+  const int total = (K + RP_R * RP_THREADS - 1) / (RP_R * RP_THREADS) * nblk;  // (pass over k, row block) steps
+  int fk = threadIdx.x, fj = 0, fst = 0;  // next step to fetch: first entry, first row, stage
+  auto fetch = [&]() {
+    if (fk - (int)threadIdx.x < K) {
+      const unsigned dst = (unsigned)__cvta_generic_to_shared(ring + fst * RP_JS * RP_R * RP_THREADS + threadIdx.x);
+#pragma unroll
+      for (int jj = 0; jj < RP_JS; ++jj)
+#pragma unroll
+        for (int r = 0; r < RP_R; ++r)
+          if (fj + jj < nv && fk + r * RP_THREADS < K)
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(
+                             dst + (jj * RP_R + r) * RP_THREADS * (unsigned)sizeof(float2)),
+                         "l"(Pa + (int64_t)(fj + jj) * K + fk + r * RP_THREADS)
+                         : "memory");
+    }
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+    fst = fst + 1 == RP_NST ? 0 : fst + 1;
+    fj += RP_JS;
+    if (fj >= nv) {
+      fj = 0;
+      fk += RP_R * RP_THREADS;
+    }
+  };
+#pragma unroll 1
+  for (int q = 0; q < RP_NST - 1; ++q) fetch();
+  __syncthreads();
+  for (int q = threadIdx.x; q < 32 * TCH; q += RP_THREADS) {  // zeros past nv and past the last tile
+    const int j = q / TCH, u = q % TCH;
+    Xs[j][u] = j < nv && u < nt
+                   ? *reinterpret_cast<const float4*>(xc + (((int64_t)u * nc + chi * nv + j) * g.Vc + a) * 4)
+                   : make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  __syncthreads();
+  float2 are[RP_R][TCH], aim[RP_R][TCH];
+  int st = 0, j0 = 0, k0 = threadIdx.x;
+#pragma unroll 1
+  for (int step = 0; step < total; ++step) {
+    if (j0 == 0) {
+#pragma unroll
+      for (int r = 0; r < RP_R; ++r)
+#pragma unroll
+        for (int u = 0; u < TCH; ++u) are[r][u] = aim[r][u] = make_float2(0.f, 0.f);
+    }
+    fetch();
+    asm volatile("cp.async.wait_group %0;\n" ::"n"(RP_NST - 1) : "memory");  // this step's entries have landed
+    const float2* ps = ring + st * RP_JS * RP_R * RP_THREADS + threadIdx.x;
+#pragma unroll
+    for (int jj = 0; jj < RP_JS; ++jj) {
+      if (j0 + jj >= nv) break;
+      float2 pv[RP_R];
+#pragma unroll
+      for (int r = 0; r < RP_R; ++r) pv[r] = ps[(jj * RP_R + r) * RP_THREADS];
+#pragma unroll
+      for (int u = 0; u < TCH; ++u) {
+        const float4 x = Xs[j0 + jj][u];
+        const float2 xr = make_float2(x.x, x.y), xi = make_float2(x.z, x.w);
+#pragma unroll
+        for (int r = 0; r < RP_R; ++r) {
+          // p x = (pr xr - pi xi) + i (pr xi + pi xr), both systems at once
+          are[r][u] = __ffma2_rn(make_float2(pv[r].x, pv[r].x), xr, are[r][u]);
+          are[r][u] = __ffma2_rn(make_float2(-pv[r].y, -pv[r].y), xi, are[r][u]);
+          aim[r][u] = __ffma2_rn(make_float2(pv[r].x, pv[r].x), xi, aim[r][u]);
+          aim[r][u] = __ffma2_rn(make_float2(pv[r].y, pv[r].y), xr, aim[r][u]);
+        }
+      }
+    }
+    st = st + 1 == RP_NST ? 0 : st + 1;
+    j0 += RP_JS;
+    if (j0 < nv) continue;
+#pragma unroll
+    for (int r = 0; r < RP_R; ++r) {
+      const int k = k0 + r * RP_THREADS;
+      if (k >= K) break;
+      const int cp = k / g.asize, q = k - cp * g.asize;
+      float* out = e + (((int64_t)chi * d + cp) * g.Vp + sidx[q]) * 4;
+      const int64_t ts = (int64_t)(2 * d) * g.Vp * 4;
+#pragma unroll
+      for (int u = 0; u < TCH; ++u) {
+        if (u < nt) {
+          float4 v = make_float4(are[r][u].x, are[r][u].y, aim[r][u].x, aim[r][u].y);
+          if (accumulate) {
+            const float4 o = *reinterpret_cast<const float4*>(out + u * ts);
+            v.x += o.x; v.y += o.y; v.z += o.z; v.w += o.w;
+          }
+          *reinterpret_cast<float4*>(out + u * ts) = v;
+        }
+      }
+    }
+    j0 = 0;
+    k0 += RP_R * RP_THREADS;
+  }
+}
+
 void prolong_vec(const AggDims& g, const float2* P, const float* xc, float* e, int nv, int d, int nsys, int accumulate,
                  cudaStream_t st) {
   TM_PROF(st, d == 6 ? "prolong" : "prolong_coarse");
   const int nt = ntiles(nsys, T2);
-  prolong_kernel<<<(unsigned)(g.Vc * 2), RP_THREADS, sizeof(int) * g.asize, st>>>(P, xc, e, g, nv, d, nt, accumulate);
+  auto few = [&](auto kernel) {
+    const size_t smem = RP_RING + sizeof(int) * g.asize;
+    func_smem_optin((const void*)kernel, (int)smem);
+    kernel<<<(unsigned)(g.Vc * 2), RP_THREADS, smem, st>>>(P, xc, e, g, nv, d, nt, accumulate);
+  };
+  if (nt <= 2) few(prolong_few_kernel<2>);
+  else if (nt <= 4) few(prolong_few_kernel<4>);
+  else
+    prolong_kernel<<<(unsigned)(g.Vc * 2), RP_THREADS, sizeof(int) * g.asize, st>>>(P, xc, e, g, nv, d, nt, accumulate);
   TM_COUNT();
 }
 
