@@ -194,6 +194,13 @@ __global__ void pair_fold_kernel(double2* out, int64_t ostride, int k, int npair
   o[1] = s;
 }
 
+static void fold_pairs(double2* out, int64_t ostride, int k, int nsys, cudaStream_t st) {
+  if (!t_pair_fold) return;
+  const int np = nsys / 2;
+  pair_fold_kernel<<<(k * np + 127) / 128, 128, 0, st>>>(out, ostride, k, np);
+  TM_COUNT();
+}
+
 static int red_blocks(int64_t M, int ntile) {
   // about 4 CTAs per SM in total, at least one per tile
   int64_t want = (152 * 4 + ntile - 1) / ntile;
@@ -218,10 +225,7 @@ void mdot(const real* V, int64_t vstride, int k, const real* w, int64_t M, int n
   TM_COUNT();
   int tot = nsys * k;
   mdot_final_kernel<T><<<(tot + 3) / 4, 128, 0, st>>>(partial, nblk, k, nsys, out, ostride, 1.0); TM_COUNT();
-  if (t_pair_fold) {
-    const int np = nsys / 2;
-    pair_fold_kernel<<<(k * np + 127) / 128, 128, 0, st>>>(out, ostride, k, np); TM_COUNT();
-  }
+  fold_pairs(out, ostride, k, nsys, st);
 }
 
 size_t partial_elems(int64_t M, int nsys, int kmax, int T) {
@@ -236,10 +240,12 @@ size_t partial_elems(int64_t M, int nsys, int kmax, int T) {
 // the basis loop is unrolled so that several vector loads are in flight per thread.
 constexpr int MAXPY_K = 128;
 
-template <typename real, int T>
-__global__ void maxpy_kernel(const real* __restrict__ Vb, int64_t vstride, int k, const double2* __restrict__ c,
+// NORM: also partial = the block's sum of |y|^2 (see norm_partial_kernel), which spares an Arnoldi step a pass over its
+// new vector (24^3x48, 16 systems: 144 us of 1.1 ms at six basis vectors)
+template <typename real, int T, bool NORM>
+__global__ void __launch_bounds__(256) maxpy_kernel(const real* __restrict__ Vb, int64_t vstride, int k, const double2* __restrict__ c,
                              int64_t cstride, real sign, real* __restrict__ y, int64_t M, int nsys,
-                             const int* __restrict__ mask) {
+                             const int* __restrict__ mask, double2* __restrict__ partial) {
   __shared__ real cre[MAXPY_K][T], cim[MAXPY_K][T];
   const int tile = blockIdx.y;
   const int64_t toff = (int64_t)tile * M * 2 * T;
@@ -252,6 +258,9 @@ __global__ void maxpy_kernel(const real* __restrict__ Vb, int64_t vstride, int k
     cim[i][l] = (real)cc.y * sign;
   }
   __syncthreads();
+  real nrm[T];
+#pragma unroll
+  for (int l = 0; l < T; ++l) nrm[l] = 0;
   int64_t m0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   for (int64_t m = m0; m < M; m += (int64_t)gridDim.x * blockDim.x) {
     Ent<real, T> acc = lde<real, T>(y + toff + m * 2 * T);
@@ -266,6 +275,26 @@ __global__ void maxpy_kernel(const real* __restrict__ Vb, int64_t vstride, int k
       }
     }
     ste<real, T>(y + toff + m * 2 * T, acc);
+    if constexpr (NORM) {
+#pragma unroll
+      for (int l = 0; l < T; ++l) nrm[l] += acc.re[l] * acc.re[l] + acc.im[l] * acc.im[l];
+    }
+  }
+  if constexpr (NORM) {
+    __shared__ double red[8][T];
+#pragma unroll
+    for (int l = 0; l < T; ++l) {
+      double d = nrm[l];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+      if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][l] = d;
+    }
+    __syncthreads();
+    if (threadIdx.x < T) {
+      double s = 0;
+      for (int q = 0; q < 8; ++q) s += red[q][threadIdx.x];
+      partial[((int64_t)tile * gridDim.x + blockIdx.x) * T + threadIdx.x] = make_double2(s, 0);
+    }
   }
 }
 
@@ -309,12 +338,34 @@ void maxpy(const real* V, int64_t vstride, int k, const double2* c, int64_t cstr
   constexpr int T = Tile<real>::T;
   int nt = ntiles(nsys, T);
   if (k <= MAXPY_K)
-    maxpy_kernel<real, T><<<upd_grid(M, nt, 256), 256, 0, st>>>(V, vstride, k, c, cstride, (real)sign, y, M, nsys,
-                                                                 mask);
+    maxpy_kernel<real, T, false><<<upd_grid(M, nt, 256), 256, 0, st>>>(V, vstride, k, c, cstride, (real)sign, y, M,
+                                                                        nsys, mask, nullptr);
   else
     maxpy_long_kernel<real, T><<<upd_grid(M, nt, 256), 256, 0, st>>>(V, vstride, k, c, cstride, (real)sign, y, M,
                                                                       nsys, mask);
   TM_COUNT();
+}
+
+// maxpy on all systems, and out[n] = (|y_n|^2, 0)
+template <typename real>
+void maxpy_norm(const real* V, int64_t vstride, int k, const double2* c, int64_t cstride, double sign, real* y,
+                int64_t M, int nsys, double2* out, double2* partial, cudaStream_t st) {
+  if (k > MAXPY_K) {
+    maxpy<real>(V, vstride, k, c, cstride, sign, y, M, nsys, nullptr, st);
+    mdot<real>(y, 0, 1, y, M, nsys, out, nsys, partial, st);
+    return;
+  }
+  TM_PROF(st, "maxpy");
+  constexpr int T = Tile<real>::T;
+  const int nt = ntiles(nsys, T);
+  // four blocks per SM, rounded down: every block resident, none left for a second wave
+  const int64_t want = 152 * 4 / nt, most = (M + 255) / 256;
+  const dim3 grid((unsigned)(want < 1 ? 1 : want < most ? want : most), nt);
+  maxpy_kernel<real, T, true><<<grid, 256, 0, st>>>(V, vstride, k, c, cstride, (real)sign, y, M, nsys, nullptr, partial);
+  TM_COUNT();
+  mdot_final_kernel<T><<<(nsys + 3) / 4, 128, 0, st>>>(partial, (int)grid.x, 1, nsys, out, nsys, 1.0);
+  TM_COUNT();
+  fold_pairs(out, nsys, 1, nsys, st);
 }
 
 // y[n] = a[n] * x[n] + b[n] * y[n]; a, b complex per system (nullptr a => 0, nullptr b => y ignored,
@@ -431,6 +482,10 @@ template void maxpy<float>(const float*, int64_t, int, const double2*, int64_t, 
                            const int*, cudaStream_t);
 template void maxpy<double>(const double*, int64_t, int, const double2*, int64_t, double, double*, int64_t, int,
                             const int*, cudaStream_t);
+template void maxpy_norm<float>(const float*, int64_t, int, const double2*, int64_t, double, float*, int64_t, int,
+                                double2*, double2*, cudaStream_t);
+template void maxpy_norm<double>(const double*, int64_t, int, const double2*, int64_t, double, double*, int64_t, int,
+                                 double2*, double2*, cudaStream_t);
 template void axpby<float>(const double2*, int, const float*, const double2*, int, float*, int64_t, int, const int*,
                            cudaStream_t);
 template void axpby<double>(const double2*, int, const double*, const double2*, int, double*, int64_t, int,

@@ -12,7 +12,7 @@ void mdot(const real* V, int64_t vstride, int k, const real* w, int64_t M, int n
           double2* partial, cudaStream_t st);
 size_t partial_elems(int64_t M, int nsys, int kmax, int T);
 
-// Doublet solves: while set (on the calling host thread), every mdot adds the results of systems
+// Doublet solves: while set (on the calling host thread), every mdot and maxpy_norm adds the results of systems
 // 2p and 2p + 1 and gives the sum to both, so that a Krylov method running on per-system scalars
 // treats each doublet (its two flavours) as one system: both lanes then see identical norms, dots,
 // rotations and update coefficients.
@@ -26,6 +26,11 @@ struct PairFold {
 template <typename real>
 void maxpy(const real* V, int64_t vstride, int k, const double2* c, int64_t cstride, double sign, real* y, int64_t M,
            int nsys, const int* mask, cudaStream_t st);
+
+// maxpy on all systems, and out[n] = (|y_n|^2, 0); partial as for mdot with one vector
+template <typename real>
+void maxpy_norm(const real* V, int64_t vstride, int k, const double2* c, int64_t cstride, double sign, real* y,
+                int64_t M, int nsys, double2* out, double2* partial, cudaStream_t st);
 
 // y = a x + b y with a, b per system: mode 0 = zero, 1 = one, 2 = from the device array
 template <typename real>

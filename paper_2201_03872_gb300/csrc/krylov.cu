@@ -214,13 +214,15 @@ CycleResult gmres_cycle(GmresState& st, const LevelOpsT<real>& ops, int nsys, in
     ops.A(z, w);
     double2* Hcol = st.H + (size_t)j * (m + 1) * cap;
     mdot<real>(V, vstride, j + 1, w, M, nsys, Hcol, cap, st.partial, s);
-    maxpy<real>(V, vstride, j + 1, Hcol, cap, -1.0, w, M, nsys, nullptr, s);
-    if (cgs2) {
+    if (!cgs2) {
+      maxpy_norm<real>(V, vstride, j + 1, Hcol, cap, -1.0, w, M, nsys, st.tmp, st.partial, s);
+    } else {
+      maxpy<real>(V, vstride, j + 1, Hcol, cap, -1.0, w, M, nsys, nullptr, s);
       mdot<real>(V, vstride, j + 1, w, M, nsys, st.tmp, cap, st.partial, s);
       maxpy<real>(V, vstride, j + 1, st.tmp, cap, -1.0, w, M, nsys, nullptr, s);
       add_col_kernel<<<((j + 1) * nsys + 127) / 128, 128, 0, s>>>(Hcol, st.tmp, j + 1, nsys, cap); TM_COUNT();
+      mdot<real>(w, 0, 1, w, M, nsys, st.tmp, cap, st.partial, s);
     }
-    mdot<real>(w, 0, 1, w, M, nsys, st.tmp, cap, st.partial, s);
     norm_finish_kernel<<<(nsys + 127) / 128, 128, 0, s>>>(st.tmp, Hcol + (size_t)(j + 1) * cap, st.sc, nsys); TM_COUNT();
     axpby<real>(nullptr, 0, nullptr, st.sc, 2, w, M, nsys, nullptr, s);
     givens_kernel<<<1, 1024, 0, s>>>(st.H, st.cs, st.sn, st.g, st.resid, st.tolabs, st.kconv, st.active, st.nactive,
