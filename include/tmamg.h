@@ -339,8 +339,8 @@ int tmamg_coarse_solve(tmamg_ctx* ctx, int level, const void* rc_bundle, void* x
 /* ------------------------------------------------------------------ diagnostics */
 
 /* Launch-shape autotuning (process-wide, on by default). Kernel families with several launch
- * variants that compute identical results (the fine stencil and its residual forms: CTA shape and
- * register budget) time every variant on the first call for a lattice volume and system count,
+ * variants that compute identical results (the fine stencil and its residual forms: how the work is
+ * split, CTA shape and register budget) time every variant on the first call for a lattice volume and system count,
  * with CUDA events on that call's stream, and use the fastest from then on (per device). The first
  * call of each shape therefore synchronises its stream once. on = 0 uses the default variant
  * everywhere. Every call clears the recorded choices. Always returns TMAMG_OK. */

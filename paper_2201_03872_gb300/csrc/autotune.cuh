@@ -1,7 +1,7 @@
 // Launch-shape autotuner (host side).
 //
 // A kernel family offers several launch variants that compute identical results (the same
-// per-thread arithmetic under different CTA shapes and register budgets). The first call for a
+// arithmetic per entry, split differently and under different CTA shapes and register budgets). The first call for a
 // problem key (lattice volume and system count) times every variant on that call's own data
 // with CUDA events on the call's stream, keeps the fastest and uses it from then on; the
 // choices are kept per device for the life of the process. Only idempotent launches are tuned
