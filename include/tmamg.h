@@ -379,6 +379,10 @@ int tmamg_profile_report(char* buf, size_t len);
  * flight when the wait gives up. Returns TMAMG_ERR_ARG for limit_cycles < 0. */
 int tmamg_debug_bounded_wait(long long limit_cycles, int unreachable_next);
 
+/* Failure-path test hook (no counterpart in the paper). For the whole process, the library's next `skip` device
+ * allocations run as usual and the `count` ones after them report that there is no memory, without being tried; count = 0 ends this. Returns how many allocations were made to fail since the last call. */
+long long tmamg_debug_fail_alloc(int skip, int count);
+
 #ifdef __cplusplus
 }
 #endif

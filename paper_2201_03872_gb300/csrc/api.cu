@@ -1,4 +1,5 @@
 // C ABI of the tmamg library: context, gauge field, operator, bundles, fine stencil.
+#include <atomic>
 #include <cstdio>
 #include <cstring>
 #include <map>
@@ -57,6 +58,28 @@ void func_smem_optin(const void* func, int bytes) {
   if (cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess) have = bytes;
 }
 
+// allocations until the next one that reports no memory, how many more do so, and how many did
+static std::atomic<long long> g_alloc_skip{0}, g_alloc_fail{0}, g_alloc_failed{0};
+
+static bool alloc_refused() {
+  if (g_alloc_fail.load(std::memory_order_relaxed) <= 0) return false;
+  if (g_alloc_skip.fetch_sub(1) > 0) return false;
+  if (g_alloc_fail.fetch_sub(1) <= 0) return false;
+  ++g_alloc_failed;
+  return true;
+}
+
+cudaError_t alloc_bytes(void** p, size_t bytes, bool pinned) {
+  *p = nullptr;
+  if (!pinned && alloc_refused()) return cudaErrorMemoryAllocation;
+  const cudaError_t e = pinned ? cudaMallocHost(p, bytes) : cudaMalloc(p, bytes);
+  if (e != cudaSuccess) {
+    *p = nullptr;
+    cudaGetLastError();  // the caller reports it; a later launch check must not find it again
+  }
+  return e;
+}
+
 int set_err(tmamg_ctx* ctx, int code, const std::string& msg) {
   if (ctx) ctx->err = msg;
   return code;
@@ -73,8 +96,9 @@ int upload_mu(tmamg_ctx* ctx, const double* mu, int nsys) {
   if (nsys > ctx->mu_cap) {
     if (ctx->mu_dev) cudaFree(ctx->mu_dev);
     ctx->mu_dev = nullptr;
+    ctx->mu_cap = 0;
     int cap = nsys < 64 ? 64 : nsys;
-    int rc = check_cuda(ctx, cudaMalloc(&ctx->mu_dev, sizeof(double) * cap), "cudaMalloc(mu)");
+    int rc = check_cuda(ctx, dev_alloc(&ctx->mu_dev, sizeof(double) * cap), "cudaMalloc(mu)");
     if (rc) return rc;
     ctx->mu_cap = cap;
   }
@@ -95,7 +119,7 @@ static int grow_scratch(tmamg_ctx* ctx, size_t bytes) {
   }
   ctx->scratch_bytes = 0;
   for (int i = 0; i < 2; ++i) {
-    int rc = check_cuda(ctx, cudaMalloc(&ctx->scratch[i], bytes), "cudaMalloc(scratch)");
+    int rc = check_cuda(ctx, dev_alloc(&ctx->scratch[i], bytes), "cudaMalloc(scratch)");
     if (rc) return rc;
   }
   ctx->scratch_bytes = bytes;
@@ -168,10 +192,10 @@ int tmamg_create(const int L[4], int bc_t, void* cuda_stream, tmamg_ctx** out) {
   ctx->g.bc_t = bc_t;
   ctx->stream = (cudaStream_t)cuda_stream;
   tmamg_default_setup_params(&ctx->sp);
-  int rc = check_cuda(ctx, cudaMalloc(&ctx->U64, sizeof(double2) * 36 * ctx->g.V), "cudaMalloc(U64)");
-  if (!rc) rc = check_cuda(ctx, cudaMalloc(&ctx->U32, sizeof(float2) * 36 * ctx->g.V), "cudaMalloc(U32)");
-  if (!rc) rc = check_cuda(ctx, cudaMalloc(&ctx->C64, sizeof(double) * 72 * ctx->g.V), "cudaMalloc(C64)");
-  if (!rc) rc = check_cuda(ctx, cudaMalloc(&ctx->C32, sizeof(float) * 72 * ctx->g.V), "cudaMalloc(C32)");
+  int rc = check_cuda(ctx, dev_alloc(&ctx->U64, sizeof(double2) * 36 * ctx->g.V), "cudaMalloc(U64)");
+  if (!rc) rc = check_cuda(ctx, dev_alloc(&ctx->U32, sizeof(float2) * 36 * ctx->g.V), "cudaMalloc(U32)");
+  if (!rc) rc = check_cuda(ctx, dev_alloc(&ctx->C64, sizeof(double) * 72 * ctx->g.V), "cudaMalloc(C64)");
+  if (!rc) rc = check_cuda(ctx, dev_alloc(&ctx->C32, sizeof(float) * 72 * ctx->g.V), "cudaMalloc(C32)");
   if (rc) {
     tmamg_destroy(ctx);
     return rc;
@@ -217,7 +241,7 @@ int tmamg_load_gauge(tmamg_ctx* ctx, const double* U, int on_device) {
   double* tmp = nullptr;
   size_t bytes = sizeof(double) * 2 * 36 * ctx->g.V;
   if (!on_device) {
-    int rc = check_cuda(ctx, cudaMalloc(&tmp, bytes), "cudaMalloc(gauge staging)");
+    int rc = check_cuda(ctx, dev_alloc(&tmp, bytes), "cudaMalloc(gauge staging)");
     if (rc) return rc;
     rc = check_cuda(ctx, cudaMemcpyAsync(tmp, U, bytes, cudaMemcpyHostToDevice, ctx->stream), "upload gauge");
     if (rc) {
@@ -255,6 +279,14 @@ int tmamg_set_operator(tmamg_ctx* ctx, double kappa, double c_sw) {
   free_workspace(ctx);
   free_levels(ctx);
   return TMAMG_OK;
+}
+
+long long tmamg_debug_fail_alloc(int skip, int count) {
+  const long long failed = g_alloc_failed.exchange(0);
+  g_alloc_fail.store(0);
+  g_alloc_skip.store(skip > 0 ? skip : 0);
+  g_alloc_fail.store(count > 0 ? count : 0);
+  return failed;
 }
 
 size_t tmamg_bundle_bytes(const tmamg_ctx* ctx, int nsys, int prec) {
@@ -343,7 +375,7 @@ int tmamg_dirac_doublet(tmamg_ctx* ctx, const void* x_bundle, void* y_bundle, in
     cudaFree(ctx->eps_dev);
     ctx->eps_dev = nullptr;
     ctx->eps_cap = 0;
-    rc = check_cuda(ctx, cudaMalloc(&ctx->eps_dev, sizeof(double) * npair), "cudaMalloc(eps)");
+    rc = check_cuda(ctx, dev_alloc(&ctx->eps_dev, sizeof(double) * npair), "cudaMalloc(eps)");
     if (rc) return rc;
     ctx->eps_cap = npair;
   }

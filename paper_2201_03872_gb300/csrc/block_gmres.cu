@@ -424,7 +424,7 @@ int BlockGmres::alloc(int m_, int nsys_, int nshift_, int64_t M_) {
   if (nblk < 1) nblk = 1;
   cudaError_t e = cudaSuccess;
   auto A = [&](void** q, size_t bytes) {
-    if (e == cudaSuccess) e = cudaMalloc(q, bytes);
+    if (e == cudaSuccess) e = dev_alloc(q, bytes);
   };
   A((void**)&gram, sizeof(double2) * (size_t)(m + 1) * nsys * s);
   A((void**)&part, sizeof(double2) * (size_t)nblk * (m + 1) * nsys * s);
@@ -442,7 +442,8 @@ int BlockGmres::alloc(int m_, int nsys_, int nshift_, int64_t M_) {
   A((void**)&active, sizeof(int) * nb);
   A((void**)&steps, sizeof(int) * nb);
   A((void**)&nactive, sizeof(int));
-  if (e == cudaSuccess) e = cudaMallocHost((void**)&h_nactive, sizeof(int));
+  if (e == cudaSuccess) e = host_alloc((void**)&h_nactive, sizeof(int));
+  if (e != cudaSuccess) release();  // nothing half allocated, which a later call would take for the whole
   return e == cudaSuccess ? 0 : -1;
 }
 

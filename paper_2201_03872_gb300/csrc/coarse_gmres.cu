@@ -879,7 +879,7 @@ int CoarseGmres::alloc(int m_, int nsys_, int G_, size_t bundle_bytes, size_t x1
   x16_bytes = x16b;
   cudaError_t e = cudaSuccess;
   auto A = [&](void** q, size_t bytes) {
-    if (e == cudaSuccess) e = cudaMalloc(q, bytes);
+    if (e == cudaSuccess) e = dev_alloc(q, bytes);
   };
   A((void**)&H, sizeof(double2) * (size_t)(m + 1) * m * NS);
   A((void**)&cs, sizeof(double) * (size_t)m * NS);
@@ -899,7 +899,8 @@ int CoarseGmres::alloc(int m_, int nsys_, int G_, size_t bundle_bytes, size_t x1
   A((void**)&iters, sizeof(int));
   A((void**)&hpart, 9 * bundle_bytes);
   if (x16_bytes) A((void**)&X16, x16_bytes);
-  if (e == cudaSuccess) e = cudaMallocHost((void**)&h_flags, sizeof(int) * 2);
+  if (e == cudaSuccess) e = host_alloc((void**)&h_flags, sizeof(int) * 2);
+  if (e != cudaSuccess) release();  // nothing half allocated, which a later call would take for the whole
   return e == cudaSuccess ? 0 : -1;
 }
 

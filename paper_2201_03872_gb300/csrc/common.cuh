@@ -118,6 +118,18 @@ int device_sms();
 int device_smem_optin();
 void func_smem_optin(const void* func, int bytes);
 
+// every device and pinned host allocation of the library (tmamg_debug_fail_alloc counts the device ones): *p is null and no
+// CUDA error is left behind where there is no memory
+cudaError_t alloc_bytes(void** p, size_t bytes, bool pinned);
+template <class T>
+cudaError_t dev_alloc(T** p, size_t bytes) {
+  return alloc_bytes(reinterpret_cast<void**>(p), bytes, false);
+}
+template <class T>
+cudaError_t host_alloc(T** p, size_t bytes) {
+  return alloc_bytes(reinterpret_cast<void**>(p), bytes, true);
+}
+
 // error helpers (host)
 int set_err(tmamg_ctx* ctx, int code, const std::string& msg);
 int check_cuda(tmamg_ctx* ctx, cudaError_t e, const char* what);

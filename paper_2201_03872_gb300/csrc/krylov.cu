@@ -22,7 +22,7 @@ int GmresState::alloc(int m_, int cap_, size_t pe) {
   partial_cap = pe;
   cudaError_t e = cudaSuccess;
   auto A = [&](void** p, size_t b) {
-    if (e == cudaSuccess) e = cudaMalloc(p, b);
+    if (e == cudaSuccess) e = dev_alloc(p, b);
   };
   A((void**)&H, sizeof(double2) * (size_t)(m + 1) * m * cap);
   A((void**)&cs, sizeof(double) * (size_t)m * cap);
@@ -38,7 +38,8 @@ int GmresState::alloc(int m_, int cap_, size_t pe) {
   A((void**)&active, sizeof(int) * (size_t)cap);
   A((void**)&nactive, sizeof(int));
   A((void**)&partial, sizeof(double2) * pe);
-  if (e == cudaSuccess) e = cudaMallocHost((void**)&h_nactive, sizeof(int));
+  if (e == cudaSuccess) e = host_alloc((void**)&h_nactive, sizeof(int));
+  if (e != cudaSuccess) release();  // nothing half allocated, which a later call would take for the whole
   return e == cudaSuccess ? 0 : -1;
 }
 

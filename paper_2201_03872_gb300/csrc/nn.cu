@@ -311,7 +311,7 @@ int NNState::alloc(int64_t V, int nsys_) {
   const int nt = ntiles(nsys, NN_T);
   cudaError_t e = cudaSuccess;
   auto A = [&](void** q, size_t b) {
-    if (e == cudaSuccess) e = cudaMalloc(q, b);
+    if (e == cudaSuccess) e = dev_alloc(q, b);
   };
   const size_t per_ch = (size_t)nt * 3 * V * 4 * sizeof(float);  // one channel of a bundle
   for (int l = 0; l < 4; ++l) A((void**)&act[l], per_ch * CH[l]);
@@ -319,6 +319,7 @@ int NNState::alloc(int64_t V, int nsys_) {
   A((void**)&gbuf[1], per_ch * 8);
   const int nchunk = (int)((V + 127) / 128);
   A((void**)&part, sizeof(double2) * (size_t)nt * 9 * nchunk * 64);
+  if (e != cudaSuccess) release_buffers();  // nothing half allocated, which a later call would take for the whole
   return e == cudaSuccess ? 0 : -1;
 }
 
@@ -327,7 +328,7 @@ int NNState::alloc_weights() {
   const int n = nn_weight_offset(3);
   cudaError_t e = cudaSuccess;
   auto A = [&](void** q, size_t b) {
-    if (e == cudaSuccess) e = cudaMalloc(q, b);
+    if (e == cudaSuccess) e = dev_alloc(q, b);
   };
   A((void**)&W, sizeof(float2) * n);
   A((void**)&Winf, sizeof(float2) * n);
@@ -342,6 +343,7 @@ int NNState::alloc_weights() {
     cudaMemset(m1, 0, sizeof(float2) * n);
     cudaMemset(m2, 0, sizeof(float2) * n);
   }
+  if (e != cudaSuccess) release();  // nothing half allocated, which a later call would take for the whole
   return e == cudaSuccess ? 0 : -1;
 }
 

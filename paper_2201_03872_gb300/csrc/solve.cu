@@ -150,7 +150,7 @@ static int ensure_ws(tmamg_ctx* ctx, int nsys, const tmamg_solve_params& p) {
   w->mb32 = (size_t)ntiles(ns, 2) * ncm * Vm * 4 * sizeof(float);
   cudaError_t e = cudaSuccess;
   auto A = [&](void** p, size_t b) {
-    if (e == cudaSuccess) e = cudaMalloc(p, b);
+    if (e == cudaSuccess) e = dev_alloc(p, b);
   };
   A((void**)&w->V, w->fb32 * (mm + 1));
   A((void**)&w->Z, w->fb32 * mm);
@@ -194,7 +194,7 @@ static int ensure_ws(tmamg_ctx* ctx, int nsys, const tmamg_solve_params& p) {
     A((void**)&w->mra, sizeof(double2) * 2 * ns);
     A((void**)&w->mrd, sizeof(double2) * 2 * ns);
   }
-  if (e == cudaSuccess) e = cudaMallocHost((void**)&w->h_count, sizeof(int));
+  if (e == cudaSuccess) e = host_alloc((void**)&w->h_count, sizeof(int));
   if (e != cudaSuccess) {
     ws_free(w);
     return check_cuda(ctx, e, "workspace allocation");
@@ -217,7 +217,7 @@ static int ensure_ws(tmamg_ctx* ctx, int nsys, const tmamg_solve_params& p) {
 static int ensure_t2(tmamg_ctx* ctx) {
   Workspace* w = ctx->ws;
   if (w->t2) return TMAMG_OK;
-  return check_cuda(ctx, cudaMalloc(&w->t2, w->fb32), "cudaMalloc(learned-step scratch)");
+  return check_cuda(ctx, dev_alloc(&w->t2, w->fb32), "cudaMalloc(learned-step scratch)");
 }
 
 // the right-hand sides as FP64 bundles, one tile each (nrhs <= the workspace's system count)
@@ -229,7 +229,7 @@ static int ensure_b64(tmamg_ctx* ctx, int nrhs) {
   cudaFree(w->b64);
   w->b64 = nullptr;
   w->b64_bytes = 0;
-  int rc = check_cuda(ctx, cudaMalloc(&w->b64, need), "cudaMalloc(right-hand sides)");
+  int rc = check_cuda(ctx, dev_alloc(&w->b64, need), "cudaMalloc(right-hand sides)");
   if (!rc) w->b64_bytes = need;
   return rc;
 }
@@ -341,12 +341,12 @@ static int setup_level2(tmamg_ctx* ctx, const tmamg_setup_params* p, const float
   lv.Vc = ad.Vc;
   lv.nv = nv2;
   lv.asize = ad.asize;
-  int rc = check_cuda(ctx, cudaMalloc(&lv.P, sizeof(float2) * (size_t)ad.Vc * 2 * nv2 * ad.asize * nv1), "cudaMalloc(P2)");
-  if (!rc) rc = check_cuda(ctx, cudaMalloc(&lv.A, sizeof(float2) * 9 * (size_t)ad.Vc * nc2 * nc2), "cudaMalloc(A2)");
+  int rc = check_cuda(ctx, dev_alloc(&lv.P, sizeof(float2) * (size_t)ad.Vc * 2 * nv2 * ad.asize * nv1), "cudaMalloc(P2)");
+  if (!rc) rc = check_cuda(ctx, dev_alloc(&lv.A, sizeof(float2) * 9 * (size_t)ad.Vc * nc2 * nc2), "cudaMalloc(A2)");
   if (!rc && nc2 <= CM_MAXNC)
-    rc = check_cuda(ctx, cudaMalloc(&lv.A16, (size_t)cm_site_bytes(nc2) * ad.Vc), "cudaMalloc(A2 f16)");
-  if (!rc) rc = check_cuda(ctx, cudaMalloc(&lv.cmax, sizeof(float) * CM_MAXSYS), "cudaMalloc(cmax)");
-  if (!rc) rc = check_cuda(ctx, cudaMalloc(&lv.cerr, sizeof(int)), "cudaMalloc(cerr)");
+    rc = check_cuda(ctx, dev_alloc(&lv.A16, (size_t)cm_site_bytes(nc2) * ad.Vc), "cudaMalloc(A2 f16)");
+  if (!rc) rc = check_cuda(ctx, dev_alloc(&lv.cmax, sizeof(float) * CM_MAXSYS), "cudaMalloc(cmax)");
+  if (!rc) rc = check_cuda(ctx, dev_alloc(&lv.cerr, sizeof(int)), "cudaMalloc(cerr)");
   if (!rc) rc = check_cuda(ctx, cudaMemsetAsync(lv.cerr, 0, sizeof(int), st), "cudaMemset(cerr)");
   if (rc) {
     cudaFree(lv.P);
@@ -366,7 +366,7 @@ static int setup_level2(tmamg_ctx* ctx, const tmamg_setup_params* p, const float
   double2 *dots = nullptr, *sc = nullptr, *part = nullptr;
   cudaError_t e = cudaSuccess;
   auto A = [&](void** q, size_t b) {
-    if (e == cudaSuccess) e = cudaMalloc(q, b);
+    if (e == cudaSuccess) e = dev_alloc(q, b);
   };
   A((void**)&Wt, b1(nv2));
   A((void**)&Wc, b1(nc2));
@@ -397,7 +397,7 @@ static int setup_level2(tmamg_ctx* ctx, const tmamg_setup_params* p, const float
   }
   if (!vec2_dev) {
     const int64_t n = (int64_t)nv2 * L1.Vc * nc1;
-    e = cudaMalloc(&field, sizeof(float2) * n);
+    e = dev_alloc(&field, sizeof(float2) * n);
     if (e == cudaSuccess) device_gaussian(p->seed, 0x5eed2ULL, n, reinterpret_cast<float2*>(field), st);
     if (e != cudaSuccess) {
       cleanup();
@@ -479,12 +479,12 @@ int do_setup(tmamg_ctx* ctx, const tmamg_setup_params* p, const float* vec_field
   lv.nv = nv;
   lv.asize = ad.asize;
   const int nc = 2 * nv;
-  int rc = check_cuda(ctx, cudaMalloc(&lv.P, sizeof(float2) * (size_t)ad.Vc * 2 * nv * ad.asize * 6), "cudaMalloc(P)");
-  if (!rc) rc = check_cuda(ctx, cudaMalloc(&lv.A, sizeof(float2) * 9 * (size_t)ad.Vc * nc * nc), "cudaMalloc(A)");
+  int rc = check_cuda(ctx, dev_alloc(&lv.P, sizeof(float2) * (size_t)ad.Vc * 2 * nv * ad.asize * 6), "cudaMalloc(P)");
+  if (!rc) rc = check_cuda(ctx, dev_alloc(&lv.A, sizeof(float2) * 9 * (size_t)ad.Vc * nc * nc), "cudaMalloc(A)");
   if (!rc && nc <= CM_MAXNC)
-    rc = check_cuda(ctx, cudaMalloc(&lv.A16, (size_t)cm_site_bytes(nc) * ad.Vc), "cudaMalloc(A16)");
-  if (!rc) rc = check_cuda(ctx, cudaMalloc(&lv.cmax, sizeof(float) * CM_MAXSYS), "cudaMalloc(cmax)");
-  if (!rc) rc = check_cuda(ctx, cudaMalloc(&lv.cerr, sizeof(int)), "cudaMalloc(cerr)");
+    rc = check_cuda(ctx, dev_alloc(&lv.A16, (size_t)cm_site_bytes(nc) * ad.Vc), "cudaMalloc(A16)");
+  if (!rc) rc = check_cuda(ctx, dev_alloc(&lv.cmax, sizeof(float) * CM_MAXSYS), "cudaMalloc(cmax)");
+  if (!rc) rc = check_cuda(ctx, dev_alloc(&lv.cerr, sizeof(int)), "cudaMalloc(cerr)");
   if (!rc) rc = check_cuda(ctx, cudaMemsetAsync(lv.cerr, 0, sizeof(int), st), "cudaMemset(cerr)");
   if (rc) {
     cudaFree(lv.P);
@@ -504,7 +504,7 @@ int do_setup(tmamg_ctx* ctx, const tmamg_setup_params* p, const float* vec_field
   double2 *dots = nullptr, *sc = nullptr, *part = nullptr;
   cudaError_t e = cudaSuccess;
   auto A = [&](void** q, size_t b) {
-    if (e == cudaSuccess) e = cudaMalloc(q, b);
+    if (e == cudaSuccess) e = dev_alloc(q, b);
   };
   A((void**)&Vt, vb);
   A((void**)&R, vb);
@@ -531,7 +531,7 @@ int do_setup(tmamg_ctx* ctx, const tmamg_setup_params* p, const float* vec_field
   float* field = nullptr;
   if (!vec_field_dev) {
     const int64_t n = (int64_t)nv * g.V * 12;
-    e = cudaMalloc(&field, sizeof(float2) * n);
+    e = dev_alloc(&field, sizeof(float2) * n);
     if (e == cudaSuccess) device_gaussian(p->seed, 0x5eedULL, n, reinterpret_cast<float2*>(field), st);
     if (e != cudaSuccess) {
       cudaFree(field);
@@ -585,6 +585,8 @@ struct SolveCtx {
   int mid_iters = 0;          // middle-level FGMRES steps (three levels)
   bool timeout = false;       // a bounded device wait gave up
   bool launch_error = false;  // a cooperative launch was refused
+  bool oom = false;           // a buffer of the coarse solver found no memory
+  void failed(int rc) { (rc == TMAMG_ERR_OOM ? oom : launch_error) = true; }
   int nshift = 1;             // systems n = r * nshift + k (block GMRES groups the rhs of shift k)
   int nn = 0;                 // apply the learned step in the AMG cycle
   const double* eps = nullptr;  // doublet solves: splitting per FP32 tile (the tile = one doublet), device
@@ -603,25 +605,26 @@ __global__ void copy_beta_kernel(const double* b, double* dst, int n) {
 }
 
 // y = D_c x on level l: FP16 operator on the tensor cores (precision 16, or 0 = default) or
-// the FP32 stencil (precision 32); false if the sizes are outside the tensor-core path
-static bool coarse_apply_level(CoarseLevel& l, int precision, const float* x, float* y, const double* mu, double dmu,
+// the FP32 stencil (precision 32); TMAMG_ERR_ARG if the sizes are outside the tensor-core path, TMAMG_ERR_OOM
+// if its operand images find no memory
+static int coarse_apply_level(CoarseLevel& l, int precision, const float* x, float* y, const double* mu, double dmu,
                                int nsys, cudaStream_t st, const double* eps = nullptr) {
   const CoarseDims cd = coarse_dims(l);
   if (precision != 32) {
-    if (!l.A16 || nsys > CM_MAXSYS) return false;
+    if (!l.A16 || nsys > CM_MAXSYS) return TMAMG_ERR_ARG;
     const size_t need = cm_x16_bytes(cd.Vc, cd.nc, nsys);
     if (need > l.x16_bytes) {  // grown once per system count; later calls reuse it
       cudaStreamSynchronize(st);
       cudaFree(l.x16);
       l.x16 = nullptr;
       l.x16_bytes = 0;
-      if (cudaMalloc(&l.x16, need) != cudaSuccess) return false;
+      if (dev_alloc(&l.x16, need) != cudaSuccess) return TMAMG_ERR_OOM;
       l.x16_bytes = need;
     }
-    return coarse_apply_f16(cd, l.A16, x, y, mu, dmu, nsys, l.cmax, l.x16, l.cerr, st, eps) == 0;
+    return coarse_apply_f16(cd, l.A16, x, y, mu, dmu, nsys, l.cmax, l.x16, l.cerr, st, eps) ? TMAMG_ERR_ARG : TMAMG_OK;
   }
   coarse_apply(cd, l.A, x, y, mu, dmu, nsys, st, eps);
-  return true;
+  return TMAMG_OK;
 }
 
 // the stand-alone tensor-core stencil records a bounded wait that gave up in l.cerr: read and clear
@@ -656,7 +659,7 @@ static void coarse_solve(SolveCtx& S, const float* rc, float* xc) {
     // block GMRES: one Krylov space per shift over that shift's right-hand sides
     const int64_t M = (int64_t)cd.nc * cd.Vc;
     if (w->bg.alloc(S.sp->coarse_restart, S.nsys, S.nshift, M)) {
-      S.launch_error = true;
+      S.oom = true;
       return;
     }
     const double dmu = S.sp->delta_mu;
@@ -664,7 +667,7 @@ static void coarse_solve(SolveCtx& S, const float* rc, float* xc) {
     const int nsys = S.nsys;
     const int prec = S.sp->coarse_precision;
     auto apply = [&, dmu, mu, nsys, prec](const float* x, float* y) {
-      if (!coarse_apply_level(L1, prec, x, y, mu, dmu, nsys, st, S.eps)) S.launch_error = true;
+      if (const int rc = coarse_apply_level(L1, prec, x, y, mu, dmu, nsys, st, S.eps)) S.failed(rc);
     };
     int it = 0;
     const size_t cbytes = (size_t)ntiles(nsys, 2) * M * 4 * sizeof(float);  // the caller's bundles hold nsys systems
@@ -684,7 +687,7 @@ static void coarse_solve(SolveCtx& S, const float* rc, float* xc) {
   const double* mu = S.mu;
   const int prec = S.sp->coarse_precision;
   ops.A = [&, dmu, mu, nsys, prec](const float* x, float* y) {
-    if (!coarse_apply_level(L1, prec, x, y, mu, dmu, nsys, st, S.eps)) S.launch_error = true;
+    if (const int rc = coarse_apply_level(L1, prec, x, y, mu, dmu, nsys, st, S.eps)) S.failed(rc);
   };
   const size_t cbytes = (size_t)ntiles(nsys, 2) * M * 4 * sizeof(float);  // the caller's bundles hold nsys systems
   cudaMemsetAsync(xc, 0, cbytes, st);
@@ -738,7 +741,7 @@ static void mid_cycle(SolveCtx& S, const float* v, float* z) {
   const double dmu = 1.0;  // the twisted-mass factor delta_mu belongs to the bottom level only
   const int ns = w->nsys;
   auto apply = [&](const float* x, float* y) {
-    if (!coarse_apply_level(L1, prec, x, y, S.mu, dmu, nsys, st, S.eps)) S.launch_error = true;
+    if (const int rc = coarse_apply_level(L1, prec, x, y, S.mu, dmu, nsys, st, S.eps)) S.failed(rc);
   };
   float* rho = w->sm1;
   float* q = w->sm2;
@@ -775,7 +778,7 @@ static void mid_solve(SolveCtx& S, const float* rm, float* xm) {
   LevelOps ops;
   ops.M = M;
   ops.A = [&](const float* x, float* y) {
-    if (!coarse_apply_level(L1, prec, x, y, S.mu, dmu, nsys, st, S.eps)) S.launch_error = true;
+    if (const int rc = coarse_apply_level(L1, prec, x, y, S.mu, dmu, nsys, st, S.eps)) S.failed(rc);
   };
   ops.precond = [&](const float* v, float* z) { mid_cycle(S, v, z); };
   const size_t mbytes = (size_t)ntiles(nsys, 2) * M * 4 * sizeof(float);  // the caller's bundles hold nsys systems
@@ -938,7 +941,7 @@ static int ensure_ws64(tmamg_ctx* ctx, int nsys, int m, int mc) {
   w->cb = (size_t)ns * w->nc * w->Vc * 2 * sizeof(double);
   cudaError_t e = cudaSuccess;
   auto A = [&](void** p, size_t bytes) {
-    if (e == cudaSuccess) e = cudaMalloc(p, bytes);
+    if (e == cudaSuccess) e = dev_alloc(p, bytes);
   };
   A((void**)&w->V, w->fb * (mm + 1));
   A((void**)&w->Z, w->fb * mm);
@@ -1037,8 +1040,8 @@ int do_solve64(tmamg_ctx* ctx, const double* b, int nrhs, const double* mu, int 
   int rc = 0;
   if (!L1.P64) {
     const int64_t np = L1.Vc * 2 * L1.nv * L1.asize * 6, na = 9 * L1.Vc * nc * nc;
-    rc = check_cuda(ctx, cudaMalloc(&L1.P64, sizeof(double2) * np), "cudaMalloc(P64)");
-    if (!rc) rc = check_cuda(ctx, cudaMalloc(&L1.A64, sizeof(double2) * na), "cudaMalloc(A64)");
+    rc = check_cuda(ctx, dev_alloc(&L1.P64, sizeof(double2) * np), "cudaMalloc(P64)");
+    if (!rc) rc = check_cuda(ctx, dev_alloc(&L1.A64, sizeof(double2) * na), "cudaMalloc(A64)");
     if (rc) return rc;
     widen_f2(L1.P, L1.P64, np, st);
     widen_f2(L1.A, L1.A64, na, st);
@@ -1055,7 +1058,7 @@ int do_solve64(tmamg_ctx* ctx, const double* b, int nrhs, const double* mu, int 
   double* bstage = nullptr;
   if (!on_device) {
     const size_t bytes = sizeof(double) * 2 * M * nrhs;
-    rc = check_cuda(ctx, cudaMalloc(&bstage, bytes), "cudaMalloc(b staging)");
+    rc = check_cuda(ctx, dev_alloc(&bstage, bytes), "cudaMalloc(b staging)");
     if (rc) return rc;
     cudaMemcpyAsync(bstage, b, bytes, cudaMemcpyHostToDevice, st);
     bsrc = bstage;
@@ -1097,7 +1100,7 @@ int do_solve64(tmamg_ctx* ctx, const double* b, int nrhs, const double* mu, int 
   double* xstage = nullptr;
   const size_t xbytes = sizeof(double) * 2 * M * nsys;
   if (!on_device) {
-    cudaMalloc(&xstage, xbytes);
+    dev_alloc(&xstage, xbytes);
     xdst = xstage;
   }
   launch_unpack<double>(g, w->x, xdst, nsys, st);
@@ -1184,7 +1187,7 @@ int do_solve(tmamg_ctx* ctx, const double* b, int nrhs, const double* mu, int ns
       cudaFree(w->epsd);
       w->epsd = nullptr;
       w->eps_cap = 0;
-      rc = check_cuda(ctx, cudaMalloc(&w->epsd, sizeof(double) * np), "cudaMalloc(splittings)");
+      rc = check_cuda(ctx, dev_alloc(&w->epsd, sizeof(double) * np), "cudaMalloc(splittings)");
       if (rc) return rc;
       w->eps_cap = np;
     }
@@ -1246,7 +1249,7 @@ int do_solve(tmamg_ctx* ctx, const double* b, int nrhs, const double* mu, int ns
       gmres_cycle<float>(w->top, fine, nsys, sp->restart, w->V, vstride, w->Z, w->e32, w->mask2, w->rel_top, 1, false,
                          st);
       add_iters_kernel<<<(nsys + 127) / 128, 128, 0, st>>>(w->top.kconv, w->mask2, w->inner_it, nsys); TM_COUNT();
-      if (ic + 1 == sp->inner_cycles) break;
+      if (ic + 1 == sp->inner_cycles || S.oom) break;
       inner_check_kernel<<<1, 1024, 0, st>>>(w->top.resid, w->top.tolabs, w->mask2, w->count, nsys); TM_COUNT();
       cudaMemcpyAsync(w->h_count, w->count, sizeof(int), cudaMemcpyDeviceToHost, st);
       cudaStreamSynchronize(st);
@@ -1257,6 +1260,7 @@ int do_solve(tmamg_ctx* ctx, const double* b, int nrhs, const double* mu, int ns
       mdot<float>(w->V, 0, 1, w->V, M, nsys, w->dot, nsys, w->top.partial, st);
       inner_rel_kernel<<<(nsys + 127) / 128, 128, 0, st>>>(w->dot, w->tmpd, w->rel_top, nsys); TM_COUNT();
     }
+    if (S.oom) break;
     f32_axpy_f64(w->rn, w->e32, w->x64, M, nsys, w->mask, st);
     // r = b - D x in FP64 in one pass (the stencil's residual form)
     launch_residual64(g, ctx->U64, ctx->C64, w->x64, w->b64, nshift, w->r64, ctx->mu_dev, nsys, st, S.eps);
@@ -1281,6 +1285,7 @@ int do_solve(tmamg_ctx* ctx, const double* b, int nrhs, const double* mu, int ns
   if (!on_device) cudaMemcpyAsync(x, w->r64, xbytes, cudaMemcpyDeviceToHost, st);
   cudaError_t se = cudaStreamSynchronize(st);
   if (!rc) rc = check_cuda(ctx, se, "solve");
+  if (!rc && S.oom) rc = set_err(ctx, TMAMG_ERR_OOM, "solve: coarse-solver buffers");
   if (!rc && S.launch_error) rc = set_err(ctx, TMAMG_ERR_CUDA, "solve: cooperative coarse-solver launch failed");
   for (const CoarseLevel& l : ctx->levels)
     if (!rc && coarse_apply_timed_out(l, st)) S.timeout = true;
@@ -1372,7 +1377,7 @@ int tmamg_sap(tmamg_ctx* ctx, void* r_bundle, void* e_bundle, int nsys, const do
   if (bytes > ctx->sap_delta_bytes) {
     free_sap_delta(ctx);
     rc = with_optional_memory(ctx, [&] {
-      return check_cuda(ctx, cudaMalloc(&ctx->sap_delta, bytes), "cudaMalloc(sap scratch)");
+      return check_cuda(ctx, dev_alloc(&ctx->sap_delta, bytes), "cudaMalloc(sap scratch)");
     });
     if (rc) return rc;
     ctx->sap_delta_bytes = bytes;
@@ -1449,6 +1454,7 @@ int tmamg_coarse_solve(tmamg_ctx* ctx, int level, const void* rc_bundle, void* x
   else
     coarse_solve(S, (const float*)rc_bundle, (float*)xc_bundle);
   rc = check_cuda(ctx, cudaStreamSynchronize(ctx->stream), "coarse_solve");
+  if (!rc && S.oom) rc = set_err(ctx, TMAMG_ERR_OOM, "coarse_solve: buffers");
   if (!rc && S.launch_error) rc = set_err(ctx, TMAMG_ERR_CUDA, "coarse_solve: launch failed");
   for (const CoarseLevel& l : ctx->levels)
     if (!rc && coarse_apply_timed_out(l, ctx->stream)) S.timeout = true;
@@ -1467,9 +1473,9 @@ int tmamg_coarse_apply(tmamg_ctx* ctx, int level, const void* x_bundle, void* y_
   int rc = upload_mu(ctx, mu, nsys);
   if (rc) return rc;
   CoarseLevel& l = ctx->levels[level - 1];
-  if (!coarse_apply_level(l, precision, (const float*)x_bundle, (float*)y_bundle, ctx->mu_dev, 1.0, nsys,
-                          ctx->stream))
-    return set_err(ctx, TMAMG_ERR_ARG, "coarse_apply: sizes outside the tensor-core stencil");
+  rc = coarse_apply_level(l, precision, (const float*)x_bundle, (float*)y_bundle, ctx->mu_dev, 1.0, nsys, ctx->stream);
+  if (rc == TMAMG_ERR_OOM) return set_err(ctx, rc, "coarse_apply: operand images");
+  if (rc) return set_err(ctx, rc, "coarse_apply: sizes outside the tensor-core stencil");
   rc = check_cuda(ctx, cudaGetLastError(), "coarse_apply launch");
   if (!rc && coarse_apply_timed_out(l, ctx->stream))
     rc = set_err(ctx, TMAMG_ERR_TIMEOUT, "coarse_apply: a bounded wait timed out");
@@ -1517,7 +1523,7 @@ static int nn_upload(tmamg_ctx* ctx, const double* W) {
 static int random_bundle(tmamg_ctx* ctx, uint64_t seed, int nsys, float* bundle) {
   const int64_t n = (int64_t)nsys * ctx->g.V * 12;
   float* field = nullptr;
-  int rc = check_cuda(ctx, cudaMalloc(&field, sizeof(float2) * n), "cudaMalloc(random field)");
+  int rc = check_cuda(ctx, dev_alloc(&field, sizeof(float2) * n), "cudaMalloc(random field)");
   if (rc) return rc;
   device_gaussian(seed, 0x5eedULL, n, reinterpret_cast<float2*>(field), ctx->stream);
   launch_pack<float>(ctx->g, field, bundle, nsys, ctx->stream);
@@ -1685,8 +1691,8 @@ int tmamg_nn_train(tmamg_ctx* ctx, const tmamg_nn_params* p, tmamg_nn_report* re
   const int nb = p->pairs / nsys;
   const int win = p->window > 0 && p->window < nb ? p->window : nb;
   float *R = nullptr, *E = nullptr;
-  rc = check_cuda(ctx, cudaMalloc(&R, w->fb32 * win), "cudaMalloc(pairs)");
-  if (!rc) rc = check_cuda(ctx, cudaMalloc(&E, w->fb32 * win), "cudaMalloc(pairs)");
+  rc = check_cuda(ctx, dev_alloc(&R, w->fb32 * win), "cudaMalloc(pairs)");
+  if (!rc) rc = check_cuda(ctx, dev_alloc(&E, w->fb32 * win), "cudaMalloc(pairs)");
   if (rc) {
     cudaFree(R);
     return rc;

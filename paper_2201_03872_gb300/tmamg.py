@@ -116,6 +116,7 @@ SIGNATURES = {
     "tmamg_nn_loss_grad": (I, [P, P, P, I, ctypes.POINTER(ctypes.c_double), P]),
     "tmamg_nn_train": (I, [P, ctypes.POINTER(NNParams), ctypes.POINTER(NNReport)]),
     "tmamg_debug_bounded_wait": (I, [ctypes.c_longlong, I]),
+    "tmamg_debug_fail_alloc": (ctypes.c_longlong, [I, I]),
     "tmamg_profile_enable": (I, [I]),
     "tmamg_autotune": (I, [I]),
     "tmamg_autotune_force": (I, [I]),
@@ -389,6 +390,12 @@ def tmamg_debug_bounded_wait(limit_cycles, unreachable_next):
     unreachable barrier for the next persistent coarse solve (tests of the timeout path)."""
     return _check("tmamg_debug_bounded_wait", None, lib().tmamg_debug_bounded_wait(int(limit_cycles),
                                                                                   int(unreachable_next)))
+
+
+def tmamg_debug_fail_alloc(skip, count):
+    """Process-wide: `skip` of the library's device allocations run as usual, the `count` ones after them report no memory
+    (0 ends this). Returns how many were made to fail since the last call."""
+    return lib().tmamg_debug_fail_alloc(int(skip), int(count))
 
 
 def tmamg_default_nn_params(**kw):
