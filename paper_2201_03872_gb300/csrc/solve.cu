@@ -1042,7 +1042,11 @@ int do_solve64(tmamg_ctx* ctx, const double* b, int nrhs, const double* mu, int 
     const int64_t np = L1.Vc * 2 * L1.nv * L1.asize * 6, na = 9 * L1.Vc * nc * nc;
     rc = check_cuda(ctx, dev_alloc(&L1.P64, sizeof(double2) * np), "cudaMalloc(P64)");
     if (!rc) rc = check_cuda(ctx, dev_alloc(&L1.A64, sizeof(double2) * na), "cudaMalloc(A64)");
-    if (rc) return rc;
+    if (rc) {  // both or neither: P64 stands for the pair, widened
+      cudaFree(L1.P64);
+      L1.P64 = nullptr;
+      return rc;
+    }
     widen_f2(L1.P, L1.P64, np, st);
     widen_f2(L1.A, L1.A64, na, st);
   }
