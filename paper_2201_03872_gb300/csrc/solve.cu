@@ -1059,11 +1059,16 @@ int do_solve64(tmamg_ctx* ctx, const double* b, int nrhs, const double* mu, int 
   if (rc) return rc;
   const double* mud = ctx->mu_dev;
   const double* bsrc = b;
-  double* bstage = nullptr;
+  double *bstage = nullptr, *xstage = nullptr;
+  const size_t xbytes = sizeof(double) * 2 * M * nsys;
   if (!on_device) {
     const size_t bytes = sizeof(double) * 2 * M * nrhs;
     rc = check_cuda(ctx, dev_alloc(&bstage, bytes), "cudaMalloc(b staging)");
-    if (rc) return rc;
+    if (!rc) rc = check_cuda(ctx, dev_alloc(&xstage, xbytes), "cudaMalloc(x staging)");
+    if (rc) {
+      cudaFree(bstage);
+      return rc;
+    }
     cudaMemcpyAsync(bstage, b, bytes, cudaMemcpyHostToDevice, st);
     bsrc = bstage;
   }
@@ -1100,14 +1105,7 @@ int do_solve64(tmamg_ctx* ctx, const double* b, int nrhs, const double* mu, int 
     cudaMemcpyAsync(w->V, w->t1, w->fb, cudaMemcpyDeviceToDevice, st);
     restart_tol_kernel<<<(nsys + 127) / 128, 128, 0, st>>>(w->dot, w->bn, sp->tol, w->rel_top, nsys); TM_COUNT();
   }
-  double* xdst = x;
-  double* xstage = nullptr;
-  const size_t xbytes = sizeof(double) * 2 * M * nsys;
-  if (!on_device) {
-    dev_alloc(&xstage, xbytes);
-    xdst = xstage;
-  }
-  launch_unpack<double>(g, w->x, xdst, nsys, st);
+  launch_unpack<double>(g, w->x, on_device ? x : xstage, nsys, st);
   if (!on_device) cudaMemcpyAsync(x, xstage, xbytes, cudaMemcpyDeviceToHost, st);
   const cudaError_t le = cudaGetLastError();
   const cudaError_t se = cudaStreamSynchronize(st);

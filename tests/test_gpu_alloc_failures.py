@@ -71,8 +71,9 @@ def every_allocation(make, call, count=ALL):
     raise AssertionError("the call never ran out of allocations")
 
 
-@pytest.mark.parametrize("kw", [dict(use_nn=2), dict(coarse_solver=1), dict(coarse_solver=2), dict(precision=64)],
-                         ids=["learned step", "block GMRES", "GMRES per step", "FP64"])
+@pytest.mark.parametrize("kw", [dict(use_nn=2), dict(coarse_solver=1), dict(coarse_solver=2), dict(precision=64),
+                                dict(precision=64, host=True)],
+                         ids=["learned step", "block GMRES", "GMRES per step", "FP64", "FP64 host"])
 def test_solve_after_a_solve_without_memory(kw):
     for q, error in every_allocation(Problem, lambda q: q.solve(**kw)):
         assert error is not None and error.code == -3, error
