@@ -80,6 +80,16 @@ cudaError_t alloc_bytes(void** p, size_t bytes, bool pinned) {
   return e;
 }
 
+// the correction buffer of tmamg_sap, and the copies of the operator, without which the FP64 stencil runs in FP64
+// arithmetic
+bool give_back(tmamg_ctx* ctx) {
+  if (!ctx || !(ctx->g.fx.U || ctx->sap_delta)) return false;
+  cudaStreamSynchronize(ctx->stream);
+  free_sap_delta(ctx);
+  free_fixed(ctx->g);
+  return true;
+}
+
 int set_err(tmamg_ctx* ctx, int code, const std::string& msg) {
   if (ctx) ctx->err = msg;
   return code;
@@ -98,7 +108,7 @@ int upload_mu(tmamg_ctx* ctx, const double* mu, int nsys) {
     ctx->mu_dev = nullptr;
     ctx->mu_cap = 0;
     int cap = nsys < 64 ? 64 : nsys;
-    int rc = check_cuda(ctx, dev_alloc(&ctx->mu_dev, sizeof(double) * cap), "cudaMalloc(mu)");
+    int rc = check_cuda(ctx, dev_alloc(ctx, &ctx->mu_dev, sizeof(double) * cap), "cudaMalloc(mu)");
     if (rc) return rc;
     ctx->mu_cap = cap;
   }
@@ -112,23 +122,19 @@ void free_sap_delta(tmamg_ctx* ctx) {
   ctx->sap_delta_bytes = 0;
 }
 
-static int grow_scratch(tmamg_ctx* ctx, size_t bytes) {
+static int ensure_scratch(tmamg_ctx* ctx, size_t bytes) {
+  if (bytes <= ctx->scratch_bytes) return TMAMG_OK;
   for (int i = 0; i < 2; ++i) {
     if (ctx->scratch[i]) cudaFree(ctx->scratch[i]);
     ctx->scratch[i] = nullptr;
   }
   ctx->scratch_bytes = 0;
   for (int i = 0; i < 2; ++i) {
-    int rc = check_cuda(ctx, dev_alloc(&ctx->scratch[i], bytes), "cudaMalloc(scratch)");
+    int rc = check_cuda(ctx, dev_alloc(ctx, &ctx->scratch[i], bytes), "cudaMalloc(scratch)");
     if (rc) return rc;
   }
   ctx->scratch_bytes = bytes;
   return TMAMG_OK;
-}
-
-static int ensure_scratch(tmamg_ctx* ctx, size_t bytes) {
-  if (bytes <= ctx->scratch_bytes) return TMAMG_OK;
-  return with_optional_memory(ctx, [&] { return grow_scratch(ctx, bytes); });
 }
 
 }  // namespace tmamg
@@ -192,10 +198,10 @@ int tmamg_create(const int L[4], int bc_t, void* cuda_stream, tmamg_ctx** out) {
   ctx->g.bc_t = bc_t;
   ctx->stream = (cudaStream_t)cuda_stream;
   tmamg_default_setup_params(&ctx->sp);
-  int rc = check_cuda(ctx, dev_alloc(&ctx->U64, sizeof(double2) * 36 * ctx->g.V), "cudaMalloc(U64)");
-  if (!rc) rc = check_cuda(ctx, dev_alloc(&ctx->U32, sizeof(float2) * 36 * ctx->g.V), "cudaMalloc(U32)");
-  if (!rc) rc = check_cuda(ctx, dev_alloc(&ctx->C64, sizeof(double) * 72 * ctx->g.V), "cudaMalloc(C64)");
-  if (!rc) rc = check_cuda(ctx, dev_alloc(&ctx->C32, sizeof(float) * 72 * ctx->g.V), "cudaMalloc(C32)");
+  int rc = check_cuda(ctx, dev_alloc(ctx, &ctx->U64, sizeof(double2) * 36 * ctx->g.V), "cudaMalloc(U64)");
+  if (!rc) rc = check_cuda(ctx, dev_alloc(ctx, &ctx->U32, sizeof(float2) * 36 * ctx->g.V), "cudaMalloc(U32)");
+  if (!rc) rc = check_cuda(ctx, dev_alloc(ctx, &ctx->C64, sizeof(double) * 72 * ctx->g.V), "cudaMalloc(C64)");
+  if (!rc) rc = check_cuda(ctx, dev_alloc(ctx, &ctx->C32, sizeof(float) * 72 * ctx->g.V), "cudaMalloc(C32)");
   if (rc) {
     tmamg_destroy(ctx);
     return rc;
@@ -241,7 +247,7 @@ int tmamg_load_gauge(tmamg_ctx* ctx, const double* U, int on_device) {
   double* tmp = nullptr;
   size_t bytes = sizeof(double) * 2 * 36 * ctx->g.V;
   if (!on_device) {
-    int rc = check_cuda(ctx, dev_alloc(&tmp, bytes), "cudaMalloc(gauge staging)");
+    int rc = check_cuda(ctx, dev_alloc(ctx, &tmp, bytes), "cudaMalloc(gauge staging)");
     if (rc) return rc;
     rc = check_cuda(ctx, cudaMemcpyAsync(tmp, U, bytes, cudaMemcpyHostToDevice, ctx->stream), "upload gauge");
     if (rc) {
@@ -375,7 +381,7 @@ int tmamg_dirac_doublet(tmamg_ctx* ctx, const void* x_bundle, void* y_bundle, in
     cudaFree(ctx->eps_dev);
     ctx->eps_dev = nullptr;
     ctx->eps_cap = 0;
-    rc = check_cuda(ctx, dev_alloc(&ctx->eps_dev, sizeof(double) * npair), "cudaMalloc(eps)");
+    rc = check_cuda(ctx, dev_alloc(ctx, &ctx->eps_dev, sizeof(double) * npair), "cudaMalloc(eps)");
     if (rc) return rc;
     ctx->eps_cap = npair;
   }

@@ -410,7 +410,7 @@ __global__ void bg_steps_kernel(const int* __restrict__ active, int* steps, int 
   if (k < nblock && active[k]) steps[k] = j + 1;
 }
 
-int BlockGmres::alloc(int m_, int nsys_, int nshift_, int64_t M_) {
+int BlockGmres::alloc(tmamg_ctx* ctx, int m_, int nsys_, int nshift_, int64_t M_) {
   if (m_ <= m && nsys_ == nsys && nshift_ == nshift && M_ <= M) return 0;
   release();
   m = m_;
@@ -424,7 +424,7 @@ int BlockGmres::alloc(int m_, int nsys_, int nshift_, int64_t M_) {
   if (nblk < 1) nblk = 1;
   cudaError_t e = cudaSuccess;
   auto A = [&](void** q, size_t bytes) {
-    if (e == cudaSuccess) e = dev_alloc(q, bytes);
+    if (e == cudaSuccess) e = dev_alloc(ctx, q, bytes);
   };
   A((void**)&gram, sizeof(double2) * (size_t)(m + 1) * nsys * s);
   A((void**)&part, sizeof(double2) * (size_t)nblk * (m + 1) * nsys * s);

@@ -14,7 +14,7 @@ struct BlockGmres {
   double *cs = nullptr, *res = nullptr, *tolabs = nullptr;
   int *active = nullptr, *steps = nullptr, *nactive = nullptr;
   int* h_nactive = nullptr;
-  int alloc(int m, int nsys, int nshift, int64_t M);
+  int alloc(tmamg_ctx* ctx, int m, int nsys, int nshift, int64_t M);
   void release();
 };
 

@@ -869,7 +869,7 @@ __global__ void __launch_bounds__(CG_THREADS, 1) coarse_gmres_kernel(CGArgs p) {
   if (p.A16) cm_end(cs);
 }
 
-int CoarseGmres::alloc(int m_, int nsys_, int G_, size_t bundle_bytes, size_t x16b) {
+int CoarseGmres::alloc(tmamg_ctx* ctx, int m_, int nsys_, int G_, size_t bundle_bytes, size_t x16b) {
   if (m_ <= m && nsys_ <= NS && G_ <= G && bundle_bytes <= hbytes && x16b <= x16_bytes) return 0;
   release();
   m = m_;
@@ -879,7 +879,7 @@ int CoarseGmres::alloc(int m_, int nsys_, int G_, size_t bundle_bytes, size_t x1
   x16_bytes = x16b;
   cudaError_t e = cudaSuccess;
   auto A = [&](void** q, size_t bytes) {
-    if (e == cudaSuccess) e = dev_alloc(q, bytes);
+    if (e == cudaSuccess) e = dev_alloc(ctx, q, bytes);
   };
   A((void**)&H, sizeof(double2) * (size_t)(m + 1) * m * NS);
   A((void**)&cs, sizeof(double) * (size_t)m * NS);

@@ -17,7 +17,7 @@ struct CoarseGmres {
   size_t hbytes = 0;       // bytes of one coarse bundle the partials are sized for
   __half* X16 = nullptr;   // B images of the tensor-core stencil
   size_t x16_bytes = 0;
-  int alloc(int m, int nsys, int G, size_t bundle_bytes, size_t x16_bytes);
+  int alloc(tmamg_ctx* ctx, int m, int nsys, int G, size_t bundle_bytes, size_t x16_bytes);
   void release();
 };
 

@@ -118,12 +118,16 @@ int device_sms();
 int device_smem_optin();
 void func_smem_optin(const void* func, int bytes);
 
-// every device and pinned host allocation of the library (tmamg_debug_fail_alloc counts the device ones): *p is null and no
-// CUDA error is left behind where there is no memory
+// Every device and pinned host allocation of the library (tmamg_debug_fail_alloc counts the device ones): *p is null and no
+// CUDA error is left behind where there is no memory. Before a device allocation reports that, ctx (or null) gives
+// back what it can do without and the allocation is tried once more.
 cudaError_t alloc_bytes(void** p, size_t bytes, bool pinned);
+bool give_back(tmamg_ctx* ctx);
 template <class T>
-cudaError_t dev_alloc(T** p, size_t bytes) {
-  return alloc_bytes(reinterpret_cast<void**>(p), bytes, false);
+cudaError_t dev_alloc(tmamg_ctx* ctx, T** p, size_t bytes) {
+  cudaError_t e = alloc_bytes(reinterpret_cast<void**>(p), bytes, false);
+  if (e == cudaErrorMemoryAllocation && give_back(ctx)) e = alloc_bytes(reinterpret_cast<void**>(p), bytes, false);
+  return e;
 }
 template <class T>
 cudaError_t host_alloc(T** p, size_t bytes) {
@@ -135,23 +139,8 @@ int set_err(tmamg_ctx* ctx, int code, const std::string& msg);
 int check_cuda(tmamg_ctx* ctx, cudaError_t e, const char* what);
 int upload_mu(tmamg_ctx* ctx, const double* mu, int nsys);
 
-// runs f; if it found no device memory while the context holds some that it can do without (the correction
-// buffer of tmamg_sap, the optional copies of the operator: the FP64 stencil then runs in FP64 arithmetic),
-// gives that back and runs it again. f leaves nothing half allocated behind when it returns TMAMG_ERR_OOM.
 void free_fixed(Geom& g);
 void free_sap_delta(tmamg_ctx* ctx);
-template <class F>
-int with_optional_memory(tmamg_ctx* ctx, F f) {
-  int rc = f();
-  if (rc == TMAMG_ERR_OOM && (ctx->g.fx.U || ctx->sap_delta)) {
-    cudaStreamSynchronize(ctx->stream);
-    free_sap_delta(ctx);
-    free_fixed(ctx->g);
-    cudaGetLastError();
-    rc = f();
-  }
-  return rc;
-}
 
 // kernels launched from other translation units
 void launch_build_clover(const Geom& g, const double2* U64, double kappa, double c_sw, double* C64, float* C32,

@@ -128,10 +128,10 @@ void launch_fixed_clover(const Geom& g, const double* C64, cudaStream_t st) {
 
 int alloc_fixed(Geom& g) {
   FixedOp f;
-  cudaError_t e = dev_alloc(&f.U, sizeof(int4) * 36 * g.V);
-  if (e == cudaSuccess) e = dev_alloc(&f.nU, sizeof(int) * 4 * g.V);
-  if (e == cudaSuccess) e = dev_alloc(&f.C, sizeof(int2) * 72 * g.V);
-  if (e == cudaSuccess) e = dev_alloc(&f.nC, sizeof(int) * g.V);
+  cudaError_t e = dev_alloc(nullptr, &f.U, sizeof(int4) * 36 * g.V);
+  if (e == cudaSuccess) e = dev_alloc(nullptr, &f.nU, sizeof(int) * 4 * g.V);
+  if (e == cudaSuccess) e = dev_alloc(nullptr, &f.C, sizeof(int2) * 72 * g.V);
+  if (e == cudaSuccess) e = dev_alloc(nullptr, &f.nC, sizeof(int) * g.V);
   g.fx = f;
   if (e == cudaSuccess) return 0;
   free_fixed(g);

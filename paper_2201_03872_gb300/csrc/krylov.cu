@@ -14,7 +14,7 @@
 
 namespace tmamg {
 
-int GmresState::alloc(int m_, int cap_, size_t pe) {
+int GmresState::alloc(tmamg_ctx* ctx, int m_, int cap_, size_t pe) {
   if (m_ <= m && cap_ <= cap && pe <= partial_cap) return 0;
   release();
   m = m_;
@@ -22,7 +22,7 @@ int GmresState::alloc(int m_, int cap_, size_t pe) {
   partial_cap = pe;
   cudaError_t e = cudaSuccess;
   auto A = [&](void** p, size_t b) {
-    if (e == cudaSuccess) e = dev_alloc(p, b);
+    if (e == cudaSuccess) e = dev_alloc(ctx, p, b);
   };
   A((void**)&H, sizeof(double2) * (size_t)(m + 1) * m * cap);
   A((void**)&cs, sizeof(double) * (size_t)m * cap);

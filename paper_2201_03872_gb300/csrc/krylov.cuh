@@ -25,7 +25,7 @@ struct GmresState {
   int* h_nactive = nullptr;  // pinned host mirror
   double2* partial = nullptr;
   size_t partial_cap = 0;
-  int alloc(int m, int cap, size_t partial_elems);
+  int alloc(tmamg_ctx* ctx, int m, int cap, size_t partial_elems);
   void release();
 };
 

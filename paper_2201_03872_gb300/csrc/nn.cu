@@ -303,7 +303,7 @@ static void layer_wgrad(const NNGeom& g, const float2* U, const float* x, const 
   TM_COUNT();
 }
 
-int NNState::alloc(int64_t V, int nsys_) {
+int NNState::alloc(tmamg_ctx* ctx, int64_t V, int nsys_) {
   if (V <= Vcap && nsys_ <= nsys) return 0;
   release_buffers();
   Vcap = V;
@@ -311,7 +311,7 @@ int NNState::alloc(int64_t V, int nsys_) {
   const int nt = ntiles(nsys, NN_T);
   cudaError_t e = cudaSuccess;
   auto A = [&](void** q, size_t b) {
-    if (e == cudaSuccess) e = dev_alloc(q, b);
+    if (e == cudaSuccess) e = dev_alloc(ctx, q, b);
   };
   const size_t per_ch = (size_t)nt * 3 * V * 4 * sizeof(float);  // one channel of a bundle
   for (int l = 0; l < 4; ++l) A((void**)&act[l], per_ch * CH[l]);
@@ -323,12 +323,12 @@ int NNState::alloc(int64_t V, int nsys_) {
   return e == cudaSuccess ? 0 : -1;
 }
 
-int NNState::alloc_weights() {
+int NNState::alloc_weights(tmamg_ctx* ctx) {
   if (W) return 0;
   const int n = nn_weight_offset(3);
   cudaError_t e = cudaSuccess;
   auto A = [&](void** q, size_t b) {
-    if (e == cudaSuccess) e = dev_alloc(q, b);
+    if (e == cudaSuccess) e = dev_alloc(ctx, q, b);
   };
   A((void**)&W, sizeof(float2) * n);
   A((void**)&Winf, sizeof(float2) * n);

@@ -27,8 +27,8 @@ struct NNState {
   bool enabled = false;  // the gate: set only when the step lowered the iteration count
   int iters_plain = 0, iters_nn = 0;
   double loss_first = 0, loss_last = 0;
-  int alloc(int64_t V, int nsys);
-  int alloc_weights();
+  int alloc(tmamg_ctx* ctx, int64_t V, int nsys);
+  int alloc_weights(tmamg_ctx* ctx);
   void release_buffers();
   void release();
 };

@@ -150,7 +150,7 @@ static int ensure_ws(tmamg_ctx* ctx, int nsys, const tmamg_solve_params& p) {
   w->mb32 = (size_t)ntiles(ns, 2) * ncm * Vm * 4 * sizeof(float);
   cudaError_t e = cudaSuccess;
   auto A = [&](void** p, size_t b) {
-    if (e == cudaSuccess) e = dev_alloc(p, b);
+    if (e == cudaSuccess) e = dev_alloc(ctx, p, b);
   };
   A((void**)&w->V, w->fb32 * (mm + 1));
   A((void**)&w->Z, w->fb32 * mm);
@@ -203,11 +203,11 @@ static int ensure_ws(tmamg_ctx* ctx, int nsys, const tmamg_solve_params& p) {
     ws_free(w);
     return set_err(ctx, TMAMG_ERR_OOM, what);
   };
-  if (w->top.alloc(mm, ns, partial_elems(12 * V, ns, mm + 1, 2))) return oom("gmres state");
-  if (w->coarse.alloc(mcc, ns, partial_elems((int64_t)nc * Vc, ns, mcc + 1, 2))) return oom("gmres state");
-  if (three && w->mid.alloc(mmm, ns, partial_elems((int64_t)ncm * Vm, ns, mmm + 1, 2))) return oom("gmres state");
+  if (w->top.alloc(ctx, mm, ns, partial_elems(12 * V, ns, mm + 1, 2))) return oom("gmres state");
+  if (w->coarse.alloc(ctx, mcc, ns, partial_elems((int64_t)nc * Vc, ns, mcc + 1, 2))) return oom("gmres state");
+  if (three && w->mid.alloc(ctx, mmm, ns, partial_elems((int64_t)ncm * Vm, ns, mmm + 1, 2))) return oom("gmres state");
   // the grid for one tile is the largest any system count uses
-  if (w->cg.alloc(mcc, ns, coarse_gmres_grid(1), w->cb32, cm_x16_bytes(Vc, nc, ns))) return oom("coarse gmres state");
+  if (w->cg.alloc(ctx, mcc, ns, coarse_gmres_grid(1), w->cb32, cm_x16_bytes(Vc, nc, ns))) return oom("coarse gmres state");
   fill_c_kernel<<<(ns + 127) / 128, 128, 0, ctx->stream>>>(w->ones, ns, 1.0); TM_COUNT();
   fill_c_kernel<<<(ns + 127) / 128, 128, 0, ctx->stream>>>(w->mones, ns, -1.0); TM_COUNT();
   return check_cuda(ctx, cudaGetLastError(), "workspace init");
@@ -217,7 +217,7 @@ static int ensure_ws(tmamg_ctx* ctx, int nsys, const tmamg_solve_params& p) {
 static int ensure_t2(tmamg_ctx* ctx) {
   Workspace* w = ctx->ws;
   if (w->t2) return TMAMG_OK;
-  return check_cuda(ctx, dev_alloc(&w->t2, w->fb32), "cudaMalloc(learned-step scratch)");
+  return check_cuda(ctx, dev_alloc(ctx, &w->t2, w->fb32), "cudaMalloc(learned-step scratch)");
 }
 
 // the right-hand sides as FP64 bundles, one tile each (nrhs <= the workspace's system count)
@@ -229,7 +229,7 @@ static int ensure_b64(tmamg_ctx* ctx, int nrhs) {
   cudaFree(w->b64);
   w->b64 = nullptr;
   w->b64_bytes = 0;
-  int rc = check_cuda(ctx, dev_alloc(&w->b64, need), "cudaMalloc(right-hand sides)");
+  int rc = check_cuda(ctx, dev_alloc(ctx, &w->b64, need), "cudaMalloc(right-hand sides)");
   if (!rc) w->b64_bytes = need;
   return rc;
 }
@@ -341,12 +341,12 @@ static int setup_level2(tmamg_ctx* ctx, const tmamg_setup_params* p, const float
   lv.Vc = ad.Vc;
   lv.nv = nv2;
   lv.asize = ad.asize;
-  int rc = check_cuda(ctx, dev_alloc(&lv.P, sizeof(float2) * (size_t)ad.Vc * 2 * nv2 * ad.asize * nv1), "cudaMalloc(P2)");
-  if (!rc) rc = check_cuda(ctx, dev_alloc(&lv.A, sizeof(float2) * 9 * (size_t)ad.Vc * nc2 * nc2), "cudaMalloc(A2)");
+  int rc = check_cuda(ctx, dev_alloc(ctx, &lv.P, sizeof(float2) * (size_t)ad.Vc * 2 * nv2 * ad.asize * nv1), "cudaMalloc(P2)");
+  if (!rc) rc = check_cuda(ctx, dev_alloc(ctx, &lv.A, sizeof(float2) * 9 * (size_t)ad.Vc * nc2 * nc2), "cudaMalloc(A2)");
   if (!rc && nc2 <= CM_MAXNC)
-    rc = check_cuda(ctx, dev_alloc(&lv.A16, (size_t)cm_site_bytes(nc2) * ad.Vc), "cudaMalloc(A2 f16)");
-  if (!rc) rc = check_cuda(ctx, dev_alloc(&lv.cmax, sizeof(float) * CM_MAXSYS), "cudaMalloc(cmax)");
-  if (!rc) rc = check_cuda(ctx, dev_alloc(&lv.cerr, sizeof(int)), "cudaMalloc(cerr)");
+    rc = check_cuda(ctx, dev_alloc(ctx, &lv.A16, (size_t)cm_site_bytes(nc2) * ad.Vc), "cudaMalloc(A2 f16)");
+  if (!rc) rc = check_cuda(ctx, dev_alloc(ctx, &lv.cmax, sizeof(float) * CM_MAXSYS), "cudaMalloc(cmax)");
+  if (!rc) rc = check_cuda(ctx, dev_alloc(ctx, &lv.cerr, sizeof(int)), "cudaMalloc(cerr)");
   if (!rc) rc = check_cuda(ctx, cudaMemsetAsync(lv.cerr, 0, sizeof(int), st), "cudaMemset(cerr)");
   if (rc) {
     cudaFree(lv.P);
@@ -366,7 +366,7 @@ static int setup_level2(tmamg_ctx* ctx, const tmamg_setup_params* p, const float
   double2 *dots = nullptr, *sc = nullptr, *part = nullptr;
   cudaError_t e = cudaSuccess;
   auto A = [&](void** q, size_t b) {
-    if (e == cudaSuccess) e = dev_alloc(q, b);
+    if (e == cudaSuccess) e = dev_alloc(ctx, q, b);
   };
   A((void**)&Wt, b1(nv2));
   A((void**)&Wc, b1(nc2));
@@ -389,7 +389,7 @@ static int setup_level2(tmamg_ctx* ctx, const tmamg_setup_params* p, const float
     cg.release();
   };
   if (e == cudaSuccess && iterate &&
-      cg.alloc(m, nv2, coarse_gmres_grid(1), b1(nv2), cm_x16_bytes(L1.Vc, nc1, nv2)))
+      cg.alloc(ctx, m, nv2, coarse_gmres_grid(1), b1(nv2), cm_x16_bytes(L1.Vc, nc1, nv2)))
     e = cudaErrorMemoryAllocation;
   if (e != cudaSuccess) {
     cleanup();
@@ -397,7 +397,7 @@ static int setup_level2(tmamg_ctx* ctx, const tmamg_setup_params* p, const float
   }
   if (!vec2_dev) {
     const int64_t n = (int64_t)nv2 * L1.Vc * nc1;
-    e = dev_alloc(&field, sizeof(float2) * n);
+    e = dev_alloc(ctx, &field, sizeof(float2) * n);
     if (e == cudaSuccess) device_gaussian(p->seed, 0x5eed2ULL, n, reinterpret_cast<float2*>(field), st);
     if (e != cudaSuccess) {
       cleanup();
@@ -479,12 +479,12 @@ int do_setup(tmamg_ctx* ctx, const tmamg_setup_params* p, const float* vec_field
   lv.nv = nv;
   lv.asize = ad.asize;
   const int nc = 2 * nv;
-  int rc = check_cuda(ctx, dev_alloc(&lv.P, sizeof(float2) * (size_t)ad.Vc * 2 * nv * ad.asize * 6), "cudaMalloc(P)");
-  if (!rc) rc = check_cuda(ctx, dev_alloc(&lv.A, sizeof(float2) * 9 * (size_t)ad.Vc * nc * nc), "cudaMalloc(A)");
+  int rc = check_cuda(ctx, dev_alloc(ctx, &lv.P, sizeof(float2) * (size_t)ad.Vc * 2 * nv * ad.asize * 6), "cudaMalloc(P)");
+  if (!rc) rc = check_cuda(ctx, dev_alloc(ctx, &lv.A, sizeof(float2) * 9 * (size_t)ad.Vc * nc * nc), "cudaMalloc(A)");
   if (!rc && nc <= CM_MAXNC)
-    rc = check_cuda(ctx, dev_alloc(&lv.A16, (size_t)cm_site_bytes(nc) * ad.Vc), "cudaMalloc(A16)");
-  if (!rc) rc = check_cuda(ctx, dev_alloc(&lv.cmax, sizeof(float) * CM_MAXSYS), "cudaMalloc(cmax)");
-  if (!rc) rc = check_cuda(ctx, dev_alloc(&lv.cerr, sizeof(int)), "cudaMalloc(cerr)");
+    rc = check_cuda(ctx, dev_alloc(ctx, &lv.A16, (size_t)cm_site_bytes(nc) * ad.Vc), "cudaMalloc(A16)");
+  if (!rc) rc = check_cuda(ctx, dev_alloc(ctx, &lv.cmax, sizeof(float) * CM_MAXSYS), "cudaMalloc(cmax)");
+  if (!rc) rc = check_cuda(ctx, dev_alloc(ctx, &lv.cerr, sizeof(int)), "cudaMalloc(cerr)");
   if (!rc) rc = check_cuda(ctx, cudaMemsetAsync(lv.cerr, 0, sizeof(int), st), "cudaMemset(cerr)");
   if (rc) {
     cudaFree(lv.P);
@@ -504,7 +504,7 @@ int do_setup(tmamg_ctx* ctx, const tmamg_setup_params* p, const float* vec_field
   double2 *dots = nullptr, *sc = nullptr, *part = nullptr;
   cudaError_t e = cudaSuccess;
   auto A = [&](void** q, size_t b) {
-    if (e == cudaSuccess) e = dev_alloc(q, b);
+    if (e == cudaSuccess) e = dev_alloc(ctx, q, b);
   };
   A((void**)&Vt, vb);
   A((void**)&R, vb);
@@ -531,7 +531,7 @@ int do_setup(tmamg_ctx* ctx, const tmamg_setup_params* p, const float* vec_field
   float* field = nullptr;
   if (!vec_field_dev) {
     const int64_t n = (int64_t)nv * g.V * 12;
-    e = dev_alloc(&field, sizeof(float2) * n);
+    e = dev_alloc(ctx, &field, sizeof(float2) * n);
     if (e == cudaSuccess) device_gaussian(p->seed, 0x5eedULL, n, reinterpret_cast<float2*>(field), st);
     if (e != cudaSuccess) {
       cudaFree(field);
@@ -607,8 +607,8 @@ __global__ void copy_beta_kernel(const double* b, double* dst, int n) {
 // y = D_c x on level l: FP16 operator on the tensor cores (precision 16, or 0 = default) or
 // the FP32 stencil (precision 32); TMAMG_ERR_ARG if the sizes are outside the tensor-core path, TMAMG_ERR_OOM
 // if its operand images find no memory
-static int coarse_apply_level(CoarseLevel& l, int precision, const float* x, float* y, const double* mu, double dmu,
-                               int nsys, cudaStream_t st, const double* eps = nullptr) {
+static int coarse_apply_level(tmamg_ctx* ctx, CoarseLevel& l, int precision, const float* x, float* y,
+                              const double* mu, double dmu, int nsys, cudaStream_t st, const double* eps = nullptr) {
   const CoarseDims cd = coarse_dims(l);
   if (precision != 32) {
     if (!l.A16 || nsys > CM_MAXSYS) return TMAMG_ERR_ARG;
@@ -618,7 +618,7 @@ static int coarse_apply_level(CoarseLevel& l, int precision, const float* x, flo
       cudaFree(l.x16);
       l.x16 = nullptr;
       l.x16_bytes = 0;
-      if (dev_alloc(&l.x16, need) != cudaSuccess) return TMAMG_ERR_OOM;
+      if (dev_alloc(ctx, &l.x16, need) != cudaSuccess) return TMAMG_ERR_OOM;
       l.x16_bytes = need;
     }
     return coarse_apply_f16(cd, l.A16, x, y, mu, dmu, nsys, l.cmax, l.x16, l.cerr, st, eps) ? TMAMG_ERR_ARG : TMAMG_OK;
@@ -658,7 +658,7 @@ static void coarse_solve(SolveCtx& S, const float* rc, float* xc) {
   if (S.sp->coarse_solver == 1) {
     // block GMRES: one Krylov space per shift over that shift's right-hand sides
     const int64_t M = (int64_t)cd.nc * cd.Vc;
-    if (w->bg.alloc(S.sp->coarse_restart, S.nsys, S.nshift, M)) {
+    if (w->bg.alloc(ctx, S.sp->coarse_restart, S.nsys, S.nshift, M)) {
       S.oom = true;
       return;
     }
@@ -667,7 +667,7 @@ static void coarse_solve(SolveCtx& S, const float* rc, float* xc) {
     const int nsys = S.nsys;
     const int prec = S.sp->coarse_precision;
     auto apply = [&, dmu, mu, nsys, prec](const float* x, float* y) {
-      if (const int rc = coarse_apply_level(L1, prec, x, y, mu, dmu, nsys, st, S.eps)) S.failed(rc);
+      if (const int rc = coarse_apply_level(ctx, L1, prec, x, y, mu, dmu, nsys, st, S.eps)) S.failed(rc);
     };
     int it = 0;
     const size_t cbytes = (size_t)ntiles(nsys, 2) * M * 4 * sizeof(float);  // the caller's bundles hold nsys systems
@@ -687,7 +687,7 @@ static void coarse_solve(SolveCtx& S, const float* rc, float* xc) {
   const double* mu = S.mu;
   const int prec = S.sp->coarse_precision;
   ops.A = [&, dmu, mu, nsys, prec](const float* x, float* y) {
-    if (const int rc = coarse_apply_level(L1, prec, x, y, mu, dmu, nsys, st, S.eps)) S.failed(rc);
+    if (const int rc = coarse_apply_level(ctx, L1, prec, x, y, mu, dmu, nsys, st, S.eps)) S.failed(rc);
   };
   const size_t cbytes = (size_t)ntiles(nsys, 2) * M * 4 * sizeof(float);  // the caller's bundles hold nsys systems
   cudaMemsetAsync(xc, 0, cbytes, st);
@@ -741,7 +741,7 @@ static void mid_cycle(SolveCtx& S, const float* v, float* z) {
   const double dmu = 1.0;  // the twisted-mass factor delta_mu belongs to the bottom level only
   const int ns = w->nsys;
   auto apply = [&](const float* x, float* y) {
-    if (const int rc = coarse_apply_level(L1, prec, x, y, S.mu, dmu, nsys, st, S.eps)) S.failed(rc);
+    if (const int rc = coarse_apply_level(ctx, L1, prec, x, y, S.mu, dmu, nsys, st, S.eps)) S.failed(rc);
   };
   float* rho = w->sm1;
   float* q = w->sm2;
@@ -778,7 +778,7 @@ static void mid_solve(SolveCtx& S, const float* rm, float* xm) {
   LevelOps ops;
   ops.M = M;
   ops.A = [&](const float* x, float* y) {
-    if (const int rc = coarse_apply_level(L1, prec, x, y, S.mu, dmu, nsys, st, S.eps)) S.failed(rc);
+    if (const int rc = coarse_apply_level(ctx, L1, prec, x, y, S.mu, dmu, nsys, st, S.eps)) S.failed(rc);
   };
   ops.precond = [&](const float* v, float* z) { mid_cycle(S, v, z); };
   const size_t mbytes = (size_t)ntiles(nsys, 2) * M * 4 * sizeof(float);  // the caller's bundles hold nsys systems
@@ -941,7 +941,7 @@ static int ensure_ws64(tmamg_ctx* ctx, int nsys, int m, int mc) {
   w->cb = (size_t)ns * w->nc * w->Vc * 2 * sizeof(double);
   cudaError_t e = cudaSuccess;
   auto A = [&](void** p, size_t bytes) {
-    if (e == cudaSuccess) e = dev_alloc(p, bytes);
+    if (e == cudaSuccess) e = dev_alloc(ctx, p, bytes);
   };
   A((void**)&w->V, w->fb * (mm + 1));
   A((void**)&w->Z, w->fb * mm);
@@ -966,8 +966,8 @@ static int ensure_ws64(tmamg_ctx* ctx, int nsys, int m, int mc) {
     ws64_free(w);
     return check_cuda(ctx, e, "FP64 workspace allocation");
   }
-  if (w->top.alloc(mm, ns, partial_elems(12 * V, ns, mm + 1, 1)) ||
-      w->coarse.alloc(mcc, ns, partial_elems((int64_t)w->nc * w->Vc, ns, mcc + 1, 1))) {
+  if (w->top.alloc(ctx, mm, ns, partial_elems(12 * V, ns, mm + 1, 1)) ||
+      w->coarse.alloc(ctx, mcc, ns, partial_elems((int64_t)w->nc * w->Vc, ns, mcc + 1, 1))) {
     ws64_free(w);
     return set_err(ctx, TMAMG_ERR_OOM, "FP64 gmres state");
   }
@@ -1040,8 +1040,8 @@ int do_solve64(tmamg_ctx* ctx, const double* b, int nrhs, const double* mu, int 
   int rc = 0;
   if (!L1.P64) {
     const int64_t np = L1.Vc * 2 * L1.nv * L1.asize * 6, na = 9 * L1.Vc * nc * nc;
-    rc = check_cuda(ctx, dev_alloc(&L1.P64, sizeof(double2) * np), "cudaMalloc(P64)");
-    if (!rc) rc = check_cuda(ctx, dev_alloc(&L1.A64, sizeof(double2) * na), "cudaMalloc(A64)");
+    rc = check_cuda(ctx, dev_alloc(ctx, &L1.P64, sizeof(double2) * np), "cudaMalloc(P64)");
+    if (!rc) rc = check_cuda(ctx, dev_alloc(ctx, &L1.A64, sizeof(double2) * na), "cudaMalloc(A64)");
     if (rc) {  // both or neither: P64 stands for the pair, widened
       cudaFree(L1.P64);
       L1.P64 = nullptr;
@@ -1063,8 +1063,8 @@ int do_solve64(tmamg_ctx* ctx, const double* b, int nrhs, const double* mu, int 
   const size_t xbytes = sizeof(double) * 2 * M * nsys;
   if (!on_device) {
     const size_t bytes = sizeof(double) * 2 * M * nrhs;
-    rc = check_cuda(ctx, dev_alloc(&bstage, bytes), "cudaMalloc(b staging)");
-    if (!rc) rc = check_cuda(ctx, dev_alloc(&xstage, xbytes), "cudaMalloc(x staging)");
+    rc = check_cuda(ctx, dev_alloc(ctx, &bstage, bytes), "cudaMalloc(b staging)");
+    if (!rc) rc = check_cuda(ctx, dev_alloc(ctx, &xstage, xbytes), "cudaMalloc(x staging)");
     if (rc) {
       cudaFree(bstage);
       return rc;
@@ -1189,7 +1189,7 @@ int do_solve(tmamg_ctx* ctx, const double* b, int nrhs, const double* mu, int ns
       cudaFree(w->epsd);
       w->epsd = nullptr;
       w->eps_cap = 0;
-      rc = check_cuda(ctx, dev_alloc(&w->epsd, sizeof(double) * np), "cudaMalloc(splittings)");
+      rc = check_cuda(ctx, dev_alloc(ctx, &w->epsd, sizeof(double) * np), "cudaMalloc(splittings)");
       if (rc) return rc;
       w->eps_cap = np;
     }
@@ -1223,7 +1223,7 @@ int do_solve(tmamg_ctx* ctx, const double* b, int nrhs, const double* mu, int ns
   S.nn = sp->use_nn == 2 || (sp->use_nn == 1 && ctx->nn && ctx->nn->enabled);
   if (S.nn && (!ctx->nn || !ctx->nn->trained)) return set_err(ctx, TMAMG_ERR_STATE, "solve: no trained network");
   if (S.nn) {
-    if (ctx->nn->alloc(ctx->g.V, nsys)) return set_err(ctx, TMAMG_ERR_OOM, "solve: network buffers");
+    if (ctx->nn->alloc(ctx, ctx->g.V, nsys)) return set_err(ctx, TMAMG_ERR_OOM, "solve: network buffers");
     rc = ensure_t2(ctx);
     if (rc) return rc;
   }
@@ -1328,13 +1328,13 @@ int tmamg_debug_bounded_wait(long long limit_cycles, int unreachable_next) {
 int tmamg_setup(tmamg_ctx* ctx, const tmamg_setup_params* p, const float* start_vectors) {
   if (!ctx || !p) return set_err(ctx, TMAMG_ERR_ARG, "setup: null argument");
   if (!ctx->have_op) return set_err(ctx, TMAMG_ERR_STATE, "setup: operator not set");
-  return with_optional_memory(ctx, [&] { return do_setup(ctx, p, start_vectors, true); });
+  return do_setup(ctx, p, start_vectors, true);
 }
 
 int tmamg_setup_from_vectors(tmamg_ctx* ctx, const tmamg_setup_params* p, const float* test_vectors) {
   if (!ctx || !p || !test_vectors) return set_err(ctx, TMAMG_ERR_ARG, "setup_from_vectors: null argument");
   if (!ctx->have_op) return set_err(ctx, TMAMG_ERR_STATE, "setup_from_vectors: operator not set");
-  return with_optional_memory(ctx, [&] { return do_setup(ctx, p, test_vectors, false); });
+  return do_setup(ctx, p, test_vectors, false);
 }
 
 int tmamg_solve(tmamg_ctx* ctx, const double* b, int nrhs, const double* mu, int nshift, double* x, int on_device,
@@ -1344,7 +1344,7 @@ int tmamg_solve(tmamg_ctx* ctx, const double* b, int nrhs, const double* mu, int
   if (!ctx->have_setup) return set_err(ctx, TMAMG_ERR_STATE, "solve: no multigrid setup");
   tmamg_solve_params def;
   tmamg_default_solve_params(&def);
-  return with_optional_memory(ctx, [&] { return do_solve(ctx, b, nrhs, mu, nshift, x, on_device, p ? p : &def, stats, nullptr); });
+  return do_solve(ctx, b, nrhs, mu, nshift, x, on_device, p ? p : &def, stats, nullptr);
 }
 
 int tmamg_solve_doublet(tmamg_ctx* ctx, const double* b, int nrhs, const double* mu, const double* eps, int nshift,
@@ -1355,7 +1355,7 @@ int tmamg_solve_doublet(tmamg_ctx* ctx, const double* b, int nrhs, const double*
   if (!ctx->have_setup) return set_err(ctx, TMAMG_ERR_STATE, "solve_doublet: no multigrid setup");
   tmamg_solve_params def;
   tmamg_default_solve_params(&def);
-  return with_optional_memory(ctx, [&] { return do_solve(ctx, b, nrhs, mu, nshift, x, on_device, p ? p : &def, stats, eps); });
+  return do_solve(ctx, b, nrhs, mu, nshift, x, on_device, p ? p : &def, stats, eps);
 }
 
 size_t tmamg_coarse_bundle_bytes(const tmamg_ctx* ctx, int level, int nsys) {
@@ -1378,9 +1378,7 @@ int tmamg_sap(tmamg_ctx* ctx, void* r_bundle, void* e_bundle, int nsys, const do
   const size_t bytes = (size_t)ntiles(nsys, 2) * 12 * ctx->g.V * 4 * sizeof(float);
   if (bytes > ctx->sap_delta_bytes) {
     free_sap_delta(ctx);
-    rc = with_optional_memory(ctx, [&] {
-      return check_cuda(ctx, dev_alloc(&ctx->sap_delta, bytes), "cudaMalloc(sap scratch)");
-    });
+    rc = check_cuda(ctx, dev_alloc(ctx, &ctx->sap_delta, bytes), "cudaMalloc(sap scratch)");
     if (rc) return rc;
     ctx->sap_delta_bytes = bytes;
   }
@@ -1443,7 +1441,7 @@ int tmamg_coarse_solve(tmamg_ctx* ctx, int level, const void* rc_bundle, void* x
       p->coarse_restart < 1 || p->coarse_restart > 64 || p->coarse_maxiter < 1 ||
       (p->coarse_precision != 0 && p->coarse_precision != 16 && p->coarse_precision != 32))
     return set_err(ctx, TMAMG_ERR_ARG, "coarse_solve: bad parameters");
-  int rc = with_optional_memory(ctx, [&] { return ensure_ws(ctx, nsys, *p); });
+  int rc = ensure_ws(ctx, nsys, *p);
   if (rc) return rc;
   std::vector<double> musys(nsys);
   for (int n = 0; n < nsys; ++n) musys[n] = mu[n % nshift];
@@ -1475,7 +1473,8 @@ int tmamg_coarse_apply(tmamg_ctx* ctx, int level, const void* x_bundle, void* y_
   int rc = upload_mu(ctx, mu, nsys);
   if (rc) return rc;
   CoarseLevel& l = ctx->levels[level - 1];
-  rc = coarse_apply_level(l, precision, (const float*)x_bundle, (float*)y_bundle, ctx->mu_dev, 1.0, nsys, ctx->stream);
+  rc = coarse_apply_level(ctx, l, precision, (const float*)x_bundle, (float*)y_bundle, ctx->mu_dev, 1.0, nsys,
+                          ctx->stream);
   if (rc == TMAMG_ERR_OOM) return set_err(ctx, rc, "coarse_apply: operand images");
   if (rc) return set_err(ctx, rc, "coarse_apply: sizes outside the tensor-core stencil");
   rc = check_cuda(ctx, cudaGetLastError(), "coarse_apply launch");
@@ -1503,7 +1502,7 @@ static NNGeom nn_geom(const tmamg_ctx* ctx) {
 
 static int nn_ready(tmamg_ctx* ctx) {
   if (!ctx->nn) ctx->nn = new NNState();
-  return ctx->nn->alloc_weights();
+  return ctx->nn->alloc_weights(ctx);
 }
 
 // host weights (complex double, three layers concatenated) <-> device FP32 master weights
@@ -1525,7 +1524,7 @@ static int nn_upload(tmamg_ctx* ctx, const double* W) {
 static int random_bundle(tmamg_ctx* ctx, uint64_t seed, int nsys, float* bundle) {
   const int64_t n = (int64_t)nsys * ctx->g.V * 12;
   float* field = nullptr;
-  int rc = check_cuda(ctx, dev_alloc(&field, sizeof(float2) * n), "cudaMalloc(random field)");
+  int rc = check_cuda(ctx, dev_alloc(ctx, &field, sizeof(float2) * n), "cudaMalloc(random field)");
   if (rc) return rc;
   device_gaussian(seed, 0x5eedULL, n, reinterpret_cast<float2*>(field), ctx->stream);
   launch_pack<float>(ctx->g, field, bundle, nsys, ctx->stream);
@@ -1632,7 +1631,7 @@ int tmamg_nn_forward(tmamg_ctx* ctx, const void* r_bundle, void* y_bundle, int n
   if (!ctx) return TMAMG_ERR_ARG;
   if (!r_bundle || !y_bundle || nsys < 1 || r_bundle == y_bundle) return set_err(ctx, TMAMG_ERR_ARG, "nn_forward: bad argument");
   if (!ctx->nn || !ctx->nn->trained) return set_err(ctx, TMAMG_ERR_STATE, "nn_forward: no weights");
-  if (ctx->nn->alloc(ctx->g.V, nsys)) return set_err(ctx, TMAMG_ERR_OOM, "nn_forward: buffers");
+  if (ctx->nn->alloc(ctx, ctx->g.V, nsys)) return set_err(ctx, TMAMG_ERR_OOM, "nn_forward: buffers");
   nn_forward(*ctx->nn, nn_geom(ctx), ctx->U32, (const float*)r_bundle, (float*)y_bundle, nsys, bf16 != 0, ctx->stream);
   return check_cuda(ctx, cudaGetLastError(), "nn_forward");
 }
@@ -1646,7 +1645,7 @@ int tmamg_nn_loss_grad(tmamg_ctx* ctx, const void* r_bundle, const void* e_bundl
   tmamg_default_solve_params(&def);
   int rc = ensure_ws(ctx, nsys, def);
   if (rc) return rc;
-  if (ctx->nn->alloc(ctx->g.V, nsys)) return set_err(ctx, TMAMG_ERR_OOM, "nn_loss_grad: buffers");
+  if (ctx->nn->alloc(ctx, ctx->g.V, nsys)) return set_err(ctx, TMAMG_ERR_OOM, "nn_loss_grad: buffers");
   rc = ensure_t2(ctx);
   if (rc) return rc;
   Workspace* w = ctx->ws;
@@ -1681,7 +1680,7 @@ int tmamg_nn_train(tmamg_ctx* ctx, const tmamg_nn_params* p, tmamg_nn_report* re
   tmamg_default_solve_params(&sp);
   int rc = ensure_ws(ctx, nsys, sp);
   if (rc) return rc;
-  if (nns.alloc(ctx->g.V, nsys)) return set_err(ctx, TMAMG_ERR_OOM, "nn_train: buffers");
+  if (nns.alloc(ctx, ctx->g.V, nsys)) return set_err(ctx, TMAMG_ERR_OOM, "nn_train: buffers");
   rc = ensure_t2(ctx);
   if (rc) return rc;
   Workspace* w = ctx->ws;
@@ -1693,8 +1692,8 @@ int tmamg_nn_train(tmamg_ctx* ctx, const tmamg_nn_params* p, tmamg_nn_report* re
   const int nb = p->pairs / nsys;
   const int win = p->window > 0 && p->window < nb ? p->window : nb;
   float *R = nullptr, *E = nullptr;
-  rc = check_cuda(ctx, dev_alloc(&R, w->fb32 * win), "cudaMalloc(pairs)");
-  if (!rc) rc = check_cuda(ctx, dev_alloc(&E, w->fb32 * win), "cudaMalloc(pairs)");
+  rc = check_cuda(ctx, dev_alloc(ctx, &R, w->fb32 * win), "cudaMalloc(pairs)");
+  if (!rc) rc = check_cuda(ctx, dev_alloc(ctx, &E, w->fb32 * win), "cudaMalloc(pairs)");
   if (rc) {
     cudaFree(R);
     return rc;

@@ -7,31 +7,40 @@ import numpy as np
 import pytest
 
 import synth
-from oracle import dirac
+from oracle import dirac, doublet
 from oracle import nn as onn
-from tests.gpu_util import Lattice, from_dev, to_dev
+from tests.gpu_util import Lattice, from_dev, to_dev, torch_cuda
 
 pytestmark = pytest.mark.gpu
 
 L = (8, 4, 4, 8)
 KAPPA = 0.125
 ALL = 1 << 30
+REFUSALS = 1  # of the copies of the operator
 U = synth.gauge_field(L, 0.3, seed=401)
 
 
 class Problem:
-    """A context with a two-level setup, one right-hand side and two masses."""
+    """A context with a two-level setup, one right-hand side and two masses; or one without copies of the operator
+    and without a setup."""
 
-    def __init__(self, agg=(2, 2, 2, 2), weights=True):
-        self.lat = Lattice(L, U, KAPPA, 1.0)
-        T = self.T = self.lat.T
+    def __init__(self, weights=True, copies=True):
+        torch_cuda()
+        from paper_2201_03872_gb300 import tmamg as T
+        self.T = T
+        refuse = 0 if copies else REFUSALS
+        T.tmamg_debug_fail_alloc(4, refuse)  # create makes four arrays that it needs, then the copies
+        self.lat = Lattice(L, to_dev(U), KAPPA, 1.0)
+        assert T.tmamg_debug_fail_alloc(0, 0) == refuse
         self.ctx = self.lat.ctx
-        tv = to_dev(synth.gaussian_spinors(L, 4, seed=402).astype(np.complex64))
-        T.tmamg_setup_from_vectors(self.ctx, T.setup_params(agg=agg, nv=4, sap_block=(2, 2, 2, 2)), tv)
-        if weights:
-            T.tmamg_nn_init(self.ctx, 11)
         self.mu = np.array([0.01, 0.2])
         self.b = synth.gaussian_spinors(L, 1, seed=403)
+        if not copies:
+            return
+        tv = to_dev(synth.gaussian_spinors(L, 4, seed=402).astype(np.complex64))
+        T.tmamg_setup_from_vectors(self.ctx, T.setup_params(agg=(2, 2, 2, 2), nv=4, sap_block=(2, 2, 2, 2)), tv)
+        if weights:
+            T.tmamg_nn_init(self.ctx, 11)
 
     def solve(self, host=False, **kw):
         p = self.T.solve_params(tol=1e-10, **kw)
@@ -90,3 +99,79 @@ def test_network_weights_after_a_failure():
         y = q.lat.torch.zeros_like(r)
         q.T.tmamg_nn_forward(q.ctx, r, y, 1, bf16=True)
         assert np.isfinite(q.lat.from_fine_bundle(y, 1)).all()
+
+
+def fp64_application(q):
+    """D x in FP64 on two systems and on a doublet, against the oracle."""
+    T, torch = q.T, q.lat.torch
+    x = synth.gaussian_spinors(L, 2, seed=404)
+    xb = torch.empty(T.tmamg_bundle_bytes(q.ctx, 2, 64) // 8, dtype=torch.float64, device="cuda")
+    yb, yf = torch.empty_like(xb), to_dev(x)
+    T.tmamg_pack(q.ctx, to_dev(x), xb, 2, 64)
+    op = dirac.Operator(U, KAPPA, 1.0)
+    T.tmamg_dirac(q.ctx, xb, yb, 2, q.mu, 64)
+    T.tmamg_unpack(q.ctx, yb, yf, 2, 64)
+    y, ref = from_dev(yf, x.shape), op.apply(x, q.mu)
+    assert np.linalg.norm(y - ref) <= 1e-14 * np.linalg.norm(ref)  # about 80 roundings at 2^-53 on both sides
+    T.tmamg_dirac_doublet(q.ctx, xb, yb, 1, q.mu[:1], np.array([0.3]), 64)
+    T.tmamg_unpack(q.ctx, yb, yf, 2, 64)
+    ref = np.stack(doublet.apply(op, x[0], x[1], q.mu[0], 0.3))
+    assert np.linalg.norm(from_dev(yf, x.shape) - ref) <= 1e-14 * np.linalg.norm(ref)
+    return y
+
+
+def _bundles(q, make, n=1):
+    x = make(n)
+    x.normal_()
+    return x, q.lat.torch.zeros_like(x)
+
+
+def _fine(q, n):
+    return q.lat.fine_bundle(synth.gaussian_spinors(L, n, seed=405))
+
+
+def _apply(q):
+    x = to_dev(q.b)
+    q.T.tmamg_apply(q.ctx, x, q.lat.torch.zeros_like(x), 1, q.mu[:1], 64)
+
+
+def _setup(q):
+    q.T.tmamg_setup(q.ctx, q.T.setup_params(agg=(2, 2, 2, 2), nv=4, sap_block=(2, 2, 2, 2), setup_iters=1))
+
+
+CALLS = {
+    "load_gauge": lambda q: (q.T.tmamg_load_gauge(q.ctx, U), q.T.tmamg_set_operator(q.ctx, KAPPA, 1.0)),
+    "apply": _apply,
+    "sap": lambda q: q.T.tmamg_sap(q.ctx, *_bundles(q, lambda n: _fine(q, n)), 1, q.mu[:1], (2, 2, 2, 2), 1, 2),
+    "coarse_apply": lambda q: q.T.tmamg_coarse_apply(q.ctx, 1, *_bundles(q, q.lat.coarse_buffer), 1, q.mu[:1], 16),
+    "setup": _setup,
+    "solve": lambda q: q.solve(host=True),
+    "solve64": lambda q: q.solve(host=True, precision=64),
+    "learned step": lambda q: q.solve(use_nn=2),
+    "block GMRES": lambda q: q.solve(coarse_solver=1),
+    "nn_forward": lambda q: q.T.tmamg_nn_forward(q.ctx, *_bundles(q, lambda n: _fine(q, n)), 1),
+    "nn_loss_grad": lambda q: q.T.tmamg_nn_loss_grad(q.ctx, _fine(q, 1), _fine(q, 1), 1),
+}
+
+
+@pytest.mark.parametrize("name", list(CALLS))
+def test_an_allocation_that_finds_no_memory_gets_what_the_context_can_spare(name):
+    for q, error in every_allocation(Problem, CALLS[name], count=1):
+        assert error is None, error
+        fp64_application(q)  # without the copies of the operator
+
+
+def test_context_without_room_for_the_copies_of_the_operator():
+    torch_cuda()
+    from paper_2201_03872_gb300 import tmamg as T
+    try:
+        for k in range(4):
+            T.tmamg_debug_fail_alloc(k, ALL)
+            with pytest.raises(T.TmamgError) as e:
+                T.tmamg_create(L, -1)
+            assert e.value.code == -3
+    finally:
+        T.tmamg_debug_fail_alloc(0, 0)
+    q = Problem(copies=False)
+    fp64_application(q)
+    q.lat.close()
