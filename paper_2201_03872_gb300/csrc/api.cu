@@ -81,12 +81,14 @@ cudaError_t alloc_bytes(void** p, size_t bytes, bool pinned) {
 }
 
 // the correction buffer of tmamg_sap, and the copies of the operator, without which the FP64 stencil runs in FP64
-// arithmetic
+// arithmetic, unless a captured graph reads them
 bool give_back(tmamg_ctx* ctx) {
-  if (!ctx || !(ctx->g.fx.U || ctx->sap_delta)) return false;
+  if (!ctx) return false;
+  const bool fixed = ctx->g.fx.U && !ctx->fixed_captured;
+  if (!fixed && !ctx->sap_delta) return false;
   cudaStreamSynchronize(ctx->stream);
   free_sap_delta(ctx);
-  free_fixed(ctx->g);
+  if (fixed) free_fixed(ctx->g);
   return true;
 }
 
@@ -318,12 +320,20 @@ int tmamg_unpack(tmamg_ctx* ctx, const void* x_bundle, void* x_field, int nsys, 
   return check_cuda(ctx, cudaGetLastError(), "unpack launch");
 }
 
+static bool capturing(tmamg_ctx* ctx) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  return cudaStreamIsCapturing(ctx->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone;
+}
+
 // whether the FP32 stencil takes this call's masses as values (not while the stream is being captured: a replay
 // reads them where the caller keeps them)
 static bool takes_values(tmamg_ctx* ctx, int nsys, int prec) {
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  return prec == 32 && dirac32_takes_values(ctx->g, nsys) &&
-         cudaStreamIsCapturing(ctx->stream, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
+  return prec == 32 && dirac32_takes_values(ctx->g, nsys) && !capturing(ctx);
+}
+
+// before a stencil launch of precision prec
+static void keep_if_captured(tmamg_ctx* ctx, int prec) {
+  if (prec == 64 && ctx->g.fx.U && !ctx->fixed_captured) ctx->fixed_captured = capturing(ctx);
 }
 
 int tmamg_dirac(tmamg_ctx* ctx, const void* x_bundle, void* y_bundle, int nsys, const double* mu, int prec) {
@@ -339,6 +349,7 @@ int tmamg_dirac(tmamg_ctx* ctx, const void* x_bundle, void* y_bundle, int nsys, 
   }
   int rc = upload_mu(ctx, mu, nsys);
   if (rc) return rc;
+  keep_if_captured(ctx, prec);
   if (prec == 32)
     launch_dirac<float>(ctx->g, ctx->U32, ctx->C32, (const float*)x_bundle, (float*)y_bundle, ctx->mu_dev, nsys,
                         ctx->stream);
@@ -388,6 +399,7 @@ int tmamg_dirac_doublet(tmamg_ctx* ctx, const void* x_bundle, void* y_bundle, in
   rc = check_cuda(ctx, cudaMemcpyAsync(ctx->eps_dev, eps, sizeof(double) * npair, cudaMemcpyHostToDevice,
                                        ctx->stream), "upload eps");
   if (rc) return rc;
+  keep_if_captured(ctx, prec);
   if (prec == 32)
     launch_dirac<float>(ctx->g, ctx->U32, ctx->C32, (const float*)x_bundle, (float*)y_bundle, ctx->mu_dev, nsys,
                         ctx->stream, ctx->eps_dev);
@@ -406,6 +418,7 @@ int tmamg_dirac_eo(tmamg_ctx* ctx, const void* x_bundle, void* y_bundle, int nsy
   int rc = upload_mu(ctx, mu, nsys);
   if (!rc) rc = ensure_scratch(ctx, tmamg_bundle_bytes(ctx, nsys, prec));
   if (rc) return rc;
+  keep_if_captured(ctx, prec);
   if (prec == 32)
     launch_dirac_eo<float>(ctx->g, ctx->U32, ctx->C32, (const float*)x_bundle, (float*)y_bundle, ctx->mu_dev, nsys,
                            (float*)ctx->scratch[0], (float*)ctx->scratch[1], ctx->stream);

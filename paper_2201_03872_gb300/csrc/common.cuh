@@ -85,6 +85,8 @@ struct tmamg_ctx {
   float* C32 = nullptr;
   double kappa = 0.0, c_sw = 0.0;
   bool have_gauge = false, have_op = false, have_setup = false;
+  // a launch that reads the fixed-point copies was captured into a graph: a replay needs them where they are
+  bool fixed_captured = false;
   // twisted masses on the device (per system), cached
   double* mu_dev = nullptr;
   int mu_cap = 0;

@@ -175,3 +175,40 @@ def test_context_without_room_for_the_copies_of_the_operator():
     q = Problem(copies=False)
     fp64_application(q)
     q.lat.close()
+
+
+def test_captured_fp64_application_keeps_its_copies_of_the_operator():
+    torch = torch_cuda()
+    from paper_2201_03872_gb300 import tmamg as T
+    st = torch.cuda.Stream()
+    mu = np.array([0.01])
+    x = synth.gaussian_spinors(L, 1, seed=406)
+    with torch.cuda.stream(st):
+        ctx = T.tmamg_create(L, -1, st.cuda_stream)
+        T.tmamg_load_gauge(ctx, U)
+        T.tmamg_set_operator(ctx, KAPPA, 1.0)
+        xb = torch.empty(T.tmamg_bundle_bytes(ctx, 1, 64) // 8, dtype=torch.float64, device="cuda")
+        yb = torch.empty_like(xb)
+        T.tmamg_pack(ctx, to_dev(x), xb, 1, 64)
+        T.tmamg_dirac(ctx, xb, yb, 1, mu, 64)  # the launch variants are timed outside the capture
+        st.synchronize()
+        ref = yb.clone()
+        graph = torch.cuda.CUDAGraph()
+        graph.capture_begin(capture_error_mode="thread_local")
+        T.tmamg_dirac(ctx, xb, yb, 1, mu, 64)
+        graph.capture_end()
+        T.tmamg_debug_fail_alloc(0, 1)
+        try:  # nothing to spare
+            with pytest.raises(T.TmamgError) as e:
+                T.tmamg_dirac_eo(ctx, xb, yb, 1, mu, 64)
+            assert e.value.code == -3 and T.tmamg_debug_fail_alloc(0, 0) == 1
+        finally:
+            T.tmamg_debug_fail_alloc(0, 0)
+        taken = torch.full((1 << 24,), float("nan"), device="cuda")  # memory that a copy given back would be in
+        for _ in range(2):
+            yb.zero_()
+            graph.replay()
+            st.synchronize()
+            assert torch.equal(yb, ref)
+        del taken
+        T.tmamg_destroy(ctx)
