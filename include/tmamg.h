@@ -121,7 +121,13 @@ void tmamg_default_solve_params(tmamg_solve_params* p);
 
 /* Create a context for an Lx x Ly x Lz x Lt lattice (L[0..3] = x, y, z, t; each even, >= 2).
  * bc_t: -1 antiperiodic or +1 periodic in t. cuda_stream: a cudaStream_t (NULL = default stream).
- * The context owns every device buffer it allocates; tmamg_destroy frees them. */
+ * The context owns every device buffer it allocates; tmamg_destroy frees them. Besides the operator in
+ * both precisions (1728 bytes per site) it holds, where they fit, fixed-point copies for the FP64 stencil
+ * (1172 bytes per site), and from the first tmamg_sap on that call's correction buffer. It gives these
+ * back when one of its allocations finds no memory; without the copies the FP64 stencil runs in FP64
+ * arithmetic, about four times slower. Copies given back are made again, where they fit, at the end of
+ * a call that did not keep their memory, and by tmamg_load_gauge, tmamg_set_operator and tmamg_setup.
+ * Once an FP64 application has been captured into a CUDA graph they stay where they are. */
 int tmamg_create(const int L[4], int bc_t, void* cuda_stream, tmamg_ctx** out);
 int tmamg_destroy(tmamg_ctx* ctx);
 const char* tmamg_last_error(const tmamg_ctx* ctx);

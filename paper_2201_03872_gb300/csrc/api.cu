@@ -88,8 +88,23 @@ bool give_back(tmamg_ctx* ctx) {
   if (!fixed && !ctx->sap_delta) return false;
   cudaStreamSynchronize(ctx->stream);
   free_sap_delta(ctx);
-  if (fixed) free_fixed(ctx->g);
+  if (fixed) {
+    free_fixed(ctx->g);
+    ctx->gave_back = true;
+  }
   return true;
+}
+
+void take_again(tmamg_ctx* ctx) {
+  if (ctx->g.fx.U || !ctx->have_gauge || alloc_fixed(ctx->g)) return;
+  launch_fixed_links(ctx->g, ctx->U64, ctx->stream);
+  if (ctx->have_op) launch_fixed_clover(ctx->g, ctx->C64, ctx->stream);
+}
+
+TakeAgain::~TakeAgain() {
+  if (!ctx || !ctx->gave_back) return;
+  ctx->gave_back = false;
+  take_again(ctx);
 }
 
 int set_err(tmamg_ctx* ctx, int code, const std::string& msg) {
@@ -244,6 +259,7 @@ int tmamg_volume(const tmamg_ctx* ctx, int64_t* V) {
 }
 
 int tmamg_load_gauge(tmamg_ctx* ctx, const double* U, int on_device) {
+  const TakeAgain at_end(ctx);
   if (!ctx || !U) return set_err(ctx, TMAMG_ERR_ARG, "load_gauge: null argument");
   const double* src = U;
   double* tmp = nullptr;
@@ -269,7 +285,8 @@ int tmamg_load_gauge(tmamg_ctx* ctx, const double* U, int on_device) {
   ctx->have_gauge = true;
   ctx->have_op = false;
   ctx->have_setup = false;
-  return TMAMG_OK;
+  take_again(ctx);
+  return check_cuda(ctx, cudaGetLastError(), "load_gauge launch");
 }
 
 int tmamg_set_operator(tmamg_ctx* ctx, double kappa, double c_sw) {
@@ -286,7 +303,8 @@ int tmamg_set_operator(tmamg_ctx* ctx, double kappa, double c_sw) {
   ctx->have_setup = false;
   free_workspace(ctx);
   free_levels(ctx);
-  return TMAMG_OK;
+  take_again(ctx);
+  return check_cuda(ctx, cudaGetLastError(), "set_operator launch");
 }
 
 long long tmamg_debug_fail_alloc(int skip, int count) {
@@ -337,6 +355,7 @@ static void keep_if_captured(tmamg_ctx* ctx, int prec) {
 }
 
 int tmamg_dirac(tmamg_ctx* ctx, const void* x_bundle, void* y_bundle, int nsys, const double* mu, int prec) {
+  const TakeAgain at_end(ctx);
   if (!ctx) return TMAMG_ERR_ARG;
   if (!x_bundle || !y_bundle || !mu || nsys <= 0) return set_err(ctx, TMAMG_ERR_ARG, "dirac: bad argument");
   if (x_bundle == y_bundle) return set_err(ctx, TMAMG_ERR_ARG, "dirac: x and y must not overlap");
@@ -363,6 +382,7 @@ int tmamg_dirac(tmamg_ctx* ctx, const void* x_bundle, void* y_bundle, int nsys, 
 
 int tmamg_dirac_doublet(tmamg_ctx* ctx, const void* x_bundle, void* y_bundle, int npair, const double* mu,
                         const double* eps, int prec) {
+  const TakeAgain at_end(ctx);
   if (!ctx) return TMAMG_ERR_ARG;
   if (!x_bundle || !y_bundle || !mu || !eps || npair <= 0 || (prec != 32 && prec != 64))
     return set_err(ctx, TMAMG_ERR_ARG, "dirac_doublet: bad argument");
@@ -410,6 +430,7 @@ int tmamg_dirac_doublet(tmamg_ctx* ctx, const void* x_bundle, void* y_bundle, in
 }
 
 int tmamg_dirac_eo(tmamg_ctx* ctx, const void* x_bundle, void* y_bundle, int nsys, const double* mu, int prec) {
+  const TakeAgain at_end(ctx);
   if (!ctx) return TMAMG_ERR_ARG;
   if (!x_bundle || !y_bundle || !mu || nsys <= 0 || (prec != 32 && prec != 64))
     return set_err(ctx, TMAMG_ERR_ARG, "dirac_eo: bad argument");
@@ -429,6 +450,7 @@ int tmamg_dirac_eo(tmamg_ctx* ctx, const void* x_bundle, void* y_bundle, int nsy
 }
 
 int tmamg_apply(tmamg_ctx* ctx, const void* x_field, void* y_field, int nsys, const double* mu, int prec) {
+  const TakeAgain at_end(ctx);
   if (!ctx) return TMAMG_ERR_ARG;
   if (!x_field || !y_field || !mu || nsys <= 0 || (prec != 32 && prec != 64))
     return set_err(ctx, TMAMG_ERR_ARG, "apply: bad argument");

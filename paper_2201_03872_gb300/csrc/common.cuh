@@ -85,6 +85,8 @@ struct tmamg_ctx {
   float* C32 = nullptr;
   double kappa = 0.0, c_sw = 0.0;
   bool have_gauge = false, have_op = false, have_setup = false;
+  // the fixed-point copies were given back in the present call
+  bool gave_back = false;
   // a launch that reads the fixed-point copies was captured into a graph: a replay needs them where they are
   bool fixed_captured = false;
   // twisted masses on the device (per system), cached
@@ -125,6 +127,14 @@ void func_smem_optin(const void* func, int bytes);
 // back what it can do without and the allocation is tried once more.
 cudaError_t alloc_bytes(void** p, size_t bytes, bool pinned);
 bool give_back(tmamg_ctx* ctx);
+void take_again(tmamg_ctx* ctx);  // the copies of the operator, if they were given back and fit now
+// in every entry point that allocates: where the copies were given back and the call did not keep their memory
+// (it failed, or needed it for staging), they are made again at its end
+struct TakeAgain {
+  tmamg_ctx* ctx;
+  explicit TakeAgain(tmamg_ctx* c) : ctx(c) {}
+  ~TakeAgain();
+};
 template <class T>
 cudaError_t dev_alloc(tmamg_ctx* ctx, T** p, size_t bytes) {
   cudaError_t e = alloc_bytes(reinterpret_cast<void**>(p), bytes, false);

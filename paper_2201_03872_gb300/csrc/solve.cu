@@ -572,6 +572,7 @@ int do_setup(tmamg_ctx* ctx, const tmamg_setup_params* p, const float* vec_field
     if (rc) return rc;
   }
   ctx->have_setup = true;
+  take_again(ctx);  // an earlier solve's workspace is gone
   return TMAMG_OK;
 }
 
@@ -1326,12 +1327,14 @@ int tmamg_debug_bounded_wait(long long limit_cycles, int unreachable_next) {
 }
 
 int tmamg_setup(tmamg_ctx* ctx, const tmamg_setup_params* p, const float* start_vectors) {
+  const TakeAgain at_end(ctx);
   if (!ctx || !p) return set_err(ctx, TMAMG_ERR_ARG, "setup: null argument");
   if (!ctx->have_op) return set_err(ctx, TMAMG_ERR_STATE, "setup: operator not set");
   return do_setup(ctx, p, start_vectors, true);
 }
 
 int tmamg_setup_from_vectors(tmamg_ctx* ctx, const tmamg_setup_params* p, const float* test_vectors) {
+  const TakeAgain at_end(ctx);
   if (!ctx || !p || !test_vectors) return set_err(ctx, TMAMG_ERR_ARG, "setup_from_vectors: null argument");
   if (!ctx->have_op) return set_err(ctx, TMAMG_ERR_STATE, "setup_from_vectors: operator not set");
   return do_setup(ctx, p, test_vectors, false);
@@ -1339,6 +1342,7 @@ int tmamg_setup_from_vectors(tmamg_ctx* ctx, const tmamg_setup_params* p, const 
 
 int tmamg_solve(tmamg_ctx* ctx, const double* b, int nrhs, const double* mu, int nshift, double* x, int on_device,
                 const tmamg_solve_params* p, tmamg_system_stats* stats) {
+  const TakeAgain at_end(ctx);
   if (!ctx) return TMAMG_ERR_ARG;
   if (!b || !x || !mu || nrhs < 1 || nshift < 1) return set_err(ctx, TMAMG_ERR_ARG, "solve: bad argument");
   if (!ctx->have_setup) return set_err(ctx, TMAMG_ERR_STATE, "solve: no multigrid setup");
@@ -1349,6 +1353,7 @@ int tmamg_solve(tmamg_ctx* ctx, const double* b, int nrhs, const double* mu, int
 
 int tmamg_solve_doublet(tmamg_ctx* ctx, const double* b, int nrhs, const double* mu, const double* eps, int nshift,
                         double* x, int on_device, const tmamg_solve_params* p, tmamg_system_stats* stats) {
+  const TakeAgain at_end(ctx);
   if (!ctx) return TMAMG_ERR_ARG;
   if (!b || !x || !mu || !eps || nrhs < 1 || nshift < 1)
     return set_err(ctx, TMAMG_ERR_ARG, "solve_doublet: bad argument");
@@ -1366,6 +1371,7 @@ size_t tmamg_coarse_bundle_bytes(const tmamg_ctx* ctx, int level, int nsys) {
 
 int tmamg_sap(tmamg_ctx* ctx, void* r_bundle, void* e_bundle, int nsys, const double* mu, const int block[4],
               int cycles, int mr_steps) {
+  const TakeAgain at_end(ctx);
   if (!ctx) return TMAMG_ERR_ARG;
   if (!r_bundle || !e_bundle || !mu || !block || nsys < 1 || nsys > 256 || cycles < 1 || mr_steps < 1)
     return set_err(ctx, TMAMG_ERR_ARG, "sap: bad argument");
@@ -1426,6 +1432,7 @@ int tmamg_prolong(tmamg_ctx* ctx, int level, const void* coarse_bundle, void* fi
 
 int tmamg_coarse_solve(tmamg_ctx* ctx, int level, const void* rc_bundle, void* xc_bundle, int nrhs, const double* mu,
                        int nshift, const tmamg_solve_params* p, int* iterations) {
+  const TakeAgain at_end(ctx);
   if (!ctx) return TMAMG_ERR_ARG;
   if (!ctx->have_setup) return set_err(ctx, TMAMG_ERR_STATE, "coarse_solve: no setup");
   const int nlev = (int)ctx->levels.size();
@@ -1465,6 +1472,7 @@ int tmamg_coarse_solve(tmamg_ctx* ctx, int level, const void* rc_bundle, void* x
 
 int tmamg_coarse_apply(tmamg_ctx* ctx, int level, const void* x_bundle, void* y_bundle, int nsys, const double* mu,
                        int precision) {
+  const TakeAgain at_end(ctx);
   if (!ctx) return TMAMG_ERR_ARG;
   if (!ctx->have_setup) return set_err(ctx, TMAMG_ERR_STATE, "coarse_apply: no setup");
   if (level < 1 || level > (int)ctx->levels.size() || !x_bundle || !y_bundle || !mu || nsys < 1 ||
@@ -1589,6 +1597,7 @@ void tmamg_default_nn_params(tmamg_nn_params* p) {
 }
 
 int tmamg_nn_init(tmamg_ctx* ctx, uint64_t seed) {
+  const TakeAgain at_end(ctx);
   if (!ctx) return TMAMG_ERR_ARG;
   if (!ctx->have_op) return set_err(ctx, TMAMG_ERR_STATE, "nn_init: operator not set");
   int rc = nn_ready(ctx);
@@ -1613,6 +1622,7 @@ int tmamg_nn_init(tmamg_ctx* ctx, uint64_t seed) {
 }
 
 int tmamg_nn_set_weights(tmamg_ctx* ctx, const double* W) {
+  const TakeAgain at_end(ctx);
   if (!ctx || !W) return set_err(ctx, TMAMG_ERR_ARG, "nn_set_weights: null argument");
   if (nn_ready(ctx)) return set_err(ctx, TMAMG_ERR_OOM, "nn_set_weights: weights");
   return nn_upload(ctx, W);
@@ -1628,6 +1638,7 @@ int tmamg_nn_get_weights(const tmamg_ctx* ctx, double* W) {
 }
 
 int tmamg_nn_forward(tmamg_ctx* ctx, const void* r_bundle, void* y_bundle, int nsys, int bf16) {
+  const TakeAgain at_end(ctx);
   if (!ctx) return TMAMG_ERR_ARG;
   if (!r_bundle || !y_bundle || nsys < 1 || r_bundle == y_bundle) return set_err(ctx, TMAMG_ERR_ARG, "nn_forward: bad argument");
   if (!ctx->nn || !ctx->nn->trained) return set_err(ctx, TMAMG_ERR_STATE, "nn_forward: no weights");
@@ -1638,6 +1649,7 @@ int tmamg_nn_forward(tmamg_ctx* ctx, const void* r_bundle, void* y_bundle, int n
 
 int tmamg_nn_loss_grad(tmamg_ctx* ctx, const void* r_bundle, const void* e_bundle, int nsys, double* loss,
                        double* grad) {
+  const TakeAgain at_end(ctx);
   if (!ctx) return TMAMG_ERR_ARG;
   if (!r_bundle || !e_bundle || nsys < 1 || nsys > 256) return set_err(ctx, TMAMG_ERR_ARG, "nn_loss_grad: bad argument");
   if (!ctx->nn || !ctx->nn->trained) return set_err(ctx, TMAMG_ERR_STATE, "nn_loss_grad: no weights");
@@ -1664,6 +1676,7 @@ int tmamg_nn_loss_grad(tmamg_ctx* ctx, const void* r_bundle, const void* e_bundl
 }
 
 int tmamg_nn_train(tmamg_ctx* ctx, const tmamg_nn_params* p, tmamg_nn_report* rep) {
+  const TakeAgain at_end(ctx);
   if (!ctx || !p) return set_err(ctx, TMAMG_ERR_ARG, "nn_train: null argument");
   if (!ctx->have_setup) return set_err(ctx, TMAMG_ERR_STATE, "nn_train: no multigrid setup");
   if (p->batch < 1 || p->batch > 16 || p->pairs < p->batch || p->epochs < 1 || !(p->lr > 0) || p->gate_systems < 1 ||

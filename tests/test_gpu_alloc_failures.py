@@ -16,7 +16,7 @@ pytestmark = pytest.mark.gpu
 L = (8, 4, 4, 8)
 KAPPA = 0.125
 ALL = 1 << 30
-REFUSALS = 1  # of the copies of the operator
+REFUSALS = 3  # of the copies of the operator: in create, load_gauge and set_operator
 U = synth.gauge_field(L, 0.3, seed=401)
 
 
@@ -158,7 +158,7 @@ CALLS = {
 def test_an_allocation_that_finds_no_memory_gets_what_the_context_can_spare(name):
     for q, error in every_allocation(Problem, CALLS[name], count=1):
         assert error is None, error
-        fp64_application(q)  # without the copies of the operator
+        fp64_application(q)  # with or without the copies of the operator
 
 
 def test_context_without_room_for_the_copies_of_the_operator():
@@ -212,3 +212,34 @@ def test_captured_fp64_application_keeps_its_copies_of_the_operator():
             assert torch.equal(yb, ref)
         del taken
         T.tmamg_destroy(ctx)
+
+
+def test_copies_of_the_operator_are_made_again_after_a_call_that_failed():
+    q = Problem()
+    T = q.T
+    try:
+        y = fp64_application(q)
+        x = q.lat.torch.zeros(T.tmamg_bundle_bytes(q.ctx, 2, 64) // 8, dtype=q.lat.torch.float64, device="cuda")
+        T.tmamg_debug_fail_alloc(0, 2)  # the scratch bundle, with and without the copies
+        with pytest.raises(T.TmamgError) as e:
+            T.tmamg_dirac_eo(q.ctx, x, q.lat.torch.zeros_like(x), 2, q.mu, 64)
+        assert e.value.code == -3 and T.tmamg_debug_fail_alloc(0, 0) == 2
+        assert np.array_equal(fp64_application(q), y)
+    finally:
+        T.tmamg_debug_fail_alloc(0, 0)
+        q.lat.close()
+
+
+@pytest.mark.parametrize("call", ["load_gauge", "set_operator", "setup"])
+def test_copies_of_the_operator_are_made_again_with_a_new(call):
+    q = Problem()
+    y = fp64_application(q)
+    q.lat.close()
+    q = Problem(copies=False)
+    assert not np.array_equal(fp64_application(q), y)  # FP64 arithmetic rounds differently
+    if call == "set_operator":
+        q.T.tmamg_set_operator(q.ctx, KAPPA, 1.0)
+    else:
+        CALLS[call](q)
+    assert np.array_equal(fp64_application(q), y)
+    q.lat.close()
