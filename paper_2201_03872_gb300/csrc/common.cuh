@@ -168,6 +168,9 @@ void launch_convert_gauge(const Geom& g, const double* Uin, double2* U64, float2
 template <typename real>
 void launch_dirac(const Geom& g, const void* U, const real* C, const real* x, real* y, const double* mu, int nsys,
                   cudaStream_t st, const double* eps = nullptr);
+// the FP64 form on the sites of one parity (y keeps its entries on the others)
+void launch_dirac64_parity(const Geom& g, const double2* U, const double* C, const double* x, double* y, const double* mu,
+                           int nsys, int parity, cudaStream_t st);
 // Twisted masses and, for the doublet form, splittings of a stencil launch: device arrays, or, for up to
 // MASS_VALUES systems, the values themselves in the kernel's arguments.
 constexpr int MASS_VALUES = 32;

@@ -6,7 +6,7 @@
 // two FP64 lanes, so it ran at the FP64 issue rate (24^3x48 x 12 systems: 21.7 ms for 3.8 GB, 3% of the
 // HBM rate, against 13.1 ms if every FP64 slot were used). Here the products run as 32 x 32 -> 64-bit
 // integer multiply-adds (measured 59 lanes per cycle and SM on GB300, FP64 multiply-add 2.0), about 2600
-// of them and 8000 shifts, additions and logic operations per site and system: 5.05 ms for the same
+// of them and 8300 shifts, additions and logic operations per site and system: 5.24 ms for the same
 // case. It is bound by the integer pipes and their latency (multiply pipe 59% busy, issue 42%).
 //
 // Arithmetic. Block fixed point with one exponent S per (site, system): every contribution to the
@@ -22,6 +22,15 @@
 // 2^60), eight of them below 2^61; the local term is below 2^60 (2^59 x 2^58 / 2^57), the twist and the
 // doublet coupling below 2^58 each: no 64-bit sum can wrap. Inside a row the mixed products sum to less
 // than 2^60 + 6 2^58 (hops) and 5/4 2^59 + 12 2^57 (local term).
+//
+// Entries. The unit is that of the site's largest contributions, so an entry whose own contributions are all
+// small would be left with few bits or none (unit links without clover: the colours do not mix). The magnitudes
+// of what is added to every real and imaginary part are therefore summed beside it, and a component of which
+// one part has received less than 2^52 units is computed in FP64 arithmetic from its own terms
+// (fine_entry_f64; the whole site where there are more than five). The others are off by 2 units or so (45 if
+// every rounding went the same way): as FP64 sums of their terms. Gaussian fields have next to no such
+// components; the sums cost 4% (24^3x48 x 12 systems, 5.04 to 5.24 ms). A field with three of four spins zero
+// takes 21.2 ms (5.07 without this, 21.7 in FP64 arithmetic throughout).
 //
 // A site whose spinors, links or masses are outside the range of this form (infinities and NaN, entries
 // beyond about 2^900 or below 2^-840, |mu| of the size of the clover block) is computed in FP64
@@ -161,7 +170,8 @@ struct FineSite {
   bool last_t, first_t;
 };
 
-__device__ __noinline__ void fine_site_f64(const FineSite& f) {
+// writes the components in `which` (in the residual form in place, the others hold results already)
+__device__ __noinline__ void fine_site_f64(const FineSite& f, unsigned which) {
   Spinor<double, 1> acc;
 #pragma unroll
   for (int k = 0; k < 12; ++k) {
@@ -181,6 +191,7 @@ __device__ __noinline__ void fine_site_f64(const FineSite& f) {
   local_term<double, 1>(acc, f.x + f.s * 2, f.V, f.C, f.V, f.s, &f.mu, f.xp ? f.xp + f.s * 2 : nullptr, f.ep);
 #pragma unroll
   for (int k = 0; k < 12; ++k) {
+    if (!(which >> k & 1)) continue;
     if (f.b) {
       CV<double, 1> bv;
       ldcv(bv, f.b + (f.s + (int64_t)k * f.V) * 2);
@@ -189,6 +200,75 @@ __device__ __noinline__ void fine_site_f64(const FineSite& f) {
     }
     stcv(f.y + (f.s + (int64_t)k * f.V) * 2, acc.c[k]);
   }
+}
+
+// Component k of the same, by spin and colour at run time
+__device__ __noinline__ void fine_entry_f64(const FineSite& f, int k) {
+  // multipliers (as in mulc) of the projection and of the lower spins for a forward hop, two bits per direction
+  // and half spinor: Proj's c0, c1 and b0, b1; a backward hop has the opposite signs
+  constexpr unsigned KC = 0x5E4Au, KB = 0x5B1Fu;
+  const int spin = k / 3, col = k % 3;
+  double re = 0, im = 0;
+#pragma unroll 1
+  for (int hop = 0; hop < 8; ++hop) {
+    const int nu = hop >> 1, back = hop & 1;
+    const int half = spin < 2 ? spin : (nu < 2 ? 3 - spin : spin - 2);  // Proj's p0, p1
+    const int low = 2 + (nu < 2 ? 1 - half : half);                     // the lower spin in that half spinor
+    const int kc = ((KC >> (4 * nu + 2 * half)) & 3) ^ back;
+    const int kb = spin < 2 ? 0 : ((KB >> (4 * nu + 2 * (spin - 2))) & 3) ^ back;
+    const int64_t at = f.nb[hop], ls = back ? at : f.s;
+    double gr = 0, gi = 0;
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      const double2 u = *reinterpret_cast<const double2*>(f.x + ((int64_t)(half * 3 + b) * f.V + at) * 2);
+      const double2 d = *reinterpret_cast<const double2*>(f.x + ((int64_t)(low * 3 + b) * f.V + at) * 2);
+      const double dr = kc & 2 ? -d.y : d.x, di = kc & 2 ? d.x : d.y;
+      const double hr = kc & 1 ? u.x - dr : u.x + dr, hi = kc & 1 ? u.y - di : u.y + di;
+      double2 w = f.U[((int64_t)nu * 9 + (back ? b * 3 + col : col * 3 + b)) * f.V + ls];
+      if (back) w.y = -w.y;
+      gr += w.x * hr - w.y * hi;
+      gi += w.x * hi + w.y * hr;
+    }
+    if ((hop == 6 && f.last_t) || (hop == 7 && f.first_t)) {
+      gr *= f.bc_t;
+      gi *= f.bc_t;
+    }
+    const double tr = kb & 2 ? -gi : gr, ti = kb & 2 ? gr : gi;
+    re += kb & 1 ? -tr : tr;
+    im += kb & 1 ? -ti : ti;
+  }
+  const int chi = k / 6, i = k % 6;
+  const double* Cc = f.C + (int64_t)chi * 36 * f.V + f.s;
+  const double* xc = f.x + ((int64_t)chi * 6 * f.V + f.s) * 2;
+  double orr = 0, oi = 0;
+#pragma unroll 1
+  for (int j = 0; j < 6; ++j) {
+    const double2 x = *reinterpret_cast<const double2*>(xc + (int64_t)j * f.V * 2);
+    double ar, ai;
+    if (i == j) {
+      ar = Cc[(int64_t)i * f.V];
+      ai = chi == 0 ? f.mu : -f.mu;
+    } else {
+      const int q = i > j ? 6 + 2 * (i * (i - 1) / 2 + j) : 6 + 2 * (j * (j - 1) / 2 + i);
+      ar = Cc[(int64_t)q * f.V];
+      ai = Cc[(int64_t)(q + 1) * f.V];
+      if (i < j) ai = -ai;
+    }
+    orr += ar * x.x - ai * x.y;
+    oi += ar * x.y + ai * x.x;
+  }
+  const int64_t at = ((int64_t)k * f.V + f.s) * 2;
+  if (f.xp) {
+    orr -= f.ep * f.xp[at];
+    oi -= f.ep * f.xp[at + 1];
+  }
+  orr -= 0.5 * re;
+  oi -= 0.5 * im;
+  if (f.b) {
+    orr = f.b[at] - orr;
+    oi = f.b[at + 1] - oi;
+  }
+  *reinterpret_cast<double2*>(f.y + at) = make_double2(orr, oi);
 }
 
 // ---------------------------------------------------------------- fixed-point building blocks
@@ -253,12 +333,23 @@ __device__ __forceinline__ unsigned raw_max(const RawD& r) {
   return t;
 }
 
+// The magnitudes of what is added to an entry, |re| and |im| in two halves of a word that counts 2^48 units
+// (they add up to less than 2^14 counts, by the bounds of the sums)
+__device__ __forceinline__ unsigned fx_mag(i64 re, i64 im) {
+  return __byte_perm((unsigned)abs((int)(re >> 32)), (unsigned)abs((int)(im >> 32)), 0x7632);
+}
+constexpr unsigned FX_LEAST = 1u << 4;  // 2^52 units
+constexpr int FX_ENTRIES = 5;  // components computed one by one; the whole site does less than half the work for each
+
 // raise the common exponent to at least `want` (the sums keep their value)
-__device__ __forceinline__ void fx_raise(i64 (&acc)[24], int& S, int want) {
+__device__ __forceinline__ void fx_raise(i64 (&acc)[24], unsigned (&mag)[12], int& S, int want) {
   if (want > S) {
     const int d = want - S;
 #pragma unroll
     for (int k = 0; k < 24; ++k) acc[k] = sar64(acc[k], d);
+    const unsigned keep = d < 16 ? (0xffffu >> d) * 0x10001u : 0u;
+#pragma unroll
+    for (int k = 0; k < 12; ++k) mag[k] = (mag[k] >> (d & 15)) & keep;
     S = want;
   }
 }
@@ -293,10 +384,17 @@ __device__ __forceinline__ void fx_sub(i64& ar, i64& ai, const i64 (&g)[2]) {
   if (K == 3) { ar -= g[1]; ai += g[0]; }
 }
 template <int NU, bool FWD>
-__device__ __forceinline__ void fx_scatter(i64 (&acc)[24], const i64 (&g)[2][3][2]) {
+__device__ __forceinline__ void fx_scatter(i64 (&acc)[24], unsigned (&mag)[12], const i64 (&g)[2][3][2]) {
   using P = Proj<NU, FWD>;
+  static_assert((P::b0 & 2) == (P::b1 & 2), "both lower spins take real for real, or both real for imaginary parts");
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
+    const unsigned m0 = fx_mag(g[0][a][0], g[0][a][1]), m1 = fx_mag(g[1][a][0], g[1][a][1]);
+    mag[a] += m0;
+    mag[3 + a] += m1;
+    const unsigned l0 = P::p0 == 0 ? m0 : m1, l1 = P::p1 == 0 ? m0 : m1;
+    mag[6 + a] += P::b0 & 2 ? __byte_perm(l0, 0, 0x1032) : l0;
+    mag[9 + a] += P::b1 & 2 ? __byte_perm(l1, 0, 0x1032) : l1;
     fx_sub<0>(acc[2 * a], acc[2 * a + 1], g[0][a]);
     fx_sub<0>(acc[6 + 2 * a], acc[6 + 2 * a + 1], g[1][a]);
     fx_sub<P::b0>(acc[12 + 2 * a], acc[12 + 2 * a + 1], g[P::p0][a]);
@@ -401,7 +499,8 @@ __global__ void __launch_bounds__(MAXT, MINB) dirac64_kernel(FixedOp fx, const d
                                                              const double* __restrict__ C, const double* __restrict__ x,
                                                              double* y, const double* __restrict__ mu, int ntile, int Lx,
                                                              int Ly, int Lz, int Lt, int bc_t, const double* bsub,
-                                                             int nshift, const double* __restrict__ eps) {
+                                                             int nshift, const double* __restrict__ eps, int parity) {
+  // parity 0 or 1: y on the sites of that parity only (the others are not written); else -1.
   // y is not restrict-qualified: the residual form may run in place (bsub == y), every thread
   // reading b at its own site before it writes y there; x never overlaps y
   const int64_t V = (int64_t)Lx * Ly * Lz * Lt;
@@ -411,6 +510,7 @@ __global__ void __launch_bounds__(MAXT, MINB) dirac64_kernel(FixedOp fx, const d
   const int L[4] = {Lx, Ly, Lz, Lt};
   int c[4];
   site_coords(s, L, c);
+  if (parity >= 0 && ((c[0] + c[1] + c[2] + c[3]) & 1) != parity) return;
   const int64_t tstride = (int64_t)24 * V;
   const double* xt = x + tile * tstride;
   // neighbours as offsets from s (32 bits: a lattice of 2^31 sites would need 800 GB per FP64 vector)
@@ -431,6 +531,7 @@ __global__ void __launch_bounds__(MAXT, MINB) dirac64_kernel(FixedOp fx, const d
 
   bool ok = fx.U != nullptr;
   i64 acc[24];
+  unsigned mag[12];
   int S = FX_ZERO;
   if (ok) {
     RawD raw;
@@ -455,12 +556,18 @@ __global__ void __launch_bounds__(MAXT, MINB) dirac64_kernel(FixedOp fx, const d
         if (chi == 0) acc[i] = o[i];
         else acc[12 + i] = o[i];
       }
+#pragma unroll
+      for (int i = 0; i < 6; ++i) {
+        const unsigned m = fx_mag(o[2 * i], o[2 * i + 1]);
+        if (chi == 0) mag[i] = m;
+        else mag[6 + i] = m;
+      }
     }
     if (ep != 0.0) {
       // - eps times the partner flavour, at the clover's scale
       ld_rawd(raw, xp + s * 2, V);
       const int tp = fx_top(raw_max(raw));
-      if (tp != FX_ZERO) fx_raise(acc, S, tp - 1022 + nC - 2);
+      if (tp != FX_ZERO) fx_raise(acc, mag, S, tp - 1022 + nC - 2);
       const int2 en = fx_split(-fx_scalar(ep, nC));
       const int ec = S - nC + 2 + 1026;
 #pragma unroll
@@ -468,8 +575,10 @@ __global__ void __launch_bounds__(MAXT, MINB) dirac64_kernel(FixedOp fx, const d
         FxSum re = {0, 1ll << 26}, im = {0, 1ll << 26};
         fx_mad(re, en.x, en.y, fx_conv(raw.v[k].x, raw.v[k].y, ec));
         fx_mad(im, en.x, en.y, fx_conv(raw.v[k].z, raw.v[k].w, ec));
-        acc[2 * k] += (re.hi << 3) + (re.mid >> 27);
-        acc[2 * k + 1] += (im.hi << 3) + (im.mid >> 27);
+        const i64 er = (re.hi << 3) + (re.mid >> 27), ei = (im.hi << 3) + (im.mid >> 27);
+        acc[2 * k] += er;
+        acc[2 * k + 1] += ei;
+        mag[k] += fx_mag(er, ei);
       }
     }
     // the eight hops in one loop (its body is small enough for the instruction cache; the unrolled form
@@ -485,7 +594,7 @@ __global__ void __launch_bounds__(MAXT, MINB) dirac64_kernel(FixedOp fx, const d
       const int nU = fx.nU[(int64_t)(hop >> 1) * V + ls];
       ok &= nU != FX_BAD;
       const int t = fx_top(raw_max(raw));
-      if (t != FX_ZERO) fx_raise(acc, S, t - 1022 + nU);
+      if (t != FX_ZERO) fx_raise(acc, mag, S, t - 1022 + nU);
       const int ec = S - nU + 1026;
       Limb v[12][2];
 #pragma unroll
@@ -517,67 +626,78 @@ __global__ void __launch_bounds__(MAXT, MINB) dirac64_kernel(FixedOp fx, const d
       if (hop & 1) fx_mul<false>(g, h, Un, V);
       else fx_mul<true>(g, h, Un, V);
       switch (hop) {
-        case 0: fx_scatter<0, true>(acc, g); break;
-        case 1: fx_scatter<0, false>(acc, g); break;
-        case 2: fx_scatter<1, true>(acc, g); break;
-        case 3: fx_scatter<1, false>(acc, g); break;
-        case 4: fx_scatter<2, true>(acc, g); break;
-        case 5: fx_scatter<2, false>(acc, g); break;
-        case 6: fx_scatter<3, true>(acc, g); break;
-        default: fx_scatter<3, false>(acc, g); break;
+        case 0: fx_scatter<0, true>(acc, mag, g); break;
+        case 1: fx_scatter<0, false>(acc, mag, g); break;
+        case 2: fx_scatter<1, true>(acc, mag, g); break;
+        case 3: fx_scatter<1, false>(acc, mag, g); break;
+        case 4: fx_scatter<2, true>(acc, mag, g); break;
+        case 5: fx_scatter<2, false>(acc, mag, g); break;
+        case 6: fx_scatter<3, true>(acc, mag, g); break;
+        default: fx_scatter<3, false>(acc, mag, g); break;
       }
     }
     // all inputs zero (S never set), or every result and its unit far inside the normal range
     ok = ok && (S < FX_ZERO / 2 || (S > -900 && S < 900));
   }
-  double* yt = y + tile * tstride;
-  if (!ok) {
-    FineSite f;
-    f.U = U; f.C = C; f.x = xt; f.xp = xp; f.b = bo; f.y = yt;
-    f.mu = m; f.ep = ep; f.bc_t = bc_t;
-    f.s = s; f.V = V;
+  // the components whose contributions are too small for the units of this site (all-zero inputs have none)
+  unsigned small = 0;
+  if (S >= FX_ZERO / 2) {
 #pragma unroll
-    for (int k = 0; k < 8; ++k) f.nb[k] = s + nb[k];
-    f.last_t = c[3] == Lt - 1;
-    f.first_t = c[3] == 0;
-    fine_site_f64(f);
+    for (int k = 0; k < 12; ++k)
+      if ((mag[k] & 0xffffu) < FX_LEAST || (mag[k] >> 16) < FX_LEAST) small |= 1u << k;
+  }
+  double* yt = y + tile * tstride;
+  if (ok) {
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+      double2 o = make_double2(fx_double(acc[2 * k], S), fx_double(acc[2 * k + 1], S));
+      const int64_t at = (s + (int64_t)k * V) * 2;
+      if (small >> k & 1) continue;
+      if (RES) {
+        const double2 bv = *reinterpret_cast<const double2*>(bo + at);
+        o = make_double2(bv.x - o.x, bv.y - o.y);
+      }
+      *reinterpret_cast<double2*>(yt + at) = o;
+    }
+    if (!small) return;
+  }
+  FineSite f;
+  f.U = U; f.C = C; f.x = xt; f.xp = xp; f.b = bo; f.y = yt;
+  f.mu = m; f.ep = ep; f.bc_t = bc_t;
+  f.s = s; f.V = V;
+#pragma unroll
+  for (int k = 0; k < 8; ++k) f.nb[k] = s + nb[k];
+  f.last_t = c[3] == Lt - 1;
+  f.first_t = c[3] == 0;
+  if (!ok || __popc(small) > FX_ENTRIES) {
+    fine_site_f64(f, ok ? small : 0xfffu);
     return;
   }
-#pragma unroll
-  for (int k = 0; k < 12; ++k) {
-    double2 o = make_double2(fx_double(acc[2 * k], S), fx_double(acc[2 * k + 1], S));
-    const int64_t at = (s + (int64_t)k * V) * 2;
-    if (RES) {
-      const double2 bv = *reinterpret_cast<const double2*>(bo + at);
-      o = make_double2(bv.x - o.x, bv.y - o.y);
-    }
-    *reinterpret_cast<double2*>(yt + at) = o;
-  }
+  for (; small; small &= small - 1) fine_entry_f64(f, __ffs(small) - 1);
 }
 
 // launch variants: (sites per CTA row, largest CTA, CTAs per SM): 168 registers at 12 warps per SM, or 128
-// registers (some spills) at 16 warps per SM; measured on 24^3x48 x 12 systems 5.05 and 5.25 ms (96
-// registers at 20 warps: 5.8 ms; the sums in shared memory: 5.6 ms)
+// registers (some spills) at 16 warps per SM; measured on 24^3x48 x 12 systems 5.24 and 5.62 ms
 template <bool RES, int BX, int MAXT, int MINB>
 static void launch_variant64(const Geom& g, const double2* U, const double* C, const double* x, double* y,
-                             const double* mu, int nsys, const double* b, int nshift, const double* eps,
+                             const double* mu, int nsys, const double* b, int nshift, const double* eps, int parity,
                              cudaStream_t st) {
   const int ty = pick_ty(nsys, BX, MAXT);
   dim3 block(BX, ty);
   dim3 grid((unsigned)((g.V + BX - 1) / BX), (unsigned)(nsys / ty));
   dirac64_kernel<BX, RES, MAXT, MINB><<<grid, block, 0, st>>>(g.fx, U, C, x, y, mu, nsys, g.L[0], g.L[1], g.L[2],
-                                                              g.L[3], g.bc_t, b, nshift, eps); TM_COUNT();
+                                                              g.L[3], g.bc_t, b, nshift, eps, parity); TM_COUNT();
 }
 
 template <bool RES>
 static void launch_tuned64(const char* family, bool may_tune, const Geom& g, const void* Uv, const double* C,
                            const double* x, double* y, const double* mu, int nsys, const double* b, int nshift,
-                           const double* eps, cudaStream_t st) {
+                           const double* eps, int parity, cudaStream_t st) {
   const double2* U = reinterpret_cast<const double2*>(Uv);
   auto launch = [&](int v) {
     switch (v) {
-      case 1: launch_variant64<RES, 32, 128, 4>(g, U, C, x, y, mu, nsys, b, nshift, eps, st); return;
-      default: launch_variant64<RES, 32, 192, 2>(g, U, C, x, y, mu, nsys, b, nshift, eps, st); return;
+      case 1: launch_variant64<RES, 32, 128, 4>(g, U, C, x, y, mu, nsys, b, nshift, eps, parity, st); return;
+      default: launch_variant64<RES, 32, 192, 2>(g, U, C, x, y, mu, nsys, b, nshift, eps, parity, st); return;
     }
   };
   launch(tune_variant(family, g.V * 4096 + nsys, 2, may_tune, launch, st));
@@ -587,13 +707,19 @@ template <>
 void launch_dirac<double>(const Geom& g, const void* U, const double* C, const double* x, double* y, const double* mu,
                           int nsys, cudaStream_t st, const double* eps) {
   TM_PROF(st, "dirac_f64");
-  launch_tuned64<false>("dirac_f64", true, g, U, C, x, y, mu, nsys, nullptr, 1, eps, st);
+  launch_tuned64<false>("dirac_f64", true, g, U, C, x, y, mu, nsys, nullptr, 1, eps, -1, st);
+}
+
+void launch_dirac64_parity(const Geom& g, const double2* U, const double* C, const double* x, double* y, const double* mu,
+                           int nsys, int parity, cudaStream_t st) {
+  TM_PROF(st, "dirac_f64");
+  launch_tuned64<false>("dirac_f64", true, g, U, C, x, y, mu, nsys, nullptr, 1, nullptr, parity, st);
 }
 
 void launch_residual64(const Geom& g, const double2* U, const double* C, const double* x, const double* b, int nshift,
                        double* r, const double* mu, int nsys, cudaStream_t st, const double* eps) {
   TM_PROF(st, "residual_f64");
-  launch_tuned64<true>("residual_f64", b != r, g, U, C, x, r, mu, nsys, b, nshift, eps, st);
+  launch_tuned64<true>("residual_f64", b != r, g, U, C, x, r, mu, nsys, b, nshift, eps, -1, st);
 }
 
 }  // namespace tmamg
