@@ -550,8 +550,18 @@ static void launch_variant(const Geom& g, const float2* U, const float* C, const
       U, C, x, y, mu, nsys, nt, g.L[0], g.L[1], g.L[2], g.L[3], (float)g.bc_t, b, eps); TM_COUNT();
 }
 
-constexpr int NVARIANTS = 4, SPLIT_VARIANT = 3;
+constexpr int NVARIANTS = 4, DIRECT_VARIANT = 1, SPLIT_VARIANT = 3;
 static int64_t tune_key(const Geom& g, int nsys) { return g.V * 4096 + nsys; }
+// Where nothing is tuned (tuning is off, or the first residual of a shape in place): direct with one tile, which
+// shares no links, and below two waves of threads, where staging is latency (staged and direct: 24^3x48 one system
+// 172 and 135 us; 8^3x16 twelve systems 14.3 and 12.6, 12^3x24 four 20.5 and 18.5, five 26.8 and 28.7)
+static int untuned_variant(const Geom& g, int nsys) {
+  const int nt = ntiles(nsys, 2);
+  return nt == 1 || g.V * nt < 2ll * 384 * device_sms() ? DIRECT_VARIANT : 0;
+}
+static int peek_variant(const Geom& g, int nsys) {
+  return tune_peek("dirac_f32", tune_key(g, nsys), NVARIANTS, untuned_variant(g, nsys));
+}
 
 template <bool RES>
 static void launch_tuned(const char* family, bool may_tune, const Geom& g, const float2* U, const float* C,
@@ -559,7 +569,7 @@ static void launch_tuned(const char* family, bool may_tune, const Geom& g, const
                          cudaStream_t st) {
   auto launch = [&](int v) {
     switch (v) {
-      case 1: launch_variant<RES, 32, false, 192, 2>(g, U, C, x, y, mu, nsys, b, eps, st); return;
+      case DIRECT_VARIANT: launch_variant<RES, 32, false, 192, 2>(g, U, C, x, y, mu, nsys, b, eps, st); return;
       case 2: launch_variant<RES, 32, true, 256, 2>(g, U, C, x, y, mu, nsys, b, eps, st); return;
       case SPLIT_VARIANT: {
         MassArgs ma;
@@ -572,11 +582,11 @@ static void launch_tuned(const char* family, bool may_tune, const Geom& g, const
       default: launch_variant<RES, 32, true, 192, 2>(g, U, C, x, y, mu, nsys, b, eps, st); return;
     }
   };
-  launch(tune_variant(family, tune_key(g, nsys), NVARIANTS, may_tune, launch, st));
+  launch(tune_variant(family, tune_key(g, nsys), NVARIANTS, untuned_variant(g, nsys), may_tune, launch, st));
 }
 
 bool dirac32_to_field(const Geom& g, int nsys) {
-  const int v = tune_peek("dirac_f32", tune_key(g, nsys), NVARIANTS);
+  const int v = peek_variant(g, nsys);
   return v == 0 || v == 2;
 }
 
@@ -584,7 +594,7 @@ void launch_dirac32_field(const Geom& g, const float2* U, const float* C, const 
                           int nsys, cudaStream_t st) {
   TM_PROF(st, "dirac_f32");
   const int nt = ntiles(nsys, 2);
-  const bool wide = tune_peek("dirac_f32", tune_key(g, nsys), NVARIANTS) == 2;
+  const bool wide = peek_variant(g, nsys) == 2;
   const int ty = pick_ty(nt, 32, wide ? 256 : 192);
   const dim3 block(32, ty), grid((unsigned)((g.V + 31) / 32), (unsigned)(nt / ty));
   static_assert(8 * 32 * 26 * 4 <= dr_stage_bytes(32), "eight warps transpose in the staging space");
@@ -596,7 +606,7 @@ void launch_dirac32_field(const Geom& g, const float2* U, const float* C, const 
 }
 
 bool dirac32_takes_values(const Geom& g, int nsys) {
-  return nsys <= MASS_VALUES && tune_peek("dirac_f32", tune_key(g, nsys), NVARIANTS) == SPLIT_VARIANT;
+  return nsys <= MASS_VALUES && peek_variant(g, nsys) == SPLIT_VARIANT;
 }
 
 void launch_dirac32_values(const Geom& g, const float2* U, const float* C, const float* x, float* y, const MassArgs& ma,

@@ -39,3 +39,31 @@ def test_apply_equals_parts(L, nsys, variant):
     finally:
         T.tmamg_autotune_force(-1)
         lat.close()
+
+
+@pytest.mark.parametrize("L,nsys", [((4, 4, 4, 4), 1), ((4, 4, 4, 4), 6), ((16, 16, 16, 28), 2), ((16, 16, 16, 28), 3)])
+def test_untuned_forms_same_bits(L, nsys):
+    """With tuning off: the direct form for one tile and for few sites, else the staged one (from 116736 sites x tiles)."""
+    torch = torch_cuda()
+    lat = Lattice(L, synth.gauge_field(L, 0.4, seed=6), 0.124, 1.1)
+    T = lat.T
+    try:
+        x = torch.from_numpy(synth.gaussian_spinors(L, nsys, seed=7).astype(np.complex64).view(np.float32).ravel()).cuda()
+        xb, mu = lat.fine_bundle(synth.gaussian_spinors(L, nsys, seed=7)), np.linspace(-0.1, 0.2, nsys)
+        out = []
+        for off in (False, True):
+            if off:
+                T.tmamg_autotune(0)
+            else:
+                T.tmamg_autotune_force(1)
+            y, f = torch.full_like(xb, 7.0), torch.empty_like(x)
+            T.tmamg_dirac(lat.ctx, xb, y, nsys, mu, 32)
+            T.tmamg_apply(lat.ctx, x, f, nsys, mu, 32)
+            torch.cuda.synchronize()
+            out.append((y, f))
+            T.tmamg_autotune_force(-1)
+        assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
+    finally:
+        T.tmamg_autotune_force(-1)
+        T.tmamg_autotune(1)
+        lat.close()
