@@ -56,6 +56,7 @@ int tune_run(const char* family, int64_t key, int nvar, const std::function<void
     cudaEventRecord(b, st);
     float t = 0.f;
     if (cudaEventSynchronize(b) != cudaSuccess || cudaEventElapsedTime(&t, a, b) != cudaSuccess) t = 1e30f;
+    if (cudaGetLastError() != cudaSuccess) t = 1e30f;  // a launch that was refused took no time
     ms[v] = 0.5f * t;
     if (ms[v] < ms[best]) best = v;
   }

@@ -33,3 +33,28 @@ def test_split_form_same_bits(L, nsys):
     finally:
         T.tmamg_autotune_force(-1)
         lat.close()
+
+
+def test_more_tiles_than_a_grid_has_rows():
+    # FP32: two systems per tile; a grid's second extent ends at 65535
+    torch = torch_cuda()
+    L, nsys = (2, 2, 2, 2), 2 * 65535 + 5
+    lat = Lattice(L, synth.gauge_field(L, 0.4, seed=6), 0.124, 1.1)
+    T = lat.T
+    try:
+        x = torch.randn(T.tmamg_bundle_bytes(lat.ctx, nsys, 32) // 4, device="cuda")
+        mu = np.linspace(-0.1, 0.2, nsys)
+        out = []
+        for v in (1, 3, -1):
+            T.tmamg_autotune_force(v)
+            y = torch.full_like(x, 7.0)
+            T.tmamg_dirac(lat.ctx, x, y, nsys, mu, 32)
+            out.append(y)
+        torch.cuda.synchronize()
+        valid = torch.ones_like(x, dtype=torch.bool).view(-1, 2)
+        valid[-12 * 16 * 2:, 1] = False  # the last tile's padding lane
+        valid = valid.view(-1)
+        assert torch.equal(out[0][valid], out[1][valid]) and torch.equal(out[0][valid], out[2][valid])
+    finally:
+        T.tmamg_autotune_force(-1)
+        lat.close()
