@@ -349,10 +349,136 @@ static void launch_restrict_r(const AggDims& g, const float2* P, const float* r,
   }
 }
 
+// The same for short sums and few outputs, where the kernel above spends its time on filling its pipelines and on adding
+// its warps' sums. One CTA per (aggregate, chirality); the entries of a chunk of RH_KC values of k are staged for all
+// tiles; a thread owns 3 x 3 outputs (rows x tiles) and one of 16 interleaved slices of k, which are added by shuffles
+// in a fixed order. Two CTAs per SM (80 registers): one stages while the other computes.
+// 16^4, 2^4 aggregates (K = 96), the kernel above and this one, us: nv = 8, 1 system 65.5 and 30.7, 12 systems 158 and
+// 74; nv = 24, 6 systems 161 and 79, 16 systems 211 and 215; K = 192, nv = 8, 12 systems 96 and 69; K = 384, nv = 8,
+// 12 systems 68 and 64, 16 systems 68 and 113; 24^3x48, K = 1536, nv = 4, 1 system 234 and 153.
+constexpr int RH_KS = 16;         // k slices (lanes of a half warp)
+constexpr int RH_MAX_SLOTS = 24;  // output blocks processed at once per CTA (blockDim.x / RH_KS)
+constexpr int RH_KC = 128;        // k values staged per chunk
+constexpr int RH_MAXT = 12;       // tiles per call
+
+static bool restrict_short(int nv, int nt, int K, int asize) {
+  if (nt > RH_MAXT || asize > RS_TABLE) return false;
+  if (K <= 128) return nt <= 6 || nv <= 8;
+  if (K <= 192) return nt <= 6;
+  return K <= 384 ? nv <= 8 && nt <= 6 : nv <= 4 && nt <= 3;
+}
+
+__global__ void __launch_bounds__(RH_KS * RH_MAX_SLOTS, 2) restrict_short_kernel(const float2* __restrict__ P,
+                                                              const float* __restrict__ r, float* __restrict__ xc,
+                                                              AggDims g, int nv, int d, int nt) {
+  constexpr int kc = RH_KC;
+  extern __shared__ float4 rsm[];                             // [nt][kc] staged entries
+  int* sidx = reinterpret_cast<int*>(rsm + (size_t)nt * kc);  // [asize] lattice site of each member
+  const int64_t a = blockIdx.x >> 1;
+  const int chi = blockIdx.x & 1;
+  const int K = g.asize * d;
+  for (int q = threadIdx.x; q < g.asize; q += blockDim.x) {
+    int c[4];
+    agg_site(a, q, g.Lc, g.agg, g.L, c);
+    sidx[q] = (int)site_index(c, g.L);
+  }
+  const int ks = threadIdx.x % RH_KS, slot = threadIdx.x / RH_KS;
+  const int nslots = blockDim.x / RH_KS;
+  const int JG = (nv + 2) / 3, TG = (nt + 2) / 3;
+  const float2* Pa = P + ((a * 2 + chi) * nv) * (int64_t)K;
+  for (int og0 = 0; og0 < JG * TG; og0 += nslots) {
+    const int og = og0 + slot;
+    const bool live = og < JG * TG;
+    const int jg = live ? og / TG : 0, tg = live ? og % TG : 0;
+    const int j0 = 3 * jg, t0 = 3 * tg;
+    float2 are[9], aim[9];
+#pragma unroll
+    for (int u = 0; u < 9; ++u) {
+      are[u] = make_float2(0.f, 0.f);
+      aim[u] = make_float2(0.f, 0.f);
+    }
+    for (int kc0 = 0; kc0 < K; kc0 += kc) {
+      const int kn = K - kc0 < kc ? K - kc0 : kc;
+      __syncthreads();  // sidx ready / the previous chunk consumed
+      for (int e = threadIdx.x; e < nt * kn; e += blockDim.x) {
+        const int t = e / kn, kk = e - t * kn;
+        const int k = kc0 + kk;
+        const int cp = k / g.asize, q = k - cp * g.asize;
+        rsm[t * kc + kk] =
+            __ldg(reinterpret_cast<const float4*>(r + (((int64_t)t * (2 * d) + chi * d + cp) * g.Vp + sidx[q]) * 4));
+      }
+      __syncthreads();
+      if (live) {
+#pragma unroll 4
+        for (int kk = ks; kk < kn; kk += RH_KS) {
+          float2 p[3];
+          float4 v[3];
+#pragma unroll
+          for (int jj = 0; jj < 3; ++jj)
+            p[jj] = j0 + jj < nv ? __ldg(Pa + (int64_t)(j0 + jj) * K + kc0 + kk) : make_float2(0.f, 0.f);
+#pragma unroll
+          for (int tt = 0; tt < 3; ++tt)
+            v[tt] = t0 + tt < nt ? rsm[(t0 + tt) * kc + kk] : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+          for (int jj = 0; jj < 3; ++jj) {
+            const float2 pr = make_float2(p[jj].x, p[jj].x), pi = make_float2(p[jj].y, p[jj].y);
+            const float2 npi = make_float2(-p[jj].y, -p[jj].y);
+#pragma unroll
+            for (int tt = 0; tt < 3; ++tt) {
+              const float2 vr = make_float2(v[tt].x, v[tt].y), vi = make_float2(v[tt].z, v[tt].w);
+              // conj(p) v = (pr vr + pi vi) + i (pr vi - pi vr), both systems at once
+              are[jj * 3 + tt] = __ffma2_rn(pr, vr, are[jj * 3 + tt]);
+              are[jj * 3 + tt] = __ffma2_rn(pi, vi, are[jj * 3 + tt]);
+              aim[jj * 3 + tt] = __ffma2_rn(pr, vi, aim[jj * 3 + tt]);
+              aim[jj * 3 + tt] = __ffma2_rn(npi, vr, aim[jj * 3 + tt]);
+            }
+          }
+        }
+      }
+    }
+    // sum of the 16 slices (lanes ks of the half warp), fixed order
+#pragma unroll
+    for (int u = 0; u < 9; ++u) {
+#pragma unroll
+      for (int o = RH_KS / 2; o > 0; o >>= 1) {
+        are[u].x += __shfl_xor_sync(0xffffffffu, are[u].x, o);
+        are[u].y += __shfl_xor_sync(0xffffffffu, are[u].y, o);
+        aim[u].x += __shfl_xor_sync(0xffffffffu, aim[u].x, o);
+        aim[u].y += __shfl_xor_sync(0xffffffffu, aim[u].y, o);
+      }
+    }
+    if (live && ks == 0) {
+#pragma unroll
+      for (int jj = 0; jj < 3; ++jj)
+#pragma unroll
+        for (int tt = 0; tt < 3; ++tt)
+          if (j0 + jj < nv && t0 + tt < nt)
+            *reinterpret_cast<float4*>(xc + (((int64_t)(t0 + tt) * (2 * nv) + chi * nv + j0 + jj) * g.Vc + a) * 4) =
+                make_float4(are[jj * 3 + tt].x, are[jj * 3 + tt].y, aim[jj * 3 + tt].x, aim[jj * 3 + tt].y);
+    }
+  }
+}
+
+static void launch_restrict_short(const AggDims& g, const float2* P, const float* r, float* xc, int nv, int d, int nt,
+                                  cudaStream_t st) {
+  // every output block of the aggregate in one pass over P and the staged chunks when they fit one CTA (rounds of
+  // RH_MAX_SLOTS blocks otherwise)
+  const int nblk = ((nv + 2) / 3) * ((nt + 2) / 3);
+  const int rounds = (nblk + RH_MAX_SLOTS - 1) / RH_MAX_SLOTS;
+  const int slots = (nblk + rounds - 1) / rounds;
+  const size_t smem = sizeof(float4) * (size_t)nt * RH_KC + sizeof(int) * g.asize;  // at most 40 KB
+  restrict_short_kernel<<<(unsigned)(g.Vc * 2), RH_KS * slots, smem, st>>>(P, r, xc, g, nv, d, nt);
+  TM_COUNT();
+}
+
 void restrict_vec(const AggDims& g, const float2* P, const float* r, float* xc, int nv, int d, int nsys,
                   cudaStream_t st) {
   const int nt = ntiles(nsys, T2);
   TM_PROF(st, d == 6 ? "restrict" : "restrict_coarse");
+  if (restrict_short(nv, nt, g.asize * d, g.asize)) {
+    launch_restrict_short(g, P, r, xc, nv, d, nt, st);
+    return;
+  }
   switch ((nv + 7) / 8) {  // nv <= 32
     case 1: launch_restrict_r<1>(g, P, r, xc, nv, d, nt, st); return;
     case 2: launch_restrict_r<2>(g, P, r, xc, nv, d, nt, st); return;
@@ -445,6 +571,9 @@ constexpr size_t RP_RING = sizeof(float2) * RP_NST * RP_JS * RP_R * RP_THREADS;
 // thread keeps 160 KB per SM of its own P entries on their way to shared memory, and two entries k share each
 // broadcast of the coarse vector. 24^3x48, nv = 24: 1 system 494 -> 335 us, 4 systems 513 -> 357, 8 systems 540 -> 452;
 // at 16 systems the general kernel is the faster one (615 against 698 us, its arithmetic has fewer other instructions).
+// A CTA's 256 threads need enough entries to share that ring: with 96 (16^4, 2^4 aggregates, nv = 24) the general kernel
+// takes 133 us for 1 system and 141 for 6, this one 144 and 203; with 192 85 and 90, 76 and 107; with 384 72 and 76, 48
+// and 63.
 template <int TCH>
 __global__ void __launch_bounds__(RP_THREADS, 2) prolong_few_kernel(const float2* __restrict__ P,
                                                                     const float* __restrict__ xc,
@@ -566,8 +695,9 @@ void prolong_vec(const AggDims& g, const float2* P, const float* xc, float* e, i
     func_smem_optin((const void*)kernel, (int)smem);
     kernel<<<(unsigned)(g.Vc * 2), RP_THREADS, smem, st>>>(P, xc, e, g, nv, d, nt, accumulate);
   };
-  if (nt <= 2) few(prolong_few_kernel<2>);
-  else if (nt <= 4) few(prolong_few_kernel<4>);
+  const int K = g.asize * d;
+  if (nt <= 2 && K > RP_THREADS / 2) few(prolong_few_kernel<2>);
+  else if (nt <= 4 && K > RP_THREADS) few(prolong_few_kernel<4>);
   else
     prolong_kernel<<<(unsigned)(g.Vc * 2), RP_THREADS, sizeof(int) * g.asize, st>>>(P, xc, e, g, nv, d, nt, accumulate);
   TM_COUNT();

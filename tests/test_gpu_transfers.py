@@ -63,6 +63,48 @@ def test_transfers_against_dense_p(nv, nsys):
         lat.close()
 
 
+@pytest.mark.parametrize("agg,nv,nsys", [
+    ((2, 2, 2, 2), 1, 1), ((2, 2, 2, 2), 8, 24), ((2, 2, 2, 2), 9, 12), ((2, 2, 2, 2), 9, 13), ((2, 2, 2, 2), 32, 5),
+    ((2, 2, 2, 2), 4, 25), ((4, 2, 2, 2), 24, 12), ((4, 2, 2, 2), 24, 14), ((4, 2, 2, 2), 7, 4), ((4, 4, 2, 2), 8, 11),
+    ((4, 4, 2, 2), 9, 3), ((4, 4, 2, 2), 5, 14), ((2, 2, 2, 4), 3, 8), ((2, 2, 1, 1), 11, 7)])
+def test_transfers_with_short_sums(agg, nv, nsys):
+    """The forms for small aggregates, and the ones beside them."""
+    torch = torch_cuda()
+    L = (8, 4, 4, 4)
+    lat = Lattice(L, synth.gauge_field(L, 0.3, seed=3), 0.125, 1.0)
+    try:
+        T = lat.T
+        tv = synth.gaussian_spinors(L, nv, seed=5).astype(np.complex64)
+        p = T.setup_params(nv=nv, agg=agg, sap_block=(4, 2, 2, 2))
+        T.tmamg_setup_from_vectors(lat.ctx, p, torch.from_numpy(tv.view(np.float32).copy()).cuda())
+        Lc = tuple(L[d] // agg[d] for d in range(4))
+        Vc, nc = int(np.prod(Lc)), 2 * nv
+
+        def prolong(xc):
+            n = xc.shape[0]
+            cb = torch.from_numpy(coarse_to_bundle(xc, nc, Vc)).cuda()
+            fb = torch.full((T.tmamg_bundle_bytes(lat.ctx, n, 32) // 4,), 7.0, device="cuda")
+            T.tmamg_prolong(lat.ctx, 1, cb, fb, n)
+            return lat.from_fine_bundle(fb, n)
+
+        P = _dense(prolong, nc, Vc)
+        assert np.abs(P.conj().T @ P - np.eye(Vc * nc)).max() < TOL32
+        x = synth.gaussian_spinors(L, nsys, seed=6)
+        cb = lat.coarse_buffer(nsys)
+        T.tmamg_restrict(lat.ctx, 1, lat.fine_bundle(x), cb, nsys)
+        torch.cuda.synchronize()
+        got = coarse_from_bundle(cb.cpu().numpy(), nsys, nc, Vc)
+        want = (P.conj().T @ x.astype(np.complex64).reshape(nsys, -1).T).T.reshape(nsys, Vc, nc)
+        for n in range(nsys):
+            assert relerr(got[n], want[n]) <= TOL32, n
+        xc = synth.gaussian_coarse(Lc, nsys, nv, seed=9).reshape(nsys, Vc, nc)
+        up = prolong(xc).reshape(nsys, -1)
+        for n in range(nsys):
+            assert relerr(up[n], P @ xc[n].ravel()) <= TOL32, n
+    finally:
+        lat.close()
+
+
 @pytest.mark.parametrize("nsys", [1, 6, 19])
 def test_level_two_transfers_with_odd_k(nsys):
     torch = torch_cuda()
