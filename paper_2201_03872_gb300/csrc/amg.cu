@@ -352,7 +352,8 @@ static void launch_restrict_r(const AggDims& g, const float2* P, const float* r,
 // The same for short sums and few outputs, where the kernel above spends its time on filling its pipelines and on adding
 // its warps' sums. One CTA per (aggregate, chirality); the entries of a chunk of RH_KC values of k are staged for all
 // tiles; a thread owns 3 x 3 outputs (rows x tiles) and one of 16 interleaved slices of k, which are added by shuffles
-// in a fixed order. Two CTAs per SM (80 registers): one stages while the other computes.
+// in a fixed order. Two CTAs per SM (80 registers; with kc known to the compiler they spill): one stages while the other
+// computes.
 // 16^4, 2^4 aggregates (K = 96), the kernel above and this one, us: nv = 8, 1 system 65.5 and 30.7, 12 systems 158 and
 // 74; nv = 24, 6 systems 161 and 79, 16 systems 211 and 215; K = 192, nv = 8, 12 systems 96 and 69; K = 384, nv = 8,
 // 12 systems 68 and 64, 16 systems 68 and 113; 24^3x48, K = 1536, nv = 4, 1 system 234 and 153.
@@ -370,8 +371,7 @@ static bool restrict_short(int nv, int nt, int K, int asize) {
 
 __global__ void __launch_bounds__(RH_KS * RH_MAX_SLOTS, 2) restrict_short_kernel(const float2* __restrict__ P,
                                                               const float* __restrict__ r, float* __restrict__ xc,
-                                                              AggDims g, int nv, int d, int nt) {
-  constexpr int kc = RH_KC;
+                                                              AggDims g, int nv, int d, int nt, int kc) {
   extern __shared__ float4 rsm[];                             // [nt][kc] staged entries
   int* sidx = reinterpret_cast<int*>(rsm + (size_t)nt * kc);  // [asize] lattice site of each member
   const int64_t a = blockIdx.x >> 1;
@@ -467,7 +467,7 @@ static void launch_restrict_short(const AggDims& g, const float2* P, const float
   const int rounds = (nblk + RH_MAX_SLOTS - 1) / RH_MAX_SLOTS;
   const int slots = (nblk + rounds - 1) / rounds;
   const size_t smem = sizeof(float4) * (size_t)nt * RH_KC + sizeof(int) * g.asize;  // at most 40 KB
-  restrict_short_kernel<<<(unsigned)(g.Vc * 2), RH_KS * slots, smem, st>>>(P, r, xc, g, nv, d, nt);
+  restrict_short_kernel<<<(unsigned)(g.Vc * 2), RH_KS * slots, smem, st>>>(P, r, xc, g, nv, d, nt, RH_KC);
   TM_COUNT();
 }
 
