@@ -6,7 +6,7 @@
 // two FP64 lanes, so it ran at the FP64 issue rate (24^3x48 x 12 systems: 21.7 ms for 3.8 GB, 3% of the
 // HBM rate, against 13.1 ms if every FP64 slot were used). Here the products run as 32 x 32 -> 64-bit
 // integer multiply-adds (measured 59 lanes per cycle and SM on GB300, FP64 multiply-add 2.0), about 2600
-// of them and 8300 shifts, additions and logic operations per site and system: 5.24 ms for the same
+// of them and 8300 shifts, additions and logic operations per site and system: 5.12 ms for the same
 // case. It is bound by the integer pipes and their latency (multiply pipe 59% busy, issue 42%).
 //
 // Arithmetic. Block fixed point with one exponent S per (site, system): every contribution to the
@@ -29,8 +29,8 @@
 // one part has received less than 2^52 units is computed in FP64 arithmetic from its own terms
 // (fine_entry_f64; the whole site where there are more than five). The others are off by 2 units or so (45 if
 // every rounding went the same way): as FP64 sums of their terms. Gaussian fields have next to no such
-// components; the sums cost 4% (24^3x48 x 12 systems, 5.04 to 5.24 ms). A field with three of four spins zero
-// takes 21.2 ms (5.07 without this, 21.7 in FP64 arithmetic throughout).
+// components; the sums cost 1.5 to 4.5% (24^3x48, 12 systems 5.04 to 5.12 ms, 1 system 0.507 to 0.526). A field with
+// three of four spins zero takes 21.0 ms (5.07 without this, 21.7 in FP64 arithmetic throughout).
 //
 // A site whose spinors, links or masses are outside the range of this form (infinities and NaN, entries
 // beyond about 2^900 or below 2^-840, |mu| of the size of the clover block) is computed in FP64
@@ -347,7 +347,8 @@ __device__ __forceinline__ unsigned fx_mag(i64 re, i64 im) {
   return __byte_perm((unsigned)abs((int)(re >> 32)), (unsigned)abs((int)(im >> 32)), 0x7632);
 }
 constexpr unsigned FX_LEAST = 1u << 4;  // 2^52 units
-constexpr int FX_ENTRIES = 5;  // components computed one by one; the whole site does less than half the work for each
+// components computed one by one: the whole site does less for each (with 3, the field with one spin takes 23.6 ms)
+constexpr int FX_ENTRIES = 5;
 
 // raise the common exponent to at least `want` (the sums keep their value)
 __device__ __forceinline__ void fx_raise(i64 (&acc)[24], unsigned (&mag)[12], int& S, int want) {
@@ -554,9 +555,10 @@ __global__ void __launch_bounds__(MAXT, MINB) dirac64_kernel(FixedOp fx, const d
     // one copy of the code for both chiralities: the kernel has to fit the instruction cache
 #pragma unroll 1
     for (int chi = 0; chi < 2; ++chi) {
-      uint4 r[6];
+      uint4 r[6];  // loaded again: all twelve entries kept beside the sums spilled (24^3x48 x 12 systems 5.25 against 5.12 ms)
 #pragma unroll
-      for (int i = 0; i < 6; ++i) r[i] = chi == 0 ? raw.v[i] : raw.v[6 + i];
+      for (int i = 0; i < 6; ++i)
+        r[i] = *reinterpret_cast<const uint4*>(xt + (s + (int64_t)(6 * chi + i) * V) * 2);
       i64 o[12];
       fx_local(o, r, fx.C + (int64_t)chi * 36 * V + s, V, S - nC + 2 + 1026, fx_split(chi == 0 ? mq : -mq));
 #pragma unroll
@@ -685,7 +687,7 @@ __global__ void __launch_bounds__(MAXT, MINB) dirac64_kernel(FixedOp fx, const d
 }
 
 // launch variants: (sites per CTA row, largest CTA, CTAs per SM): 168 registers at 12 warps per SM, or 128
-// registers (some spills) at 16 warps per SM; measured on 24^3x48 x 12 systems 5.24 and 5.62 ms
+// registers (some spills) at 16 warps per SM; measured on 24^3x48 x 12 systems 5.12 and 5.54 ms
 template <bool RES, int BX, int MAXT, int MINB>
 static void launch_variant64(const Geom& g, const double2* U, const double* C, const double* x, double* y,
                              const double* mu, int nsys, const double* b, int nshift, const double* eps, int parity,
