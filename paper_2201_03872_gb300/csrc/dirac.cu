@@ -411,7 +411,7 @@ __global__ void __launch_bounds__(MAXT, MINB) dirac_kernel(const float2* __restr
 // It is then one or two load latencies long instead of eight: 8^3x16, one system, 9.0 -> 8.0 us with cold caches and
 // 10.3 -> 8.2 us per call of many; with four times the sites 20.5 us against 12.0, so it is a launch variant.
 constexpr int DS_WARPS = 12;
-constexpr int DS_TILES = 32768;  // tiles per layer of the grid, whose extent in y ends at 65535
+constexpr int DS_TILES = 65535;  // tiles per launch: the grid's extent in y
 
 template <int NU, bool FWD>
 __device__ __forceinline__ void split_hop(float4* g, const float2* __restrict__ U, const float* __restrict__ xt, int V,
@@ -459,8 +459,7 @@ __global__ void __launch_bounds__(DS_WARPS * 32, 2) dirac_split_kernel(
     const __grid_constant__ MassArgs ma, int nsys, int Lx, int Ly, int Lz, int Lt, float bc_t, const float* bsub) {
   __shared__ float4 gs[8 * 192];  // [hop][half spinor component][site]
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int V = Lx * Ly * Lz * Lt, tile = blockIdx.z * DS_TILES + blockIdx.y;
-  if (2 * tile >= nsys) return;  // (the whole block)
+  const int V = Lx * Ly * Lz * Lt, tile = blockIdx.y;
   const int s0 = blockIdx.x * 32 + lane;
   const bool live = s0 < V;
   const int s = live ? s0 : V - 1;
@@ -533,11 +532,19 @@ __global__ void __launch_bounds__(DS_WARPS * 32, 2) dirac_split_kernel(
 template <bool RES>
 static void launch_split(const Geom& g, const float2* U, const float* C, const float* x, float* y, const MassArgs& ma,
                          int nsys, const float* b, cudaStream_t st) {
-  const int nt = ntiles(nsys, 2);
-  const dim3 grid((unsigned)((g.V + 31) / 32), nt < DS_TILES ? nt : DS_TILES, (nt + DS_TILES - 1) / DS_TILES);
-  dirac_split_kernel<RES><<<grid, DS_WARPS * 32, 0, st>>>(
-      U, C, x, y, ma, nsys, g.L[0], g.L[1], g.L[2], g.L[3], (float)g.bc_t, b);
-  TM_COUNT();
+  MassArgs m = ma;
+  for (int t0 = 0, nt = ntiles(nsys, 2); t0 < nt; t0 += DS_TILES) {
+    const int n = nt - t0 < DS_TILES ? nt - t0 : DS_TILES;
+    dirac_split_kernel<RES><<<dim3((unsigned)((g.V + 31) / 32), n), DS_WARPS * 32, 0, st>>>(
+        U, C, x, y, m, nsys - 2 * t0, g.L[0], g.L[1], g.L[2], g.L[3], (float)g.bc_t, b);
+    TM_COUNT();
+    const int64_t step = (int64_t)n * 48 * g.V;
+    x += step;
+    y += step;
+    if (b) b += step;
+    if (m.mu) m.mu += 2 * n;  // (the masses in the arguments are those of at most 32 systems)
+    if (m.eps) m.eps += n;
+  }
 }
 
 // launch variants: (sites per CTA row, staged, largest CTA, CTAs per SM): 168 registers at 12 warps per SM,
