@@ -24,23 +24,25 @@ int tune_lookup(const char* family, int64_t key);
 int tune_run(const char* family, int64_t key, int nvar, const std::function<void(int)>& launch, cudaStream_t st);
 
 // the variant to use: the forced one, else the one tuned on first use when tuning is on; tuning (which
-// runs every variant on this call's data) only when `may_tune`, i.e. when the launch is repeatable. untuned: the
-// family's variant for this call where nothing was tuned
-inline int tune_variant(const char* family, int64_t key, int nvar, int untuned, bool may_tune,
-                        const std::function<void(int)>& launch, cudaStream_t st) {
+// runs every variant on this call's data) only when `may_tune`, i.e. when the launch is repeatable. untuned():
+// the family's variant for this call where nothing was tuned
+template <class Untuned>
+int tune_variant(const char* family, int64_t key, int nvar, Untuned untuned, bool may_tune,
+                 const std::function<void(int)>& launch, cudaStream_t st) {
   const int f = tune_forced();
   if (f >= 0) return f < nvar ? f : 0;
-  if (!autotune_on() || nvar < 2) return untuned;
+  if (!autotune_on() || nvar < 2) return untuned();
   const int v = tune_lookup(family, key);
   if (v >= 0) return v;
-  return may_tune ? tune_run(family, key, nvar, launch, st) : untuned;
+  return may_tune ? tune_run(family, key, nvar, launch, st) : untuned();
 }
 
 // the variant that a launch would use now without tuning first, or -1 if it would tune
-inline int tune_peek(const char* family, int64_t key, int nvar, int untuned) {
+template <class Untuned>
+int tune_peek(const char* family, int64_t key, int nvar, Untuned untuned) {
   const int f = tune_forced();
   if (f >= 0) return f < nvar ? f : 0;
-  return autotune_on() ? tune_lookup(family, key) : untuned;
+  return autotune_on() ? tune_lookup(family, key) : untuned();
 }
 
 // largest divisor of nt that keeps a CTA of bx x ty threads at <= maxthreads threads

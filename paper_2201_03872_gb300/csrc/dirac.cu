@@ -571,7 +571,7 @@ static int untuned_variant(const Geom& g, int nsys) {
   return nt == 1 || g.V * nt < 2ll * 384 * device_sms() ? DIRECT_VARIANT : 0;
 }
 static int peek_variant(const Geom& g, int nsys) {
-  return tune_peek("dirac_f32", tune_key(g, nsys), NVARIANTS, untuned_variant(g, nsys));
+  return tune_peek("dirac_f32", tune_key(g, nsys), NVARIANTS, [&] { return untuned_variant(g, nsys); });
 }
 
 template <bool RES>
@@ -593,7 +593,8 @@ static void launch_tuned(const char* family, bool may_tune, const Geom& g, const
       default: launch_variant<RES, 32, true, 192, 2>(g, U, C, x, y, mu, nsys, b, eps, st); return;
     }
   };
-  launch(tune_variant(family, tune_key(g, nsys), NVARIANTS, untuned_variant(g, nsys), may_tune, launch, st));
+  launch(tune_variant(family, tune_key(g, nsys), NVARIANTS, [&] { return untuned_variant(g, nsys); }, may_tune, launch,
+                      st));
 }
 
 bool dirac32_to_field(const Geom& g, int nsys) {

@@ -710,7 +710,7 @@ static void launch_tuned64(const char* family, bool may_tune, const Geom& g, con
       default: launch_variant64<RES, 32, 192, 2>(g, U, C, x, y, mu, nsys, b, nshift, eps, parity, st); return;
     }
   };
-  launch(tune_variant(family, g.V * 4096 + nsys, 2, 0, may_tune, launch, st));
+  launch(tune_variant(family, g.V * 4096 + nsys, 2, [] { return 0; }, may_tune, launch, st));
 }
 
 template <>
