@@ -495,6 +495,8 @@ def timed_solves(pb, sp, steps, stream, nrhs=None):
 
 FP32_ALU_PEAK_TFLOPS = 152 * 128 * 2 * 2.070e9 / 1e12   # 152 SMs x 128 FP32 lanes x FMA x 2070 MHz
 DIRAC_FLOP_PER_SITE_SYSTEM = 1896                         # hops 1320 + clover 2 x 252 + twist/diag 48 + combine 24
+WIDE_MAD_PEAK_T = 152 * 59 * 2.070e9 / 1e12
+DIRAC64_MAD_PER_SITE_SYSTEM = 2592                        # hops 8 x 216 + clover and twist 864
 
 
 def kernel_profile(pb, sp, stream):
@@ -517,7 +519,7 @@ def kernel_profile(pb, sp, stream):
 
 def kernel_rooflines(pb, rec, total_ms, stats):
     """Per-kernel time share of one profiled solve and, where an algorithmic count is defined, the
-    achieved rate against its peak (HBM copy bandwidth, FP32 or FP64 ALU rate)."""
+    achieved rate against its peak (HBM copy bandwidth, FP32 or integer rate)."""
     hbm, _, peak_src = read_peaks()
     V, N = pb.V, pb.nsys
     st = pb.wl["setup"]
@@ -532,10 +534,10 @@ def kernel_rooflines(pb, rec, total_ms, stats):
             b = dirac_bytes_per_site(N, 32) * V
             e.update(bound="hbm", algorithmic_bytes_per_launch=b, achieved=b / per / 1e9, peak=hbm, unit="GB/s")
         elif name == "residual_f64":
-            # runs on the integer pipes (block fixed point): against the bytes of the FP64 form, which reads
-            # the right-hand sides once each as well
-            b = (dirac_bytes_per_site(N, 64) + 192 * pb.nrhs) * V
-            e.update(bound="hbm", algorithmic_bytes_per_launch=b, achieved=b / per / 1e9, peak=hbm, unit="GB/s")
+            # block fixed point: bound by the integer pipes, of which the wide multiply-adds are counted
+            f = DIRAC64_MAD_PER_SITE_SYSTEM * V * N
+            e.update(bound="int", algorithmic_mads_per_launch=f, achieved=f / per / 1e12, peak=WIDE_MAD_PEAK_T,
+                     unit="Tmad/s", peak_source="152 SMs x 59 lanes (measured) of 32 x 32 + 64-bit multiply-add x 2070 MHz")
         elif name in ("restrict", "prolong"):
             # P (FP32 complex, 12 Nv per site) plus the fine vectors (FP32, 96 B per site and system)
             b = V * (12 * nv * 8 + 96 * N)
@@ -669,7 +671,7 @@ def dominant_roofline(kernels):
     r = {k: e[k] for k in ("bound", "achieved", "peak", "unit", "frac", "peak_source")}
     r.update(kernel=best, share_of_solve=e["share"], launches_in_solve=e["launches"], launch_ms=e["ms_per_launch"],
              traffic=e.get("traffic"))
-    for k in ("algorithmic_bytes_per_launch", "algorithmic_flops_per_launch"):
+    for k in ("algorithmic_bytes_per_launch", "algorithmic_flops_per_launch", "algorithmic_mads_per_launch"):
         if k in e:
             r[k] = e[k]
     return r

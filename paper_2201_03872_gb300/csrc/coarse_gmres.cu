@@ -74,7 +74,6 @@ struct CGArgs {
   int* kconv;
   int* active;
   int* done;      // converged (no restart needed)
-  int* nactive;   // [1]
   double2* part;  // [G][m + 2][2 lanes]
   float* hpart;   // [9][nt][nc][Vc][4] hop partials of the stencil
   unsigned* bar;  // [2]: count, generation
@@ -277,8 +276,8 @@ __device__ void cg_apply_sum(const CGArgs& p, const float* in, float* out, int t
 }
 
 // The warp's sums of N floats per thread (N a power of two up to 32): value k of the sums ends up in lane k's
-// return value (lanes k + N, ... hold it too). Halving exchanges the values not kept: 31 shuffles for 16 values
-// and 32 lanes instead of 80.
+// return value (lanes k + N, ... hold it too). Halving exchanges the values not kept: 16 shuffles for 16 values
+// instead of 80, 31 for 32 instead of 160.
 template <int N>
 __device__ __forceinline__ float warp_sums(const float (&v)[N], int lane) {
   float t[N];
@@ -678,7 +677,7 @@ __device__ __forceinline__ void cg_body(const CGArgs& p, CmShared& cs, float4* d
     cta_part(p, 1, 0, sm);
   }
   if (!grid_barrier(p)) return;
-  // norms sit in the real slot of each lane's partial (see cta_reduce_store)
+  // norms sit in the real slot of each lane's partial (see cta_part)
   if (gtid < p.nsys) {
     const int n = gtid;
     const double2 s = part_sum(p, 0, n);
@@ -834,7 +833,7 @@ __device__ __forceinline__ void cg_body(const CGArgs& p, CmShared& cs, float4* d
         nrm[0].y += w.y * w.y + w.w * w.w;
       }
       warp_part(nrm, 0, sm);
-    cta_part(p, 1, 0, sm);
+      cta_part(p, 1, 0, sm);
     }
     if (!grid_barrier(p)) return;
     if (gtid < p.nsys) {
@@ -892,7 +891,6 @@ int CoarseGmres::alloc(tmamg_ctx* ctx, int m_, int nsys_, int G_, size_t bundle_
   A((void**)&kconv, sizeof(int) * NS);
   A((void**)&active, sizeof(int) * NS);
   A((void**)&done, sizeof(int) * NS);
-  A((void**)&nactive, sizeof(int));
   A((void**)&part, sizeof(double2) * (size_t)G * (m + 2) * 2);
   A((void**)&bar, sizeof(unsigned) * 2);
   A((void**)&err, sizeof(int));
@@ -905,17 +903,17 @@ int CoarseGmres::alloc(tmamg_ctx* ctx, int m_, int nsys_, int G_, size_t bundle_
 }
 
 void CoarseGmres::release() {
-  void* ptrs[] = {H, cs, sn, g, y, tolabs, b0, sc, kconv, active, done, nactive, part, bar, err, iters, hpart, X16};
+  void* ptrs[] = {H, cs, sn, g, y, tolabs, b0, sc, kconv, active, done, part, bar, err, iters, hpart, X16};
   for (void* q : ptrs) cudaFree(q);
   if (h_flags) cudaFreeHost(h_flags);
   H = nullptr; cs = nullptr; sn = nullptr; g = nullptr; y = nullptr; tolabs = nullptr; b0 = nullptr; sc = nullptr;
-  kconv = nullptr; active = nullptr; done = nullptr; nactive = nullptr; part = nullptr; bar = nullptr;
+  kconv = nullptr; active = nullptr; done = nullptr; part = nullptr; bar = nullptr;
   err = nullptr; iters = nullptr; h_flags = nullptr; hpart = nullptr; X16 = nullptr;
   m = 0; NS = 0; G = 0; hbytes = 0; x16_bytes = 0;
 }
 
-// dynamic shared memory: back substitution, and the stencil phase (FP32 per-warp staging, or
-// the tensor-core operand buffers with nbuf operator copies)
+// dynamic shared memory: back substitution, reductions, and the stencil phase (FP32 per-warp staging, or the
+// tensor-core stencil's ring of nstage stages)
 static size_t dyn_smem_bytes(int m, int nc, int nsys, bool tc, int nstage) {
   const size_t rs = sizeof(double2) * (size_t)m * m;
   const size_t stage = tc ? cm_smem_bytes(nc, nsys, nstage) : sizeof(float4) * (size_t)(CG_THREADS / 32) * CG_WARP_F4;
@@ -989,7 +987,7 @@ int coarse_gmres_solve(CoarseGmres& s, const CoarseDims& cd, const float2* A, co
   p.maxiter = maxiter;
   p.tol = tol;
   p.H = s.H; p.cs = s.cs; p.sn = s.sn; p.g = s.g; p.y = s.y; p.tolabs = s.tolabs; p.sc = s.sc;
-  p.kconv = s.kconv; p.active = s.active; p.done = s.done; p.nactive = s.nactive; p.part = s.part;
+  p.kconv = s.kconv; p.active = s.active; p.done = s.done; p.part = s.part;
   p.bar = s.bar; p.err = s.err; p.iters = s.iters; p.hpart = s.hpart;
   p.wait_limit = g_wait_limit.load();
   p.extra = (unsigned)g_unreachable_next.exchange(0);

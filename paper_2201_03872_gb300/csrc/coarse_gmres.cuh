@@ -10,7 +10,7 @@ struct CoarseGmres {
   int m = 0, NS = 0, G = 0;
   double2 *H = nullptr, *sn = nullptr, *g = nullptr, *y = nullptr, *part = nullptr;
   double *cs = nullptr, *tolabs = nullptr, *b0 = nullptr, *sc = nullptr;
-  int *kconv = nullptr, *active = nullptr, *done = nullptr, *nactive = nullptr, *err = nullptr, *iters = nullptr;
+  int *kconv = nullptr, *active = nullptr, *done = nullptr, *err = nullptr, *iters = nullptr;
   unsigned* bar = nullptr;
   int* h_flags = nullptr;
   float* hpart = nullptr;  // 9 coarse bundles: hop partials of the stencil

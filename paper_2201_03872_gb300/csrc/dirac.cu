@@ -5,13 +5,11 @@
 // with A_chi = 1/(2 kappa) + c_sw C restricted to chirality chi (the operator of the
 // paper's Fig. 6 caption, D_TM = D_W + i mu gamma5, at delta mu = 1).
 //
-// Design: one thread per (site, tile of T systems). The gauge links and the
-// clover blocks of a site are loaded once per thread and applied to all T
-// systems of the tile; the T threads of one site that differ only in the tile
-// sit in the same CTA, so the re-reads of links and clover hit L1 (paper
-// Sec. 3: the matrix data is loaded once for all right-hand sides). Spin
-// projection in the chiral basis halves the SU(3) work: each hop multiplies
-// two colour vectors.
+// Design: one thread per (site, tile of two systems), a CTA holding 32 sites and several tiles. The links and the
+// clover blocks of the sites come to shared memory once per CTA and are applied to all its tiles (paper Sec. 3: the
+// matrix data is loaded once for all right-hand sides); with a single tile every thread loads them itself, and on small
+// lattices a site is split over twelve warps. Spin projection in the chiral basis halves the SU(3) work: each hop
+// multiplies two colour vectors. The FP64 form is in dirac64.cu.
 #include "autotune.cuh"
 #include "stencil.cuh"
 #include "profile.cuh"

@@ -30,7 +30,8 @@
 // (fine_entry_f64; the whole site where there are more than five). The others are off by 2 units or so (45 if
 // every rounding went the same way): as FP64 sums of their terms. Gaussian fields have next to no such
 // components; the sums cost 1.5 to 4.5% (24^3x48, 12 systems 5.04 to 5.12 ms, 1 system 0.507 to 0.526). A field with
-// three of four spins zero takes 21.0 ms (5.07 without this, 21.7 in FP64 arithmetic throughout).
+// three of four spins zero takes 21.0 ms (5.07 without this, 21.7 in FP64 arithmetic throughout); the residuals of a
+// point source's solution, whose colours and spins differ in size, 1.49 ms each on 16^3x32 x 12 systems (1.10 without).
 //
 // A site whose spinors, links or masses are outside the range of this form (infinities and NaN, entries
 // beyond about 2^900 or below 2^-840, |mu| of the size of the clover block) is computed in FP64
@@ -65,7 +66,8 @@ __device__ __forceinline__ int2 fx_limbs(double v, int n) {
 
 // the larger of two numbers that are not negative (a NaN of either sign counts as larger)
 __device__ __forceinline__ double fx_larger(double a, double b) {
-  const unsigned long long x = (unsigned long long)__double_as_longlong(a), y = (unsigned long long)__double_as_longlong(b);
+  const unsigned long long x = (unsigned long long)__double_as_longlong(a);
+  const unsigned long long y = (unsigned long long)__double_as_longlong(b);
   return __longlong_as_double((long long)(x > y ? x : y));
 }
 
@@ -555,7 +557,8 @@ __global__ void __launch_bounds__(MAXT, MINB) dirac64_kernel(FixedOp fx, const d
     // one copy of the code for both chiralities: the kernel has to fit the instruction cache
 #pragma unroll 1
     for (int chi = 0; chi < 2; ++chi) {
-      uint4 r[6];  // loaded again: all twelve entries kept beside the sums spilled (24^3x48 x 12 systems 5.25 against 5.12 ms)
+      // loaded again: all twelve entries kept beside the sums spilled (24^3x48 x 12 systems 5.25 against 5.12 ms)
+      uint4 r[6];
 #pragma unroll
       for (int i = 0; i < 6; ++i)
         r[i] = *reinterpret_cast<const uint4*>(xt + (s + (int64_t)(6 * chi + i) * V) * 2);

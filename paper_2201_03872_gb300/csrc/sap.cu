@@ -112,7 +112,7 @@ __device__ __forceinline__ void sap_cp_async_wait() {
 // packed FP32x2 arithmetic; CTA of ceil(bv / 32) * 32 threads (the threads past bv only take
 // part in the reductions and barriers).
 //
-// What bounds it: a 4^4 block fills the shared memory and, at 246 registers, the register file of an SM, so 8
+// What bounds it: a 4^4 block fills the shared memory and, at 248 registers, the register file of an SM, so 8
 // warps have to cover their own waits (34% of the issue slots used; spills would go to L2, the L1 being all
 // shared memory). Hence asynchronous staging, few loads of rho (the dot products are taken while the local
 // term holds it), a reduction of 15 shuffles, no load of e in the first cycle, and e on its way to L2 while
@@ -573,7 +573,7 @@ void sap_apply(const Geom& g, const int bs[4], const float2* U32, const float* C
       if (!last && d.pdim >= 0) {
         TM_PROF(st, "sap_face");
         const int64_t nsite = (int64_t)(nblocks / 2) * d.bv;  // sites of the blocks of the other colour
-sap_face_kernel<<<dim3((unsigned)((nsite + 127) / 128), nt), 128, 0, st>>>(U32, fresh ? e : delta, r, d,
+        sap_face_kernel<<<dim3((unsigned)((nsite + 127) / 128), nt), 128, 0, st>>>(U32, fresh ? e : delta, r, d,
                                                                                    1 - colour, nt);
         TM_COUNT();
       }

@@ -1,11 +1,10 @@
 // SAP smoother entry point that allocates no device memory.
 //
-// tmamg_sap allocates its scratch (the per-colour correction buffer) and may grow the
-// context's twisted-mass array on every call. Some callers cannot allow that: code that
-// runs while a CUDA stream is being captured into a graph (cudaMalloc is not a legal
-// operation there), code that must not touch the allocator once a memory budget has been
-// fixed, or code running under a memory pool it does not own. This file gives them a
-// variant whose scratch lives in file-scope device arrays of a fixed maximum size, which
+// tmamg_sap may grow the context's correction buffer and twisted-mass array, and waits for
+// the stream. Some callers cannot allow that: code that runs while a CUDA stream is being
+// captured into a graph (cudaMalloc is not a legal operation there), code that must not
+// touch the allocator once a memory budget has been fixed, or code running under a memory
+// pool it does not own. This file gives them a variant whose scratch lives in file-scope device arrays of a fixed maximum size, which
 // every GPU that loads the library holds until the process exits.
 #include <cstring>
 #include <mutex>
