@@ -114,11 +114,11 @@ def dirac_bytes_per_site(nsys, prec):
 # the same kernel on another volume is reported as the captured bytes times the volume ratio.
 # Valid only for the kernel sources the capture was taken on (SHA-1 of the files), else null.
 KERNEL_TRAFFIC = {
-    "dirac_f32": {"bytes": 1974231040 + 996510976, "L": (24, 24, 24, 48), "nsys": 16,
-                  "sha1": {"dirac.cu": "3518cd22c7b3457717bb9a2f27be1eeacde28a04",
+    "dirac_f32": {"bytes": 1977324288 + 996668160, "L": (24, 24, 24, 48), "nsys": 16,
+                  "sha1": {"dirac.cu": "046989ca82652c6e380938cb72d96520bb0a1f79",
                            "stencil.cuh": "76df2d28f1ae9c55ef0539b804f08d293db5940f"}},
-    "sap_mr": {"bytes": 2211575552 + 1500810240, "L": (24, 24, 24, 48), "nsys": 16,
-               "sha1": {"sap.cu": "0d16cf72354ebde8b86ec57456174d79eaed40f0",
+    "sap_mr": {"bytes": 2225249024 + 1500130560, "L": (24, 24, 24, 48), "nsys": 16,
+               "sha1": {"sap.cu": "1820f62864afafc32899b792c5e1b5a7d86d5807",
                         "stencil.cuh": "76df2d28f1ae9c55ef0539b804f08d293db5940f"}},
 }
 

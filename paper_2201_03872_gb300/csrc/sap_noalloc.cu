@@ -4,8 +4,9 @@
 // the stream. Some callers cannot allow that: code that runs while a CUDA stream is being
 // captured into a graph (cudaMalloc is not a legal operation there), code that must not
 // touch the allocator once a memory budget has been fixed, or code running under a memory
-// pool it does not own. This file gives them a variant whose scratch lives in file-scope device arrays of a fixed maximum size, which
-// every GPU that loads the library holds until the process exits.
+// pool it does not own. This file gives them a variant whose scratch lives in file-scope
+// device arrays of a fixed maximum size, which every GPU that loads the library holds until
+// the process exits.
 #include <cstring>
 #include <mutex>
 #include <string>
