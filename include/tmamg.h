@@ -349,8 +349,8 @@ int tmamg_coarse_solve(tmamg_ctx* ctx, int level, const void* rc_bundle, void* x
  * variants that compute identical results (the fine stencil and its residual forms: how the work is
  * split, CTA shape and register budget) time every variant on the first call for a lattice volume and system count,
  * with CUDA events on that call's stream, and use the fastest from then on (per device). The first
- * call of each shape therefore synchronises its stream once. on = 0 uses the default variant
- * everywhere. Every call clears the recorded choices. Always returns TMAMG_OK. */
+ * call of each shape therefore synchronises its stream once. on = 0 takes the
+ * variant that each family's rule on sizes gives. Every call clears the recorded choices. Always returns TMAMG_OK. */
 int tmamg_autotune(int on);
 
 /* Holds every tuned kernel family to launch variant `variant` (a family with fewer variants uses
