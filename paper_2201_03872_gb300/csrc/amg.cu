@@ -308,13 +308,16 @@ __global__ void __launch_bounds__(rs_warps(TG) * 32, 16 / rs_warps(TG)) restrict
   __syncthreads();
   for (int e = threadIdx.x; e < nv * ntc; e += blockDim.x) {
     const int j = e / ntc, t = e % ntc;
-    float4 s = rsm[j * TILES + t];
+    float4 v[WARPS];  // added in pairs: one after the other they were 2% less exact than the form with slices of k
 #pragma unroll
-    for (int w = 1; w < WARPS; ++w) {
-      const float4 v = rsm[(w * ROWS + j) * TILES + t];
-      s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
-    }
-    *reinterpret_cast<float4*>(xc + (((int64_t)(t0 + t) * (2 * nv) + chi * nv + j) * g.Vc + a) * 4) = s;
+    for (int w = 0; w < WARPS; ++w) v[w] = rsm[(w * ROWS + j) * TILES + t];
+#pragma unroll
+    for (int h = 1; h < WARPS; h *= 2)
+#pragma unroll
+      for (int w = 0; w < WARPS; w += 2 * h) {
+        v[w].x += v[w + h].x; v[w].y += v[w + h].y; v[w].z += v[w + h].z; v[w].w += v[w + h].w;
+      }
+    *reinterpret_cast<float4*>(xc + (((int64_t)(t0 + t) * (2 * nv) + chi * nv + j) * g.Vc + a) * 4) = v[0];
   }
 }
 
