@@ -359,17 +359,19 @@ static void launch_restrict_r(const AggDims& g, const float2* P, const float* r,
 // computes.
 // 16^4, 2^4 aggregates (K = 96), the kernel above and this one, us: nv = 8, 1 system 65.5 and 30.7, 12 systems 158 and
 // 74; nv = 24, 6 systems 161 and 79, 16 systems 211 and 215; K = 192, nv = 8, 12 systems 96 and 69; K = 384, nv = 8,
-// 12 systems 68 and 64, 16 systems 68 and 113; 24^3x48, K = 1536, nv = 4, 1 system 234 and 153.
+// 12 systems 68 and 64, 16 systems 68 and 113; 24^3x48, K = 1536, nv = 4, 1 system 234 and 153. It takes the CTAs of many
+// aggregates to hide one's chain: 32 aggregates, K = 192, 6 systems 6.1 and 10.4; 512, K = 1536, nv = 4, 6 systems 66 and
+// 138; 1024, K = 768, 82 and 80.
 constexpr int RH_KS = 16;         // k slices (lanes of a half warp)
 constexpr int RH_MAX_SLOTS = 24;  // output blocks processed at once per CTA (blockDim.x / RH_KS)
 constexpr int RH_KC = 128;        // k values staged per chunk
 constexpr int RH_MAXT = 12;       // tiles per call
 
-static bool restrict_short(int nv, int nt, int K, int asize) {
-  if (nt > RH_MAXT || asize > RS_TABLE) return false;
+static bool restrict_short(const AggDims& g, int nv, int nt, int K) {
+  if (nt > RH_MAXT || g.asize > RS_TABLE || g.Vc < device_sms()) return false;
   if (K <= 128) return nt <= 6 || nv <= 8;
   if (K <= 192) return nt <= 6;
-  return K <= 384 ? nv <= 8 && nt <= 6 : nv <= 4 && nt <= 3;
+  return K <= 384 ? nv <= 8 && nt <= 6 : nv <= 4 && nt <= 3 && g.Vc >= 6 * device_sms();
 }
 
 __global__ void __launch_bounds__(RH_KS * RH_MAX_SLOTS, 2) restrict_short_kernel(const float2* __restrict__ P,
@@ -478,7 +480,7 @@ void restrict_vec(const AggDims& g, const float2* P, const float* r, float* xc, 
                   cudaStream_t st) {
   const int nt = ntiles(nsys, T2);
   TM_PROF(st, d == 6 ? "restrict" : "restrict_coarse");
-  if (restrict_short(nv, nt, g.asize * d, g.asize)) {
+  if (restrict_short(g, nv, nt, g.asize * d)) {
     launch_restrict_short(g, P, r, xc, nv, d, nt, st);
     return;
   }
