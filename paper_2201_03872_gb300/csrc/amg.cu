@@ -152,7 +152,7 @@ void build_P(const AggDims& g, const float* Vb, float2* P, int nv, int d, cudaSt
 //  * Every tile of the call is in the CTA's registers (up to 40 systems): P and the vector are read once.
 //    The warps' partial sums are added in a fixed order at the end.
 // 24^3x48, nv = 24, 40 systems: 5.88 ms with 3 x 3 outputs per thread, 16 slices of k per half warp and the
-// vector staged behind CTA barriers in three rounds, 1.29 ms in this form (FP32 arithmetic alone
+// vector staged behind CTA barriers in three rounds, 1.28 ms in this form (FP32 arithmetic alone
 // 0.76 ms, the bytes 0.61 ms); 1 system 0.357 -> 0.30 ms (bytes 0.24 ms), 16 systems 1.31 -> 0.65 ms.
 // warps per CTA: 16 (one CTA per SM) when the lanes hold four tile groups, so that a warp sums at most 96
 // values of k at nv = 24, d = 6, 4^4 aggregates (8 warps and two CTAs: 1.24 against 1.29 ms, but sums twice
